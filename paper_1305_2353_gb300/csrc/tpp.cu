@@ -1,47 +1,55 @@
 // tpp.cu -- K4: threshold partial pivoting on the whole supernode (Listing 1,
 // Section 2), i.e. without compression: every test takes its column maxima over
 // all n rows, which must be up to date.  This is the comparator of the
-// compressed path.
+// compressed path, and the pivoting of a chain's or a root's last resort.
 //
-// GB300 design.  One cooperative, persistent launch (all CTAs co-resident) with
-// a software grid barrier whose spin is bounded.  Per accepted pivot:
-//   decide  CTA 0 runs the tests of Listing 1 on a full symmetric copy of A11
-//           (W11, p x p in the workspace) and on the column maxima of the
-//           trailing A21 (integer keys of |a|, one per column); rejected
-//           candidates change nothing, so it tests windows of 8 candidates (one
-//           warp each) and loops until it accepts a pivot or the sweep ends;
-//   update  every CTA applies that pivot to its share of all n rows (W11 rows
-//           and A21 rows, coalesced along the rows of each column), writes the
-//           L21 entries of the pivot column(s), and takes the new column maxima
-//           of A21 in the same pass.
-// So each accepted pivot costs one pass over the trailing A21 -- the traffic
-// the paper's compressed pivoting avoids (Section 6).  At the end the A21
-// columns are permuted into pivot order through shared memory and L11 / D /
-// the delayed block are written from W11, in the same layout as the compressed
-// path.  All grid barriers give up after a bounded number of polls; a timeout
-// sets CTP_ETIMEOUT in the info word and every CTA leaves the main loop.
+// GB300 design.  One cooperative, persistent launch (one CTA of 16 warps per SM
+// at most, all co-resident).  The rows of A21 are dealt out in contiguous runs,
+// one per CTA, held in shared memory when they fit (n p up to about 3.6 million
+// entries on 152 SMs) and streamed from memory otherwise; the elements of W11,
+// a full symmetric copy of A11, are dealt out one by one, each owned by one
+// thread, which keeps it in a register.  Per accepted pivot:
+//   barrier  one software grid barrier, its spin bounded;
+//   decide   every CTA runs the tests of Listing 1 itself, on W11 and the
+//            column maxima of the trailing A21 (integer keys of |a|) in L2:
+//            the inputs are the same, so is the outcome, and nothing has to be
+//            sent back (a decision by one CTA costs a second barrier per
+//            pivot).  Rejected candidates change nothing, so a window of up to
+//            16 candidates (one warp each) is tested per step; the window is one
+//            candidate after an acceptance and grows fourfold while all fail;
+//   update   every CTA applies the pivot to its rows of A21 (a warp per column,
+//            which leaves the column's new maximum in the warp: one atomicMax
+//            per column and CTA) and to its elements of W11, written to the other
+//            of two W11 buffers, since slower CTAs may still be reading this
+//            one; maxima are triple-buffered for the same reason.
+// What bounds a pivot at moderate n is latency: the barrier (an atomic and a poll
+// in L2), two dependent L2 reads of the tests and their FP64 chain; at large n
+// the pass over the trailing A21, the traffic that the paper's compressed
+// pivoting avoids (Section 6).  The column loop keeps four loads per lane in
+// flight.  Measured: 11.3 us per pivot at n = 20011, p = 127 (FP64 work 2 us) and
+// 9.1 us in the 256-wide panels of a dense system of order 1999; with one CTA
+// deciding, and a warp per 128 rows going through the columns one load at a
+// time, it was 62 and 105 us.
+// At the end the A21 columns are scaled and permuted into pivot order and
+// L11 / D / the delayed block are written from W11, in the same layout as the
+// compressed path.  A barrier that gives up sets the abort flag and
+// CTP_ETIMEOUT in the info word, and every CTA leaves the main loop.
 #include "ctp_internal.cuh"
+#include "pivot_tests.cuh"
 
 namespace ctp {
 
 namespace {
 
-constexpr int kT = 256;
+constexpr int kT = 512;
 constexpr int kNW = kT / 32;
-constexpr long kBarSpin = 1L << 24;  // default polls of ~100 ns: about a second and a half
-constexpr int kTilesPerWarp = 4;     // 32-row tiles a warp keeps pivot values for
-
-enum { D_STOP = -2, D_ZERO = -1, D_REJECT = 0, D_1X1 = 1, D_2X2 = 2 };
-
-struct Dec {
-    int kind, t, m, pad;
-    double d0, d1, d2, i0, i1, i2;
-};
+constexpr int kOwn = 8;              // elements of W11 a thread owns at most
+constexpr long kBarSpin = 1L << 22;  // default polls (an L2 round trip each): about two seconds
+constexpr size_t kTileBytes = 200 * 1024;  // shared memory for a CTA's rows of A21
 
 struct Ctl {
-    unsigned bar_count, bar_gen;
-    int abort, pad0;
-    Dec dec;
+    unsigned bar_count;
+    int abort;
 };
 
 struct TppArgs {
@@ -49,53 +57,42 @@ struct TppArgs {
     int64_t lda, n;
     int p;
     double u, small;
-    double *W11;                 // p x p, column c at W11 + c*p
-    unsigned long long *M21;     // [2][p] column-maximum keys of the trailing A21
-    int *live_g;                 // [p] live flags published by CTA 0
+    double *W11;                 // three p x p: two buffers by turns, then the pivots' frozen columns
+    unsigned long long *M21;     // [3][p] column-maximum keys of the trailing A21
     Ctl *ctl;
     int32_t *perm, *piv, *nelim;
     double *D, *Dinv;
     int32_t *info;
     long spin;                   // polls a grid barrier waits before it gives up
+    int64_t rows;                // A21 rows per CTA
 };
 
-__device__ __forceinline__ unsigned long long akey(double x) {
-    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-}
-__device__ __forceinline__ double key_val(unsigned long long k) { return __longlong_as_double((long long)k); }
-__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
-}
+struct Shared {
+    Decision res[kNW];
+    double sD[2 * kMaxP + 2], sInv[2 * kMaxP + 2];
+    double b0[kMaxP], b1[kMaxP], s0[kMaxP], s1[kMaxP];  // pivot column(s) on the A11 rows; times D^-1
+    int order[kMaxP], kind[kMaxP], pos_of[kMaxP];
+    unsigned char live[kMaxP];
+    unsigned short lcol[kMaxP];  // the live columns after the pivot at hand
+    int nlive, ok;
+};
 
-// software grid barrier for a cooperative launch; false on timeout (more than
-// `spin` polls) or when another CTA gave up
-__device__ bool grid_sync(Ctl *ctl, int *s_ok, long spin) {
+// Software grid barrier for a cooperative launch (arrivals are counted up, never
+// reset: the epoch's target is epoch * CTAs); false on timeout (more than
+// `spin` polls) or when another CTA gave up.
+__device__ __forceinline__ bool grid_sync(Ctl *ctl, unsigned target, int *s_ok, long spin) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned *genp = &ctl->bar_gen;
-        const unsigned gen = *genp;
         __threadfence();
-        const unsigned arrived = atomicAdd(&ctl->bar_count, 1u) + 1u;
+        unsigned seen = atomicAdd(&ctl->bar_count, 1u) + 1u;
         int ok = 1;
-        if (arrived == gridDim.x) {
-            ctl->bar_count = 0;
-            __threadfence();
-            atomicAdd(&ctl->bar_gen, 1u);
-        } else {
-            long it = 0;
-            while (*genp == gen) {
-                if (++it > spin) {
-                    ok = 0;
-                    atomicExch(&ctl->abort, 1);
-                    break;
-                }
-                __nanosleep(64);
+        for (long it = 0; (int)(seen - target) < 0; it++) {
+            if (it >= spin) {
+                ok = 0;
+                atomicExch(&ctl->abort, 1);
+                break;
             }
+            seen = *(volatile unsigned *)&ctl->bar_count;
         }
         __threadfence();
         *s_ok = ok && (*(volatile int *)&ctl->abort == 0);
@@ -104,482 +101,405 @@ __device__ bool grid_sync(Ctl *ctl, int *s_ok, long spin) {
     return *s_ok != 0;
 }
 
-// Listing 1's test_2x2 (readings Q3-Q5), explicitly rounded.
-__device__ __forceinline__ bool test_2x2(double a_tt, double a_tm, double a_mm, double maxt,
-                                         double maxm, double u, double small, Dec &d) {
-    double amax = fmax(fabs(a_tt), fmax(fabs(a_tm), fabs(a_mm)));
-    if (amax < small) return false;
-    double detscale = __ddiv_rn(1.0, amax);
-    double detpiv1 = __dmul_rn(__dmul_rn(a_tm, detscale), a_tm);
-    double detpiv0 = __dmul_rn(__dmul_rn(a_mm, detscale), a_tt);
-    double detpiv = __dsub_rn(detpiv0, detpiv1);
-    double guard = fmax(small, fmax(0.5 * fabs(detpiv0), 0.5 * fabs(detpiv1)));
-    if (fabs(detpiv) <= guard) return false;
-    bool ok;
-    if (fmax(maxm, maxt) < small) {
-        ok = true;
-    } else {
-        double ad = fabs(detpiv);
-        double gt = __ddiv_rn(__dmul_rn(__dadd_rn(__dmul_rn(fabs(a_mm), maxt), __dmul_rn(fabs(a_tm), maxm)), detscale), ad);
-        double gm = __ddiv_rn(__dmul_rn(__dadd_rn(__dmul_rn(fabs(a_tm), maxt), __dmul_rn(fabs(a_tt), maxm)), detscale), ad);
-        double iu = __ddiv_rn(1.0, u);
-        ok = (gt <= iu) && (gm <= iu);
-    }
-    if (ok) {
-        d.d0 = a_tt;
-        d.d1 = a_tm;
-        d.d2 = a_mm;
-        d.i0 = __ddiv_rn(__dmul_rn(a_mm, detscale), detpiv);
-        d.i1 = __ddiv_rn(__dmul_rn(-a_tm, detscale), detpiv);
-        d.i2 = __ddiv_rn(__dmul_rn(a_tt, detscale), detpiv);
-    }
-    return ok;
-}
-
-// Tests of Listing 1 for candidate c (one warp): the A11 part of every column
-// maximum comes from W11, the A21 part is the precomputed key M[c].
-__device__ Dec test_candidate(int c, const double *W11, const unsigned long long *M,
-                              const unsigned char *live, int p, double u, double small) {
+// Tests of Listing 1 for candidate c (one warp, p <= 256: eight entries of a column
+// per lane, loaded together): the A11 part of every column maximum comes from
+// W11, the A21 part is the key M[c].
+__device__ __forceinline__ Decision tpp_test(int c, const double *W, const unsigned long long *M,
+                                             const unsigned char *live, int p, double u, double rcp_u,
+                                             unsigned long long small_k) {
+    constexpr int NE = kMaxP / 32;
     const int lane = threadIdx.x & 31;
-    const double *cm = W11 + (size_t)c * p;
-    Dec d;
-    d.kind = D_REJECT;
+    const double *cm = W + (size_t)c * p;
+    Decision d;
+    d.kind = DEC_REJECT;
     d.t = -1;
     d.m = c;
     d.pad = 0;
     d.d0 = d.d1 = d.d2 = d.i0 = d.i1 = d.i2 = 0.0;
-    unsigned long long v = 0;
-    for (int i = lane; i < p; i += 32)
-        if (live[i]) {
-            const unsigned long long k = akey(__ldcg(cm + i));
-            v = k > v ? k : v;
-        }
-    v = warp_max_key(v);
-    const unsigned long long mc = M[c];
-    if (key_val(v > mc ? v : mc) < small) {
-        d.kind = D_ZERO;
-        return d;
+    unsigned long long km[NE];
+    bool lv[NE];
+#pragma unroll
+    for (int q = 0; q < NE; q++) {
+        const int i = lane + 32 * q;
+        lv[q] = i < p && live[i];
+        km[q] = i < p ? akey(__ldcg(cm + i)) : 0ull;
     }
+    const double amm = __ldcg(cm + c);
+    const unsigned long long mc = __ldcg(M + c);
+    // partner t: largest |a(c, j)| over live j < c, lowest j on ties
     unsigned long long bv = 0;
     int bi = -1;
-    for (int j = lane; j < c; j += 32)
-        if (live[j]) {
-            const unsigned long long k = akey(__ldcg(cm + j));
-            if (bi < 0 || k > bv) {
-                bv = k;
-                bi = j;
-            }
-        }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (oi >= 0 && (bi < 0 || ov > bv || (ov == bv && oi < bi))) {
-            bv = ov;
-            bi = oi;
+    for (int q = 0; q < NE; q++) {
+        const int i = lane + 32 * q;
+        if (lv[q] && i < c && (bi < 0 || km[q] > bv)) {
+            bv = km[q];
+            bi = i;
         }
     }
-    const int t = bi;
-    double maxm2 = 0.0;
+    const unsigned bh = bi >= 0 ? (unsigned)(bv >> 32) : 0u, bl = bi >= 0 ? (unsigned)bv : 0u;
+    const unsigned BH = __reduce_max_sync(0xffffffffu, bh);
+    const unsigned BL = __reduce_max_sync(0xffffffffu, bh == BH ? bl : 0u);
+    const int t0 = __reduce_min_sync(0xffffffffu, (bi >= 0 && bh == BH && bl == BL) ? bi : 0x7fffffff);
+    const int t = t0 == 0x7fffffff ? -1 : t0;
+    unsigned long long vt = 0, ktm = 0;
+    double att = 0.0, atm = 0.0;
     if (t >= 0) {
-        const double *ct = W11 + (size_t)t * p;
-        unsigned long long vm = 0, vt = 0;
-        for (int i = lane; i < p; i += 32)
-            if (live[i] && i != t && i != c) {
-                const unsigned long long km = akey(__ldcg(cm + i)), kt = akey(__ldcg(ct + i));
-                vm = km > vm ? km : vm;
-                vt = kt > vt ? kt : vt;
-            }
-        vm = warp_max_key(vm);
+        const double *ct = W + (size_t)t * p;
+        unsigned long long kt[NE];
+#pragma unroll
+        for (int q = 0; q < NE; q++) {
+            const int i = lane + 32 * q;
+            kt[q] = i < p ? akey(__ldcg(ct + i)) : 0ull;
+        }
+        att = __ldcg(ct + t);
+        atm = __ldcg(cm + t);
+        const unsigned long long mt = __ldcg(M + t);
+#pragma unroll
+        for (int q = 0; q < NE; q++) {
+            const int i = lane + 32 * q;
+            if (lv[q] && i != t && i != c) vt = kt[q] > vt ? kt[q] : vt;
+        }
         vt = warp_max_key(vt);
-        vm = vm > mc ? vm : mc;
-        vt = vt > M[t] ? vt : M[t];
-        maxm2 = key_val(vm);
-        if (test_2x2(__ldcg(ct + t), __ldcg(cm + t), __ldcg(cm + c), key_val(vt), maxm2, u, small, d)) {
-            d.kind = D_2X2;
+        vt = vt > mt ? vt : mt;
+        ktm = akey(atm);
+    }
+    unsigned long long vm = 0;
+#pragma unroll
+    for (int q = 0; q < NE; q++) {
+        const int i = lane + 32 * q;
+        if (lv[q] && i != t && i != c) vm = km[q] > vm ? km[q] : vm;
+    }
+    vm = warp_max_key(vm);
+    vm = vm > mc ? vm : mc;
+    const unsigned long long kmm = akey(amm);
+    unsigned long long vall = vm > kmm ? vm : kmm;
+    vall = ktm > vall ? ktm : vall;
+    if (vall < small_k) {
+        d.kind = DEC_ZERO;
+        return d;
+    }
+    unsigned long long maxm1 = vm;
+    if (t >= 0) {
+        if (test_2x2(att, atm, amm, vt, vm, rcp_u, small_k, d)) {
+            d.kind = DEC_2X2;
             d.t = t;
             return d;
         }
+        maxm1 = ktm > vm ? ktm : vm;
     }
-    double maxm1;
-    if (t >= 0) {
-        maxm1 = fmax(maxm2, fabs(__ldcg(cm + t)));
-    } else {
-        unsigned long long w = 0;
-        for (int i = lane; i < p; i += 32)
-            if (live[i] && i != c) {
-                const unsigned long long k = akey(__ldcg(cm + i));
-                w = k > w ? k : w;
-            }
-        w = warp_max_key(w);
-        maxm1 = key_val(w > mc ? w : mc);
-    }
-    const double amm = __ldcg(cm + c);
-    if (fabs(amm) >= __dmul_rn(u, maxm1)) {
-        d.kind = D_1X1;
+    const int f1 = test_1x1_f32(kmm, maxm1, u);
+    if (f1 == 1 || (f1 < 0 && kmm >= akey(__dmul_rn(u, key_val(maxm1))))) {
+        d.kind = DEC_1X1;
         d.d0 = amm;
-        d.i0 = __ddiv_rn(1.0, amm);
+        d.i0 = __drcp_rn(amm);
     }
     return d;
 }
 
-struct Cta0 {  // decision state, kept by CTA 0 across rounds
-    unsigned char live[kMaxP];
-    int order[kMaxP], kind[kMaxP];
-    double sD[2 * kMaxP + 2], sInv[2 * kMaxP + 2];
-    unsigned long long M[kMaxP];
-    int cand[kNW];
-    Dec res[kNW];
-    int nelim, m, accepted, hi, cstar;
-};
+// A pivot's update of this CTA's rows of A21: column k of the live list, entry
+// r: a(r,k) - x0(r) s0(k) - x1(r) s1(k), one fused multiply-add per term, with
+// x the pivot column(s) and s = D^-1 times the pivot row(s); the new maximum of
+// the column goes to Mn[k].
+template <bool k2x2>
+__device__ __forceinline__ void update_rows(double *T, int64_t ldt, int64_t rows, int q0, int q1, const Shared &sh,
+                                            unsigned long long *Mn) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double *x0 = T + q0 * ldt, *x1 = k2x2 ? T + q1 * ldt : x0;
+    for (int ci = warp; ci < sh.nlive; ci += kNW) {
+        const int k = sh.lcol[ci];
+        const double s0 = sh.s0[k], s1 = k2x2 ? sh.s1[k] : 0.0;
+        double *col = T + k * ldt;
+        unsigned long long mx = 0;
+        constexpr int U = 4;
+        for (int64_t r0 = lane; r0 < rows; r0 += 32 * U) {
+            double v[U], a[U], b[U];
+#pragma unroll
+            for (int q = 0; q < U; q++) {
+                const bool in = r0 + 32 * q < rows;
+                v[q] = in ? col[r0 + 32 * q] : 0.0;
+                a[q] = in ? x0[r0 + 32 * q] : 0.0;
+                b[q] = (k2x2 && in) ? x1[r0 + 32 * q] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < U; q++) {
+                if (r0 + 32 * q >= rows) break;
+                double w = fma(-a[q], s0, v[q]);
+                if (k2x2) w = fma(-b[q], s1, w);
+                col[r0 + 32 * q] = w;
+                const unsigned long long kk = akey(w);
+                mx = kk > mx ? kk : mx;
+            }
+        }
+        mx = warp_max_key(mx);
+        if (lane == 0 && mx) atomicMax(Mn + k, mx);
+    }
+}
 
-__global__ void __launch_bounds__(kT) k_tpp(TppArgs a) {
-    extern __shared__ __align__(16) double dsm[];
-    __shared__ Cta0 st;
-    __shared__ int s_ok;
-    __shared__ Dec s_dec;
+template <bool kSmem>
+__global__ void __launch_bounds__(kT, 1) k_tpp(TppArgs a) {
+    extern __shared__ __align__(16) double dsm[];  // kSmem: the CTA's rows [p][rows]; else staging [p][33]
+    __shared__ Shared sh;
     const int p = a.p;
     const int64_t n = a.n, m = n - p, lda = a.lda;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    unsigned long long *ckey = reinterpret_cast<unsigned long long *>(dsm);  // [p] column maxima
-    double *s0 = dsm + p, *s1 = s0 + p;                                       // [p] folded pivot row
-    unsigned char *live = reinterpret_cast<unsigned char *>(s1 + p);         // [p]
     Ctl *ctl = a.ctl;
+    const int64_t row0 = min((int64_t)blockIdx.x * a.rows, m), rows = min(a.rows, m - row0);
+    double *T = kSmem ? dsm : a.A + p + row0;
+    const int64_t ldt = kSmem ? a.rows : lda;
+    const int pp = p * p;
+    double *fin = a.W11 + 2 * (size_t)pp;
 
-    // ---- phase 0: W11 (full symmetric) and the initial column maxima of A21
-    for (int64_t idx = (int64_t)blockIdx.x * kT + tid; idx < (int64_t)p * p; idx += (int64_t)gridDim.x * kT) {
-        const int c = (int)(idx / p), i = (int)(idx % p);
-        a.W11[idx] = (i >= c) ? a.A[(int64_t)c * lda + i] : a.A[(int64_t)i * lda + c];
+    // ---- this thread's elements of W11 (full symmetric), this CTA's rows of A21
+    // and their initial column maxima
+    const int e0 = (int)blockIdx.x * kT + tid, estep = (int)gridDim.x * kT;
+    double own[kOwn];
+#pragma unroll
+    for (int j = 0; j < kOwn; j++) {
+        const int idx = e0 + j * estep;
+        own[j] = 0.0;
+        if (idx < pp) {
+            const int k = idx / p, i = idx - k * p;
+            own[j] = i >= k ? a.A[(int64_t)k * lda + i] : a.A[(int64_t)i * lda + k];
+            a.W11[idx] = own[j];
+        }
     }
-    for (int k = tid; k < p; k += kT) ckey[k] = 0;
-    __syncthreads();
     bool nonfinite = false;
-    {
-        const int64_t ntiles = (m + 31) / 32;
-        const int64_t gw = (int64_t)blockIdx.x * kNW + warp, nw = (int64_t)gridDim.x * kNW;
-        for (int k = 0; k < p; k++) {
-            unsigned long long mx = 0;
-            for (int64_t tl = gw; tl < ntiles; tl += nw) {
-                const int64_t r = tl * 32 + lane;
-                if (r < m) {
-                    const unsigned long long kk = akey(a.A[(int64_t)k * lda + p + r]);
-                    nonfinite |= kk >= 0x7FF0000000000000ull;
-                    mx = kk > mx ? kk : mx;
-                }
+    for (int k = warp; k < p; k += kNW) {
+        const double *src = a.A + (int64_t)k * lda + p + row0;
+        unsigned long long mx = 0;
+        for (int64_t r0 = lane; r0 < rows; r0 += 128) {
+            double v[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) v[q] = r0 + 32 * q < rows ? src[r0 + 32 * q] : 0.0;
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const unsigned long long kk = akey(v[q]);
+                nonfinite |= kk >= 0x7FF0000000000000ull;
+                mx = kk > mx ? kk : mx;
+                if (kSmem && r0 + 32 * q < rows) T[k * ldt + r0 + 32 * q] = v[q];
             }
-            mx = warp_max_key(mx);
-            if (lane == 0 && mx) atomicMax(&ckey[k], mx);
         }
+        mx = warp_max_key(mx);
+        if (lane == 0 && mx) atomicMax(a.M21 + k, mx);
     }
-    __syncthreads();
-    for (int k = tid; k < p; k += kT)
-        if (ckey[k]) atomicMax(&a.M21[k], ckey[k]);
     if (nonfinite) atomicCAS(a.info, kInfoOk, (int32_t)CTP_ENONFINITE);
-    if (blockIdx.x == 0) {
-        for (int i = tid; i < p; i += kT) {
-            st.live[i] = 1;
-            a.live_g[i] = 1;
-        }
-        if (tid == 0) {
-            st.nelim = 0;
-            st.m = p >= 2 ? 1 : 0;
-            st.accepted = 0;
-        }
-    }
-    int round = 0;
-    if (!grid_sync(ctl, &s_ok, a.spin)) goto done;
+    for (int i = tid; i < p; i += kT) sh.live[i] = 1;
 
-    for (;;) {
-        const int cur = round & 1, nxt = cur ^ 1;
-        // ---------------- decide (CTA 0)
-        if (blockIdx.x == 0) {
-            for (int k = tid; k < p; k += kT) {
-                st.M[k] = __ldcg(&a.M21[cur * p + k]);
-                a.M21[nxt * p + k] = 0;  // next maxima start from zero
+    const double u = a.u, rcp_u = __drcp_rn(a.u);
+    const unsigned long long small_k = akey(a.small);
+    int nelim = 0, c0 = p >= 2 ? 1 : 0, accepted = 0, win = 1, from = c0;
+    unsigned round = 0;
+    bool ok;
+    while ((ok = grid_sync(ctl, (round + 1) * gridDim.x, &sh.ok, a.spin))) {
+        const double *W = a.W11 + (size_t)(round & 1) * pp;
+        double *Wn = a.W11 + (size_t)((round & 1) ^ 1) * pp;
+        const unsigned long long *M = a.M21 + (round % 3) * p;
+        unsigned long long *Mn = a.M21 + ((round + 1) % 3) * p;
+        // ---------------- decide: the same steps and outcome in every CTA
+        bool stop = false;
+        Decision dv;
+        for (;;) {
+            if (nelim >= p) {
+                stop = true;
+                break;
             }
-            __syncthreads();
-            Dec out;
-            out.kind = D_STOP;
-            for (;;) {
-                // uniform control state read by all threads
-                int nl = st.nelim, mm = st.m;
-                if (nl >= p) break;
-                while (mm < p && !st.live[mm]) mm++;
-                if (mm >= p) {
-                    if (!st.accepted) break;
-                    __syncthreads();
-                    if (tid == 0) {
-                        st.accepted = 0;
-                        st.m = 0;
-                    }
-                    __syncthreads();
-                    continue;
-                }
-                if (tid == 0) {
-                    int k = 0, hi = p;
-                    for (int c = mm; c < p; c++) {
-                        if (!st.live[c]) continue;
-                        if (k < kNW)
-                            st.cand[k++] = c;
-                        else {
-                            hi = c;
-                            break;
-                        }
-                    }
-                    for (int w = k; w < kNW; w++) st.cand[w] = -1;
-                    st.hi = hi;
-                }
-                __syncthreads();
-                {
-                    const int c = st.cand[warp];
-                    if (c >= 0) {
-                        Dec d = test_candidate(c, a.W11, st.M, st.live, p, a.u, a.small);
-                        if (lane == 0) st.res[warp] = d;
-                    }
-                }
-                __syncthreads();
-                if (tid == 0) {
-                    int cs = -1;
-                    for (int w = 0; w < kNW; w++)
-                        if (st.cand[w] >= 0 && st.res[w].kind != D_REJECT) {
-                            cs = w;
-                            break;
-                        }
-                    st.cstar = cs;
-                    if (cs < 0) {
-                        st.m = st.hi;
-                    } else {
-                        const Dec d = st.res[cs];
-                        const int e = st.nelim;
-                        st.accepted = 1;
-                        st.m = d.m + 1;
-                        if (d.kind == D_ZERO) {
-                            st.live[d.m] = 0;
-                            st.order[e] = d.m;
-                            st.kind[e] = CTP_PIVKIND_ZERO;
-                            st.sD[2 * e] = st.sD[2 * e + 1] = 0.0;
-                            st.sInv[2 * e] = st.sInv[2 * e + 1] = 0.0;
-                            st.nelim = e + 1;
-                        } else if (d.kind == D_1X1) {
-                            st.live[d.m] = 0;
-                            st.order[e] = d.m;
-                            st.kind[e] = CTP_PIVKIND_1X1;
-                            st.sD[2 * e] = d.d0;
-                            st.sD[2 * e + 1] = 0.0;
-                            st.sInv[2 * e] = d.i0;
-                            st.sInv[2 * e + 1] = 0.0;
-                            st.nelim = e + 1;
-                        } else {
-                            st.live[d.t] = 0;
-                            st.live[d.m] = 0;
-                            st.order[e] = d.t;
-                            st.order[e + 1] = d.m;
-                            st.kind[e] = CTP_PIVKIND_2X2_FIRST;
-                            st.kind[e + 1] = CTP_PIVKIND_2X2_SECOND;
-                            st.sD[2 * e] = d.d0;
-                            st.sD[2 * e + 1] = d.d1;
-                            st.sD[2 * e + 2] = d.d2;
-                            st.sD[2 * e + 3] = 0.0;
-                            st.sInv[2 * e] = d.i0;
-                            st.sInv[2 * e + 1] = d.i1;
-                            st.sInv[2 * e + 2] = d.i2;
-                            st.sInv[2 * e + 3] = 0.0;
-                            st.nelim = e + 2;
-                        }
-                    }
-                }
-                __syncthreads();
-                const int cs = st.cstar;
-                if (cs >= 0 && st.res[cs].kind != D_ZERO) {
-                    out = st.res[cs];
+            while (c0 < p && !sh.live[c0]) c0++;
+            if (c0 >= p) {
+                if (!accepted) {  // a whole sweep without a pivot
+                    stop = true;
                     break;
                 }
+                accepted = 0;
+                c0 = from = 0;
+                continue;
             }
-            if (out.kind == D_STOP) {
-                // publish the pivot order: accepted pivots, then delayed columns in order
-                if (tid == 0) {
-                    int k = st.nelim;
-                    for (int c = 0; c < p; c++)
-                        if (st.live[c]) {
-                            st.order[k] = c;
-                            st.kind[k] = CTP_PIVKIND_DELAYED;
-                            st.sD[2 * k] = st.sD[2 * k + 1] = 0.0;
-                            st.sInv[2 * k] = st.sInv[2 * k + 1] = 0.0;
-                            k++;
-                        }
-                    *a.nelim = st.nelim;
+            const int hi = min(p, c0 + win);
+            {
+                const int c = c0 + warp;
+                int kind = DEC_REJECT;
+                if (c < hi && sh.live[c]) {
+                    const Decision d = tpp_test(c, W, M, sh.live, p, u, rcp_u, small_k);
+                    kind = d.kind;
+                    if (lane == 0) sh.res[warp] = d;
                 }
+                if (lane == 0 && kind == DEC_REJECT) sh.res[warp].kind = DEC_REJECT;
+            }
+            __syncthreads();
+            int w = 0;
+            while (w < hi - c0 && sh.res[w].kind == DEC_REJECT) w++;
+            if (w >= hi - c0) {
+                c0 = hi;
+                win = win * 4 < kNW ? win * 4 : kNW;
                 __syncthreads();
-                for (int k = tid; k < p; k += kT) {
-                    a.perm[k] = st.order[k];
-                    a.piv[k] = st.kind[k];
-                    a.D[2 * k] = st.sD[2 * k];
-                    a.D[2 * k + 1] = st.sD[2 * k + 1];
-                    a.Dinv[2 * k] = st.sInv[2 * k];
-                    a.Dinv[2 * k + 1] = st.sInv[2 * k + 1];
-                }
+                continue;
             }
-            for (int k = tid; k < p; k += kT) a.live_g[k] = st.live[k];
-            if (tid == 0) ctl->dec = out;
+            dv = sh.res[w];
+            // the next window: twice the distance that this search covered
+            const int gap = dv.m - from;
+            win = 1;
+            while (win < 2 * gap && win < kNW) win *= 2;
+            c0 = from = dv.m + 1;
+            accepted = 1;
+            __syncthreads();
+            if (dv.kind != DEC_ZERO) break;
+            if (tid == 0) {
+                sh.live[dv.m] = 0;
+                sh.order[nelim] = dv.m;
+                sh.kind[nelim] = CTP_PIVKIND_ZERO;
+                sh.sD[2 * nelim] = sh.sD[2 * nelim + 1] = 0.0;
+                sh.sInv[2 * nelim] = sh.sInv[2 * nelim + 1] = 0.0;
+            }
+            nelim++;
+            __syncthreads();
         }
-        if (!grid_sync(ctl, &s_ok, a.spin)) break;
+        if (stop) break;
+        // ---------------- the pivot's records, its column(s) and the live list
+        const bool two = dv.kind == DEC_2X2;
+        const int q0 = two ? dv.t : dv.m, q1 = two ? dv.m : -1;
         if (tid == 0) {
-            volatile Dec *vd = &ctl->dec;
-            s_dec.kind = vd->kind;
-            s_dec.t = vd->t;
-            s_dec.m = vd->m;
-            s_dec.i0 = vd->i0;
-            s_dec.i1 = vd->i1;
-            s_dec.i2 = vd->i2;
-        }
-        __syncthreads();
-        const Dec dv = s_dec;
-        if (dv.kind == D_STOP) break;
-
-        // ---------------- update: every row of [W11; A21] against the pivot
-        const int q0 = dv.kind == D_2X2 ? dv.t : dv.m;
-        const int q1 = dv.kind == D_2X2 ? dv.m : -1;
-        for (int k = tid; k < p; k += kT) {
-            live[k] = (unsigned char)__ldcg(&a.live_g[k]);
-            const double b0 = __ldcg(&a.W11[(size_t)q0 * p + k]);
-            if (q1 < 0) {
-                s0[k] = b0 * dv.i0;
-                s1[k] = 0.0;
-            } else {
-                const double b1 = __ldcg(&a.W11[(size_t)q1 * p + k]);
-                s0[k] = dv.i0 * b0 + dv.i1 * b1;
-                s1[k] = dv.i1 * b0 + dv.i2 * b1;
+            sh.order[nelim] = q0;
+            sh.kind[nelim] = two ? CTP_PIVKIND_2X2_FIRST : CTP_PIVKIND_1X1;
+            sh.sD[2 * nelim] = dv.d0;
+            sh.sD[2 * nelim + 1] = two ? dv.d1 : 0.0;
+            sh.sInv[2 * nelim] = dv.i0;
+            sh.sInv[2 * nelim + 1] = two ? dv.i1 : 0.0;
+            if (two) {
+                sh.order[nelim + 1] = q1;
+                sh.kind[nelim + 1] = CTP_PIVKIND_2X2_SECOND;
+                sh.sD[2 * nelim + 2] = dv.d2;
+                sh.sD[2 * nelim + 3] = 0.0;
+                sh.sInv[2 * nelim + 2] = dv.i2;
+                sh.sInv[2 * nelim + 3] = 0.0;
             }
-            ckey[k] = 0;
         }
-        __syncthreads();
-        {
-            // rows 0..p-1 are W11 rows, rows p..n-1 are A21 rows (A21 row r-p is
-            // at A + r); warp gw owns 32-row tiles gw, gw + nw, ...
-            const int64_t ntiles = (n + 31) / 32;
-            const int64_t gw = (int64_t)blockIdx.x * kNW + warp, nw = (int64_t)gridDim.x * kNW;
-            for (int64_t t0 = gw; t0 < ntiles; t0 += nw * kTilesPerWarp) {
-                double x0[kTilesPerWarp], x1[kTilesPerWarp];
-                bool act[kTilesPerWarp], isw[kTilesPerWarp];
-                int64_t rr[kTilesPerWarp];
-#pragma unroll
-                for (int q = 0; q < kTilesPerWarp; q++) {
-                    const int64_t r = (t0 + (int64_t)q * nw) * 32 + lane;
-                    rr[q] = r;
-                    isw[q] = r < p;
-                    act[q] = r < n && (r >= p || (live[r] && r != q0 && r != q1));
-                    x0[q] = x1[q] = 0.0;
-                    if (act[q]) {
-                        const double *src0 = isw[q] ? a.W11 + (size_t)q0 * p + r : a.A + (int64_t)q0 * lda + r;
-                        x0[q] = __ldcg(src0);
-                        if (q1 >= 0) {
-                            const double *src1 = isw[q] ? a.W11 + (size_t)q1 * p + r : a.A + (int64_t)q1 * lda + r;
-                            x1[q] = __ldcg(src1);
-                        }
-                    }
-                }
-                for (int k = 0; k < p; k++) {
-                    if (!live[k] || k == q0 || k == q1) continue;
-                    const double sk0 = s0[k], sk1 = s1[k];
-                    unsigned long long mx = 0;
-#pragma unroll
-                    for (int q = 0; q < kTilesPerWarp; q++) {
-                        if (!act[q]) continue;
-                        double *dst = isw[q] ? a.W11 + (size_t)k * p + rr[q] : a.A + (int64_t)k * lda + rr[q];
-                        const double v = __ldcg(dst) - (x0[q] * sk0 + x1[q] * sk1);
-                        *dst = v;
-                        if (!isw[q]) {
-                            const unsigned long long kk = akey(v);
-                            mx = kk > mx ? kk : mx;
-                        }
-                    }
-                    mx = warp_max_key(mx);
-                    if (lane == 0 && mx) atomicMax(&ckey[k], mx);
-                }
-                // L21 entries of the pivot column(s) in place (A21 rows only)
-#pragma unroll
-                for (int q = 0; q < kTilesPerWarp; q++) {
-                    if (!act[q] || isw[q]) continue;
-                    if (q1 < 0) {
-                        a.A[(int64_t)q0 * lda + rr[q]] = x0[q] * dv.i0;
-                    } else {
-                        a.A[(int64_t)q0 * lda + rr[q]] = x0[q] * dv.i0 + x1[q] * dv.i1;
-                        a.A[(int64_t)q1 * lda + rr[q]] = x0[q] * dv.i1 + x1[q] * dv.i2;
-                    }
+        if (warp == 0) {
+            int r = 0;
+            for (int j0 = 0; j0 < p; j0 += 32) {
+                const int j = j0 + lane;
+                const bool l = j < p && sh.live[j] && j != q0 && j != q1;
+                const unsigned bal = __ballot_sync(0xffffffffu, l);
+                if (l) sh.lcol[r + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)j;
+                if (j < p) sh.live[j] = l;
+                r += __popc(bal);
+            }
+            if (lane == 0) sh.nlive = r;
+        } else {
+            for (int k = tid - 32; k < p; k += kT - 32) {
+                const double x = __ldcg(W + (size_t)q0 * p + k);
+                sh.b0[k] = x;
+                if (!two) {
+                    sh.s0[k] = x * dv.i0;
+                } else {
+                    const double y = __ldcg(W + (size_t)q1 * p + k);
+                    sh.b1[k] = y;
+                    sh.s0[k] = dv.i0 * x + dv.i1 * y;
+                    sh.s1[k] = dv.i1 * x + dv.i2 * y;
                 }
             }
         }
+        if (blockIdx.x == 0)  // read last in the decision before this one
+            for (int k = tid; k < p; k += kT) a.M21[((round + 2) % 3) * p + k] = 0;
         __syncthreads();
-        for (int k = tid; k < p; k += kT)
-            if (ckey[k]) atomicMax(&a.M21[nxt * p + k], ckey[k]);
+        // ---------------- update: the own elements of W11 (an entry above the
+        // diagonal takes its mirror's operands, so W11 stays exactly symmetric;
+        // the pivot columns are frozen), then the own rows of A21
+#pragma unroll
+        for (int j = 0; j < kOwn; j++) {
+            const int idx = e0 + j * estep;
+            if (idx < pp) {
+                const int k = idx / p, i = idx - k * p;
+                if (k == q0 || k == q1) {
+                    fin[idx] = own[j];
+                } else if (sh.live[k] && sh.live[i]) {
+                    const int r = i > k ? i : k, c = i > k ? k : i;
+                    own[j] = fma(-sh.b0[r], sh.s0[c], own[j]);
+                    if (two) own[j] = fma(-sh.b1[r], sh.s1[c], own[j]);
+                    Wn[idx] = own[j];
+                }
+            }
+        }
+        if (two)
+            update_rows<true>(T, ldt, rows, q0, q1, sh, Mn);
+        else
+            update_rows<false>(T, ldt, rows, q0, q0, sh, Mn);
+        nelim += two ? 2 : 1;
         round++;
-        if (!grid_sync(ctl, &s_ok, a.spin)) break;
     }
-
-done:
-    if (*(volatile int *)&ctl->abort) {
+    if (!ok) {
         if (blockIdx.x == 0 && tid == 0) atomicCAS(a.info, kInfoOk, (int32_t)CTP_ETIMEOUT);
         return;
     }
-    // ---- output: A21 columns into pivot order (zero pivots give zero columns),
-    // then the A11 block from W11 (frozen pivot columns, delayed Schur block)
-    {
-        double *tile = dsm + 3 * p + (p + 64) / 8;  // [p][33]
-        int *sperm = reinterpret_cast<int *>(tile + (size_t)p * 33);
-        int *spiv = sperm + p;
+
+    // ---- the final order: accepted pivots, then the delayed columns in original order
+    if (tid == 0) {
+        int k = nelim;
+        for (int c = 0; c < p; c++)
+            if (sh.live[c]) {
+                sh.order[k] = c;
+                sh.kind[k] = CTP_PIVKIND_DELAYED;
+                sh.sD[2 * k] = sh.sD[2 * k + 1] = 0.0;
+                sh.sInv[2 * k] = sh.sInv[2 * k + 1] = 0.0;
+                k++;
+            }
+    }
+    __syncthreads();
+    for (int k = tid; k < p; k += kT) sh.pos_of[sh.order[k]] = k;
+    if (blockIdx.x == 0) {
         for (int k = tid; k < p; k += kT) {
-            sperm[k] = __ldcg(&a.perm[k]);
-            spiv[k] = __ldcg(&a.piv[k]);
+            a.perm[k] = sh.order[k];
+            a.piv[k] = sh.kind[k];
+            a.D[2 * k] = sh.sD[2 * k];
+            a.D[2 * k + 1] = sh.sD[2 * k + 1];
+            a.Dinv[2 * k] = sh.sInv[2 * k];
+            a.Dinv[2 * k + 1] = sh.sInv[2 * k + 1];
         }
-        __syncthreads();
-        const int64_t ntiles = (m + 31) / 32;
-        for (int64_t tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
-            const int64_t r = tl * 32 + lane;
-            for (int k = warp; k < p; k += kNW) tile[k * 33 + lane] = (r < m) ? __ldcg(a.A + (int64_t)k * lda + p + r) : 0.0;
+        if (tid == 0) *a.nelim = nelim;
+    }
+    __syncthreads();
+
+    // ---- output: A21 in pivot order, the pivots' columns times D^-1 (zero
+    // pivots give zero columns)
+    auto l21_entry = [&](const double *t, int64_t ld, int pos, int64_t r) -> double {
+        const int kd = sh.kind[pos];
+        const double x = t[sh.order[pos] * ld + r];
+        if (kd == CTP_PIVKIND_1X1) return x * sh.sInv[2 * pos];
+        if (kd == CTP_PIVKIND_2X2_FIRST)
+            return x * sh.sInv[2 * pos] + t[sh.order[pos + 1] * ld + r] * sh.sInv[2 * pos + 1];
+        if (kd == CTP_PIVKIND_2X2_SECOND)
+            return t[sh.order[pos - 1] * ld + r] * sh.sInv[2 * pos - 1] + x * sh.sInv[2 * pos];
+        return kd == CTP_PIVKIND_ZERO ? 0.0 : x;
+    };
+    if (kSmem) {
+        for (int pos = warp; pos < p; pos += kNW)
+            for (int64_t r = lane; r < rows; r += 32)
+                a.A[(int64_t)pos * lda + p + row0 + r] = l21_entry(T, ldt, pos, r);
+    } else {
+        for (int64_t t0 = 0; t0 < rows; t0 += 32) {
+            const int64_t r = t0 + lane;
+            for (int k = warp; k < p; k += kNW) dsm[k * 33 + lane] = r < rows ? T[k * lda + r] : 0.0;
             __syncthreads();
-            if (r < m)
-                for (int pos = warp; pos < p; pos += kNW)
-                    a.A[(int64_t)pos * lda + p + r] = spiv[pos] == CTP_PIVKIND_ZERO ? 0.0 : tile[sperm[pos] * 33 + lane];
+            if (r < rows)
+                for (int pos = warp; pos < p; pos += kNW) T[pos * lda + r] = l21_entry(dsm, 33, pos, lane);
             __syncthreads();
         }
     }
-    {
-        int *sperm = reinterpret_cast<int *>(dsm + 3 * p + (p + 64) / 8 + (size_t)p * 33);
-        int *spiv = sperm + p;
-        int *pos_of = spiv + p;
-        for (int k = tid; k < p; k += kT) pos_of[sperm[k]] = k;
-        __syncthreads();
-        for (int c = blockIdx.x; c < p; c += gridDim.x) {
-            const int pos = pos_of[c];
-            const int kd = spiv[pos];
-            const double *col = a.W11 + (size_t)c * p;
-            double *out = a.A + (int64_t)pos * lda;
+    // the A11 block from W11: frozen pivot columns, delayed Schur block
+    const double *Wd = a.W11 + (size_t)(round & 1) * pp;
+    for (int c = blockIdx.x; c < p; c += gridDim.x) {
+        const int pos = sh.pos_of[c], kd = sh.kind[pos];
+        double *out = a.A + (int64_t)pos * lda;
+        for (int i = tid; i < p; i += kT) {
+            const int pi = sh.pos_of[i];
             if (kd == CTP_PIVKIND_DELAYED) {
-                for (int i = tid; i < p; i += kT)
-                    if (pos_of[i] >= pos) out[pos_of[i]] = __ldcg(col + i);
+                if (pi >= pos) out[pi] = __ldcg(Wd + (size_t)c * p + i);
             } else if (kd == CTP_PIVKIND_ZERO) {
-                for (int i = tid; i < p; i += kT)
-                    if (pos_of[i] >= pos) out[pos_of[i]] = 0.0;
-            } else if (kd == CTP_PIVKIND_1X1) {
-                const double inv = __ldcg(&a.Dinv[2 * pos]);
-                for (int i = tid; i < p; i += kT)
-                    if (pos_of[i] > pos) out[pos_of[i]] = __ldcg(col + i) * inv;
-                if (tid == 0) out[pos] = __ldcg(&a.D[2 * pos]);
-            } else if (kd == CTP_PIVKIND_2X2_FIRST) {
-                const double *cmo = a.W11 + (size_t)sperm[pos + 1] * p;
-                const double i11 = __ldcg(&a.Dinv[2 * pos]), i21 = __ldcg(&a.Dinv[2 * pos + 1]);
-                for (int i = tid; i < p; i += kT)
-                    if (pos_of[i] > pos + 1) out[pos_of[i]] = __ldcg(col + i) * i11 + __ldcg(cmo + i) * i21;
-                if (tid == 0) {
-                    out[pos] = __ldcg(&a.D[2 * pos]);
-                    out[pos + 1] = __ldcg(&a.D[2 * pos + 1]);
-                }
+                if (pi >= pos) out[pi] = 0.0;
             } else {
-                const double *cto = a.W11 + (size_t)sperm[pos - 1] * p;
-                const double i21 = __ldcg(&a.Dinv[2 * (pos - 1) + 1]), i22 = __ldcg(&a.Dinv[2 * (pos - 1) + 2]);
-                for (int i = tid; i < p; i += kT)
-                    if (pos_of[i] > pos) out[pos_of[i]] = __ldcg(cto + i) * i21 + __ldcg(col + i) * i22;
-                if (tid == 0) out[pos] = __ldcg(&a.D[2 * pos]);
+                const bool first = kd == CTP_PIVKIND_2X2_FIRST;
+                if (pi > (first ? pos + 1 : pos)) out[pi] = l21_entry(fin, p, pos, i);
+                if (pi == pos) out[pi] = sh.sD[2 * pos];
+                if (first && pi == pos + 1) out[pi] = sh.sD[2 * pos + 1];
             }
         }
     }
@@ -588,13 +508,7 @@ done:
 }  // namespace
 
 size_t tpp_ws_bytes(int p) {
-    return 256 + align256(sizeof(double) * (size_t)p * p) + align256(2 * sizeof(unsigned long long) * (size_t)p) +
-           align256(sizeof(int) * (size_t)p);
-}
-
-static size_t tpp_smem(int p) {
-    // ckey, s0, s1 (3p doubles), live (p bytes, padded), tile [p][33], perm/piv/pos_of
-    return sizeof(double) * (3 * (size_t)p + (p + 64) / 8 + (size_t)p * 33) + 3 * sizeof(int) * (size_t)p;
+    return 256 + align256(3 * sizeof(double) * (size_t)p * p) + align256(3 * sizeof(unsigned long long) * (size_t)p);
 }
 
 cudaError_t launch_tpp(double *A, int64_t n, int p, int64_t lda, double u, double small, void *ws,
@@ -611,9 +525,7 @@ cudaError_t launch_tpp(double *A, int64_t n, int p, int64_t lda, double u, doubl
     a.small = small;
     a.ctl = reinterpret_cast<Ctl *>(w);
     a.W11 = reinterpret_cast<double *>(w + 256);
-    a.M21 = reinterpret_cast<unsigned long long *>(w + 256 + align256(sizeof(double) * (size_t)p * p));
-    a.live_g = reinterpret_cast<int *>(reinterpret_cast<char *>(a.M21) +
-                                       align256(2 * sizeof(unsigned long long) * (size_t)p));
+    a.M21 = reinterpret_cast<unsigned long long *>(w + 256 + align256(3 * sizeof(double) * (size_t)p * p));
     a.perm = perm;
     a.piv = piv;
     a.nelim = nelim;
@@ -622,19 +534,25 @@ cudaError_t launch_tpp(double *A, int64_t n, int p, int64_t lda, double u, doubl
     a.info = info;
     cudaError_t err = cudaMemsetAsync(w, 0, 256, st);
     if (err != cudaSuccess) return err;
-    err = cudaMemsetAsync(a.M21, 0, 2 * sizeof(unsigned long long) * (size_t)p, st);
+    err = cudaMemsetAsync(a.M21, 0, 3 * sizeof(unsigned long long) * (size_t)p, st);
     if (err != cudaSuccess) return err;
-    const size_t smem = tpp_smem(p);
-    err = smem_at_least((const void *)k_tpp, smem);
+    // CTAs: 32 rows of A21 each (a warp's width) until the SMs run out -- fewer
+    // CTAs make the barrier cheaper -- and no more than four elements of W11 per thread
+    const int64_t m = n - p;
+    int64_t G = (m + 31) / 32;
+    const int64_t gw = ((int64_t)p * p + 4 * kT - 1) / (4 * kT);
+    if (G < gw) G = gw;
+    if (G > num_sms) G = num_sms;
+    if (G * kT * kOwn < (int64_t)p * p) return cudaErrorLaunchOutOfResources;  // fewer than 16 SMs
+    a.rows = (m + G - 1) / G;
+    const size_t tile = sizeof(double) * (size_t)p * (size_t)a.rows;
+    const bool in_smem = tile <= kTileBytes;
+    const size_t smem = in_smem ? (tile > 0 ? tile : 16) : sizeof(double) * (size_t)p * 33;
+    const void *fn = in_smem ? (const void *)k_tpp<true> : (const void *)k_tpp<false>;
+    err = smem_at_least(fn, smem);
     if (err != cudaSuccess) return err;
-    int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tpp, kT, smem);
-    if (err != cudaSuccess) return err;
-    if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-    if (per_sm > 2) per_sm = 2;
-    dim3 grid(num_sms * per_sm), block(kT);
     void *args[] = {&a};
-    return cudaLaunchCooperativeKernel((void *)k_tpp, grid, block, args, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)G), dim3(kT), args, smem, st);
 }
 
 }  // namespace ctp
