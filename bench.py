@@ -53,10 +53,6 @@ MEASURED = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # number of S entries; the Solve's is proportional to the rows of A21): see
 # profiles/ for the captures.
 NCU_TRAFFIC = {
-    # ncu --set full, n=20000 p=256 relaxed, S FP64 lower-packed: 163.66 MB read +
-    # 1512.10 MB written for m(m+1)/2 = 194,921,640 entries
-    "form_fp64": {"file": "form.cu", "sha1": "bed329d47e2e3d13657366883dcf61b1968adf7a",
-                  "unit": "packed_entry", "bytes_per_unit": (163.662592e6 + 1512.099e6) / 194921640},
     # ncu --set full, n=40000 p=256 relaxed, split BF16 on SM pairs, S FP32 in 128x128
     # blocks: 89.63 MB read + 3118.79 MB written for 48,516 blocks of 16,384 entries
     "form_tc_bf16x3": {"file": "form_tc.cu", "sha1": "488eb8cb39a135fe2b96ff90b589d43a008cdf37",
@@ -342,9 +338,20 @@ def kernel_roofline(name, launches, ms, a, e, peaks, prec="fp64"):
         out["traffic"] = ncu_traffic(name, m, prec)
         out["launch_ms"] = ms / launches
         return out
-    elif name in ("form_fp64", "solve_fp64"):
-        fs, form = flops_model(n, p, e)
-        work = form if name == "form_fp64" else fs
+    elif name == "form_fp64":
+        # exact digit slices on the BF16 tensor cores: 36 products of slices per
+        # product of the method; S (8 bytes an entry) is the algorithmic traffic
+        _, form = flops_model(n, p, e)
+        tensor = 36 * form / t / 1e12
+        hbm = (8.0 * m * (m + 1) / 2 + 2 * 16.0 * m * ((e + 31) // 32 * 32)) / t / 1e9
+        return {"kernel": name, "bound": "tensor", "achieved": tensor, "peak": peaks["bf16_tflops"],
+                "unit": "TFLOP/s", "frac": tensor / peaks["bf16_tflops"],
+                "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst)", "work_per_launch": 36 * form,
+                "products_per_flop": 36, "method_tflops": tensor / 36, "hbm_gbs": hbm,
+                "hbm_frac": hbm / peaks["hbm_gbs"], "traffic": ncu_traffic(name, m, prec),
+                "launch_ms": ms / launches}
+    elif name == "solve_fp64":
+        work, _ = flops_model(n, p, e)
         bound, unit, peak = "alu", "TFLOP/s", peaks["fp64_tflops"]
         src = "measured in this run: torch.matmul float64 6144^3, best of 10"
         achieved = work / t / 1e12

@@ -16,7 +16,7 @@ const char *kKernelNames[K_NUM_IDS] = {"compress_strict", "keys_to_rowmajor", "c
                                        "tpp_full_column", "batch_prepare", "batch_compress_strict",
                                        "batch_factor_cta", "batch_factor_g2", "batch_factor_g4",
                                        "batch_factor_g8", "batch_factor_g16", "batch_solve_fp64",
-                                       "batch_form", "w21_from_l", "sys_forward", "sys_backward",
+                                       "batch_form", "slices_from_l", "sys_forward", "sys_backward",
                                        "symv_residual", "backward_error", "axpy", "form_tc_bf16x3",
                                        "sym_grad", "mf_assemble", "mf_extend_add", "spmv_residual",
                                        "form_tc_bf16x6", "solve_tc", "batch_factor_warp"};
@@ -49,8 +49,15 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     L.Dinv = off;
     off += align256(sizeof(double) * (2 * (size_t)p + 2));
     const bool tc = opt->prec != CTP_FP64 && opt->smode != CTP_S_NONE;
-    L.W21 = off;
-    off += align256(opt->smode != CTP_S_NONE && !tc ? sizeof(double) * (size_t)m * p : 0);
+    const int64_t ms = opt->smode != CTP_S_NONE && !tc ? m : 0;  // digit slices of the FP64 Form
+    L.Ws = off;
+    off += align256(slice_w_bytes(ms, p));
+    L.Ls = off;
+    off += align256(slice_l_bytes(ms, p));
+    L.ew = off;
+    off += align256(sizeof(int32_t) * (size_t)ms);
+    L.el = off;
+    off += align256(sizeof(int32_t) * (size_t)ms);
     // BF16 operand copies (hi, and for the split form the lo parts after them)
     const size_t nb = tc ? 2 * (size_t)m * form_tc_kpad(p) * prec_pieces(opt->prec) : 0;
     L.Wb = off;
@@ -247,7 +254,10 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
     char *ws = (char *)workspace;
     int32_t *info = (int32_t *)(ws + L.info);
     double *Dinv = (double *)(ws + L.Dinv);
-    double *W21 = (opt->smode != CTP_S_NONE && !tc) ? (double *)(ws + L.W21) : nullptr;
+    SliceBuf sb = {nullptr, nullptr, nullptr, nullptr, 0};
+    if (opt->smode != CTP_S_NONE && !tc)
+        sb = {(unsigned char *)(ws + L.Ws), (unsigned char *)(ws + L.Ls), (int32_t *)(ws + L.ew),
+              (int32_t *)(ws + L.el), slice_kb(p)};
     void *Wb = tc ? (void *)(ws + L.Wb) : nullptr;
     void *Lbf = tc ? (void *)(ws + L.Lb) : nullptr;
     const int Kp = form_tc_kpad(p);
@@ -263,10 +273,11 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
         }));
         if (opt->smode != CTP_S_NONE && m > 0) {
             CTP_CUDA(timed(ctx, K_W21, st, [&] {
-                return launch_w21_from_l(A, lda, p, m, piv, D, nelim, W21, m, st);
+                return launch_slices_from_l(A, lda, p, m, piv, D, Dinv, nelim, sb, st);
             }));
             CTP_CUDA(timed(ctx, K_FORM, st, [&] {
-                return launch_form_fp64(A + p, lda, W21, m, m, nelim, S, lds, opt->smode, st);
+                return launch_form_fp64(sb, A + p, lda, piv, D, m, nelim, S, lds, opt->smode, info, ctx->num_sms,
+                                        st);
             }));
         }
         return CTP_OK;
@@ -328,8 +339,7 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
         }));
     else if (m > 0)
         CTP_CUDA(timed(ctx, K_SOLVE, st, [&] {
-            return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, W21, m, Wb, Lbf, Kp, lo_off, pieces,
-                                     st);
+            return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, sb, Wb, Lbf, Kp, lo_off, pieces, st);
         }));
     if (opt->smode != CTP_S_NONE && m > 0) {
         if (tc)
@@ -341,7 +351,8 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
             }));
         else
             CTP_CUDA(timed(ctx, K_FORM, st, [&] {
-                return launch_form_fp64(A + p, lda, W21, m, m, nelim, S, lds, opt->smode, st);
+                return launch_form_fp64(sb, A + p, lda, piv, D, m, nelim, S, lds, opt->smode, info, ctx->num_sms,
+                                        st);
             }));
     }
     return CTP_OK;

@@ -591,7 +591,8 @@ cudaError_t batch_form_class(const ctp_plan *P, int ci, const ctp_front *fr, cha
         return launch_form_tc_batch(fr, tab, fitem, c.f_count, P->total_rows, w + P->off_wb, w + P->off_lb,
                                     P->bo.pieces, P->opt.smode == CTP_S_FP64_SUB ? 3 : 2,
                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st, ftile);
-    return launch_form_fp64_batch(fr, tab, w, fitem, c.f_count, P->bo, st, ftile);
+    return launch_form_fp64_batch(fr, tab, w, fitem, c.f_count, P->bo,
+                                  reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st, ftile);
 }
 cudaError_t batch_form(const ctp_plan *P, const ctp_front *fr, char *w, int num_sms, cudaStream_t st) {
     if (P->opt.smode == CTP_S_NONE) return cudaSuccess;
@@ -601,7 +602,8 @@ cudaError_t batch_form(const ctp_plan *P, const ctp_front *fr, char *w, int num_
         return launch_form_tc_batch(fr, tab, fitem, P->f_items, P->total_rows, w + P->off_wb, w + P->off_lb,
                                     P->bo.pieces, P->opt.smode == CTP_S_FP64_SUB ? 3 : 2,
                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
-    return launch_form_fp64_batch(fr, tab, w, fitem, P->f_items, P->bo, st);
+    return launch_form_fp64_batch(fr, tab, w, fitem, P->f_items, P->bo,
+                                  reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
 }
 
 }  // namespace ctp

@@ -15,15 +15,39 @@ constexpr int kMaxP = 256;
 // Device info word codes (first int32 of the workspace).
 constexpr int kInfoOk = 0;
 
+// Digit slices of the FP64 Form's operands (slices.cuh).
+constexpr int kSlices = 8;
+constexpr int kSliceK = 32;                       // pivots per K block
+constexpr int kWRows = 128, kLRows = 64;          // rows per block
+constexpr uint32_t kWSlice = kWRows * 64, kLSlice = kLRows * 64;  // bytes of one slice of one K block
+constexpr uint32_t kWBlock = kSlices * kWSlice, kLBlock = kSlices * kLSlice;
+constexpr int kExpZero = -100000, kExpNonfinite = 1 << 20, kExpWide = 1 << 24;
+
+// Where a supernode's slices live: blocks at (row block * kb + K block), the
+// rows' exponents E; kb = ceil(p / 32).
+struct SliceBuf {
+    unsigned char *W, *L;
+    int32_t *ew, *el;
+    int kb;
+};
+__host__ __device__ inline int slice_kb(int p) { return (p + kSliceK - 1) / kSliceK; }
+__host__ __device__ inline size_t slice_w_bytes(int64_t m, int p) {
+    return (size_t)((m + kWRows - 1) / kWRows) * slice_kb(p) * kWBlock;
+}
+__host__ __device__ inline size_t slice_l_bytes(int64_t m, int p) {
+    return (size_t)((m + kLRows - 1) / kLRows) * slice_kb(p) * kLBlock;
+}
+
 // Workspace layout (all offsets 256-byte aligned):
 //   [0, 256)            info word + scratch counters
 //   C                   p*p doubles, row-major compressed matrix (strict: as uint64 keys)
 //   Dinv                2p doubles: inverse pivot blocks, same slots as D
-//   W21                 m*p doubles (FP64 Y = L21 D11) when the FP64 Form step runs
+//   Ws, Ls, ew, el      digit slices of Y = L21 D11 and L21 and their row exponents
+//                       (slices.cuh) when the FP64 Form step runs
 //   Wb, Lb              m*Kp BF16 copies of Y and L21 for the tensor-core Form
 //   aux                 method-specific scratch (relaxed candidate lists)
 struct WsLayout {
-    size_t info, C, Dinv, W21, Wb, Lb, aux, Xs, flags, total;
+    size_t info, C, Dinv, Ws, Ls, ew, el, Wb, Lb, aux, Xs, flags, total;
 };
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -98,9 +122,9 @@ struct BFront {
     int32_t kbx, nwz;
 };
 // offsets inside a front's section: info word, compressed matrix (strict),
-// Dinv, and W21 = L21 D11 when an FP64 Form follows
+// Dinv, and the digit slices of L21 D11 and L21 when an FP64 Form follows
 struct BSection {
-    size_t info, C, Dinv, W21, nz, total;
+    size_t info, C, Dinv, Ws, Ls, ew, el, nz, total;
 };
 __host__ __device__ inline size_t align256hd(size_t x) { return (x + 255) & ~size_t(255); }
 __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options *opt) {
@@ -112,12 +136,29 @@ __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options
     off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(double) * (size_t)p * p : 0);
     s.Dinv = off;
     off += align256hd(sizeof(double) * (2 * (size_t)p + 2));
-    s.W21 = off;
-    off += align256hd((opt->smode != CTP_S_NONE && opt->prec == CTP_FP64) ? sizeof(double) * (size_t)(n - p) * p : 0);
+    const int64_t ms = opt->smode != CTP_S_NONE && opt->prec == CTP_FP64 ? n - p : 0;
+    s.Ws = off;
+    off += align256hd(slice_w_bytes(ms, p));
+    s.Ls = off;
+    off += align256hd(slice_l_bytes(ms, p));
+    s.ew = off;
+    off += align256hd(sizeof(int32_t) * (size_t)ms);
+    s.el = off;
+    off += align256hd(sizeof(int32_t) * (size_t)ms);
     s.nz = off;  // strict: which rows of C receive an A21 row (one bit per row)
     off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
     s.total = off;
     return s;
+}
+
+__host__ __device__ inline SliceBuf bsection_slices(char *base, const BSection &s, int p) {
+    SliceBuf b;
+    b.W = reinterpret_cast<unsigned char *>(base + s.Ws);
+    b.L = reinterpret_cast<unsigned char *>(base + s.Ls);
+    b.ew = reinterpret_cast<int32_t *>(base + s.ew);
+    b.el = reinterpret_cast<int32_t *>(base + s.el);
+    b.kb = slice_kb(p);
+    return b;
 }
 
 struct BatchOpts {
@@ -147,7 +188,7 @@ cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char 
 // item_tile (optional, both batched Forms): each item's tile of its front;
 // without it the items of a front are consecutive, from tab[front].f0 on
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                                   const int *item_front, int64_t items, BatchOpts o,
+                                   const int *item_front, int64_t items, BatchOpts o, int32_t *info, int num_sms,
                                    cudaStream_t st, const int *item_tile = nullptr);
 cudaError_t launch_form_tc_batch(const ctp_front *fronts, const BFront *tab, const int *item_front,
                                  int64_t items, int64_t total_rows, const void *Wb, const void *Lb,
@@ -196,8 +237,8 @@ cudaError_t launch_solve_tc_batch(const ctp_front *fronts, const BFront *tab, ch
 
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
-                              double *W21, int64_t ldw, void *Wb, void *Lb, int Kp, int64_t lo_off,
-                              int pieces, cudaStream_t st);
+                              const SliceBuf &sb, void *Wb, void *Lb, int Kp, int64_t lo_off, int pieces,
+                              cudaStream_t st);
 
 // Threshold partial pivoting on all n rows (the comparator of the compressed path).
 size_t tpp_ws_bytes(int p);
@@ -214,9 +255,15 @@ cudaError_t launch_form_tc(const void *Wb, const void *Lb, int64_t piece_off, in
                            int layout /* 0 full, 1 packed, 2 tiled, 3 subtract from FP64 */,
                            int32_t *info, int num_sms, int walk /* ctp_walk */, cudaStream_t st);
 
-cudaError_t launch_form_fp64(const double *L21, int64_t ldl, const double *W21, int64_t ldw,
-                             int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
-                             cudaStream_t st);
+// S = W21 L21^T in FP64 from the operands' slices (form.cu)
+// (L21, D and the pivot kinds serve the rows that the slices do not represent)
+cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda, const int32_t *piv,
+                             const double *D, int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
+                             int32_t *info, int num_sms, cudaStream_t st);
+// the slices from a stored L21 and its D, D^-1 (full-column pivoting)
+cudaError_t launch_slices_from_l(const double *A, int64_t lda, int p, int64_t m, const int32_t *piv,
+                                 const double *D, const double *Dinv, const int32_t *nelim, const SliceBuf &sb,
+                                 cudaStream_t st);
 
 // Complete systems: front-list solve, residual, backward error (system.cu).
 size_t sys_solve_ws_bytes(int64_t nmax, int nrhs);
@@ -243,8 +290,5 @@ cudaError_t launch_spmv_csc_residual(int64_t N, const int64_t *colptr, const int
                                      int64_t ldr, cudaStream_t st);
 cudaError_t launch_spmv_csc_abs_rowsum(int64_t N, const int64_t *colptr, const int32_t *rowind,
                                        const double *val, double *rowsum, cudaStream_t st);
-cudaError_t launch_w21_from_l(const double *A, int64_t lda, int p, int64_t m, const int32_t *piv,
-                              const double *D, const int32_t *nelim, double *W21, int64_t ldw,
-                              cudaStream_t st);
 
 }  // namespace ctp

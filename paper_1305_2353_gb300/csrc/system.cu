@@ -330,29 +330,6 @@ __global__ void k_axpy(int64_t N, int nrhs, double *X, int64_t ldx, const double
         X[(int64_t)r * ldx + i] += Dx[(int64_t)r * ldd + i];
 }
 
-// W21 = L21 D11 from the stored L21 and D (used where the pivoting kernel does
-// not produce W21 itself, i.e. full-column threshold partial pivoting).
-__global__ void __launch_bounds__(kTh) k_w21_from_l(const double *A, int64_t lda, int p, int64_t m,
-                                                    const int32_t *piv, const double *D,
-                                                    const int32_t *nelim, double *W21, int64_t ldw) {
-    const int e = *nelim;
-    const int64_t i = (int64_t)blockIdx.x * kTh + threadIdx.x;
-    if (i >= m) return;
-    const double *L = A + p + i;
-    for (int q = 0; q < e; q++) {
-        const int k = piv[q];
-        double w = 0.0;
-        if (k == CTP_PIVKIND_1X1) {
-            w = L[(int64_t)q * lda] * D[2 * q];
-        } else if (k == CTP_PIVKIND_2X2_FIRST) {
-            w = L[(int64_t)q * lda] * D[2 * q] + L[(int64_t)(q + 1) * lda] * D[2 * q + 1];
-        } else if (k == CTP_PIVKIND_2X2_SECOND) {
-            w = L[(int64_t)(q - 1) * lda] * D[2 * q - 1] + L[(int64_t)q * lda] * D[2 * q];
-        }
-        W21[(int64_t)q * ldw + i] = w;
-    }
-}
-
 // Gradient of a loss through x = M^{-1} b with respect to the stored lower
 // triangle of the symmetric M (each stored off-diagonal entry stands for both
 // m_ij and m_ji): dL/dm_ij = -sum_r (g_ir x_jr + g_jr x_ir) for i > j and
@@ -538,14 +515,6 @@ cudaError_t launch_spmv_csc_abs_rowsum(int64_t N, const int64_t *colptr, const i
                                        const double *val, double *rowsum, cudaStream_t st) {
     const int64_t g = (N + 7) / 8 < 4096 ? (N + 7) / 8 : 4096;
     k_spmv_csc<true><<<(unsigned)g, kTh, 0, st>>>(N, colptr, rowind, val, 1, nullptr, 0, rowsum, N);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_w21_from_l(const double *A, int64_t lda, int p, int64_t m, const int32_t *piv,
-                              const double *D, const int32_t *nelim, double *W21, int64_t ldw,
-                              cudaStream_t st) {
-    if (m == 0) return cudaSuccess;
-    k_w21_from_l<<<blocks_for(m), kTh, 0, st>>>(A, lda, p, m, piv, D, nelim, W21, ldw);
     return cudaGetLastError();
 }
 
