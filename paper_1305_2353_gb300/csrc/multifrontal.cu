@@ -46,7 +46,6 @@ struct ctp_mf {
         std::vector<int32_t> cb;  // contribution-block variables (new numbering); delayed first
         int64_t ndel = 0;
         int64_t pa = 0, pb = 0;  // this block's panels in the panel list
-        int last_level = -1;     // solve level of its last panel
     };
     std::vector<Blk> blk;
     // assembly lists: local codes (own variables 0..p_own-1, struct rows p_own + t)
@@ -57,7 +56,7 @@ struct ctp_mf {
     std::vector<ctp_sfront> fronts;
     std::vector<PanelRec> panels;
     std::vector<int32_t> panel_block;  // block of each panel
-    SolvePlan plan;  // the panels grouped into levels of independent panels
+    SolvePlan plan;  // the factors repacked for solving
     bool factored = false;
     bool mixed = false;  // the last factorization's Form ran on the tensor cores
     ~ctp_mf() {
@@ -623,27 +622,11 @@ ctp_status ctp_mf_factor(ctp_ctx *ctx, ctp_mf *mf, const double *val, const ctp_
         return rc;
     }
     for (const PanelRec &r : mf->panels) mf->fronts.push_back(r.f);
-    // solve levels: a block's first panel follows its children's last panels,
-    // each further panel follows the one before
-    std::vector<int> level(mf->panels.size());
-    for (ctp_mf::Blk &b : mf->blk) {
-        int lv = -1;
-        for (int c : b.children) lv = std::max(lv, mf->blk[c].last_level);
-        for (int64_t k = b.pa; k < b.pb; k++) level[k] = ++lv;
-        b.last_level = lv;
-    }
-    std::vector<int> order(mf->panels.size());
-    for (size_t k = 0; k < order.size(); k++) order[k] = (int)k;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return level[a] < level[c]; });
-    std::vector<ctp_sfront> pf;
-    std::vector<int> pl;
+    std::vector<SolveChain> chains;
+    for (const ctp_mf::Blk &b : mf->blk) chains.push_back({b.pa, b.pb, b.parent});
     std::vector<int32_t> pe;
-    for (int k : order) {
-        pf.push_back(mf->panels[k].f);
-        pl.push_back(level[k]);
-        pe.push_back(mf->panels[k].e);
-    }
-    rc = mf->plan.build(pf, pl, pe, st);
+    for (const PanelRec &r : mf->panels) pe.push_back(r.e);
+    rc = mf->plan.build(mf->fronts, pe, chains, mf->perm, mf->inv, opt->prec != CTP_FP64, st);
     if (rc != CTP_OK) return rc;
     mf->factored = true;
     mf->mixed = opt->prec != CTP_FP64;

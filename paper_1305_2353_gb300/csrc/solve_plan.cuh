@@ -1,7 +1,7 @@
-// solve_plan.cuh -- a front-list solve planned by levels (fronts of a level are
-// independent: one launch per level and sweep), and FP64 iterative refinement
-// (Section 7) around any solve: the helpers shared by the ABI's complete-system
-// entry points.
+// solve_plan.cuh -- the solve with a multifrontal factorization, planned by levels of
+// groups of pivots (groups of a level are independent: one launch per level and
+// sweep), and FP64 iterative refinement (Section 7) around any solve: the
+// helpers shared by the ABI's complete-system entry points.
 #pragma once
 
 #include <vector>
@@ -10,27 +10,47 @@
 
 namespace ctp {
 
-// Fronts in an elimination order grouped by level: the fronts of a level are
-// independent (none updates another's pivot rows), so a level is one launch
-// per sweep over items (front, chunk of rows below its pivots).
+// A device buffer that only grows.
+struct DevBuf {
+    void *p = nullptr;
+    size_t cap = 0;
+    bool need(size_t bytes);
+    void release();
+    template <typename T>
+    T *as() const { return static_cast<T *>(p); }
+};
+
+// A front's panels, in order: panels [pa, pb) of the list, and its parent front
+// (-1: a root; children come before parents).
+struct SolveChain {
+    int64_t pa, pb;
+    int parent;
+};
+
+// The factors repacked for solving.  The pivots of a front's panels, in
+// elimination order, are cut into groups of at most 64; a group's L11 and its
+// rows below (L21, in chunks of rows) are copied into contiguous blocks, with
+// the rows in the order they have after the group's last panel, so that a
+// sweep needs one launch per level of groups instead of one per panel
+// (strict pivoting makes panels of about 15 pivots), and an item's factor entries
+// are one contiguous copy.
 struct SolvePlan {
-    int nf = 0, nlev = 0;
-    std::vector<int64_t> item_ptr;  // items of level l: [item_ptr[l], item_ptr[l+1])
-    void *d_F = nullptr;            // the fronts' descriptors (solve_plan.cu)
-    int2 *d_items = nullptr;        // (front, chunk)
-    int32_t *d_pvar = nullptr;      // per front: the variables of its pivot positions
-    int *d_cnt = nullptr;           // per front: items done in the backward sweep (0 between solves)
-    int64_t z_per_rhs = 0;          // doubles per right-hand side: z of every front
-    int64_t part_per_rhs = 0;       // doubles per right-hand side: the largest level's partial sums
+    int ngrp = 0, nlev = 0;
+    int64_t N = 0, npiv = 0;
+    std::vector<int64_t> item_ptr;  // items (group, chunk) of level l: [item_ptr[l], item_ptr[l+1])
+    std::vector<int> level_e;       // largest group of each level
+    DevBuf grp, items, vars, perm, pack64, pack32, kind, D;
     SolvePlan() = default;
     SolvePlan(const SolvePlan &) = delete;
     SolvePlan &operator=(const SolvePlan &) = delete;
-    ~SolvePlan() { clear(); }
-    void clear();
-    // fronts with their levels (nondecreasing) and eliminated counts; perm and
-    // rows are read on `st` (synchronised before returning)
-    ctp_status build(const std::vector<ctp_sfront> &fronts, const std::vector<int> &level,
-                     const std::vector<int32_t> &nelim, cudaStream_t st);
+    ~SolvePlan();
+    void clear() { ngrp = nlev = 0; }  // forgets the plan, keeps its memory for the next one
+    // panels of all fronts; perm_host: the elimination order (variable of position i),
+    // inv_host its inverse; fp32: also pack for FP32 sweeps.  Reads the panels'
+    // device arrays on `st` (synchronised before returning).
+    ctp_status build(const std::vector<ctp_sfront> &panels, const std::vector<int32_t> &nelim,
+                     const std::vector<SolveChain> &fronts, const std::vector<int32_t> &perm_host,
+                     const std::vector<int32_t> &inv_host, bool fp32, cudaStream_t st);
     size_t ws_bytes(int nrhs) const;
     // X <- M^{-1} X; fp32: the sweeps' arithmetic in FP32 (X read and written in FP64)
     cudaError_t solve(ctp_ctx *ctx, double *X, int64_t ldx, int nrhs, void *ws, cudaStream_t st,
