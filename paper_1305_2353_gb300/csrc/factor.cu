@@ -25,7 +25,10 @@
 //                (largest |a(m, j)| over live j < m) and the 1x1 test for one
 //                candidate; a passing warp pushes (candidate, warp) into every
 //                CTA's slot with a DSMEM atomicMin, so after the barrier each
-//                CTA finds the winner in its own shared memory;
+//                CTA finds the winner in its own shared memory.  A round of one
+//                candidate (every round while pivots are accepted as they come)
+//                pushes its whole outcome instead, with nothing to hand out or
+//                collect: 100 us of 1628 at p = 256, all pivots accepted;
 //   update       every CTA copies the pivot column(s), takes the per-column
 //                scalars from them and applies the 1x1 or 2x2 update to its own
 //                live columns (one CTA barrier, then the team barrier).
@@ -62,7 +65,7 @@ constexpr int kNoKey = 0x7fffffff;
 
 struct Shared {
     Decision res[2][kNW];  // per warp's candidate, double-buffered by round
-    Decision cur;
+    Decision one[2];       // the accepted decision, double-buffered by round
     int cmin[2];           // lowest (candidate * kNW + warp) that passed, pushed by every CTA
     unsigned char live[kMaxP];
     int order[kMaxP];
@@ -333,23 +336,31 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
         // of rejections are tested in parallel (a rejection is cheap: most are
         // settled by the FP32 filters).
         const int hi = min(p, m + win);  // the same on every CTA
-        if (warp == 0) {
-            // this CTA's live columns in [m, hi), in order, go to its warps
-            // (win <= kNW * G, so no CTA owns more than kNW of them)
-            const int j0 = m > rank ? (m - rank + gm) >> gs : 0;
-            const int c = rank + G * (j0 + lane);
-            const bool ok = c < hi && sh.live[c];
-            const unsigned int bal = __ballot_sync(0xffffffffu, ok);
-            if (ok) sh.cand[__popc(bal & ((1u << lane) - 1u))] = c;
-            if (lane >= __popc(bal) && lane < kNW) sh.cand[lane] = -1;
+        // A round of one candidate (every round while pivots are accepted as they
+        // come): the first warp of the CTA that owns column m tests it and writes
+        // the outcome to every CTA; nothing to hand out or to collect.
+        const bool one = win == 1;
+        if (!one) {
+            if (warp == 0) {
+                // this CTA's live columns in [m, hi), in order, go to its warps
+                // (win <= kNW * G, so no CTA owns more than kNW of them)
+                const int j0 = m > rank ? (m - rank + gm) >> gs : 0;
+                const int c = rank + G * (j0 + lane);
+                const bool ok = c < hi && sh.live[c];
+                const unsigned int bal = __ballot_sync(0xffffffffu, ok);
+                if (ok) sh.cand[__popc(bal & ((1u << lane) - 1u))] = c;
+                if (lane >= __popc(bal) && lane < kNW) sh.cand[lane] = -1;
+            }
+            __syncthreads();
         }
-        __syncthreads();
         {
-            const int c = sh.cand[warp];
+            const int c = one ? ((warp == 0 && (m & gm) == rank) ? m : -1) : sh.cand[warp];
             if (c >= 0) {
                 Decision d = test_candidate(c, cols + (size_t)(c >> gs) * LD, colptr, sh.live, p, LD, u, rcp_u,
                                             small_k);
-                if (d.kind != DEC_REJECT) {
+                if (one) {
+                    if (lane < G) *team.at(&sh.one[buf], lane) = d;
+                } else if (d.kind != DEC_REJECT) {
                     // publish: the decision stays here, (candidate, warp) goes to
                     // every CTA's slot for this round
                     if (lane == 0) sh.res[buf][warp] = d;
@@ -359,24 +370,29 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             }
         }
         team.sync();
-        // the lowest passing candidate: read the own slot (and clear it for the
-        // round after next), fetch the winner's decision from its CTA
-        if (warp == 0) {
-            int key = 0;
-            if (lane == 0) {
-                key = sh.cmin[buf];
-                sh.cmin[buf] = kNoKey;
+        int cstar;
+        if (one) {
+            cstar = sh.one[buf].kind != DEC_REJECT ? m : p;
+        } else {
+            // the lowest passing candidate: read the own slot (and clear it for the
+            // round after next), fetch the winner's decision from its CTA
+            if (warp == 0) {
+                int key = 0;
+                if (lane == 0) {
+                    key = sh.cmin[buf];
+                    sh.cmin[buf] = kNoKey;
+                }
+                key = __shfl_sync(0xffffffffu, key, 0);
+                const int cs = key == kNoKey ? p : key / kNW;
+                if (cs < p && lane < 8) {
+                    const Decision *src = team.at(&sh.res[buf][key % kNW], cs & gm);
+                    reinterpret_cast<double *>(&sh.one[buf])[lane] = reinterpret_cast<const double *>(src)[lane];
+                }
+                if (lane == 0) sh.cstar = cs;
             }
-            key = __shfl_sync(0xffffffffu, key, 0);
-            const int cs = key == kNoKey ? p : key / kNW;
-            if (cs < p && lane < 8) {
-                const Decision *src = team.at(&sh.res[buf][key % kNW], cs & gm);
-                reinterpret_cast<double *>(&sh.cur)[lane] = reinterpret_cast<const double *>(src)[lane];
-            }
-            if (lane == 0) sh.cstar = cs;
+            __syncthreads();
+            cstar = sh.cstar;
         }
-        __syncthreads();
-        const int cstar = sh.cstar;
         if (cstar >= hi) {
             // every tested candidate before the window's end failed: the sweep
             // continues there, with a wider window
@@ -394,7 +410,7 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             if (win > win_max) win = win_max;
             m0 = cstar + 1;
         }
-        const Decision dv = sh.cur;
+        const Decision dv = sh.one[buf];
         if (dv.kind == DEC_ZERO) {
             // the live-row list without cstar (every thread reads its own rows'
             // old positions only)
@@ -443,6 +459,7 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             const double *s1 = q1 >= 0 ? colptr(q1) : s0;
             const double ad0 = abs_bits(dv.d0), ai0 = abs_bits(dv.i0), ai1 = abs_bits(dv.i1), ai2 = abs_bits(dv.i2);
             for (int i = tid; i < LD; i += kT) {
+                if (i < p && !sh.live[i]) continue;  // rows of earlier pivots take no part any more
                 if (i < p) {
                     // the live-row list without the pivot rows: the rank of a
                     // row drops by the pivots above it (the pivots' own flags
@@ -456,7 +473,7 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
                 const bool ab = abs_rows && i >= p;
                 if (i < p) apc0[i] = abs_bits(x);
                 if (q1 < 0) {
-                    const double l = __ddiv_rn(x, ab ? ad0 : dv.d0);
+                    const double l = div_by(x, ab ? ad0 : dv.d0, ab ? ai0 : dv.i0);
                     rl0[i] = ab ? l : neg_bits(l);
                 } else {
                     const double y = s1[i];
@@ -498,33 +515,48 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             }
         }
         __syncthreads();
-        // the update: warp w takes the own live columns w, w + kNW, ...; column
-        // c gets its live A11 rows from the diagonal down and the R outer rows,
-        // one fused multiply-add per pivot column: -l(i) a(c,q), or +l(i)
-        // |a(c,q)| on the abs rows (eq. (4.3)).  The entry (c, i) above the
-        // diagonal, in row i's column, is the same product (row i's multiplier,
-        // row c's pivot entry) on the same old value (the working matrix is
-        // symmetric), so column c's owner stores the result there too (in
-        // another CTA's shared memory when column i lives there): the upper half
-        // costs a store instead of a second FP64 update, and both halves stay
-        // bit-identical.  Only live rows are visited, so no lane of an FP64
-        // instruction idles on a retired row.
+        // the update: warp w takes the own live columns w, w + kNW, ...; one fused
+        // multiply-add per pivot column: -l(i) a(c,q), or +l(i) |a(c,q)| on the
+        // abs rows (eq. (4.3)).  The entry (c, i) above the diagonal, in row i's
+        // column, is the same product (row i's multiplier, row c's pivot entry)
+        // on the same old value (the working matrix is symmetric).  One CTA
+        // updates the live A11 rows from the diagonal down and stores each result
+        // into its mirror too, so the upper half costs a store instead of a
+        // second FP64 update.  In a cluster the mirror lies in another CTA's
+        // shared memory, and a few hundred remote stores per pivot and CTA cost
+        // more than they save: each CTA computes both halves, the upper from its
+        // mirror's operands (p = 256 on 16 CTAs, all pivots accepted: 1652 -> 1612
+        // us).  Either way both halves stay bit-identical.  Only live rows are
+        // visited, so no lane of an FP64 instruction idles on a retired row, and
+        // 1x1 and 2x2 pivots have loops of their own: a predicated-off FP64
+        // instruction takes its turn in the pipe all the same.  (Several rows per
+        // lane in flight were slower: 1882 us with four.)
         {
             const int nl = sh.nlive;
             for (int lc = warp; lc < ncl; lc += kNW) {
                 const int c = (lc << gs) + rank;
                 if (c >= p || !sh.live[c]) continue;  // warp-uniform
-                const int a0 = sh.lpos[c], lenA = nl - a0, len = lenA + R;
+                const int a0 = kSingle ? sh.lpos[c] : 0, lenA = nl - a0, len = lenA + R;
                 double *col = cols + (size_t)lc * LD;
-                const double q0c = pc0[c], aq0c = apc0[c];
-                const double q1c = q1 >= 0 ? pc1[c] : 0.0, aq1c = q1 >= 0 ? apc1[c] : 0.0;
-                for (int j = lane; j < len; j += 32) {
-                    const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
-                    const bool ab = abs_rows && i >= p;
-                    double v = fma(rl0[i], ab ? aq0c : q0c, col[i]);
-                    if (q1 >= 0) v = fma(rl1[i], ab ? aq1c : q1c, v);
-                    col[i] = v;
-                    if (i < p && i != c) team.at(cols, i & gm)[(size_t)(i >> gs) * LD + c] = v;
+                const double q0c = pc0[c], aq0c = abs_rows ? apc0[c] : q0c, l0c = rl0[c];
+                if (q1 < 0) {
+                    for (int j = lane; j < len; j += 32) {
+                        const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
+                        const bool up = !kSingle && i < c;
+                        const double v = fma(up ? l0c : rl0[i], up ? pc0[i] : (i >= p ? aq0c : q0c), col[i]);
+                        col[i] = v;
+                        if (kSingle && i < p && i != c) cols[(size_t)i * LD + c] = v;
+                    }
+                } else {
+                    const double q1c = pc1[c], aq1c = abs_rows ? apc1[c] : q1c, l1c = rl1[c];
+                    for (int j = lane; j < len; j += 32) {
+                        const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
+                        const bool up = !kSingle && i < c;
+                        double v = fma(up ? l0c : rl0[i], up ? pc0[i] : (i >= p ? aq0c : q0c), col[i]);
+                        v = fma(up ? l1c : rl1[i], up ? pc1[i] : (i >= p ? aq1c : q1c), v);
+                        col[i] = v;
+                        if (kSingle && i < p && i != c) cols[(size_t)i * LD + c] = v;
+                    }
                 }
             }
         }
@@ -751,7 +783,7 @@ __global__ void __launch_bounds__(32 * kWarpFronts)
                 const bool ab = abs_rows && i >= p;
                 const double x = p0[i];
                 if (q1 < 0) {
-                    const double l = __ddiv_rn(x, ab ? ad0 : dv.d0);
+                    const double l = div_by(x, ab ? ad0 : dv.d0, ab ? ai0 : dv.i0);
                     l0[h] = ab ? l : neg_bits(l);
                 } else {
                     const double y = p1[i];
