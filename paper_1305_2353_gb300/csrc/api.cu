@@ -58,6 +58,16 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     off += align256(sizeof(int32_t) * (size_t)ms);
     L.el = off;
     off += align256(sizeof(int32_t) * (size_t)ms);
+    // the blocked FP64 Solve
+    const int blocks = opt->pivot != CTP_PIV_TPP && !solve_on_tc(opt) ? solve_blocks(m, p, opt->pivot) : 0;
+    L.Yb = off;
+    off += align256(slice_w_bytes(blocks > 0 ? m : 0, kSliceK));
+    L.Lx = off;
+    off += align256(blocks * slice_l_bytes(p, kSliceK));
+    L.ey = off;
+    off += align256(sizeof(int32_t) * (size_t)(blocks > 0 ? m : 0));
+    L.ex = off;
+    off += align256(sizeof(int32_t) * (size_t)blocks * kMaxP);
     // BF16 operand copies (hi, and for the split form the lo parts after them)
     const size_t nb = tc ? 2 * (size_t)m * form_tc_kpad(p) * prec_pieces(opt->prec) : 0;
     L.Wb = off;
@@ -339,7 +349,10 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
         }));
     else if (m > 0)
         CTP_CUDA(timed(ctx, K_SOLVE, st, [&] {
-            return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, sb, Wb, Lbf, Kp, lo_off, pieces, st);
+            const SliceBuf blk = {(unsigned char *)(ws + L.Yb), (unsigned char *)(ws + L.Lx),
+                                  (int32_t *)(ws + L.ey), (int32_t *)(ws + L.ex), 1};
+            return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, sb, blk, solve_blocks(m, p, opt->pivot), Wb,
+                                     Lbf, Kp, lo_off, pieces, info, ctx->num_sms, st);
         }));
     if (opt->smode != CTP_S_NONE && m > 0) {
         if (tc)
@@ -465,7 +478,7 @@ ctp_status ctp_factor_batch(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front 
             CTP_CUDA(cudaStreamWaitEvent(s, ctx->fork_ev, 0));
             CTP_CUDA(batch_factor_class(plan, c, fronts, w, s));
             if (per_class) {
-                CTP_CUDA(batch_solve_class(plan, c, fronts, w, s));
+                CTP_CUDA(batch_solve_class(plan, c, fronts, w, ctx->num_sms, s));
                 CTP_CUDA(batch_form_class(plan, c, fronts, w, ctx->num_sms, s));
             }
             CTP_CUDA(cudaEventRecord(ctx->join_ev[i % kSideStreams], s));
@@ -483,7 +496,12 @@ ctp_status ctp_factor_batch(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front 
                          : K_B_FACTOR_G1 + (G == 1 ? 0 : G == 2 ? 1 : G == 4 ? 2 : G == 8 ? 3 : 4);
             CTP_CUDA(timed(ctx, id, st, [&] { return batch_factor_class(plan, c, fronts, w, st); }));
         }
-        CTP_CUDA(timed(ctx, K_B_SOLVE, st, [&] { return batch_solve(plan, fronts, w, ctx->num_sms, st); }));
+        if (batch_solve_per_class(plan))
+            for (int c = 0; c < ncls; c++)
+                CTP_CUDA(timed(ctx, K_B_SOLVE, st,
+                               [&] { return batch_solve_class(plan, c, fronts, w, ctx->num_sms, st); }));
+        else
+            CTP_CUDA(timed(ctx, K_B_SOLVE, st, [&] { return batch_solve(plan, fronts, w, ctx->num_sms, st); }));
     }
     CTP_CUDA(timed(ctx, K_B_FORM, st, [&] { return batch_form(plan, fronts, w, ctx->num_sms, st); }));
     return CTP_OK;

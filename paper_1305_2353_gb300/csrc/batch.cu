@@ -26,6 +26,11 @@ namespace {
 
 constexpr int kTR = 32;     // rows per compression item
 constexpr int kThreads = 256;
+// A class's Solve is blocked (solve.cu) when its fronts hold this many entries of A21
+// right of their first 32 columns: the Solves of a mixed 64^3 multifrontal
+// factorization took 67.8 ms whole, 45.9 with the line at 1e6, 46.4 at 1e5, those
+// of a 36^3 one 9.5, 9.3 and 8.3 ms, those of 1024 uneven fronts 0.79, 0.64, 0.68 ms
+constexpr double kBlockedEntries = 3e5;
 constexpr unsigned long long kAbsMask = 0x7FFFFFFFFFFFFFFFull;
 
 __device__ __forceinline__ unsigned long long abs_key(double x) {
@@ -217,7 +222,7 @@ struct ctp_plan {
     bool tc;
     // workspace layout
     size_t off_ginfo, off_tab, off_citem, off_sitem, off_fitem, off_lists, off_flags, off_sections, off_wb,
-        off_lb, off_qitem, off_ritem, off_xt, off_zt, off_csitem, off_cstile, off_cfitem, off_cftile;
+        off_lb, off_qitem, off_ritem, off_xt, off_zt, off_csitem, off_cstile, off_cfitem, off_cftile, off_cuitem, off_cutile;
     size_t total;
     int64_t c_items, s_items, f_items, total_rows, q_items, r_items, nxt, nzt;
     int64_t cbucket[5] = {0, 0, 0, 0, 0};  // compression items of fronts with p <= 32, 64, 128, 256
@@ -228,6 +233,7 @@ struct ctp_plan {
         size_t list_off;     // element offset in the class-list array
         int pmax;            // largest p of the class
         int64_t s_off, s_count;  // the class's Solve items (front, tile) in the class Solve lists
+        int64_t u_off, u_count;  // blocked Solve: the class's update items (none: a whole pass per tile)
         int64_t f_off, f_count;  // the class's Form items (front, tile) in the class Form lists
     };
     std::vector<Class> classes;
@@ -372,7 +378,7 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
         };
         std::stable_sort(byKey[key].begin(), byKey[key].end(), [&](int x, int y) { return work(x) > work(y); });
     }
-    std::vector<int> lists, csitem, cstile, cfitem, cftile;
+    std::vector<int> lists, csitem, cstile, cfitem, cftile, cuitem, cutile;
     for (int key = 0; key < kNumKeys; key++) {
         if (byKey[key].empty()) continue;
         ctp_plan::Class c;
@@ -384,6 +390,18 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
                 cstile.push_back((int)t);
             }
         c.s_count = (int64_t)csitem.size() - c.s_off;
+        // the class's Solve is blocked (three more launches, one more pass over its
+        // rows) when its fronts hold enough entries of A21 right of the first block
+        c.u_off = (int64_t)cuitem.size();
+        double right = 0.0;
+        for (int f : byKey[key]) right += tab[f].p > kSliceK ? (double)tab[f].m * (tab[f].p - kSliceK) : 0.0;
+        if (!stc && right >= kBlockedEntries)
+            for (int f : byKey[key])
+                for (int64_t t = 0; t < update_tiles(tab[f].m, tab[f].p); t++) {
+                    cuitem.push_back(f);
+                    cutile.push_back((int)t);
+                }
+        c.u_count = (int64_t)cuitem.size() - c.u_off;
         c.f_off = (int64_t)cfitem.size();
         if (opt->smode != CTP_S_NONE)
             for (int f : byKey[key]) {
@@ -438,6 +456,10 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     off += align256(sizeof(int) * cfitem.size());
     P->off_cftile = off;
     off += align256(sizeof(int) * cftile.size());
+    P->off_cuitem = off;
+    off += align256(sizeof(int) * cuitem.size());
+    P->off_cutile = off;
+    off += align256(sizeof(int) * cutile.size());
     P->off_flags = off;
     off += align256(sizeof(int32_t) * (size_t)nb);
     const size_t tables_end = off;
@@ -477,6 +499,10 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     if (!cfitem.empty()) {
         memcpy(P->blob.data() + P->off_cfitem, cfitem.data(), sizeof(int) * cfitem.size());
         memcpy(P->blob.data() + P->off_cftile, cftile.data(), sizeof(int) * cftile.size());
+    }
+    if (!cuitem.empty()) {
+        memcpy(P->blob.data() + P->off_cuitem, cuitem.data(), sizeof(int) * cuitem.size());
+        memcpy(P->blob.data() + P->off_cutile, cutile.data(), sizeof(int) * cutile.size());
     }
     *plan = P;
     if (ws_bytes) *ws_bytes = P->total;
@@ -556,24 +582,31 @@ cudaError_t batch_factor_class(const ctp_plan *P, int ci, const ctp_front *fr, c
                                reinterpret_cast<const int *>(w + P->off_lists) + c.list_off, c.count, c.kind,
                                c.G, c.smem, c.pcap, c.ldcap, P->bo, st);
 }
+// The tensor-core Solve of all fronts
 cudaError_t batch_solve(const ctp_plan *P, const ctp_front *fr, char *w, int num_sms, cudaStream_t st) {
-    if (P->bo.stc)
-        return launch_solve_tc_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
-                                     reinterpret_cast<const int *>(w + P->off_sitem), P->s_items,
-                                     reinterpret_cast<const int *>(w + P->off_qitem), P->q_items,
-                                     reinterpret_cast<const int *>(w + P->off_ritem), P->r_items, P->bo,
-                                     w + P->off_xt, w + P->off_zt, P->nxt, P->nzt, w + P->off_wb, w + P->off_lb,
-                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
-    return launch_solve_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
-                              reinterpret_cast<const int *>(w + P->off_sitem), P->s_items, P->bo,
-                              P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, P->pmax,
-                              st);
+    return launch_solve_tc_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
+                                 reinterpret_cast<const int *>(w + P->off_sitem), P->s_items,
+                                 reinterpret_cast<const int *>(w + P->off_qitem), P->q_items,
+                                 reinterpret_cast<const int *>(w + P->off_ritem), P->r_items, P->bo,
+                                 w + P->off_xt, w + P->off_zt, P->nxt, P->nzt, w + P->off_wb, w + P->off_lb,
+                                 reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
 }
 // The FP64 Solve of one pivot-search class's fronts (false when the batch
 // solves on the tensor cores: that Solve runs once over all fronts)
 bool batch_solve_per_class(const ctp_plan *P) { return !P->bo.stc; }
-cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, cudaStream_t st) {
+cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, int num_sms,
+                              cudaStream_t st) {
     const ctp_plan::Class &c = P->classes[ci];
+    if (c.u_count > 0)
+        return launch_solve_batch_blocked(
+            fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
+            reinterpret_cast<const int *>(w + P->off_lists) + c.list_off, c.count,
+            reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off,
+            reinterpret_cast<const int *>(w + P->off_cstile) + c.s_off, c.s_count,
+            reinterpret_cast<const int *>(w + P->off_cuitem) + c.u_off,
+            reinterpret_cast<const int *>(w + P->off_cutile) + c.u_off, c.u_count, P->bo,
+            P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax,
+            reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
     return launch_solve_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
                               reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off, c.s_count, P->bo,
                               P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax, st,

@@ -44,10 +44,12 @@ __host__ __device__ inline size_t slice_l_bytes(int64_t m, int p) {
 //   Dinv                2p doubles: inverse pivot blocks, same slots as D
 //   Ws, Ls, ew, el      digit slices of Y = L21 D11 and L21 and their row exponents
 //                       (slices.cuh) when the FP64 Form step runs
+//   Yb, Lx, ey, ex      digit slices of one block's y and of L11, and their row
+//                       exponents, for the blocked FP64 Solve
 //   Wb, Lb              m*Kp BF16 copies of Y and L21 for the tensor-core Form
 //   aux                 method-specific scratch (relaxed candidate lists)
 struct WsLayout {
-    size_t info, C, Dinv, Ws, Ls, ew, el, Wb, Lb, aux, Xs, flags, total;
+    size_t info, C, Dinv, Ws, Ls, ew, el, Yb, Lx, ey, ex, Wb, Lb, aux, Xs, flags, total;
 };
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -124,7 +126,7 @@ struct BFront {
 // offsets inside a front's section: info word, compressed matrix (strict),
 // Dinv, and the digit slices of L21 D11 and L21 when an FP64 Form follows
 struct BSection {
-    size_t info, C, Dinv, Ws, Ls, ew, el, nz, total;
+    size_t info, C, Dinv, Ws, Ls, ew, el, Yb, Lx, ey, ex, nz, total;
 };
 __host__ __device__ inline size_t align256hd(size_t x) { return (x + 255) & ~size_t(255); }
 __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options *opt) {
@@ -145,6 +147,16 @@ __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options
     off += align256hd(sizeof(int32_t) * (size_t)ms);
     s.el = off;
     off += align256hd(sizeof(int32_t) * (size_t)ms);
+    // the blocked Solve's first block: slices of y and of L11's rows below it
+    const int64_t mb = p > kSliceK ? n - p : 0;
+    s.Yb = off;
+    off += align256hd(slice_w_bytes(mb, kSliceK));
+    s.Lx = off;
+    off += align256hd(mb > 0 ? slice_l_bytes(p, kSliceK) : 0);
+    s.ey = off;
+    off += align256hd(sizeof(int32_t) * (size_t)mb);
+    s.ex = off;
+    off += align256hd(mb > 0 ? sizeof(int32_t) * (size_t)p : 0);
     s.nz = off;  // strict: which rows of C receive an A21 row (one bit per row)
     off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
     s.total = off;
@@ -158,6 +170,16 @@ __host__ __device__ inline SliceBuf bsection_slices(char *base, const BSection &
     b.ew = reinterpret_cast<int32_t *>(base + s.ew);
     b.el = reinterpret_cast<int32_t *>(base + s.el);
     b.kb = slice_kb(p);
+    return b;
+}
+
+__host__ __device__ inline SliceBuf bsection_block(char *base, const BSection &s) {
+    SliceBuf b;
+    b.W = reinterpret_cast<unsigned char *>(base + s.Yb);
+    b.L = reinterpret_cast<unsigned char *>(base + s.Lx);
+    b.ew = reinterpret_cast<int32_t *>(base + s.ey);
+    b.el = reinterpret_cast<int32_t *>(base + s.ex);
+    b.kb = 1;
     return b;
 }
 
@@ -180,11 +202,10 @@ cudaError_t launch_factor_batch(const ctp_front *fronts, const BFront *tab, char
 cudaError_t launch_compress_strict_batch(const ctp_front *fronts, const BFront *tab, char *ws,
                                          const int *item_front, const int64_t (&bucket)[5], BatchOpts o,
                                          cudaStream_t st);
-// item_tile (optional): each item's 32-row tile of its front; without it the
-// items of a front are consecutive, from tab[front].s0 on
+// items: (front, 32-row tile) pairs
 cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char *ws,
                                const int *item_front, int64_t items, BatchOpts o, void *Wb, void *Lb,
-                               int pmax, cudaStream_t st, const int *item_tile = nullptr);
+                               int pmax, cudaStream_t st, const int *item_tile);
 // item_tile (optional, both batched Forms): each item's tile of its front;
 // without it the items of a front are consecutive, from tab[front].f0 on
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
@@ -206,7 +227,7 @@ cudaError_t batch_compress(const ctp_plan *P, const ctp_front *fr, char *w, int 
 cudaError_t batch_factor_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, cudaStream_t st);
 cudaError_t batch_solve(const ctp_plan *P, const ctp_front *fr, char *w, int num_sms, cudaStream_t st);
 bool batch_solve_per_class(const ctp_plan *P);
-cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, cudaStream_t st);
+cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, int num_sms, cudaStream_t st);
 cudaError_t batch_form_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, int num_sms, cudaStream_t st);
 cudaError_t batch_form(const ctp_plan *P, const ctp_front *fr, char *w, int num_sms, cudaStream_t st);
 
@@ -237,8 +258,22 @@ cudaError_t launch_solve_tc_batch(const ctp_front *fronts, const BFront *tab, ch
 
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
-                              const SliceBuf &sb, void *Wb, void *Lb, int Kp, int64_t lo_off, int pieces,
-                              cudaStream_t st);
+                              const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
+                              int64_t lo_off, int pieces, int32_t *info, int num_sms, cudaStream_t st);
+int solve_blocks(int64_t m, int p, int pivot);  // 0: a whole pass
+// A21(:, 32 (blk+1)..p-1) -= y_blk L11(32 (blk+1).., block blk)^T from the slices (form.cu)
+cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int64_t m, int blk, const int32_t *piv,
+                          const int32_t *nelim, int32_t *info, int num_sms, cudaStream_t st);
+// the same for block 0 of a batch's fronts, by (front, tile) items
+cudaError_t launch_update_batch(const ctp_front *fronts, const BFront *tab, char *ws, const int *item_front,
+                                const int *item_tile, int64_t items, BatchOpts o, int32_t *info, int num_sms,
+                                cudaStream_t st);
+int64_t update_tiles(int64_t m, int p);  // of a front, for block 0
+// a batch class's Solve in one block of 32 columns, its update and the tail
+cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
+                                       int count, const int *item_front, const int *item_tile, int64_t items,
+                                       const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
+                                       void *Lb, int pmax, int32_t *info, int num_sms, cudaStream_t st);
 
 // Threshold partial pivoting on all n rows (the comparator of the compressed path).
 size_t tpp_ws_bytes(int p);

@@ -22,8 +22,15 @@
 //   warps 2-17  epilogue: a thread holds 16 columns of one row of S as 64-bit
 //               integers; the accumulators are handed back as soon as they have
 //               been added up, and rounding and stores overlap the next tile.
-// Bound: tensor pipe for e from about 100 on, S traffic and the epilogue's integer
-// instructions below.  FP64 multiply-adds ran at 0.99 of the FP64 pipe's rate.
+// The same kernel, kMode kUpdate, is the Solve's update of the later columns of A21
+// with a block of 32 columns: A21(:, c0 + j) -= y L11(c0 + j, block)^T, all rows
+// by all j, one K block.
+// Bound: tensor pipe for e from about 100 on (n = 20000, p = e = 256: 2.26 ms, 1.6
+// PFLOP/s of executed products, against 80.6 ms for FP64 multiply-adds at 0.99 of
+// their pipe's rate); below, S traffic and the epilogue's instructions: the
+// update of 224 columns of 200000 rows took 446 us with 144 instructions per entry,
+// 210 with the test-free path, the 32-bit sums of neighbouring groups and the old
+// values brought to L2 ahead (HBM's share: 121 us).
 // Every mbarrier wait is bounded; on timeout the kernel records CTP_ETIMEOUT,
 // waits (bounded) for its copies in flight, frees its tensor memory and returns.
 #include "slices.cuh"
@@ -42,6 +49,7 @@ constexpr int kStages = 2;
 constexpr uint32_t kStageBytes = kWBlock + kLBlock;
 constexpr size_t kSmem = kStages * (size_t)kStageBytes + 1024;
 constexpr int kPanel = 8;  // column blocks of a panel of the walk
+constexpr int kUpdate = 100;  // kMode of the Solve's update (the others are a ctp_smode)
 
 struct Bars {
     unsigned long long full[kStages], empty[kStages], acc_full, acc_empty;
@@ -68,18 +76,16 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    tmem_wait_ld();
 }
 
 struct Tile {
-    int ti, tj, e;
-    int64_t m, lds, ldl;
+    int ti, tj, e, m, nc;  // m, nc: rows, columns (a Form: nc = m)
+    int64_t lds, ldl;
     SliceBuf sb;
     const double *L21, *D;
     const int32_t *piv;
@@ -102,6 +108,8 @@ struct Work {
     const int *item_front, *item_tile;
     BatchOpts o;
     int64_t count;  // items, or slots of the walk
+    int c0;         // kUpdate: first column updated, 32 past the block's first
+    int64_t nc;     // kUpdate, one supernode: columns updated
 };
 
 // The walk over one supernode's tiles: panels of kPanel column blocks, inside a
@@ -118,9 +126,45 @@ __host__ __device__ inline int64_t walk_slots(int64_t m) {
 }
 
 // The k-th tile of this CTA; false past the end.  ti < 0: a slot without a tile.
+template <bool kUpd>
 __device__ __forceinline__ bool tile_at(const Work &w, int64_t k, Tile &x) {
     const int64_t t = blockIdx.x + k * (int64_t)gridDim.x;
     if (t >= w.count) return false;
+    if (kUpd) {
+        // row block by row block, its column blocks one after another
+        int64_t q = t;
+        x.nc = (int)w.nc;
+        x.sb = w.sb;
+        x.m = (int)w.m;
+        x.e = w.fronts != nullptr ? 0 : *w.nelim;
+        x.L21 = w.L21;
+        x.ldl = w.ldl;
+        x.piv = w.piv;
+        if (w.fronts != nullptr) {
+            const int f = w.item_front[t];
+            const BFront b = w.tab[f];
+            const ctp_front &fr = w.fronts[f];
+            q = w.item_tile[t];
+            ctp_options oo;
+            oo.pivot = w.o.pivot;
+            oo.smode = w.o.smode;
+            oo.prec = w.o.prec;
+            x.sb = bsection_block(w.ws + b.ws, bsection(b.n, b.p, &oo));
+            x.m = (int)b.m;
+            x.nc = b.p - w.c0;
+            x.e = *fr.nelim;
+            x.L21 = fr.A + b.p;
+            x.ldl = fr.lda;
+            x.piv = fr.piv;
+        }
+        x.e = min(x.e - (w.c0 - kSliceK), kSliceK);
+        x.S = const_cast<double *>(x.L21 + (int64_t)w.c0 * x.ldl);
+        x.lds = x.ldl;
+        const int nN = (x.nc + kBN - 1) / kBN;
+        x.ti = x.e > 0 ? (int)(q / nN) : -1;  // nothing eliminated in the block: nothing to do
+        x.tj = (int)(q % nN);
+        return true;
+    }
     if (w.fronts != nullptr) {
         const int f = w.item_front[t];
         const BFront b = w.tab[f];
@@ -138,7 +182,7 @@ __device__ __forceinline__ bool tile_at(const Work &w, int64_t k, Tile &x) {
         const BSection sec = bsection(b.n, b.p, &oo);
         x.sb = bsection_slices(w.ws + b.ws, sec, b.p);
         const ctp_front &fr = w.fronts[f];
-        x.m = b.m;
+        x.m = x.nc = (int)b.m;
         x.e = *fr.nelim;
         x.L21 = fr.A + b.p;
         x.ldl = fr.lda;
@@ -149,7 +193,7 @@ __device__ __forceinline__ bool tile_at(const Work &w, int64_t k, Tile &x) {
         return true;
     }
     x.sb = w.sb;
-    x.m = w.m;
+    x.m = x.nc = (int)w.m;
     x.e = *w.nelim;
     x.L21 = w.L21;
     x.ldl = w.ldl;
@@ -173,49 +217,116 @@ __device__ __forceinline__ bool tile_at(const Work &w, int64_t k, Tile &x) {
     return true;
 }
 
-// V = 0, or V 2^ex outside the normal range of FP64
-__device__ __noinline__ double to_fp64_rare(long long V, int ex) {
-    return V == 0 ? 0.0 : scalbn((double)V, ex);
-}
-// V 2^ex rounded to nearest even, in integer instructions (the FP64 pipe takes
-// about 20 cycles per warp instruction and SM)
+// V 2^ex rounded to nearest even in integer instructions, for results in the normal
+// range of FP64 (the FP64 pipe takes 17 cycles per warp instruction and SM)
 __device__ __forceinline__ double to_fp64(long long V, int ex) {
     const unsigned long long a = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
     const int lz = __clzll((long long)a) & 63;
-    const unsigned long long n = a << lz;
-    unsigned long long mant = n >> 11;
-    mant += ((n >> 10) & 1u) & (((n & 0x3FFull) != 0ull ? 1u : 0u) | (unsigned)(mant & 1u));
-    const int be = 63 - lz + ex + 1022;  // biased exponent - 1: the hidden bit adds the 1
-    if ((unsigned)be >= 2045u || V == 0) return to_fp64_rare(V, ex);
-    const unsigned long long bits = ((unsigned long long)be << 52) + mant;
-    return __longlong_as_double((long long)(bits | ((unsigned long long)V & 0x8000000000000000ull)));
+    const unsigned long long n = a << lz, t = n >> 11;
+    const unsigned up = ((unsigned)n & 0x7FFu) + ((unsigned)t & 1u) > 0x400u ? 1u : 0u;
+    // biased exponent - 1 (the hidden bit adds the 1) and sign in the high word
+    const unsigned he = ((unsigned)(63 - lz + ex + 1022) << 20) | ((unsigned)(V >> 32) & 0x80000000u);
+    const unsigned long long bits = ((unsigned long long)he << 32) + t + up;
+    return V == 0 ? 0.0 : __longlong_as_double((long long)bits);
+}
+// any result
+__device__ __noinline__ double to_fp64_any(long long V, int ex) {
+    return ex > -900 && ex < 900 ? to_fp64(V, ex) : (V == 0 ? 0.0 : scalbn((double)V, ex));
 }
 
-// Entries (i, j..j+7) of S by FP64 multiply-adds over the stored L21 and D11 (i < m;
-// columns past i count as 0): the marked rows' path.
-__device__ __noinline__ void plain_entries(const double *L21, int64_t ldl, const double *D, const int32_t *piv, int e,
-                                          int64_t i, int64_t j, double (&acc)[8]) {
+// Entries (i, j..j+7) of the k-th tile's result by FP64 multiply-adds (i < m; columns
+// past the result count as 0): the marked rows' path.  It looks its tile up again,
+// so that the epilogue keeps no registers for it.
+template <bool kUpd>
+__device__ __noinline__ void plain_entries(const Work &wk, int64_t kt, int64_t i, int64_t j, double (&acc)[8]) {
+    Tile x;
+    tile_at<kUpd>(wk, kt, x);
 #pragma unroll
     for (int c = 0; c < 8; c++) acc[c] = 0.0;
-    for (int k = 0; k < e; k++) {
-        const int kd = piv[k];
+    const int first = kUpd ? wk.c0 - kSliceK : 0;
+    for (int k = first; k < first + x.e; k++) {
+        const int kd = x.piv[k];
         if (kd == CTP_PIVKIND_ZERO) continue;
-        const double *col = L21 + (int64_t)k * ldl;
-        double w = col[i] * D[2 * k];
-        if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(col[i + ldl], D[2 * k + 1], w);
-        if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(col[i - ldl], D[2 * k - 1], w);
+        const double *col = x.L21 + (int64_t)k * x.ldl;
+        double w = col[i];  // kUpd: y itself, in the block's columns of A21
+        const double *l = col;
+        if (kUpd) {
+            l = col - (x.nc + wk.c0) + wk.c0;  // rows c0.. of L11's column
+        } else {
+            w *= x.D[2 * k];
+            if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(col[i + x.ldl], x.D[2 * k + 1], w);
+            if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(col[i - x.ldl], x.D[2 * k - 1], w);
+        }
 #pragma unroll
-        for (int c = 0; c < 8; c++)
-            if (j + c <= i) acc[c] = fma(w, col[j + c], acc[c]);
+        for (int c = 0; c < 8; c++) {
+            const bool d21 = kUpd && wk.c0 + j + c == k + 1 && kd == CTP_PIVKIND_2X2_FIRST;  // that slot holds D
+            if (j + c <= (kUpd ? x.nc - 1 : i) && !d21) acc[c] = fma(w, l[j + c], acc[c]);
+        }
     }
 }
 
-// kMode: ctp_smode of S
+// The eight accumulators of 8 columns (group g at column g kBN) added up: V = sum_g
+// T_g 2^(40 + f - 8 g), the last two groups rounded to whole units.  kSmall (K
+// <= 32: every |T_g| <= 2^22): a float becomes an integer by adding 1.5 2^23 (its
+// mantissa bits then hold the integer, offset by a constant that is taken off at
+// the end), and two neighbouring groups fit one 32-bit integer; otherwise by the
+// conversion instruction, a quarter as fast.
+template <bool kSmall>
+__device__ __forceinline__ void add_groups(uint32_t ta, int f, long long *V) {
+    uint32_t r[8];
+    float low[8];
+    tmem_ld8(ta + 7 * kBN, r);
+    const float w7 = __int_as_float((127 + f - 16) << 23), w6 = __int_as_float((127 + f - 8) << 23);
+#pragma unroll
+    for (int c = 0; c < 8; c++) low[c] = __uint_as_float(r[c]) * w7;
+    tmem_ld8(ta + 6 * kBN, r);
+    if (kSmall) {
+        constexpr float kMagic = 12582912.0f;   // 1.5 2^23
+        constexpr unsigned kOff = 0x4B400000u;  // its bits
+        unsigned pr[8];
+#pragma unroll
+        for (int c = 0; c < 8; c++)  // |low| < 2^21: two groups of at most 2^22 by 2^(f - 8), f <= 6
+            V[c] = (int)(__float_as_uint(fmaf(__uint_as_float(r[c]), w6, low[c]) + kMagic) - kOff);
+#pragma unroll
+        for (int g = 4; g >= 0; g -= 2) {
+            tmem_ld8(ta + g * kBN, r);
+#pragma unroll
+            for (int c = 0; c < 8; c++) pr[c] = __float_as_uint(__uint_as_float(r[c]) + kMagic) * 256u - 257u * kOff;
+            tmem_ld8(ta + (g + 1) * kBN, r);
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                const int two = (int)(pr[c] + __float_as_uint(__uint_as_float(r[c]) + kMagic));
+                if (g > 0)  // groups 4, 5 weigh 2^f, groups 2, 3 2^(16 + f)
+                    V[c] += (long long)two * (1 << (32 - 8 * g + f));
+                else        // groups 0, 1 2^(32 + f): the high word
+                    V[c] += (long long)((unsigned long long)(unsigned)(two << f) << 32);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 8; c++) V[c] = __float2int_rn(fmaf(__uint_as_float(r[c]), w6, low[c]));
+#pragma unroll
+        for (int g = 5; g >= 0; g--) {
+            tmem_ld8(ta + g * kBN, r);
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                const int d = __float2int_rn(__uint_as_float(r[c]));
+                if (g > 1)
+                    V[c] += (long long)d * (1 << ((40 - 8 * g + f) & 31));
+                else  // weights 2^(32 + f) and 2^(40 + f): the high word
+                    V[c] += (long long)((unsigned long long)(unsigned)(d << (8 - 8 * g + f)) << 32);
+            }
+        }
+    }
+}
+
+// kMode: ctp_smode of S, or kUpdate
 template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_t *__restrict__ info) {
     using OutT = typename std::conditional<kMode == CTP_S_FP32 || kMode == CTP_S_FP32_PACKED, float, double>::type;
     constexpr bool kPacked = kMode == CTP_S_FP64_PACKED || kMode == CTP_S_FP32_PACKED;
-    constexpr bool kSub = kMode == CTP_S_FP64_SUB;
+    constexpr bool kUpd = kMode == kUpdate;
+    constexpr bool kSub = kMode == CTP_S_FP64_SUB || kUpd;
     extern __shared__ unsigned char smraw[];
     __shared__ Bars bars;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
@@ -243,11 +354,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
             uint32_t phase = 0;
             Tile x;
             bool ok = true;
-            for (int64_t k = 0; ok && tile_at(wk, k, x); k++) {
+            for (int64_t k = 0; ok && tile_at<kUpd>(wk, k, x); k++) {
                 if (x.ti < 0) continue;
                 // rows of the tile in use, in groups of 8
-                const uint32_t rw = (uint32_t)(min((int64_t)kBM, x.m - (int64_t)x.ti * kBM) + 7) & ~7u;
-                const uint32_t rl = (uint32_t)(min((int64_t)kBN, x.m - (int64_t)x.tj * kBN) + 7) & ~7u;
+                const uint32_t rw = (uint32_t)(min(kBM, x.m - x.ti * kBM) + 7) & ~7u;
+                const uint32_t rl = (uint32_t)(min(kBN, x.nc - x.tj * kBN) + 7) & ~7u;
                 const int KB = (x.e + kSliceK - 1) / kSliceK;
                 const unsigned char *srcW = x.sb.W + (size_t)x.ti * x.sb.kb * kWBlock;
                 const unsigned char *srcL = x.sb.L + (size_t)x.tj * x.sb.kb * kLBlock;
@@ -294,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
             uint32_t phase = 0, accphase = 0;
             Tile x;
             bool ok = true;
-            for (int64_t k = 0; ok && tile_at(wk, k, x); k++) {
+            for (int64_t k = 0; ok && tile_at<kUpd>(wk, k, x); k++) {
                 if (x.ti < 0) continue;
                 if (!mbar_wait(&bars.acc_empty, accphase ^ 1u, &bars.abort)) {
                     ok = false;
@@ -341,17 +452,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
         const int cg = (warp - 2) >> 2;                // its 16 columns of the tile
         uint32_t accphase = 0;
         Tile x;
-        for (int64_t k = 0; tile_at(wk, k, x); k++) {
+        for (int64_t k = 0; tile_at<kUpd>(wk, k, x); k++) {
             if (x.ti < 0) continue;
-            const int64_t i = (int64_t)x.ti * kBM + q * 32 + lane, j0 = (int64_t)x.tj * kBN + cg * kCols;
-            const int64_t m = x.m;
-            const bool any = j0 < m && j0 <= (int64_t)x.ti * kBM + q * 32 + 31 && i - lane < m;  // warp-uniform
-            const bool interior = (j0 + kCols - 1 <= (int64_t)x.ti * kBM + q * 32) && (i - lane + 31 < m);
-            OutT *S = reinterpret_cast<OutT *>(x.S);
-            OutT *ptr = S + (kPacked ? j0 * m - j0 * (j0 + 1) / 2 : j0 * x.lds) + i;
+            const int i = x.ti * kBM + q * 32 + lane, j0 = x.tj * kBN + cg * kCols, m = x.m;
+            // entries (i, j) with i < m and j <= jmax belong to the result
+            const int jmax = kUpd ? x.nc - 1 : i;
+            const bool any = j0 <= (kUpd ? jmax : i - lane + 31) && j0 < x.nc && i - lane < m;  // warp-uniform
+            const bool interior = j0 + kCols - 1 <= (kUpd ? jmax : i - lane) && i - lane + 31 < m;
+            OutT *ptr = reinterpret_cast<OutT *>(x.S) +
+                        (kPacked ? (int64_t)j0 * m - (int64_t)j0 * (j0 + 1) / 2 : j0 * x.lds) + i;
             int ei = kExpZero, ej = kExpZero;
             if (x.e > 0 && i < m) ei = x.sb.ew[i];
-            if (x.e > 0 && lane < kCols && j0 + lane < m) ej = x.sb.el[j0 + lane];
+            if (x.e > 0 && lane < kCols && j0 + lane < x.nc) ej = x.sb.el[j0 + lane];
+            // subtracting: the old values come to L2 while the products are computed
+            if (kSub && any && i < m) {
+#pragma unroll
+                for (int c = 0; c < kCols; c++)
+                    if (interior || j0 + c <= jmax)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr + (int64_t)c * x.lds));
+            }
             if (!mbar_wait(&bars.acc_full, accphase, &bars.abort)) {
                 if (lane == 0) atomicExch(&bars.abort, 1);
                 break;
@@ -363,30 +482,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
             long long V[kCols];
             if (any && x.e > 0) {
                 const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * kCols);
-                uint32_t r[16];
-                float low[kCols];
-                tmem_ld16_nowait(ta + 7 * kBN, r);
-                tmem_wait_ld();
-                const float w7 = __int_as_float((127 + f - 16) << 23), w6 = __int_as_float((127 + f - 8) << 23);
 #pragma unroll
-                for (int c = 0; c < kCols; c++) low[c] = __uint_as_float(r[c]) * w7;
-                tmem_ld16_nowait(ta + 6 * kBN, r);
-                tmem_wait_ld();
-#pragma unroll
-                for (int c = 0; c < kCols; c++) V[c] = __float2int_rn(fmaf(__uint_as_float(r[c]), w6, low[c]));
-#pragma unroll
-                for (int g = 5; g >= 0; g--) {
-                    tmem_ld16_nowait(ta + g * kBN, r);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < kCols; c++) {
-                        const int d = __float2int_rn(__uint_as_float(r[c]));
-                        if (g > 1)
-                            V[c] += (long long)d * (1 << ((40 - 8 * g + f) & 31));
-                        else  // weights 2^(32 + f) and 2^(40 + f): the high word
-                            V[c] += (long long)((unsigned long long)(unsigned)(d << (8 - 8 * g + f)) << 32);
-                    }
-                }
+                for (int h = 0; h < kCols; h += 8)
+                    if (kUpd || x.e <= 32)
+                        add_groups<true>(ta + h, f, V + h);
+                    else
+                        add_groups<false>(ta + h, f, V + h);
             }
             tc_fence_before();
             __syncwarp();
@@ -396,27 +497,47 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
             const bool wide_i = ei >= kExpWide / 2, wide_j = ej >= kExpWide / 2;
             const unsigned wides = __ballot_sync(0xffffffffu, wide_j);
             const bool any_wide = wides != 0u || __any_sync(0xffffffffu, wide_i);
+            // the plain case -- every entry of the warp's block belongs to the result, no
+            // row is marked, exponents are moderate -- has no test in its loop
+            const bool mild = abs(ei) < 400 && (lane >= kCols || abs(ej) < 400);
+            if (interior && !any_wide && __all_sync(0xffffffffu, mild)) {
 #pragma unroll
-            for (int h = 0; h < kCols; h += 8) {
-                double pl[8];
-                if (any_wide) {
-                    if (i < m) plain_entries(x.L21, x.ldl, x.D, x.piv, x.e, i, j0 + h, pl);
-                }
-                // subtracting: eight old values loaded before any is stored
-                double old[8];
-                if (kSub) {
+                for (int h = 0; h < kCols; h += 8) {
+                    double old[8];  // eight old values loaded before any is stored
+                    OutT *pl = ptr;
+                    if (kSub) {
+#pragma unroll
+                        for (int c = 0; c < 8; c++) {
+                            old[c] = *pl;
+                            pl += x.lds;
+                        }
+                    }
 #pragma unroll
                     for (int c = 0; c < 8; c++) {
-                        old[c] = 0.0;
-                        if (interior || (i < m && j0 + h + c <= i)) old[c] = ptr[(int64_t)c * x.lds];
+                        const double v = to_fp64(V[h + c], ei + __shfl_sync(0xffffffffu, ej, h + c) - 52 - f);
+                        if (kSub)
+                            *ptr = (OutT)(old[c] - v);
+                        else
+                            __stcs(ptr, (OutT)v);
+                        ptr += kPacked ? m - 1 - (j0 + h + c) : x.lds;
                     }
+                }
+                continue;
+            }
+#pragma unroll
+            for (int h = 0; h < kCols; h += 8) {
+                double pl[8], old[8];
+                if (any_wide && i < m) plain_entries<kUpd>(wk, k, i, j0 + h, pl);
+                if (kSub) {
+#pragma unroll
+                    for (int c = 0; c < 8; c++) old[c] = i < m && j0 + h + c <= jmax ? ptr[(int64_t)c * x.lds] : 0.0;
                 }
 #pragma unroll
                 for (int c = 0; c < 8; c++) {
                     const int ex = ei + __shfl_sync(0xffffffffu, ej, h + c) - 52 - f;
-                    double v = x.e > 0 ? to_fp64(V[h + c], ex) : 0.0;
-                    if (any_wide && (wide_i || ((wides >> (h + c)) & 1u))) v = pl[c];
-                    if (interior || (i < m && j0 + h + c <= i)) {
+                    if (i < m && j0 + h + c <= jmax) {
+                        double v = x.e > 0 ? to_fp64_any(V[h + c], ex) : 0.0;
+                        if (any_wide && (wide_i || ((wides >> (h + c)) & 1u))) v = pl[c];
                         if (kSub)
                             *ptr = (OutT)(old[c] - v);
                         else
@@ -481,6 +602,7 @@ cudaError_t launch_any(const Work &wk, int smode, int32_t *info, int num_sms, cu
     case CTP_S_FP64: return launch_mode<CTP_S_FP64>(wk, info, num_sms, st);
     case CTP_S_FP32: return launch_mode<CTP_S_FP32>(wk, info, num_sms, st);
     case CTP_S_FP64_SUB: return launch_mode<CTP_S_FP64_SUB>(wk, info, num_sms, st);
+    case kUpdate: return launch_mode<kUpdate>(wk, info, num_sms, st);
     case CTP_S_FP64_PACKED: return launch_mode<CTP_S_FP64_PACKED>(wk, info, num_sms, st);
     default: return launch_mode<CTP_S_FP32_PACKED>(wk, info, num_sms, st);
     }
@@ -519,6 +641,42 @@ cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, c
     wk.o = o;
     wk.count = items;
     return launch_any(wk, o.smode, info, num_sms, st);
+}
+
+cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int64_t m, int blk, const int32_t *piv,
+                          const int32_t *nelim, int32_t *info, int num_sms, cudaStream_t st) {
+    Work wk = {};
+    wk.sb = u;
+    wk.L21 = A + p;
+    wk.ldl = lda;
+    wk.piv = piv;
+    wk.m = m;
+    wk.nelim = nelim;
+    wk.c0 = (blk + 1) * kSliceK;
+    wk.nc = p - wk.c0;
+    wk.count = (m + kBM - 1) / kBM * ((wk.nc + kBN - 1) / kBN);
+    if (wk.count <= 0) return cudaSuccess;
+    return launch_any(wk, kUpdate, info, num_sms, st);
+}
+
+int64_t update_tiles(int64_t m, int p) {
+    return p > kSliceK ? (m + kBM - 1) / kBM * ((p - kSliceK + kBN - 1) / kBN) : 0;
+}
+
+cudaError_t launch_update_batch(const ctp_front *fronts, const BFront *tab, char *ws, const int *item_front,
+                                const int *item_tile, int64_t items, BatchOpts o, int32_t *info, int num_sms,
+                                cudaStream_t st) {
+    if (items == 0) return cudaSuccess;
+    Work wk = {};
+    wk.fronts = fronts;
+    wk.tab = tab;
+    wk.ws = ws;
+    wk.item_front = item_front;
+    wk.item_tile = item_tile;
+    wk.o = o;
+    wk.c0 = kSliceK;
+    wk.count = items;
+    return launch_any(wk, kUpdate, info, num_sms, st);
 }
 
 cudaError_t launch_slices_from_l(const double *A, int64_t lda, int p, int64_t m, const int32_t *piv,

@@ -19,15 +19,15 @@
 //
 // Accuracy: a digit product with s + t > 7 is dropped and X is cut at 2^-62, in
 // all about 2^-62 e^(1/2) of the two rows' scales 2^(E_i + E_j): less than the
-// rounding of e FP64 multiply-adds wherever the large entries of the two rows
-// meet in the same columns, as they do when the rows share a profile (random
-// data; the growth of the pivots' columns, common to all rows).  Rows whose
-// entries scatter widely about the profile are not good enough for that (wide
-// random scales: entries of S lost up to 8 bits): a row that lies more than
-// kWideBits per entry below its tile's profile (per column the largest entry,
-// relative to its row's scale, of the tile's 32 rows) is marked, as is one with
-// an Inf or NaN, by kExpWide added to its exponent, and the Form takes its
-// entries of S by FP64 multiply-adds.
+// rounding of e FP64 multiply-adds wherever the large entries of one row meet
+// entries of the other that are not much below its own largest, as they do in
+// random data and under the growth of the pivots' columns, which all rows share.
+// A row is marked, by kExpWide added to its exponent, when none of its entries
+// does -- in no column is its entry, relative to its scale, times the typical
+// entry (the geometric mean of the nonzero ones of the tile's 32 rows, relative
+// to theirs) above 2^-kWideBits -- or when it holds an Inf or NaN, and the Form
+// takes its entries of S by FP64 multiply-adds.  (Entries scattered over 2^40
+// lost up to 8 bits without the mark.)
 //
 // Layout (what a bulk copy puts into shared memory as the MMA reads it): W in
 // blocks of 128 rows, L in blocks of 64; per row block and block of 32 pivots
@@ -112,23 +112,22 @@ __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t ro
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kWarps; q++) E = max(E, red[q * 32 + lane]);
-    int sum = 0;  // 512 * (bits below the profile) + entries counted
+    int best = kExpZero;  // the row's best column: log2 of its entry times the typical one
     for (int k = w; k < e; k += kWarps) {
         if (cexp[k] == kSliceSkip) continue;
         const int x = slice_exp(xs[k * LDX + lane], sgn * cexp[k]);
         const bool in = x > kExpZero && x < kExpNonfinite;
-        const int rel = in ? x - E : -kExpNonfinite;
-        const int prof = __reduce_max_sync(0xffffffffu, rel);
-        if (in) sum += 512 * (prof - rel) + 1;
+        const int cnt = __popc(__ballot_sync(0xffffffffu, in));
+        const int sum = __reduce_add_sync(0xffffffffu, in ? E - x : 0);
+        if (in) best = max(best, x - E - sum / cnt);
     }
-    red[(kWarps + w) * 32 + lane] = sum;
+    red[(kWarps + w) * 32 + lane] = best;
     __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int q = 1; q < kWarps; q++) sum += red[(kWarps + q) * 32 + lane];
+        for (int q = 1; q < kWarps; q++) best = max(best, red[(kWarps + q) * 32 + lane]);
         rexp[lane] = E;
-        const int cnt = sum & 511;
-        const bool wide = E >= kExpNonfinite || (sum >> 9) > kWideBits * cnt + 8;
+        const bool wide = E >= kExpNonfinite || (E > kExpZero && best < -kWideBits);
         if (lane < nrows) rowexp[row0 + lane] = wide ? E + kExpWide : E;
     }
     __syncthreads();

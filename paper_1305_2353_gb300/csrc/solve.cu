@@ -65,6 +65,25 @@ __device__ __forceinline__ void write_pieces(__nv_bfloat16 *__restrict__ B, int6
     }
 }
 
+// What a pass over a tile does.  A whole Solve in one pass updates every later
+// column with every y_j in FP64: p^2/2 multiply-adds per row on a pipe of 2 per
+// clock and SM (n = 200000, p = e = 256: 12.9 ms, 0.8 of that pipe).  The blocked
+// Solve (3.4 ms: 1.9 ms in the diagonal blocks, 0.84 in the updates, 0.3 in the
+// tail) keeps only the 32-column diagonal blocks of
+// that and leaves the rest -- columns times y's block by block -- to the
+// tensor cores, as products of exact digit slices (k_update in form.cu):
+//   kFirst  gather through perm, eliminate the first block inside itself, write
+//           the row in pivot order and the block's slices;
+//   kNext   the same for block blk (its columns are in place by now);
+//   kTail   after the last block's update: the rest of the elimination, if blocks
+//           were left out, then the outputs as in a whole pass.
+enum { kWhole, kFirst, kNext, kTail };
+struct SolvePass {
+    int mode;
+    int blk;      // kNext: the block; kTail: how many blocks are done
+    SliceBuf yb;  // slices of the block's y (kFirst, kNext)
+};
+
 // Right-looking substitution over a tile of 32 rows: for each eliminated
 // position j, every warp reads y_j of its lane's row and updates its share of
 // the later columns (four independent updates in flight per warp); a CTA
@@ -77,7 +96,7 @@ __device__ __forceinline__ void write_pieces(__nv_bfloat16 *__restrict__ B, int6
 // pieces > 1: also write the further BF16 pieces of the split operands (piece
 // k rounds what pieces 0..k-1 left), lo_off elements apart.  sb: the slices of
 // the FP64 Form (sb.W null: none).
-__device__ __forceinline__ void solve_tile(double *__restrict__ A, int64_t n, int p, int64_t lda,
+__device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                                            const int32_t *__restrict__ perm,
                                            const int32_t *__restrict__ piv,
                                            const double *__restrict__ Dinv, int e, const SliceBuf &sb,
@@ -91,42 +110,74 @@ __device__ __forceinline__ void solve_tile(double *__restrict__ A, int64_t n, in
     const int64_t row = row0 + lane;
     const bool valid = row < m;
     double *A21 = A + p;
+    const bool part = ps.mode == kFirst || ps.mode == kNext;
+    // pivots j0..j1-1 update columns below ku; xs holds columns c0..c1-1
+    const int c0 = ps.mode == kNext ? ps.blk * kSliceK : 0;
+    const int j0 = ps.mode == kTail ? min(ps.blk * kSliceK, e) : c0;
+    const int j1 = part ? min(c0 + kSliceK, e) : e;
+    const int ku = part ? min(c0 + kSliceK, p) : p;
+    const int c1 = ps.mode == kNext ? ku : (ps.mode == kTail && j0 == e ? e : p);
+    if (ps.mode == kNext && c0 >= e) return;  // the whole CTA
 
     // gather x = A21(rows, perm): each warp reads 32 consecutive rows of a column
-    for (int k = w; k < p; k += kWarps) {
-        const int c = perm[k];
-        xs[k * LDX + lane] = valid ? A21[(int64_t)c * lda + row] : 0.0;
+    // (eight columns' loads in flight per warp)
+#pragma unroll 1
+    for (int k0 = c0 + w; k0 < c1; k0 += 8 * kWarps) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const int k = k0 + q * kWarps;
+            v[q] = 0.0;
+            if (k < c1 && valid) v[q] = A21[(int64_t)(ps.mode <= kFirst ? perm[k] : k) * lda + row];
+        }
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+            if (k0 + q * kWarps < c1) xs[(k0 + q * kWarps - c0) * LDX + lane] = v[q];
     }
     __syncthreads();
 
-    for (int j = 0; j < e;) {
+    for (int j = j0; j < j1;) {
         const int kd = piv[j];
-        if (kd == CTP_PIVKIND_2X2_FIRST) {
-            const double y0 = xs[j * LDX + lane], y1 = xs[(j + 1) * LDX + lane];
+        if (kd == CTP_PIVKIND_2X2_FIRST && j + 1 < j1) {
+            const double y0 = xs[(j - c0) * LDX + lane], y1 = xs[(j + 1 - c0) * LDX + lane];
             const double *l0 = A + (int64_t)j * lda, *l1 = A + (int64_t)(j + 1) * lda;
 #pragma unroll 4
-            for (int k = j + 2 + w; k < p; k += kWarps)
-                xs[k * LDX + lane] -= y0 * __ldg(l0 + k) + y1 * __ldg(l1 + k);
+            for (int k = j + 2 + w; k < ku; k += kWarps)
+                xs[(k - c0) * LDX + lane] -= y0 * __ldg(l0 + k) + y1 * __ldg(l1 + k);
             j += 2;
         } else {
-            if (kd == CTP_PIVKIND_1X1) {
-                const double y0 = xs[j * LDX + lane];
+            // (a 2x2 pair that a block boundary cuts: its first column has nothing left
+            // to update in its block, its second is a column like any other)
+            if (kd == CTP_PIVKIND_1X1 || kd == CTP_PIVKIND_2X2_SECOND) {
+                const double y0 = xs[(j - c0) * LDX + lane];
                 const double *l0 = A + (int64_t)j * lda;
 #pragma unroll 4
-                for (int k = j + 1 + w; k < p; k += kWarps) xs[k * LDX + lane] -= y0 * __ldg(l0 + k);
+                for (int k = j + 1 + w; k < ku; k += kWarps) xs[(k - c0) * LDX + lane] -= y0 * __ldg(l0 + k);
             }
             j += 1;  // zero pivots have an all-zero L column
         }
         __syncthreads();
     }
 
+    const int tile_rows = m - row0 < kRows ? (int)(m - row0) : kRows;
+    __shared__ short cexp[kMaxP];
+    __shared__ int red[2 * kWarps * 32], rexp[32];
+    if (part) {
+        if (c0 + kSliceK < p) {  // columns are left to update
+            for (int k = c0 + threadIdx.x; k < j1; k += blockDim.x) cexp[k - c0] = (short)slice_col_exp(piv, Dinv, k);
+            __syncthreads();
+            write_slices<kWRows, kWarps>(xs, j1 - c0, row0, tile_rows, cexp, -1, ps.yb.W, ps.yb.ew, ps.yb.kb, red,
+                                         rexp);
+        }
+        if (valid)
+            for (int k = c0 + w; k < c1; k += kWarps) A21[(int64_t)k * lda + row] = xs[(k - c0) * LDX + lane];
+        return;
+    }
+
     // the Form's copies of Y = W21.  BF16 pieces: row-major, K contiguous,
     // zero from e to the end of e's last 64-wide K block (the Form reads no
     // further; a batch's rows are 256 wide whatever the front's p)
     const int Kz = min(Kp, (e + 63) / 64 * 64);
-    const int tile_rows = m - row0 < kRows ? (int)(m - row0) : kRows;
-    __shared__ short cexp[kMaxP];
-    __shared__ int red[2 * kWarps * 32], rexp[32];
     if (sb.W != nullptr) {
         for (int k = threadIdx.x; k < e; k += blockDim.x) cexp[k] = (short)slice_col_exp(piv, Dinv, k);
         __syncthreads();
@@ -136,7 +187,7 @@ __device__ __forceinline__ void solve_tile(double *__restrict__ A, int64_t n, in
     __syncthreads();
     // L21 = Y D11^{-1} in place (1x1 and 2x2 blocks; zero pivots give 0), written
     // back with the delayed columns as they are
-    for (int k = w; k < p; k += kWarps) {
+    for (int k = w; k < c1; k += kWarps) {
         const int kd = k < e ? piv[k] : CTP_PIVKIND_DELAYED;
         if (kd == CTP_PIVKIND_2X2_SECOND) continue;  // with its first column
         double out = xs[k * LDX + lane];
@@ -162,20 +213,19 @@ __device__ __forceinline__ void solve_tile(double *__restrict__ A, int64_t n, in
 }
 
 __global__ void __launch_bounds__(kRows * kWarps)
-    k_solve_fp64(double *__restrict__ A, int64_t n, int p, int64_t lda,
+    k_solve_fp64(SolvePass ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                  const int32_t *__restrict__ perm, const int32_t *__restrict__ piv,
                  const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p,
                  SliceBuf sb, __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb, int Kp,
                  int64_t lo_off, int pieces) {
-    extern __shared__ __align__(16) double xs[];  // [p][kRows+1]
-    solve_tile(A, n, p, lda, perm, piv, Dinv, *nelim_p, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
+    extern __shared__ __align__(16) double xs[];  // [columns][kRows+1]
+    solve_tile(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
 }
 
 // Batched: CTA b takes work item b = (front, 32-row tile of its A21): the
-// front is item_front[b], the tile item_tile[b] (or, without that list, the
-// item's place among the front's consecutive items).
+// front is item_front[b], the tile item_tile[b].
 __global__ void __launch_bounds__(kRows * kWarps)
-    k_solve_batch(const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
+    k_solve_batch(int mode, const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
                   const int *__restrict__ item_front, const int *__restrict__ item_tile, BatchOpts o,
                   __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb) {
     extern __shared__ __align__(16) double xs[];
@@ -190,28 +240,115 @@ __global__ void __launch_bounds__(kRows * kWarps)
     char *base = ws + bt.ws;
     SliceBuf sb = {nullptr, nullptr, nullptr, nullptr, 0};
     if (o.smode != CTP_S_NONE && o.prec == CTP_FP64) sb = bsection_slices(base, sec, bt.p);
-    solve_tile(fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
+    SolvePass ps = {mode, mode == kTail ? 1 : 0, {nullptr, nullptr, nullptr, nullptr, 0}};
+    if (mode == kFirst) ps.yb = bsection_block(base, sec);
+    solve_tile(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
                *fr.nelim, sb, Wb, Lb, kBatchKp, bt.row0, o.lo_off, o.pieces,
-               item_tile != nullptr ? (int64_t)item_tile[blockIdx.x] : (int64_t)blockIdx.x - bt.s0, xs);
+               item_tile[blockIdx.x], xs);
 }
 
+// Slices of L11's rows below block blk, columns of the block: what the block's y
+// are multiplied with.  One 32-row tile (rows r0.. in pivot order) per CTA; row r
+// is row r - 32 (blk + 1) of the image.
+__device__ __forceinline__ void l11_tile(const double *__restrict__ A, int64_t lda, int p, int blk, int r0,
+                                         const int32_t *__restrict__ piv, const double *__restrict__ Dinv, int e,
+                                         const SliceBuf &lb) {
+    constexpr int LDX = kRows + 1;
+    __shared__ double xs[kSliceK * LDX];
+    __shared__ short cexp[kSliceK];
+    __shared__ int red[2 * kWarps * 32], rexp[32];
+    const int c0 = blk * kSliceK, cnt = min(kSliceK, e - c0), first = c0 + kSliceK;
+    if (cnt <= 0 || r0 < first || r0 >= p) return;  // the whole CTA
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r = r0 + lane;
+    for (int k = threadIdx.x; k < cnt; k += kRows * kWarps) cexp[k] = (short)slice_col_exp(piv, Dinv, c0 + k);
+    for (int k = w; k < cnt; k += kWarps) {
+        const int c = c0 + k;
+        const bool d21 = r == c + 1 && piv[c] == CTP_PIVKIND_2X2_FIRST;  // that slot holds D
+        xs[k * LDX + lane] = (r < p && !d21) ? A[(int64_t)c * lda + r] : 0.0;
+    }
+    __syncthreads();
+    write_slices<kLRows, kWarps>(xs, cnt, r0 - first, min(kRows, p - r0), cexp, 1, lb.L, lb.el, lb.kb, red, rexp);
+}
+__global__ void __launch_bounds__(kRows * kWarps)
+    k_l11_slices(const double *__restrict__ A, int64_t lda, int p, const int32_t *__restrict__ piv,
+                 const double *__restrict__ Dinv, const int32_t *__restrict__ nelim, SliceBuf lb, size_t blk_bytes) {
+    lb.L += blockIdx.y * blk_bytes;
+    lb.el += blockIdx.y * kMaxP;
+    l11_tile(A, lda, p, blockIdx.y, blockIdx.x * kRows, piv, Dinv, *nelim, lb);
+}
+__global__ void __launch_bounds__(kRows * kWarps)
+    k_l11_slices_batch(const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
+                       const int *__restrict__ list, BatchOpts o) {
+    const int f = list[blockIdx.x];
+    const ctp_front fr = fronts[f];
+    const BFront bt = tab[f];
+    ctp_options oo;
+    oo.pivot = o.pivot;
+    oo.smode = o.smode;
+    oo.prec = o.prec;
+    if (bt.m == 0) return;  // no rows to solve for, and no room for slices in its section
+    const BSection sec = bsection(bt.n, bt.p, &oo);
+    char *base = ws + bt.ws;
+    l11_tile(fr.A, fr.lda, bt.p, 0, (blockIdx.y + 1) * kRows, fr.piv,
+             reinterpret_cast<const double *>(base + sec.Dinv), *fr.nelim, bsection_block(base, sec));
+}
 
 }  // namespace
 
+// How many 32-column blocks the blocked Solve of an m x p supernode takes, 0 for a
+// whole pass.  Blocked, a Solve is 2 + 2 blocks launches (e is not known on the
+// host; blocks past it exit at once, about 2 us each).  Strict and single-row
+// pivoting accept few columns (12 of 256 on random data, 30 in large
+// multifrontal panels): one block, and what it leaves goes with the tail.
+// Measured, whole / blocked, all columns accepted: p = 256 from m = 344 on (498 /
+// 313 us; n = 200000: 12869 / 3413); p = 160, m = 240: 254 / 205; p = 128, m = 1372:
+// 170 / 164; p = 96, m = 2904: 108 / 117, m = 11904: 160 / 133; p = 64, m = 11936: 84 / 88,
+// m = 23936: 113 / 104.  A dozen accepted: p = 192, m = 208: 45 / 43; p = 160, m =
+// 2840: 41 / 41, m = 11840: 70 / 53; p = 128, m = 5872: 41 / 43, m = 11872: 57 / 53; p = 96, m
+// = 11904: 43 / 49; p = 64, m = 23936: 41 / 53, m = 99936: 149 / 131.
+int solve_blocks(int64_t m, int p, int pivot) {
+    if (p <= kSliceK || m <= 0) return 0;
+    const double right = (double)m * (p - kSliceK);  // entries the first block's update touches
+    if (pivot == CTP_PIV_STRICT || pivot == CTP_PIV_SINGLE_ROW)
+        return p > 176 || right >= (p > 96 ? 1e6 : 2.5e6) ? 1 : 0;
+    return p > 128 || right * (p - kSliceK) >= 1.6e7 ? (p + kSliceK - 1) / kSliceK : 0;
+}
+
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
-                              const SliceBuf &sb, void *Wb, void *Lb, int Kp, int64_t lo_off, int pieces,
-                              cudaStream_t st) {
+                              const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
+                              int64_t lo_off, int pieces, int32_t *info, int num_sms, cudaStream_t st) {
     const int64_t m = n - p;
     if (m <= 0) return cudaSuccess;
-    size_t smem = sizeof(double) * (size_t)p * (kRows + 1);
-    cudaError_t err =
-        smem_at_least((const void *)k_solve_fp64, smem);
+    cudaError_t err = smem_at_least((const void *)k_solve_fp64, sizeof(double) * (size_t)p * (kRows + 1));
     if (err != cudaSuccess) return err;
-    int64_t grid = (m + kRows - 1) / kRows;
-    k_solve_fp64<<<(unsigned)grid, kRows * kWarps, smem, st>>>(
-        A, n, p, lda, perm, piv, Dinv, nelim, sb, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, Kp, lo_off, pieces);
-    return cudaGetLastError();
+    const unsigned grid = (unsigned)((m + kRows - 1) / kRows);
+    auto pass = [&](int mode, int b, int cols) {
+        const SolvePass ps = {mode, b, blk};
+        k_solve_fp64<<<grid, kRows * kWarps, sizeof(double) * (size_t)cols * (kRows + 1), st>>>(
+            ps, A, n, p, lda, perm, piv, Dinv, nelim, sb, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, Kp, lo_off, pieces);
+        return cudaGetLastError();
+    };
+    if (blocks == 0) return pass(kWhole, 0, p);
+    const size_t lbytes = slice_l_bytes(p, kSliceK);
+    if (p > kSliceK) {
+        const int nb = blocks < (p - 1) / kSliceK ? blocks : (p - 1) / kSliceK;  // the last block has nothing below
+        k_l11_slices<<<dim3((unsigned)((p + kRows - 1) / kRows), (unsigned)nb), kRows * kWarps, 0, st>>>(
+            A, lda, p, piv, Dinv, nelim, blk, lbytes);
+        err = cudaGetLastError();
+        if (err != cudaSuccess) return err;
+    }
+    for (int b = 0; b < blocks; b++) {
+        err = b == 0 ? pass(kFirst, 0, p) : pass(kNext, b, kSliceK);
+        if (err != cudaSuccess) return err;
+        if ((b + 1) * kSliceK >= p) break;
+        SliceBuf u = blk;
+        u.L += b * lbytes;
+        u.el += b * kMaxP;
+        err = launch_update(u, A, lda, p, m, b, piv, nelim, info, num_sms, st);
+        if (err != cudaSuccess) return err;
+    }
+    return pass(kTail, blocks, p);
 }
 
 cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char *ws,
@@ -223,7 +360,30 @@ cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char 
         smem_at_least((const void *)k_solve_batch, smem);
     if (err != cudaSuccess) return err;
     k_solve_batch<<<(unsigned)items, kRows * kWarps, smem, st>>>(
-        fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
+        kWhole, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
+                                       int count, const int *item_front, const int *item_tile, int64_t items,
+                                       const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
+                                       void *Lb, int pmax, int32_t *info, int num_sms, cudaStream_t st) {
+    if (items == 0) return cudaSuccess;
+    const size_t smem = sizeof(double) * (size_t)pmax * (kRows + 1);
+    cudaError_t err = smem_at_least((const void *)k_solve_batch, smem);
+    if (err != cudaSuccess) return err;
+    if (pmax > kSliceK) {
+        const unsigned tiles = (unsigned)((pmax - 1) / kRows);  // 32-row tiles below the first block
+        k_l11_slices_batch<<<dim3((unsigned)count, tiles), kRows * kWarps, 0, st>>>(fronts, tab, ws, list, o);
+        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    }
+    k_solve_batch<<<(unsigned)items, kRows * kWarps, smem, st>>>(
+        kFirst, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    err = launch_update_batch(fronts, tab, ws, uitem, utile, uitems, o, info, num_sms, st);
+    if (err != cudaSuccess) return err;
+    k_solve_batch<<<(unsigned)items, kRows * kWarps, smem, st>>>(
+        kTail, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
     return cudaGetLastError();
 }
 
