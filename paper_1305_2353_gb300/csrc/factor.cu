@@ -32,6 +32,14 @@
 //   update       every CTA copies the pivot column(s), takes the per-column
 //                scalars from them and applies the 1x1 or 2x2 update to its own
 //                live columns (one CTA barrier, then the team barrier).
+// When the next candidate has no partner (no live column before it, as while
+// pivots are accepted in order), its test needs its own column only: the
+// update brings that column up to date first and one warp tests it while the others go
+// on, which saves the test round and its barrier: 1527 -> 1134 us at p = 256 on
+// 16 CTAs, 504 -> 403 at p = 128 on 8, 227 -> 188 at p = 64 on one (relaxed, all
+// accepted), with the columns split between warps once there are fewer of them.
+// What is left of a pivot at p = 256 (8400 clocks) is the multipliers, which every CTA
+// computes for all rows (4700 with the remote reads), and the update (FP64 work 1700).
 // The warp kernel runs the same tests one candidate at a time.
 // Columns are never moved: accepted pivots leave the live set, and because the
 // paper's stable shift never reorders the remaining columns, the candidate
@@ -81,6 +89,8 @@ struct Shared {
     unsigned short lrow[kMaxP];  // the live A11 rows, ascending (rebuilt before each update)
     unsigned short lpos[kMaxP];  // lpos[i]: how many live rows lie above row i
     int nlive;
+    unsigned short ocol[kMaxP];  // this CTA's live columns, ascending (rebuilt with lrow)
+    int nown;
 };
 
 // The team that owns one front: a cluster of G CTAs, or one CTA.
@@ -209,6 +219,44 @@ __device__ __forceinline__ Decision test_candidate(int c, const double *cm, ColP
     return d;
 }
 
+// The same for a candidate without partner, the first of the nl live rows in lrow:
+// its own column is all the test needs.
+__device__ __forceinline__ Decision test_first(const double *cm, const unsigned short *lrow, int nl, int p, int R,
+                                               double u, unsigned long long small_k) {
+    const int lane = threadIdx.x & 31, c = lrow[0], len = nl + R;
+    Decision d;
+    d.kind = DEC_REJECT;
+    d.t = -1;
+    d.m = c;
+    d.pad = 0;
+    d.d1 = d.d2 = d.i1 = d.i2 = 0.0;
+    const double amm = cm[c];
+    d.d0 = amm;
+    d.i0 = __drcp_rn(amm);
+    unsigned long long vm = 0;
+    constexpr int U = 4;
+    for (int j0 = 1 + lane; j0 < len; j0 += 32 * U) {
+        double x[U];
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            const int j = j0 + 32 * q;
+            x[q] = j < len ? cm[j < nl ? (int)lrow[j] : p + (j - nl)] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            const unsigned long long k = akey(x[q]);
+            vm = k > vm ? k : vm;
+        }
+    }
+    vm = warp_max_key(vm);
+    const unsigned long long kmm = akey(amm);
+    if ((vm > kmm ? vm : kmm) < small_k)
+        d.kind = DEC_ZERO;
+    else if (kmm >= akey(__dmul_rn(u, key_val(vm))))
+        d.kind = DEC_1X1;
+    return d;
+}
+
 template <bool kSingle>
 __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
     Team<kSingle> team;
@@ -317,6 +365,7 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
     int win = 1;                  // candidates tested in the next round
     const int win_max = kNW * G;  // no CTA owns more than kNW of them
     int m0 = m;                   // where the search for the next pivot began
+    bool pre = false;             // candidate m was tested behind the last update
     for (;;) {
         if (nelim >= p) break;
         while (m < p && !sh.live[m]) m++;
@@ -335,11 +384,11 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
         // with no pass, so accepted-first candidates cost a single test and runs
         // of rejections are tested in parallel (a rejection is cheap: most are
         // settled by the FP32 filters).
-        const int hi = min(p, m + win);  // the same on every CTA
+        const int hi = pre ? m + 1 : min(p, m + win);  // the same on every CTA
         // A round of one candidate (every round while pivots are accepted as they
         // come): the first warp of the CTA that owns column m tests it and writes
         // the outcome to every CTA; nothing to hand out or to collect.
-        const bool one = win == 1;
+        const bool one = pre || win == 1;
         if (!one) {
             if (warp == 0) {
                 // this CTA's live columns in [m, hi), in order, go to its warps
@@ -353,7 +402,7 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             }
             __syncthreads();
         }
-        {
+        if (!pre) {
             const int c = one ? ((warp == 0 && (m & gm) == rank) ? m : -1) : sh.cand[warp];
             if (c >= 0) {
                 Decision d = test_candidate(c, cols + (size_t)(c >> gs) * LD, colptr, sh.live, p, LD, u, rcp_u,
@@ -369,7 +418,8 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
                 }
             }
         }
-        team.sync();
+        if (!pre) team.sync();
+        pre = false;
         int cstar;
         if (one) {
             cstar = sh.one[buf].kind != DEC_REJECT ? m : p;
@@ -486,6 +536,17 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
                     rl1[i] = ab ? l1 : neg_bits(l1);
                 }
             }
+            if (warp == kNW - 1) {  // the own live columns without the pivots'
+                int r = 0;
+                for (int l0 = 0; l0 < ncl; l0 += 32) {
+                    const int c = ((l0 + lane) << gs) + rank;
+                    const bool ok = l0 + lane < ncl && c < p && c != q0 && c != q1 && sh.live[c];
+                    const unsigned int bal = __ballot_sync(0xffffffffu, ok);
+                    if (ok) sh.ocol[r + __popc(bal & ((1u << lane) - 1u))] = (unsigned short)c;
+                    r += __popc(bal);
+                }
+                if (lane == 0) sh.nown = r;
+            }
             if (tid == 0) {
                 sh.nlive -= q1 < 0 ? 1 : 2;
                 if (q1 < 0) {
@@ -515,11 +576,10 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             }
         }
         __syncthreads();
-        // the update: warp w takes the own live columns w, w + kNW, ...; one fused
-        // multiply-add per pivot column: -l(i) a(c,q), or +l(i) |a(c,q)| on the
-        // abs rows (eq. (4.3)).  The entry (c, i) above the diagonal, in row i's
-        // column, is the same product (row i's multiplier, row c's pivot entry)
-        // on the same old value (the working matrix is symmetric).  One CTA
+        // the update: one fused multiply-add per pivot column: -l(i) a(c,q), or
+        // +l(i) |a(c,q)| on the abs rows (eq. (4.3)).  The entry (c, i) above the
+        // diagonal, in row i's column, is the same product (row i's multiplier, row c's
+        // pivot entry) on the same old value (the working matrix is symmetric).  One CTA
         // updates the live A11 rows from the diagonal down and stores each result
         // into its mirror too, so the upper half costs a store instead of a
         // second FP64 update.  In a cluster the mirror lies in another CTA's
@@ -531,33 +591,64 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
         // 1x1 and 2x2 pivots have loops of their own: a predicated-off FP64
         // instruction takes its turn in the pipe all the same.  (Several rows per
         // lane in flight were slower: 1882 us with four.)
-        {
-            const int nl = sh.nlive;
-            for (int lc = warp; lc < ncl; lc += kNW) {
-                const int c = (lc << gs) + rank;
-                if (c >= p || !sh.live[c]) continue;  // warp-uniform
-                const int a0 = kSingle ? sh.lpos[c] : 0, lenA = nl - a0, len = lenA + R;
-                double *col = cols + (size_t)lc * LD;
-                const double q0c = pc0[c], aq0c = abs_rows ? apc0[c] : q0c, l0c = rl0[c];
-                if (q1 < 0) {
-                    for (int j = lane; j < len; j += 32) {
-                        const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
-                        const bool up = !kSingle && i < c;
-                        const double v = fma(up ? l0c : rl0[i], up ? pc0[i] : (i >= p ? aq0c : q0c), col[i]);
-                        col[i] = v;
-                        if (kSingle && i < p && i != c) cols[(size_t)i * LD + c] = v;
-                    }
-                } else {
-                    const double q1c = pc1[c], aq1c = abs_rows ? apc1[c] : q1c, l1c = rl1[c];
-                    for (int j = lane; j < len; j += 32) {
-                        const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
-                        const bool up = !kSingle && i < c;
-                        double v = fma(up ? l0c : rl0[i], up ? pc0[i] : (i >= p ? aq0c : q0c), col[i]);
-                        v = fma(up ? l1c : rl1[i], up ? pc1[i] : (i >= p ? aq1c : q1c), v);
-                        col[i] = v;
-                        if (kSingle && i < p && i != c) cols[(size_t)i * LD + c] = v;
-                    }
+        const int nl = sh.nlive;
+        auto update_column = [&](int c, int j0, int step) {
+            const int a0 = kSingle ? sh.lpos[c] : 0, lenA = nl - a0, len = lenA + R;
+            double *col = cols + (size_t)(c >> gs) * LD;
+            const double q0c = pc0[c], aq0c = abs_rows ? apc0[c] : q0c, l0c = rl0[c];
+            if (q1 < 0) {
+                for (int j = j0; j < len; j += step) {
+                    const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
+                    const bool up = !kSingle && i < c;
+                    const double v = fma(up ? l0c : rl0[i], up ? pc0[i] : (i >= p ? aq0c : q0c), col[i]);
+                    col[i] = v;
+                    if (kSingle && i < p && i != c) cols[(size_t)i * LD + c] = v;
                 }
+            } else {
+                const double q1c = pc1[c], aq1c = abs_rows ? apc1[c] : q1c, l1c = rl1[c];
+                for (int j = j0; j < len; j += step) {
+                    const int i = j < lenA ? (int)sh.lrow[a0 + j] : p + (j - lenA);
+                    const bool up = !kSingle && i < c;
+                    double v = fma(up ? l0c : rl0[i], up ? pc0[i] : (i >= p ? aq0c : q0c), col[i]);
+                    v = fma(up ? l1c : rl1[i], up ? pc1[i] : (i >= p ? aq1c : q1c), v);
+                    col[i] = v;
+                    if (kSingle && i < p && i != c) cols[(size_t)i * LD + c] = v;
+                }
+            }
+        };
+        // When the next candidate is the first live column, it has no partner and its test
+        // needs its own column only: its CTA updates that column first, all warps
+        // together, and the first warp tests it and pushes the outcome while the
+        // others go on.  The round of the next pivot then needs no test and no
+        // barrier before its update.  (A copy of the column in every CTA, tested by
+        // each, saves the push and the remote reads of the pivot column, but every CTA then
+        // waits for a test that shares its FP64 pipe: 1164 us, not 1134.)
+        const int cn = nl > 0 ? (int)sh.lrow[0] : 0;
+        pre = nl > 0 && cn > cstar;
+        const int mine = pre && (cn & gm) == rank ? 1 : 0;
+        if (mine) {
+            update_column(cn, tid, kT);
+            if (warp == 0) {
+                __syncwarp();
+                asm volatile("bar.sync 1, %0;" ::"n"(kT) : "memory");
+                const Decision d = test_first(cols + (size_t)(cn >> gs) * LD, sh.lrow, nl, p, R, u, small_k);
+                if (lane < G) *team.at(&sh.one[round & 1], lane) = d;
+            } else {
+                __syncwarp();
+                asm volatile("bar.arrive 1, %0;" ::"n"(kT) : "memory");
+            }
+        }
+        // the other live columns to the other warps, several warps to a column when
+        // there are fewer columns than warps
+        {
+            const int nw = kNW - mine, w = warp - mine, no = sh.nown - mine;
+            const int S = no > 0 && no < nw ? nw / no : 1;
+            if (S == 1) {
+                if (w >= 0)
+                    for (int o = w; o < no; o += nw) update_column(sh.ocol[o + mine], lane, 32);
+            } else if (w >= 0 && w < no * S) {
+                const int s = w / no;
+                update_column(sh.ocol[w - s * no + mine], lane + 32 * s, 32 * S);
             }
         }
         nelim += (q1 < 0) ? 1 : 2;
