@@ -261,6 +261,37 @@ static ClassKey batch_class_of(int p, int64_t m, int pivot, size_t budget) {
     return {kFactorCluster, G, 0};
 }
 
+// Classes (CTA: keys 2 to 4, clusters of 2 to 16: keys 5 to 8) move to wider clusters
+// while the batch leaves SMs idle: a front's pivot search is quicker on more
+// CTAs, but takes more CTA time.  One strict front of p = 256 on 8 / 16 CTAs
+// takes 166 / 126 us, p = 128 on 2 / 4 / 8: 149 / 112 / 92, p = 64 on 1 / 2 / 4 / 8:
+// 81 / 67 / 61 / 57, p = 32 on 1 / 2: 61 / 68, so p <= 32 stays on one.  112 CTAs: seven
+// clusters of 16, which the GPU's processing clusters hold side by side.  The
+// results do not depend on the width.
+constexpr int64_t kWidenCtas = 112;
+
+static void widen_classes(std::vector<std::vector<int>> &byKey, const std::vector<BFront> &tab) {
+    auto width = [](int key) { return key < 5 ? 1 : 2 << (key - 5); };
+    int64_t ctas = 0;
+    for (int key = 2; key < (int)byKey.size(); key++) ctas += (int64_t)byKey[key].size() * width(key);
+    for (bool moved = true; moved;) {
+        moved = false;
+        for (int key = 7; key >= 2; key--) {  // the widest, whose fronts take longest, first
+            std::vector<int> &from = byKey[key];
+            int p = 0;
+            for (int f : from) p = std::max(p, tab[f].p);
+            const int want = p > 128 ? 16 : (p > 64 ? 8 : (p > 32 ? 4 : 1));
+            const int to = key < 5 ? 5 : key + 1;
+            const int64_t more = (int64_t)from.size() * (width(to) - width(key));
+            if (from.empty() || width(key) >= want || ctas + more > kWidenCtas) continue;
+            byKey[to].insert(byKey[to].end(), from.begin(), from.end());
+            from.clear();
+            ctas += more;
+            moved = true;
+        }
+    }
+}
+
 extern "C" {
 
 ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host,
@@ -356,17 +387,20 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     std::vector<int> pmaxK(kNumKeys, 1), ldmaxK(kNumKeys, 1);
     std::vector<size_t> smemK(kNumKeys, 0);
     for (int f = 0; f < nb; f++) {
-        const int p = tab[f].p;
-        const int64_t m = tab[f].m;
-        const ClassKey k = batch_class_of(p, m, opt->pivot, budget);
-        const int R = opt->pivot == CTP_PIV_STRICT ? (int)(m < p ? m : p) : 0;
+        const ClassKey k = batch_class_of(tab[f].p, tab[f].m, opt->pivot, budget);
         const int gi = k.G == 2 ? 0 : k.G == 4 ? 1 : k.G == 8 ? 2 : 3;
-        const int key = k.kind == kFactorWarp ? k.bucket : (k.kind == kFactorCta ? 2 + k.bucket : 5 + gi);
-        byKey[key].push_back(f);
-        pmaxK[key] = std::max(pmaxK[key], p);
-        ldmaxK[key] = std::max(ldmaxK[key], p + R);
-        if (k.kind != kFactorWarp) smemK[key] = std::max(smemK[key], factor_smem_bytes(p, R, k.G));
+        byKey[k.kind == kFactorWarp ? k.bucket : (k.kind == kFactorCta ? 2 + k.bucket : 5 + gi)].push_back(f);
     }
+    widen_classes(byKey, tab);
+    for (int key = 0; key < kNumKeys; key++)
+        for (int f : byKey[key]) {
+            const int p = tab[f].p;
+            const int64_t m = tab[f].m;
+            const int R = opt->pivot == CTP_PIV_STRICT ? (int)(m < p ? m : p) : 0;
+            pmaxK[key] = std::max(pmaxK[key], p);
+            ldmaxK[key] = std::max(ldmaxK[key], p + R);
+            if (key >= 2) smemK[key] = std::max(smemK[key], factor_smem_bytes(p, R, key < 5 ? 1 : 2 << (key - 5)));
+        }
     // within a class, the fronts with the most pivot-search work first (about
     // p^2 (p + R) terms), so that no large front starts in the launch's last
     // wave; the results do not depend on the order
