@@ -114,7 +114,7 @@ ctp_status ctp_create(ctp_ctx **ctx, int32_t device) {
     c->profiling = false;
     c->nrec = 0;
     c->events_made = false;
-    c->side_made = false;
+    c->sides[0].made = c->sides[1].made = false;
     *ctx = c;
     return CTP_OK;
 }
@@ -122,12 +122,15 @@ ctp_status ctp_create(ctp_ctx **ctx, int32_t device) {
 ctp_status ctp_destroy(ctp_ctx *ctx) {
     if (ctx != nullptr && ctx->events_made)
         for (int i = 0; i < 2 * kMaxRec; i++) cudaEventDestroy(ctx->ev[i]);
-    if (ctx != nullptr && ctx->side_made) {
+    for (int k = 0; ctx != nullptr && k < 2; k++) {
+        ctp_ctx::SideSet &s = ctx->sides[k];
+        if (!s.made) continue;
         for (int i = 0; i < kSideStreams; i++) {
-            cudaStreamDestroy(ctx->side[i]);
-            cudaEventDestroy(ctx->join_ev[i]);
+            cudaStreamDestroy(s.side[i]);
+            cudaEventDestroy(s.join_ev[i]);
         }
-        cudaEventDestroy(ctx->fork_ev);
+        cudaStreamDestroy(s.main);
+        cudaEventDestroy(s.fork_ev);
     }
     free(ctx);
     return CTP_OK;
@@ -428,42 +431,59 @@ ctp_status ctp_profile_end(ctp_ctx *ctx, int32_t max_kernels, char *names, doubl
 // device is current the batch does not fork (the caller's stream is on the
 // current device, and events cannot join streams across devices).  A partial
 // failure releases what it made, so a later call may try again.
-static bool side_streams(ctp_ctx *ctx, cudaStream_t st) {
+static bool side_streams(ctp_ctx *ctx, cudaStream_t st, int set) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != ctx->device) return false;
-    if (ctx->side_made) return true;
+    ctp_ctx::SideSet &s = ctx->sides[set];
+    if (s.made) return true;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
     int ns = 0, ne = 0;
-    bool fork = false, ok = true;
+    bool main = false, fork = false, ok = true;
     for (; ok && ns < kSideStreams; ns++)
-        ok = cudaStreamCreateWithFlags(&ctx->side[ns], cudaStreamNonBlocking) == cudaSuccess;
+        ok = cudaStreamCreateWithFlags(&s.side[ns], cudaStreamNonBlocking) == cudaSuccess;
     if (!ok) ns--;
     for (; ok && ne < kSideStreams; ne++)
-        ok = cudaEventCreateWithFlags(&ctx->join_ev[ne], cudaEventDisableTiming) == cudaSuccess;
+        ok = cudaEventCreateWithFlags(&s.join_ev[ne], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) ne--;
-    if (ok) ok = fork = cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming) == cudaSuccess;
+    if (ok) ok = main = cudaStreamCreateWithFlags(&s.main, cudaStreamNonBlocking) == cudaSuccess;
+    if (ok) ok = fork = cudaEventCreateWithFlags(&s.fork_ev, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
-        for (int i = 0; i < ns; i++) cudaStreamDestroy(ctx->side[i]);
-        for (int i = 0; i < ne; i++) cudaEventDestroy(ctx->join_ev[i]);
-        if (fork) cudaEventDestroy(ctx->fork_ev);
+        for (int i = 0; i < ns; i++) cudaStreamDestroy(s.side[i]);
+        for (int i = 0; i < ne; i++) cudaEventDestroy(s.join_ev[i]);
+        if (main) cudaStreamDestroy(s.main);
+        if (fork) cudaEventDestroy(s.fork_ev);
         (void)cudaGetLastError();
         return false;
     }
-    ctx->side_made = true;
+    s.made = true;
     return true;
 }
 
-ctp_status ctp_factor_batch(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *fronts,
-                            void *workspace, size_t ws_bytes, void *stream) {
-    if (ctx == nullptr || plan == nullptr || fronts == nullptr || workspace == nullptr) return CTP_EINVAL;
+}  // extern "C"
+
+namespace ctp {
+
+bool second_stream(ctp_ctx *ctx, cudaStream_t st, cudaStream_t *out) {
+    if (ctx->profiling || !side_streams(ctx, st, 1)) return false;
+    ctp_ctx::SideSet &s = ctx->sides[1];
+    if (cudaEventRecord(s.fork_ev, st) != cudaSuccess || cudaStreamWaitEvent(s.main, s.fork_ev, 0) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    *out = s.main;
+    return true;
+}
+
+ctp_status factor_batch_on(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *fronts, void *workspace,
+                           size_t ws_bytes, cudaStream_t st, int set) {
     if (ws_bytes < batch_total(plan)) return CTP_ENOMEM;
-    cudaStream_t st = (cudaStream_t)stream;
     char *w = (char *)workspace;
     CTP_CUDA(timed(ctx, K_B_PREPARE, st, [&] { return batch_prepare(plan, w, st); }));
     CTP_CUDA(timed(ctx, K_B_COMPRESS, st, [&] { return batch_compress(plan, fronts, w, ctx->num_sms, st); }));
     const int ncls = batch_num_classes(plan);
-    if (!ctx->profiling && ncls > 1 && side_streams(ctx, st)) {
+    if (!ctx->profiling && ncls > 1 && side_streams(ctx, st, set)) {
+        ctp_ctx::SideSet &sd = ctx->sides[set];
         // the classes touch disjoint fronts: run them side by side (the plan
         // lists the widest last: launched first, its clusters take SMs before
         // the narrow CTAs fill the rest), each followed on its stream by the
@@ -471,19 +491,19 @@ ctp_status ctp_factor_batch(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front 
         // classes still searching), joined back into st; capturable as a
         // fork/join
         const bool per_class = batch_solve_per_class(plan);
-        CTP_CUDA(cudaEventRecord(ctx->fork_ev, st));
+        CTP_CUDA(cudaEventRecord(sd.fork_ev, st));
         for (int i = 0; i < ncls; i++) {
             const int c = ncls - 1 - i;
-            cudaStream_t s = ctx->side[i % kSideStreams];
-            CTP_CUDA(cudaStreamWaitEvent(s, ctx->fork_ev, 0));
+            cudaStream_t s = sd.side[i % kSideStreams];
+            CTP_CUDA(cudaStreamWaitEvent(s, sd.fork_ev, 0));
             CTP_CUDA(batch_factor_class(plan, c, fronts, w, s));
             if (per_class) {
                 CTP_CUDA(batch_solve_class(plan, c, fronts, w, ctx->num_sms, s));
                 CTP_CUDA(batch_form_class(plan, c, fronts, w, ctx->num_sms, s));
             }
-            CTP_CUDA(cudaEventRecord(ctx->join_ev[i % kSideStreams], s));
+            CTP_CUDA(cudaEventRecord(sd.join_ev[i % kSideStreams], s));
         }
-        for (int i = 0; i < ncls && i < kSideStreams; i++) CTP_CUDA(cudaStreamWaitEvent(st, ctx->join_ev[i], 0));
+        for (int i = 0; i < ncls && i < kSideStreams; i++) CTP_CUDA(cudaStreamWaitEvent(st, sd.join_ev[i], 0));
         if (!per_class) {
             CTP_CUDA(timed(ctx, K_B_SOLVE, st, [&] { return batch_solve(plan, fronts, w, ctx->num_sms, st); }));
             CTP_CUDA(timed(ctx, K_B_FORM, st, [&] { return batch_form(plan, fronts, w, ctx->num_sms, st); }));
@@ -505,6 +525,16 @@ ctp_status ctp_factor_batch(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front 
     }
     CTP_CUDA(timed(ctx, K_B_FORM, st, [&] { return batch_form(plan, fronts, w, ctx->num_sms, st); }));
     return CTP_OK;
+}
+
+}  // namespace ctp
+
+extern "C" {
+
+ctp_status ctp_factor_batch(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *fronts,
+                            void *workspace, size_t ws_bytes, void *stream) {
+    if (ctx == nullptr || plan == nullptr || fronts == nullptr || workspace == nullptr) return CTP_EINVAL;
+    return factor_batch_on(ctx, plan, fronts, workspace, ws_bytes, (cudaStream_t)stream, 0);
 }
 
 /* ---------------------------------------------------------------------- */

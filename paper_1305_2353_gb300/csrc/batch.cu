@@ -292,6 +292,34 @@ static void widen_classes(std::vector<std::vector<int>> &byKey, const std::vecto
     }
 }
 
+namespace ctp {
+
+size_t batch_blob_bytes(const ctp_plan *P) { return P->blob.size(); }
+const void *batch_blob(const ctp_plan *P) { return P->blob.data(); }
+
+// the plan's tables, from `blob` (a copy of batch_blob that outlives the copy), into the workspace
+cudaError_t batch_upload(const ctp_plan *P, const void *blob, char *w, cudaStream_t st) {
+    cudaError_t e = cudaMemcpyAsync(w, blob, P->blob.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && P->tc) {
+        // padding rows of the stacked operands must read as zero
+        e = cudaMemsetAsync(w + P->off_wb, 0, P->off_lb - P->off_wb, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(w + P->off_lb, 0, P->off_xt - P->off_lb, st);
+    }
+    return e;
+}
+
+// every front's status to flags_host
+cudaError_t batch_flags(const ctp_plan *P, char *w, int32_t *flags_host, cudaStream_t st) {
+    k_batch_flags<<<(P->nb + 255) / 256, 256, 0, st>>>(
+        reinterpret_cast<const BFront *>(w + P->off_tab), w, P->bo, P->nb,
+        reinterpret_cast<const int32_t *>(w + P->off_ginfo), reinterpret_cast<int32_t *>(w + P->off_flags));
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(flags_host, w + P->off_flags, sizeof(int32_t) * (size_t)P->nb, cudaMemcpyDeviceToHost, st);
+}
+
+}  // namespace ctp
+
 extern "C" {
 
 ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host,
@@ -553,15 +581,7 @@ ctp_status ctp_batch_upload(ctp_ctx *ctx, const ctp_plan *plan, void *workspace,
     if (ctx == nullptr || plan == nullptr || workspace == nullptr) return CTP_EINVAL;
     if (ws_bytes < plan->total) return CTP_ENOMEM;
     cudaStream_t st = (cudaStream_t)stream;
-    char *w = (char *)workspace;
-    if (cudaMemcpyAsync(w, plan->blob.data(), plan->blob.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
-        return CTP_ECUDA;
-    if (plan->tc) {
-        // padding rows of the stacked operands must read as zero
-        if (cudaMemsetAsync(w + plan->off_wb, 0, plan->off_lb - plan->off_wb, st) != cudaSuccess ||
-            cudaMemsetAsync(w + plan->off_lb, 0, plan->off_xt - plan->off_lb, st) != cudaSuccess)
-            return CTP_ECUDA;
-    }
+    if (batch_upload(plan, plan->blob.data(), (char *)workspace, st) != cudaSuccess) return CTP_ECUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return CTP_ECUDA;  // the blob is pageable
     return CTP_OK;
 }
@@ -571,13 +591,7 @@ ctp_status ctp_batch_read_info(ctp_ctx *ctx, const ctp_plan *plan, const void *w
     if (ctx == nullptr || plan == nullptr || workspace == nullptr || flags_host == nullptr)
         return CTP_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    char *w = (char *)const_cast<void *>(workspace);
-    k_batch_flags<<<(plan->nb + 255) / 256, 256, 0, st>>>(
-        reinterpret_cast<const BFront *>(w + plan->off_tab), w, plan->bo, plan->nb,
-        reinterpret_cast<const int32_t *>(w + plan->off_ginfo), reinterpret_cast<int32_t *>(w + plan->off_flags));
-    if (cudaGetLastError() != cudaSuccess) return CTP_ECUDA;
-    if (cudaMemcpyAsync(flags_host, w + plan->off_flags, sizeof(int32_t) * (size_t)plan->nb,
-                        cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (batch_flags(plan, (char *)const_cast<void *>(workspace), flags_host, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return CTP_ECUDA;
     return CTP_OK;

@@ -222,6 +222,15 @@ int batch_num_classes(const ctp_plan *P);
 int batch_class_kind(const ctp_plan *P, int c);  // kFactor*
 int batch_class_G(const ctp_plan *P, int c);
 size_t batch_total(const ctp_plan *P);
+size_t batch_blob_bytes(const ctp_plan *P);
+const void *batch_blob(const ctp_plan *P);
+cudaError_t batch_upload(const ctp_plan *P, const void *blob, char *w, cudaStream_t st);
+cudaError_t batch_flags(const ctp_plan *P, char *w, int32_t *flags_host, cudaStream_t st);
+// ctp_factor_batch with one of the context's two sets of side streams; the stream
+// from which a second batch in flight runs (ordered behind st; false: none)
+ctp_status factor_batch_on(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *fronts, void *workspace,
+                           size_t ws_bytes, cudaStream_t st, int set);
+bool second_stream(ctp_ctx *ctx, cudaStream_t st, cudaStream_t *out);
 cudaError_t batch_prepare(const ctp_plan *P, char *w, cudaStream_t st);
 cudaError_t batch_compress(const ctp_plan *P, const ctp_front *fr, char *w, int num_sms, cudaStream_t st);
 cudaError_t batch_factor_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, cudaStream_t st);

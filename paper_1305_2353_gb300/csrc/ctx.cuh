@@ -29,10 +29,14 @@ struct ctp_ctx {
     int rec_id[ctp::kMaxRec];
     cudaEvent_t ev[2 * ctp::kMaxRec];
     bool events_made;
-    // side streams on which a batch's pivot-search classes run side by side
-    cudaStream_t side[ctp::kSideStreams];
-    cudaEvent_t fork_ev, join_ev[ctp::kSideStreams];
-    bool side_made;
+    // Side streams on which a batch's pivot-search classes run side by side: one set
+    // for the caller's batches, one (with a stream to run them from) for
+    // the second of two batches in flight within one call.
+    struct SideSet {
+        cudaStream_t side[ctp::kSideStreams], main;
+        cudaEvent_t fork_ev, join_ev[ctp::kSideStreams];
+        bool made;
+    } sides[2];
 };
 
 namespace ctp {

@@ -57,12 +57,30 @@ struct ctp_mf {
     std::vector<PanelRec> panels;
     std::vector<int32_t> panel_block;  // block of each panel
     SolvePlan plan;  // the factors repacked for solving
+    // pinned staging of the two batches in flight (uploads and read-backs)
+    char *pin[2] = {nullptr, nullptr};
+    size_t pin_cap[2] = {0, 0};
+    bool pin_need(int g, size_t bytes) {
+        if (bytes <= pin_cap[g]) return true;
+        if (pin[g]) cudaFreeHost(pin[g]);
+        pin[g] = nullptr;
+        pin_cap[g] = 0;
+        if (cudaMallocHost((void **)&pin[g], bytes + bytes / 2) != cudaSuccess) {
+            pin[g] = nullptr;
+            (void)cudaGetLastError();
+            return false;
+        }
+        pin_cap[g] = bytes + bytes / 2;
+        return true;
+    }
     bool factored = false;
     bool mixed = false;  // the last factorization's Form ran on the tensor cores
     ~ctp_mf() {
         if (d_ci) cudaFree(d_ci);
         if (d_cj) cudaFree(d_cj);
         if (d_q) cudaFree(d_q);
+        for (char *h : pin)
+            if (h) cudaFreeHost(h);
         arena.release();
     }
 };
@@ -310,8 +328,8 @@ ctp_status ctp_mf_factor(ctp_ctx *ctx, ctp_mf *mf, const double *val, const ctp_
     std::vector<std::vector<int>> bylev(nlev);
     for (int s2 = 0; s2 < nblk; s2++) bylev[lvl[s2]].push_back(s2);
     std::vector<int32_t> loc(mf->N, -1);
-    void *bws = nullptr;
-    size_t bws_cap = 0;
+    void *bws[2] = {nullptr, nullptr};
+    size_t bws_cap[2] = {0, 0};
     struct AsmRow {
         int64_t e0, ne;
         double *F;
@@ -465,113 +483,156 @@ ctp_status ctp_mf_factor(ctp_ctx *ctx, ctp_mf *mf, const double *val, const ctp_
             if (batchable && b.parent >= 0 && b.n > b.p) bi.push_back(i);
         }
         std::vector<std::vector<int32_t>> ordb(bi.size());  // current row order (new numbering)
+        std::vector<std::vector<int32_t>> varb(bi.size());  // the same as variables: a pass uploads its tail
         for (size_t k = 0; k < bi.size(); k++) {
             ctp_mf::Blk &b = mf->blk[lv[bi[k]]];
             ordb[k] = rows[bi[k]];
+            varb[k].resize(ordb[k].size());
+            for (size_t q = 0; q < ordb[k].size(); q++) varb[k][q] = mf->perm[ordb[k][q]];
             b.elim = 0;
             b.pa = b.pb = -1;
         }
-        std::vector<int> active(bi.size());
-        for (size_t k = 0; k < bi.size(); k++) active[k] = (int)k;
         std::vector<std::vector<PanelRec>> recs(bi.size());
-        while (!active.empty() && rc == CTP_OK) {
+        // Two batches of fronts take their passes by turns, each on a stream of its own:
+        // while one runs, the host reads the other's results and prepares its next
+        // pass (about 130 us, a fifth of a 64^3 factorization when the GPU waits for it),
+        // and the latency-bound pivot searches of one run beside the Form of the other.
+        struct Group {
+            std::vector<int> active;
+            cudaStream_t st;
+            ctp_plan *plan;  // of the pass in flight
+            std::vector<int64_t> nh;
+            std::vector<int32_t> ph;
+            std::vector<ctp_front> fh;
+            int32_t *d_nel, *d_perm, *d_piv, *d_rows;
+            double *d_D;
+            int32_t *outh, *flags;  // pinned
+            int64_t sp;
+        } grp[2];
+        int ngrp = 1;
+        grp[0].st = st;
+        grp[0].plan = grp[1].plan = nullptr;
+        if (bi.size() > 1 && second_stream(ctx, st, &grp[1].st)) ngrp = 2;
+        {
+            // the fronts by work, to the two groups by turns
+            std::vector<int> byw(bi.size());
+            for (size_t k = 0; k < bi.size(); k++) byw[k] = (int)k;
+            std::stable_sort(byw.begin(), byw.end(), [&](int x, int z) {
+                const ctp_mf::Blk &bx = mf->blk[lv[bi[x]]], &bz = mf->blk[lv[bi[z]]];
+                return bx.n * bx.p > bz.n * bz.p;
+            });
+            for (size_t k = 0; k < byw.size(); k++) grp[ngrp == 1 || (k + 1) % 4 < 2 ? 0 : 1].active.push_back(byw[k]);
+        }
+        // enqueue the next pass of group gi
+        auto submit = [&](int gi) -> ctp_status {
+            Group &g = grp[gi];
+            const std::vector<int> &active = g.active;
             const int nb = (int)active.size();
-            std::vector<int64_t> nh(nb);
-            std::vector<int32_t> ph(nb);
+            g.nh.resize(nb);
+            g.ph.resize(nb);
             int64_t sp = 0, sn = 0;
             for (int k = 0; k < nb; k++) {
                 const ctp_mf::Blk &b = mf->blk[lv[bi[active[k]]]];
-                nh[k] = b.n - b.elim;
-                ph[k] = (int32_t)std::min<int64_t>(kMaxP, b.p - b.elim);
-                sp += ph[k];
-                sn += nh[k];
+                g.nh[k] = b.n - b.elim;
+                g.ph[k] = (int32_t)std::min<int64_t>(kMaxP, b.p - b.elim);
+                sp += g.ph[k];
+                sn += g.nh[k];
             }
+            g.sp = sp;
             // per-front outputs, contiguous for one read-back: nelim | perm | piv | rows, then D
             const size_t ib = align256(sizeof(int32_t) * (size_t)(nb + 2 * sp + sn));
             char *ob = (char *)mf->arena.alloc(ib + align256(sizeof(double) * 2 * (size_t)sp) +
                                                sizeof(ctp_front) * nb);
-            if (ob == nullptr) {
-                rc = CTP_ENOMEM;
-                break;
-            }
-            int32_t *d_nel = (int32_t *)ob, *d_perm = d_nel + nb, *d_piv = d_perm + sp, *d_rows = d_piv + sp;
-            double *d_D = (double *)(ob + ib);
+            if (ob == nullptr) return CTP_ENOMEM;
+            g.d_nel = (int32_t *)ob;
+            g.d_perm = g.d_nel + nb;
+            g.d_piv = g.d_perm + sp;
+            g.d_rows = g.d_piv + sp;
+            g.d_D = (double *)(ob + ib);
             ctp_front *d_fr = (ctp_front *)(ob + ib + align256(sizeof(double) * 2 * (size_t)sp));
-            std::vector<ctp_front> fh(nb);
-            std::vector<int32_t> rows_h;
-            rows_h.reserve(sn);
+            size_t need = 0;
+            ctp_status s = ctp_batch_plan_create(ctx, nb, g.nh.data(), g.ph.data(), &bopt, &g.plan, &need);
+            if (s != CTP_OK) return s;
+            // staging: rows | fronts | tables of the plan | nelim and perm | flags
+            const size_t o_fr = align256(sizeof(int32_t) * (size_t)sn), o_tab = o_fr + align256(sizeof(ctp_front) * nb),
+                         o_out = o_tab + align256(batch_blob_bytes(g.plan)),
+                         o_flag = o_out + align256(sizeof(int32_t) * (size_t)(nb + sp));
+            if (!mf->pin_need(gi, o_flag + sizeof(int32_t) * (size_t)nb)) return CTP_ENOMEM;
+            char *h = mf->pin[gi];
+            g.outh = (int32_t *)(h + o_out);
+            g.flags = (int32_t *)(h + o_flag);
+            g.fh.resize(nb);
+            int32_t *rh = (int32_t *)h;
             int64_t po = 0;
             for (int k = 0; k < nb; k++) {
                 ctp_mf::Blk &b = mf->blk[lv[bi[active[k]]]];
                 const int64_t e0 = b.elim;
-                ctp_front &f = fh[k];
-                f.n = nh[k];
-                f.p = ph[k];
+                ctp_front &f = g.fh[k];
+                f.n = g.nh[k];
+                f.p = g.ph[k];
                 f.reserved = 0;
                 f.A = b.F + e0 * b.n + e0;
                 f.lda = b.n;
-                f.perm = d_perm + po;
-                f.piv = d_piv + po;
-                f.D = d_D + 2 * po;
-                f.nelim = d_nel + k;
-                f.S = f.A + (int64_t)ph[k] * b.n + ph[k];
+                f.perm = g.d_perm + po;
+                f.piv = g.d_piv + po;
+                f.D = g.d_D + 2 * po;
+                f.nelim = g.d_nel + k;
+                f.S = f.A + (int64_t)g.ph[k] * b.n + g.ph[k];
                 f.lds = b.n;
-                for (int64_t q = e0; q < b.n; q++) rows_h.push_back(mf->perm[ordb[active[k]][q]]);
-                po += ph[k];
+                rh = std::copy(varb[active[k]].begin() + e0, varb[active[k]].end(), rh);
+                po += g.ph[k];
             }
-            if (cudaMemcpyAsync(d_rows, rows_h.data(), sizeof(int32_t) * rows_h.size(), cudaMemcpyHostToDevice,
-                                st) != cudaSuccess ||
-                cudaMemcpyAsync(d_fr, fh.data(), sizeof(ctp_front) * nb, cudaMemcpyHostToDevice, st) != cudaSuccess) {
-                rc = CTP_ECUDA;
-                break;
+            std::copy(g.fh.begin(), g.fh.end(), (ctp_front *)(h + o_fr));
+            std::copy_n((const char *)batch_blob(g.plan), batch_blob_bytes(g.plan), h + o_tab);
+            if (need > bws_cap[gi]) {
+                if (bws[gi]) cudaFree(bws[gi]);
+                bws[gi] = nullptr;
+                bws_cap[gi] = 0;
+                if (cudaMalloc(&bws[gi], need) != cudaSuccess) return CTP_ENOMEM;
+                bws_cap[gi] = need;
             }
-            ctp_plan *plan = nullptr;
-            size_t need = 0;
-            rc = ctp_batch_plan_create(ctx, nb, nh.data(), ph.data(), &bopt, &plan, &need);
-            if (rc != CTP_OK) break;
-            if (need > bws_cap) {
-                if (bws) cudaFree(bws);
-                bws = nullptr;
-                bws_cap = 0;
-                if (cudaMalloc(&bws, need) != cudaSuccess) {
-                    ctp_batch_plan_destroy(plan);
-                    rc = CTP_ENOMEM;
-                    break;
-                }
-                bws_cap = need;
-            }
-            rc = ctp_batch_upload(ctx, plan, bws, bws_cap, st);
-            if (rc == CTP_OK) rc = ctp_factor_batch(ctx, plan, d_fr, bws, bws_cap, st);
-            std::vector<int32_t> flags(nb), outh(nb + sp);
-            if (rc == CTP_OK) rc = ctp_batch_read_info(ctx, plan, bws, flags.data(), st);
-            ctp_batch_plan_destroy(plan);
-            if (rc != CTP_OK) break;
-            for (int k = 0; k < nb; k++)
-                if (flags[k] != CTP_OK) rc = (ctp_status)flags[k];
-            if (rc != CTP_OK) break;
-            if (cudaMemcpyAsync(outh.data(), d_nel, sizeof(int32_t) * (nb + sp), cudaMemcpyDeviceToHost, st) !=
+            if (cudaMemcpyAsync(g.d_rows, h, sizeof(int32_t) * (size_t)sn, cudaMemcpyHostToDevice, g.st) !=
                     cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess) {
-                rc = CTP_ECUDA;
-                break;
-            }
+                cudaMemcpyAsync(d_fr, h + o_fr, sizeof(ctp_front) * nb, cudaMemcpyHostToDevice, g.st) != cudaSuccess ||
+                batch_upload(g.plan, h + o_tab, (char *)bws[gi], g.st) != cudaSuccess)
+                return CTP_ECUDA;
+            s = factor_batch_on(ctx, g.plan, d_fr, bws[gi], bws_cap[gi], g.st, gi);
+            if (s != CTP_OK) return s;
+            if (batch_flags(g.plan, (char *)bws[gi], g.flags, g.st) != cudaSuccess ||
+                cudaMemcpyAsync(g.outh, g.d_nel, sizeof(int32_t) * (nb + sp), cudaMemcpyDeviceToHost, g.st) !=
+                    cudaSuccess)
+                return CTP_ECUDA;
+            return CTP_OK;
+        };
+        // wait for group gi's pass and take its results
+        auto finish = [&](int gi) -> ctp_status {
+            Group &g = grp[gi];
+            const int nb = (int)g.active.size();
+            const bool ran = cudaStreamSynchronize(g.st) == cudaSuccess;
+            ctp_batch_plan_destroy(g.plan);
+            g.plan = nullptr;
+            if (!ran) return CTP_ECUDA;
+            ctp_status s = CTP_OK;
+            for (int k = 0; k < nb; k++)
+                if (g.flags[k] != CTP_OK) s = (ctp_status)g.flags[k];
+            if (s != CTP_OK) return s;
             std::vector<int> next;
             std::vector<int32_t> tmp;
-            po = 0;
-            int64_t ro = 0;
+            int64_t po = 0, ro = 0;
             for (int k = 0; k < nb; k++) {
-                const int a = active[k];
+                const int a = g.active[k];
                 ctp_mf::Blk &b = mf->blk[lv[bi[a]]];
-                const int32_t e = outh[k];
-                const int64_t e0 = b.elim, pk = ph[k];
+                const int32_t e = g.outh[k], *pm = g.outh + nb + po;
+                const int64_t e0 = b.elim, pk = g.ph[k];
                 // pivot order of this pass's fully-summed rows
-                std::vector<int32_t> &o = ordb[a];
-                tmp.assign(o.begin() + e0, o.begin() + e0 + pk);
-                for (int64_t q = 0; q < pk; q++) o[e0 + q] = tmp[outh[nb + po + q]];
+                for (std::vector<int32_t> *o : {&ordb[a], &varb[a]}) {
+                    tmp.assign(o->begin() + e0, o->begin() + e0 + pk);
+                    for (int64_t q = 0; q < pk; q++) (*o)[e0 + q] = tmp[pm[q]];
+                }
                 if (e > 0) {
                     PanelRec r;
-                    r.f = {nh[k], (int32_t)pk, 0, fh[k].A, b.n, d_perm + po, d_piv + po, d_D + 2 * po, d_nel + k,
-                           d_rows + ro};
+                    r.f = {g.nh[k], (int32_t)pk, 0, g.fh[k].A, b.n, g.d_perm + po, g.d_piv + po, g.d_D + 2 * po,
+                           g.d_nel + k, g.d_rows + ro};
                     r.e = e;
                     r.w = (int32_t)pk;
                     r.pivot = opt->pivot;
@@ -580,10 +641,24 @@ ctp_status ctp_mf_factor(ctp_ctx *ctx, ctp_mf *mf, const double *val, const ctp_
                     if (b.elim < b.p) next.push_back(a);
                 }
                 po += pk;
-                ro += nh[k];
+                ro += g.nh[k];
             }
-            active.swap(next);
-        }
+            g.active.swap(next);
+            return CTP_OK;
+        };
+        for (int gi = 0; gi < ngrp && rc == CTP_OK; gi++)
+            if (!grp[gi].active.empty()) rc = submit(gi);
+        while (rc == CTP_OK && (grp[0].plan != nullptr || grp[1].plan != nullptr))
+            for (int gi = 0; gi < ngrp && rc == CTP_OK; gi++) {
+                if (grp[gi].plan == nullptr) continue;
+                rc = finish(gi);
+                if (rc == CTP_OK && !grp[gi].active.empty()) rc = submit(gi);
+            }
+        for (int gi = 0; gi < ngrp; gi++)  // after an error: nothing stays in flight
+            if (grp[gi].plan != nullptr) {
+                cudaStreamSynchronize(grp[gi].st);
+                ctp_batch_plan_destroy(grp[gi].plan);
+            }
         if (rc != CTP_OK) break;
         for (size_t k = 0; k < bi.size(); k++) {
             ctp_mf::Blk &b = mf->blk[lv[bi[k]]];
@@ -616,7 +691,8 @@ ctp_status ctp_mf_factor(ctp_ctx *ctx, ctp_mf *mf, const double *val, const ctp_
             for (int64_t k = elim; k < b.n; k++) b.cb[k - elim] = mf->inv[ord[k]];
         }
     }
-    if (bws) cudaFree(bws);
+    for (void *w : bws)
+        if (w) cudaFree(w);
     if (rc != CTP_OK) {
         cudaStreamSynchronize(st);
         return rc;
