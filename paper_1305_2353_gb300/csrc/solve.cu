@@ -68,12 +68,13 @@ __device__ __forceinline__ void write_pieces(__nv_bfloat16 *__restrict__ B, int6
 // What a pass over a tile does.  A whole Solve in one pass updates every later
 // column with every y_j in FP64: p^2/2 multiply-adds per row on a pipe of 2 per
 // clock and SM (n = 200000, p = e = 256: 12.9 ms, 0.8 of that pipe).  The blocked
-// Solve (3.4 ms: 1.9 ms in the diagonal blocks, 0.84 in the updates, 0.3 in the
-// tail) keeps only the 32-column diagonal blocks of
+// Solve (3.06 ms: 2.0 ms in the diagonal blocks, 0.84 in the updates, the rest moving
+// and scaling columns) keeps only the 32-column diagonal blocks of
 // that and leaves the rest -- columns times y's block by block -- to the
 // tensor cores, as products of exact digit slices (k_update in form.cu):
 //   kFirst  gather through perm, eliminate the first block inside itself, write
-//           the row in pivot order and the block's slices;
+//           the row in pivot order and the block's slices (large Solves move the
+//           columns in a pass of their own instead);
 //   kNext   the same for block blk (its columns are in place by now);
 //   kTail   after the last block's update: the rest of the elimination, if blocks
 //           were left out, then the outputs as in a whole pass.
@@ -247,6 +248,63 @@ __global__ void __launch_bounds__(kRows * kWarps)
                item_tile[blockIdx.x], xs);
 }
 
+// The columns of A21 into pivot order, in place: a tile of 32 rows by all columns per
+// CTA; columns that stay are left alone.
+__global__ void __launch_bounds__(kRows * kWarps)
+    k_move_columns(double *__restrict__ A21, int64_t m, int p, int64_t lda, const int32_t *__restrict__ perm) {
+    extern __shared__ __align__(16) double xs[];  // [p][kRows]
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t row = (int64_t)blockIdx.x * kRows + lane;
+    const bool valid = row < m;
+#pragma unroll 1
+    for (int k0 = w; k0 < p; k0 += 8 * kWarps) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const int k = k0 + q * kWarps;
+            v[q] = 0.0;
+            if (k < p && valid && perm[k] != k) v[q] = A21[(int64_t)perm[k] * lda + row];
+        }
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+            if (k0 + q * kWarps < p) xs[(k0 + q * kWarps) * kRows + lane] = v[q];
+    }
+    __syncthreads();
+    if (!valid) return;
+    for (int k = w; k < p; k += kWarps)
+        if (perm[k] != k) A21[(int64_t)k * lda + row] = xs[k * kRows + lane];
+}
+
+// L21 = Y D11^{-1} in place, as solve_tile's tail computes it: a thread per row and 16
+// columns (and the second of a 2x2 pair that begins with the last of them).
+constexpr int kScaleCols = 16, kScaleRows = 256;
+__global__ void __launch_bounds__(kScaleRows)
+    k_scale_columns(double *__restrict__ A21, int64_t m, int64_t lda, const int32_t *__restrict__ piv,
+                    const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p) {
+    const int e = *nelim_p, k0 = blockIdx.y * kScaleCols;
+    const int64_t row = (int64_t)blockIdx.x * kScaleRows + threadIdx.x;
+    if (k0 >= e || row >= m) return;
+    double *x = A21 + (int64_t)k0 * lda + row;
+    const int cnt = min(kScaleCols, e - k0);
+    double v[kScaleCols + 1];
+#pragma unroll
+    for (int q = 0; q < kScaleCols; q++) v[q] = q < cnt ? x[q * lda] : 0.0;
+    v[kScaleCols] = cnt == kScaleCols && piv[k0 + cnt - 1] == CTP_PIVKIND_2X2_FIRST ? x[kScaleCols * lda] : 0.0;
+#pragma unroll
+    for (int q = 0; q < kScaleCols; q++) {
+        if (q >= cnt) break;
+        const int k = k0 + q, kd = piv[k];
+        if (kd == CTP_PIVKIND_1X1) {
+            x[q * lda] = v[q] * Dinv[2 * k];
+        } else if (kd == CTP_PIVKIND_2X2_FIRST) {
+            x[q * lda] = __fma_rn(v[q + 1], Dinv[2 * k + 1], v[q] * Dinv[2 * k]);
+            x[(q + 1) * lda] = __fma_rn(v[q + 1], Dinv[2 * k + 2], v[q] * Dinv[2 * k + 1]);
+        } else if (kd == CTP_PIVKIND_ZERO) {
+            x[q * lda] = 0.0;
+        }
+    }
+}
+
 // Slices of L11's rows below block blk, columns of the block: what the block's y
 // are multiplied with.  One 32-row tile (rows r0.. in pivot order) per CTA; row r
 // is row r - 32 (blk + 1) of the image.
@@ -314,6 +372,15 @@ int solve_blocks(int64_t m, int p, int pivot) {
     return p > 128 || right * (p - kSliceK) >= 1.6e7 ? (p + kSliceK - 1) / kSliceK : 0;
 }
 
+// Entries of A21 from which a blocked Solve (p > 64) moves the columns, and scales them
+// when nothing else is left to do, in passes of their own: two launches more, but
+// the first block's elimination keeps eight CTAs per SM instead of three and the
+// scaling streams.  Together / apart, all columns accepted: n = 200000, p = 256: 3442 /
+// 3062 us (n = 24000: 547 / 510, 12000: 400 / 402), p = 128, n = 50000: 457 / 436 (24000: 232
+// / 238); a dozen accepted: p = 256, n = 200000: 567 / 444 (24000: 92 / 92, 12000: 61 / 68), p = 64,
+// n = 100000: 133 / 137.
+constexpr int64_t kApart = 6000000;
+
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
                               const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
@@ -338,8 +405,15 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
         err = cudaGetLastError();
         if (err != cudaSuccess) return err;
     }
+    const bool apart = p > 64 && m * p >= kApart;
+    if (apart) {
+        const size_t smem = sizeof(double) * (size_t)p * kRows;
+        if ((err = smem_at_least((const void *)k_move_columns, smem)) != cudaSuccess) return err;
+        k_move_columns<<<grid, kRows * kWarps, smem, st>>>(A + p, m, p, lda, perm);
+        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    }
     for (int b = 0; b < blocks; b++) {
-        err = b == 0 ? pass(kFirst, 0, p) : pass(kNext, b, kSliceK);
+        err = b == 0 && !apart ? pass(kFirst, 0, p) : pass(kNext, b, kSliceK);
         if (err != cudaSuccess) return err;
         if ((b + 1) * kSliceK >= p) break;
         SliceBuf u = blk;
@@ -347,6 +421,12 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
         u.el += b * kMaxP;
         err = launch_update(u, A, lda, p, m, b, piv, nelim, info, num_sms, st);
         if (err != cudaSuccess) return err;
+    }
+    if (apart && blocks * kSliceK >= p && sb.W == nullptr && sb.L == nullptr && Wb == nullptr && Lb == nullptr) {
+        k_scale_columns<<<dim3((unsigned)((m + kScaleRows - 1) / kScaleRows),
+                               (unsigned)((p + kScaleCols - 1) / kScaleCols)),
+                          kScaleRows, 0, st>>>(A + p, m, lda, piv, Dinv, nelim);
+        return cudaGetLastError();
     }
     return pass(kTail, blocks, p);
 }
