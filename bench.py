@@ -351,7 +351,12 @@ def kernel_roofline(name, launches, ms, a, e, peaks, prec="fp64"):
                 "hbm_frac": hbm / peaks["hbm_gbs"], "traffic": ncu_traffic(name, m, prec),
                 "launch_ms": ms / launches}
     elif name == "solve_fp64":
-        work, _ = flops_model(n, p, e)
+        # what stays on the FP64 pipe: all of a narrow Solve; of a wide one (p > 128,
+        # blocked) the 32-column diagonal blocks and the scaling by D^-1, the rest being
+        # exact digit slices on the tensor cores
+        method, _ = flops_model(n, p, e)
+        blocks = (e + 31) // 32
+        work = method if p <= 128 else 2.0 * m * (blocks * 496 + e)
         bound, unit, peak = "alu", "TFLOP/s", peaks["fp64_tflops"]
         src = "measured in this run: torch.matmul float64 6144^3, best of 10"
         achieved = work / t / 1e12

@@ -456,9 +456,12 @@ ctp_status ctp_refine_csc(ctp_ctx *ctx, int32_t nf, const ctp_sfront *fronts, in
  *   CTP_ECAPACITY.  The fronts of a tree level are assembled together, and
  *   with strict or restricted pivoting the non-root fronts of a level are
  *   factored in batched passes (one panel per front still making progress per
- *   pass).
- *   Device memory for the fronts is allocated by the call and held by *mf.
- *   Synchronises `stream` once per panel.
+ *   pass), in two batches that take their passes by turns; the second runs
+ *   on a stream of the context's, ordered behind `stream` and finished when the
+ *   call goes on to the next level.
+ *   Device memory for the fronts is allocated by the call and held by *mf, as is
+ *   pinned host memory for the passes' tables.
+ *   The host waits for every pass.
  * ctp_mf_fronts: the factored panels, in elimination order, as fronts for
  *   ctp_solve / ctp_refine_csc (host array valid until the next factor or
  *   destroy; rows name the ORIGINAL variables).
@@ -556,18 +559,20 @@ ctp_status ctp_chain_destroy(ctp_chain *chain);
  * CTP_TUNE_BATCH_SMEM_KB: shared memory (KB, 48..220; default 200) a CTA of
  *   the batched pivot search may hold (capped at what the kernel can take
  *   beside its static shared memory, about 190 KB); each front gets the
- *   narrowest cluster (1..16 CTAs) whose CTAs fit it.  A larger budget means fewer CTAs per
+ *   narrowest cluster (1..16 CTAs) whose CTAs fit it, and a wider one when the
+ *   whole batch leaves SMs idle.  A larger budget means fewer CTAs per
  *   front (cheaper cluster barriers, fewer parallel tests, fewer co-resident
  *   clusters).  Read when a batch plan is created.
  * CTP_TUNE_FACTOR_G: cluster width of the single-supernode pivot search
  *   (0 = by p, the default; else 1, 2, 4, 8 or 16, widened when the columns do
  *   not fit on chip).
- * CTP_TUNE_TPP_SPIN: how many polls (of about 100 ns) a software grid barrier
- *   of the full-column TPP kernel (CTP_PIV_TPP) waits for the other CTAs
- *   before it gives up: the kernel then stops, every CTA returns and the info
- *   word reads CTP_ETIMEOUT (0 = the default, 2^24 polls, about 1.5 s; else
+ * CTP_TUNE_TPP_SPIN: how many polls (an L2 round trip each, about half a
+ *   microsecond) a CTA of the full-column TPP kernel (CTP_PIV_TPP) waits for the
+ *   others, at a software grid barrier or in an exchange of column maxima, before
+ *   it gives up: the kernel then stops, every CTA returns and the info
+ *   word reads CTP_ETIMEOUT (0 = the default, 2^22 polls, about two seconds; else
  *   1..2^24).  Small values exist to exercise that timeout path in tests: the
- *   wait of the CTAs for CTA 0's pivot decision then runs out, and the
+ *   CTAs' waits for one another then run out, and the
  *   factorization's outputs are unspecified. */
 typedef enum {
     CTP_TUNE_FORM_WALK = 0,
