@@ -426,6 +426,10 @@ ctp_status ctp_profile_end(ctp_ctx *ctx, int32_t max_kernels, char *names, doubl
     return CTP_OK;
 }
 
+// Held while work is enqueued through a context's side streams: their events are
+// recorded and waited for in pairs, which calls from several threads must not mix.
+static std::mutex side_mutex;
+
 // The context's side streams, made on first use outside a stream capture
 // (false: run on st alone).  They belong to the context's device: when another
 // device is current the batch does not fork (the caller's stream is on the
@@ -465,6 +469,7 @@ static bool side_streams(ctp_ctx *ctx, cudaStream_t st, int set) {
 namespace ctp {
 
 bool second_stream(ctp_ctx *ctx, cudaStream_t st, cudaStream_t *out) {
+    std::lock_guard<std::mutex> lock(side_mutex);
     if (ctx->profiling || !side_streams(ctx, st, 1)) return false;
     ctp_ctx::SideSet &s = ctx->sides[1];
     if (cudaEventRecord(s.fork_ev, st) != cudaSuccess || cudaStreamWaitEvent(s.main, s.fork_ev, 0) != cudaSuccess) {
@@ -482,6 +487,8 @@ ctp_status factor_batch_on(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *
     CTP_CUDA(timed(ctx, K_B_PREPARE, st, [&] { return batch_prepare(plan, w, st); }));
     CTP_CUDA(timed(ctx, K_B_COMPRESS, st, [&] { return batch_compress(plan, fronts, w, ctx->num_sms, st); }));
     const int ncls = batch_num_classes(plan);
+    std::unique_lock<std::mutex> lock(side_mutex, std::defer_lock);
+    if (!ctx->profiling && ncls > 1) lock.lock();
     if (!ctx->profiling && ncls > 1 && side_streams(ctx, st, set)) {
         ctp_ctx::SideSet &sd = ctx->sides[set];
         // the classes touch disjoint fronts: run them side by side (the plan
@@ -510,6 +517,7 @@ ctp_status factor_batch_on(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *
         }
         return CTP_OK;
     } else {
+        if (lock.owns_lock()) lock.unlock();
         for (int c = 0; c < ncls; c++) {
             const int G = batch_class_G(plan, c), kind = batch_class_kind(plan, c);
             const int id = kind == kFactorWarp ? K_B_FACTOR_WARP

@@ -52,3 +52,41 @@ def test_two_groups(ctx, k, leaf, pivot, prec):
             assert np.array_equal(info[key], res[0][0][key])
         assert len(perms) == len(res[0][1]) and all(np.array_equal(a, b) for a, b in zip(perms, res[0][1]))
         assert np.abs(X - res[0][2]).max() <= tol * np.abs(res[0][2]).max()
+
+
+def test_two_threads_one_context(ctx):
+    """Two factorizations at once, from two threads and on two streams, share the
+    context's side streams."""
+    import threading
+    from paper_1305_2353_gb300 import ctp
+    k = 14
+    perm, blocks = inputs.nested_dissection_3d(k, 64)
+    jobs = []
+    for shift in (3.1, 2.7):
+        cp, ri, v = inputs.laplacian_3d(k, shift)
+        jobs.append((ctp.Multifrontal(ctx, cp, ri, v, perm, blocks), torch.cuda.Stream()))
+    opt = ctp.options(pivot="strict")
+    want = []
+    for mf, _ in jobs:
+        mf.factor(opt)
+        want.append((mf.info(), mf.panel_perms()))
+    errors = []
+
+    def run(mf, s):
+        try:
+            torch.cuda.set_device(ctx.device)
+            for _ in range(5):
+                mf.factor(opt, stream=s)
+        except Exception as e:  # noqa: BLE001  (reported by the assertion below)
+            errors.append(e)
+
+    ts = [threading.Thread(target=run, args=j) for j in jobs]
+    [t.start() for t in ts]
+    [t.join() for t in ts]
+    torch.cuda.synchronize()
+    assert not errors
+    for (mf, _), (info, perms) in zip(jobs, want):
+        got = mf.info()
+        for key in ("n", "p", "nelim", "delayed"):
+            assert np.array_equal(got[key], info[key])
+        assert all(np.array_equal(a, b) for a, b in zip(mf.panel_perms(), perms))
