@@ -21,6 +21,7 @@ namespace ctp {
 
 int64_t form_fp64_tiles(int64_t m);
 int64_t form_tc_tiles(int64_t m, int pieces);
+int ctx_num_sms(const ctp_ctx *ctx);
 
 namespace {
 
@@ -233,6 +234,7 @@ struct ctp_plan {
         size_t list_off;     // element offset in the class-list array
         int pmax;            // largest p of the class
         int64_t s_off, s_count;  // the class's Solve items (front, tile) in the class Solve lists
+        int s_rows;              // rows per tile
         int64_t u_off, u_count;  // blocked Solve: the class's update items (none: a whole pass per tile)
         int64_t f_off, f_count;  // the class's Form items (front, tile) in the class Form lists
     };
@@ -445,13 +447,6 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
         if (byKey[key].empty()) continue;
         ctp_plan::Class c;
         c.pmax = pmaxK[key];
-        c.s_off = (int64_t)csitem.size();
-        for (int f : byKey[key])
-            for (int64_t t = 0; t < (tab[f].m + kTR - 1) / kTR; t++) {
-                csitem.push_back(f);
-                cstile.push_back((int)t);
-            }
-        c.s_count = (int64_t)csitem.size() - c.s_off;
         // the class's Solve is blocked (three more launches, one more pass over its
         // rows) when its fronts hold enough entries of A21 right of the first block
         c.u_off = (int64_t)cuitem.size();
@@ -464,6 +459,16 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
                     cutile.push_back((int)t);
                 }
         c.u_count = (int64_t)cuitem.size() - c.u_off;
+        int64_t tiles = 0;
+        for (int f : byKey[key]) tiles += (tab[f].m + 31) / 32;
+        c.s_rows = solve_rows(tiles, c.u_count > 0, ctx_num_sms(ctx));
+        c.s_off = (int64_t)csitem.size();
+        for (int f : byKey[key])
+            for (int64_t t = 0; t < (tab[f].m + c.s_rows - 1) / c.s_rows; t++) {
+                csitem.push_back(f);
+                cstile.push_back((int)t);
+            }
+        c.s_count = (int64_t)csitem.size() - c.s_off;
         c.f_off = (int64_t)cfitem.size();
         if (opt->smode != CTP_S_NONE)
             for (int f : byKey[key]) {
@@ -650,13 +655,13 @@ cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, ch
             fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
             reinterpret_cast<const int *>(w + P->off_lists) + c.list_off, c.count,
             reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off,
-            reinterpret_cast<const int *>(w + P->off_cstile) + c.s_off, c.s_count,
+            reinterpret_cast<const int *>(w + P->off_cstile) + c.s_off, c.s_count, c.s_rows,
             reinterpret_cast<const int *>(w + P->off_cuitem) + c.u_off,
             reinterpret_cast<const int *>(w + P->off_cutile) + c.u_off, c.u_count, P->bo,
             P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax,
             reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
     return launch_solve_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
-                              reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off, c.s_count, P->bo,
+                              reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off, c.s_count, c.s_rows, P->bo,
                               P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax, st,
                               reinterpret_cast<const int *>(w + P->off_cstile) + c.s_off);
 }

@@ -204,8 +204,10 @@ cudaError_t launch_compress_strict_batch(const ctp_front *fronts, const BFront *
                                          cudaStream_t st);
 // items: (front, 32-row tile) pairs
 cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                               const int *item_front, int64_t items, BatchOpts o, void *Wb, void *Lb,
+                               const int *item_front, int64_t items, int rows, BatchOpts o, void *Wb, void *Lb,
                                int pmax, cudaStream_t st, const int *item_tile);
+// rows per tile (32, 16 or 8) of a Solve with this many 32-row tiles
+int solve_rows(int64_t tiles, bool blocked, int num_sms);
 // item_tile (optional, both batched Forms): each item's tile of its front;
 // without it the items of a front are consecutive, from tab[front].f0 on
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
@@ -281,7 +283,7 @@ int64_t update_tiles(int64_t m, int p);  // of a front, for block 0
 // a batch class's Solve in one block of 32 columns, its update and the tail
 cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
                                        int count, const int *item_front, const int *item_tile, int64_t items,
-                                       const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
+                                       int rows, const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
                                        void *Lb, int pmax, int32_t *info, int num_sms, cudaStream_t st);
 
 // Threshold partial pivoting on all n rows (the comparator of the compressed path).

@@ -92,11 +92,13 @@ struct SolvePass {
 // memory without a register copy, so that a CTA needs few
 // registers and as many CTAs fit on an SM as its shared memory allows (three at
 // p = 256, more for narrower fronts): enough warps for all four FP64 pipes.
-// One 32-row tile.  brow0: row of this front's first A21 row in the BF16
+// One tile of RT rows: 32, a lane per row, or fewer, with the lanes of a warp on several
+// columns (small supernodes, so that more SMs have a tile).  brow0: row of this front's first A21 row in the BF16
 // operand copies (0 for a single supernode; the stacked offset in a batch).
 // pieces > 1: also write the further BF16 pieces of the split operands (piece
 // k rounds what pieces 0..k-1 left), lo_off elements apart.  sb: the slices of
 // the FP64 Form (sb.W null: none).
+template <int RT>
 __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                                            const int32_t *__restrict__ perm,
                                            const int32_t *__restrict__ piv,
@@ -104,11 +106,11 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
                                            __nv_bfloat16 *__restrict__ Wb,
                                            __nv_bfloat16 *__restrict__ Lb, int Kp, int64_t brow0,
                                            int64_t lo_off, int pieces, int64_t tile, double *xs) {
-    constexpr int LDX = kRows + 1;
+    constexpr int LDX = kRows + 1, SUB = kRows / RT, CW = kWarps * SUB;
     const int64_t m = n - p;
-    const int64_t row0 = tile * kRows;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t row = row0 + lane;
+    const int64_t row0 = tile * RT;
+    const int r = (threadIdx.x & 31) % RT, w = (threadIdx.x >> 5) * SUB + (threadIdx.x & 31) / RT;
+    const int64_t row = row0 + r;
     const bool valid = row < m;
     double *A21 = A + p;
     const bool part = ps.mode == kFirst || ps.mode == kNext;
@@ -123,44 +125,48 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     // gather x = A21(rows, perm): each warp reads 32 consecutive rows of a column
     // (eight columns' loads in flight per warp)
 #pragma unroll 1
-    for (int k0 = c0 + w; k0 < c1; k0 += 8 * kWarps) {
+    for (int k0 = c0 + w; k0 < c1; k0 += 8 * CW) {
         double v[8];
 #pragma unroll
         for (int q = 0; q < 8; q++) {
-            const int k = k0 + q * kWarps;
+            const int k = k0 + q * CW;
             v[q] = 0.0;
             if (k < c1 && valid) v[q] = A21[(int64_t)(ps.mode <= kFirst ? perm[k] : k) * lda + row];
         }
 #pragma unroll
         for (int q = 0; q < 8; q++)
-            if (k0 + q * kWarps < c1) xs[(k0 + q * kWarps - c0) * LDX + lane] = v[q];
+            if (k0 + q * CW < c1) {
+                xs[(k0 + q * CW - c0) * LDX + r] = v[q];
+#pragma unroll
+                for (int z = RT; z < kRows; z += RT) xs[(k0 + q * CW - c0) * LDX + z + r] = 0.0;  // no such rows
+            }
     }
     __syncthreads();
 
     for (int j = j0; j < j1;) {
         const int kd = piv[j];
         if (kd == CTP_PIVKIND_2X2_FIRST && j + 1 < j1) {
-            const double y0 = xs[(j - c0) * LDX + lane], y1 = xs[(j + 1 - c0) * LDX + lane];
+            const double y0 = xs[(j - c0) * LDX + r], y1 = xs[(j + 1 - c0) * LDX + r];
             const double *l0 = A + (int64_t)j * lda, *l1 = A + (int64_t)(j + 1) * lda;
 #pragma unroll 4
-            for (int k = j + 2 + w; k < ku; k += kWarps)
-                xs[(k - c0) * LDX + lane] -= y0 * __ldg(l0 + k) + y1 * __ldg(l1 + k);
+            for (int k = j + 2 + w; k < ku; k += CW)
+                xs[(k - c0) * LDX + r] -= y0 * __ldg(l0 + k) + y1 * __ldg(l1 + k);
             j += 2;
         } else {
             // (a 2x2 pair that a block boundary cuts: its first column has nothing left
             // to update in its block, its second is a column like any other)
             if (kd == CTP_PIVKIND_1X1 || kd == CTP_PIVKIND_2X2_SECOND) {
-                const double y0 = xs[(j - c0) * LDX + lane];
+                const double y0 = xs[(j - c0) * LDX + r];
                 const double *l0 = A + (int64_t)j * lda;
 #pragma unroll 4
-                for (int k = j + 1 + w; k < ku; k += kWarps) xs[(k - c0) * LDX + lane] -= y0 * __ldg(l0 + k);
+                for (int k = j + 1 + w; k < ku; k += CW) xs[(k - c0) * LDX + r] -= y0 * __ldg(l0 + k);
             }
             j += 1;  // zero pivots have an all-zero L column
         }
         __syncthreads();
     }
 
-    const int tile_rows = m - row0 < kRows ? (int)(m - row0) : kRows;
+    const int tile_rows = m - row0 < RT ? (int)(m - row0) : RT;
     __shared__ short cexp[kMaxP];
     __shared__ int red[2 * kWarps * 32], rexp[32];
     if (part) {
@@ -171,7 +177,7 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
                                          rexp);
         }
         if (valid)
-            for (int k = c0 + w; k < c1; k += kWarps) A21[(int64_t)k * lda + row] = xs[(k - c0) * LDX + lane];
+            for (int k = c0 + w; k < c1; k += CW) A21[(int64_t)k * lda + row] = xs[(k - c0) * LDX + r];
         return;
     }
 
@@ -188,22 +194,22 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     __syncthreads();
     // L21 = Y D11^{-1} in place (1x1 and 2x2 blocks; zero pivots give 0), written
     // back with the delayed columns as they are
-    for (int k = w; k < c1; k += kWarps) {
+    for (int k = w; k < c1; k += CW) {
         const int kd = k < e ? piv[k] : CTP_PIVKIND_DELAYED;
         if (kd == CTP_PIVKIND_2X2_SECOND) continue;  // with its first column
-        double out = xs[k * LDX + lane];
+        double out = xs[k * LDX + r];
         if (kd == CTP_PIVKIND_2X2_FIRST) {
-            const double y0 = out, y1 = xs[(k + 1) * LDX + lane];
+            const double y0 = out, y1 = xs[(k + 1) * LDX + r];
             out = __fma_rn(y1, Dinv[2 * k + 1], y0 * Dinv[2 * k]);
             const double o1 = __fma_rn(y1, Dinv[2 * k + 2], y0 * Dinv[2 * k + 1]);
-            xs[(k + 1) * LDX + lane] = o1;
+            xs[(k + 1) * LDX + r] = o1;
             if (valid) A21[(int64_t)(k + 1) * lda + row] = o1;
         } else if (kd == CTP_PIVKIND_1X1) {
             out *= Dinv[2 * k];
         } else if (kd == CTP_PIVKIND_ZERO) {
             out = 0.0;
         }
-        if (kd != CTP_PIVKIND_DELAYED) xs[k * LDX + lane] = out;
+        if (kd != CTP_PIVKIND_DELAYED) xs[k * LDX + r] = out;
         if (valid) A21[(int64_t)k * lda + row] = out;
     }
     if (Lb == nullptr && sb.L == nullptr) return;
@@ -213,6 +219,7 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     if (Lb != nullptr) write_pieces(Lb, brow0 + row0, tile_rows, Kp, e, Kz, pieces, lo_off, xs);
 }
 
+template <int RT>
 __global__ void __launch_bounds__(kRows * kWarps)
     k_solve_fp64(SolvePass ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                  const int32_t *__restrict__ perm, const int32_t *__restrict__ piv,
@@ -220,11 +227,12 @@ __global__ void __launch_bounds__(kRows * kWarps)
                  SliceBuf sb, __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb, int Kp,
                  int64_t lo_off, int pieces) {
     extern __shared__ __align__(16) double xs[];  // [columns][kRows+1]
-    solve_tile(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
+    solve_tile<RT>(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
 }
 
-// Batched: CTA b takes work item b = (front, 32-row tile of its A21): the
+// Batched: CTA b takes work item b = (front, RT-row tile of its A21): the
 // front is item_front[b], the tile item_tile[b].
+template <int RT>
 __global__ void __launch_bounds__(kRows * kWarps)
     k_solve_batch(int mode, const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
                   const int *__restrict__ item_front, const int *__restrict__ item_tile, BatchOpts o,
@@ -243,7 +251,7 @@ __global__ void __launch_bounds__(kRows * kWarps)
     if (o.smode != CTP_S_NONE && o.prec == CTP_FP64) sb = bsection_slices(base, sec, bt.p);
     SolvePass ps = {mode, mode == kTail ? 1 : 0, {nullptr, nullptr, nullptr, nullptr, 0}};
     if (mode == kFirst) ps.yb = bsection_block(base, sec);
-    solve_tile(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
+    solve_tile<RT>(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
                *fr.nelim, sb, Wb, Lb, kBatchKp, bt.row0, o.lo_off, o.pieces,
                item_tile[blockIdx.x], xs);
 }
@@ -372,6 +380,18 @@ int solve_blocks(int64_t m, int p, int pivot) {
     return p > 128 || right * (p - kSliceK) >= 1.6e7 ? (p + kSliceK - 1) / kSliceK : 0;
 }
 
+// Rows per tile of a Solve with this many 32-row tiles: few tiles leave SMs idle, and
+// one tile per SM waits for its own chain of pivots, so they get 16 or 8 rows, up
+// to two tiles per SM.  Whole passes with 32 rows / with this rule, all columns accepted: n = 500,
+// p = 64: 61 / 45 us; n = 1000, p = 96: 113 / 70; n = 2000, p = 64: 61 / 45; n = 3500, p = 64: 61 / 49;
+// n = 9000, p = 64: 68 / 65; a dozen accepted: n = 2400, p = 96: 29 / 18; n = 2600, p = 64: 24 / 20.
+// Blocked ones (up to one tile per SM, their passes are short): p = 256, n = 600: 314 /
+// 271; n = 1500: 334 / 277; n = 5000: 334 / 314; p = 160, n = 2400: 203 / 170.
+int solve_rows(int64_t tiles, bool blocked, int num_sms) {
+    const int64_t sms = blocked ? num_sms : 2 * (int64_t)num_sms;
+    return tiles > sms ? kRows : (2 * tiles > sms ? kRows / 2 : kRows / 4);
+}
+
 // Entries of A21 from which a blocked Solve (p > 64) moves the columns, and scales them
 // when nothing else is left to do, in passes of their own: two launches more, but
 // the first block's elimination keeps eight CTAs per SM instead of three and the
@@ -387,12 +407,18 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
                               int64_t lo_off, int pieces, int32_t *info, int num_sms, cudaStream_t st) {
     const int64_t m = n - p;
     if (m <= 0) return cudaSuccess;
-    cudaError_t err = smem_at_least((const void *)k_solve_fp64, sizeof(double) * (size_t)p * (kRows + 1));
+    const size_t smem_p = sizeof(double) * (size_t)p * (kRows + 1);
+    const int rt = solve_rows((m + kRows - 1) / kRows, blocks > 0, num_sms);
+    const void *fn = rt == kRows       ? (const void *)k_solve_fp64<kRows>
+                     : rt == kRows / 2 ? (const void *)k_solve_fp64<kRows / 2>
+                                       : (const void *)k_solve_fp64<kRows / 4>;
+    cudaError_t err = smem_at_least(fn, smem_p);
     if (err != cudaSuccess) return err;
-    const unsigned grid = (unsigned)((m + kRows - 1) / kRows);
+    const unsigned grid = (unsigned)((m + rt - 1) / rt);
     auto pass = [&](int mode, int b, int cols) {
         const SolvePass ps = {mode, b, blk};
-        k_solve_fp64<<<grid, kRows * kWarps, sizeof(double) * (size_t)cols * (kRows + 1), st>>>(
+        auto *k = rt == kRows ? k_solve_fp64<kRows> : rt == kRows / 2 ? k_solve_fp64<kRows / 2> : k_solve_fp64<kRows / 4>;
+        k<<<grid, kRows * kWarps, sizeof(double) * (size_t)cols * (kRows + 1), st>>>(
             ps, A, n, p, lda, perm, piv, Dinv, nelim, sb, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, Kp, lo_off, pieces);
         return cudaGetLastError();
     };
@@ -431,42 +457,45 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
     return pass(kTail, blocks, p);
 }
 
+static decltype(&k_solve_batch<kRows>) solve_batch_kernel(int rows) {
+    return rows == kRows ? k_solve_batch<kRows> : rows == kRows / 2 ? k_solve_batch<kRows / 2> : k_solve_batch<kRows / 4>;
+}
+
 cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                               const int *item_front, int64_t items, BatchOpts o, void *Wb, void *Lb,
+                               const int *item_front, int64_t items, int rows, BatchOpts o, void *Wb, void *Lb,
                                int pmax, cudaStream_t st, const int *item_tile) {
     if (items == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (size_t)pmax * (kRows + 1);
-    cudaError_t err =
-        smem_at_least((const void *)k_solve_batch, smem);
+    auto *k = solve_batch_kernel(rows);
+    cudaError_t err = smem_at_least((const void *)k, smem);
     if (err != cudaSuccess) return err;
-    k_solve_batch<<<(unsigned)items, kRows * kWarps, smem, st>>>(
+    k<<<(unsigned)items, kRows * kWarps, smem, st>>>(
         kWhole, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
     return cudaGetLastError();
 }
 
 cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
                                        int count, const int *item_front, const int *item_tile, int64_t items,
-                                       const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
+                                       int rows, const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
                                        void *Lb, int pmax, int32_t *info, int num_sms, cudaStream_t st) {
     if (items == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (size_t)pmax * (kRows + 1);
-    cudaError_t err = smem_at_least((const void *)k_solve_batch, smem);
+    auto *k = solve_batch_kernel(rows);
+    cudaError_t err = smem_at_least((const void *)k, smem);
     if (err != cudaSuccess) return err;
     if (pmax > kSliceK) {
         const unsigned tiles = (unsigned)((pmax - 1) / kRows);  // 32-row tiles below the first block
         k_l11_slices_batch<<<dim3((unsigned)count, tiles), kRows * kWarps, 0, st>>>(fronts, tab, ws, list, o);
         if ((err = cudaGetLastError()) != cudaSuccess) return err;
     }
-    k_solve_batch<<<(unsigned)items, kRows * kWarps, smem, st>>>(
+    k<<<(unsigned)items, kRows * kWarps, smem, st>>>(
         kFirst, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     err = launch_update_batch(fronts, tab, ws, uitem, utile, uitems, o, info, num_sms, st);
     if (err != cudaSuccess) return err;
-    k_solve_batch<<<(unsigned)items, kRows * kWarps, smem, st>>>(
+    k<<<(unsigned)items, kRows * kWarps, smem, st>>>(
         kTail, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
     return cudaGetLastError();
 }
-
-int solve_rows_per_tile() { return kRows; }
 
 }  // namespace ctp
