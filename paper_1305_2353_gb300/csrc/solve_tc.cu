@@ -117,54 +117,63 @@ __device__ __forceinline__ double l21_of(const double *y, int o, const int32_t *
 }
 
 constexpr int kPrepRows = 1;  // identity rows (warps) per CTA: one, so the rows spread over the SMs' FP64 pipes
+constexpr int kPrepT = 128;   // threads: the others help to write the outputs
 
 // Z^T pieces: Zt[o * Kp + k] for output column o < kZRows, K index k < Kp.
-// One warp per identity row k (a CTA per row): the row lives in shared memory, each
-// position updated by one lane, and the warp runs the FP64 Solve's recurrence
-// with only warp barriers (row k is zero before position k, so its pivots
-// start at k's block).  The CTA then writes the Z^T column of its row.
-__global__ void __launch_bounds__(32 * kPrepRows)
+// One warp per identity row k (a CTA per row): the row lives in registers and the warp
+// runs the FP64 Solve's recurrence, a shuffle and the multiply-adds of the
+// positions behind it per pivot, the columns of L11 loaded four pivots ahead (row k is
+// zero before position k, so its pivots start at k's block).  The CTA then writes the
+// Z^T column of its row.  p = 256: 140 -> 97 us (the row in shared memory, an L2 round
+// trip and all positions' instructions per pivot before).
+__global__ void __launch_bounds__(kPrepT)
     k_stc_prep(const double *__restrict__ A, int p, int64_t lda, const int32_t *__restrict__ piv,
                const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p, __nv_bfloat16 *__restrict__ Zt,
                int Kp, int64_t zoff, int pieces) {
     __shared__ double rows[kPrepRows][kMaxP];
+    __shared__ int spiv[kMaxP];
+    constexpr int NG = kMaxP / 32;
     const int e = *nelim_p;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int k0 = blockIdx.x * kPrepRows, k = k0 + w;
-    __shared__ int spiv[kMaxP];
-    double *x = rows[w];  // this warp's row; position q is updated by lane q % 32 only
     for (int q = threadIdx.x; q < p; q += blockDim.x) spiv[q] = piv[q];
-    for (int q = lane; q < kMaxP; q += 32) x[q] = (q == k && k < e) ? 1.0 : 0.0;
+    double x[NG];  // this warp's row, positions lane + 32 s
+#pragma unroll
+    for (int s = 0; s < NG; s++) x[s] = (lane + 32 * s == k && k < e) ? 1.0 : 0.0;
     __syncthreads();
-    if (k < e) {
-        int j = (k > 0 && spiv[k] == CTP_PIVKIND_2X2_SECOND) ? k - 1 : k;
-        while (j < e) {
-            const int kd = spiv[j];
-            const double y0 = x[j];
-            // all of a lane's positions at once (predicated), so that the loads
-            // of the L column(s) are in flight together
-            if (kd == CTP_PIVKIND_2X2_FIRST) {
-                const double y1 = x[j + 1];
-                const double *l0 = A + (int64_t)j * lda, *l1 = A + (int64_t)(j + 1) * lda;
+    if (w < kPrepRows && k < e) {
+        const int start = (k > 0 && spiv[k] == CTP_PIVKIND_2X2_SECOND) ? k - 1 : k;
+        auto entry = [&](int c, int q) { return (c < e && q > c && q < p) ? __ldg(A + (int64_t)c * lda + q) : 0.0; };
+        double l[4][NG];  // the columns of L11 of this and the next three pivots
 #pragma unroll
-                for (int s2 = 0; s2 < kMaxP / 32; s2++) {
-                    const int q = lane + 32 * s2;
-                    if (q >= j + 2 && q < p) x[q] -= y0 * __ldg(l0 + q) + y1 * __ldg(l1 + q);
-                }
-                j += 2;
-            } else {
-                if (kd == CTP_PIVKIND_1X1) {
-                    const double *l0 = A + (int64_t)j * lda;
+        for (int a = 0; a < 4; a++)
 #pragma unroll
-                    for (int s2 = 0; s2 < kMaxP / 32; s2++) {
-                        const int q = lane + 32 * s2;
-                        if (q > j && q < p) x[q] -= y0 * __ldg(l0 + q);
+            for (int s = 0; s < NG; s++) l[a][s] = entry((start & ~3) + a, lane + 32 * s);
+#pragma unroll
+        for (int g = 0; g < NG; g++) {
+            const int j1 = min(e, 32 * g + 32);
+            for (int jb = max(start & ~3, 32 * g); jb < j1; jb += 4) {
+#pragma unroll
+                for (int a = 0; a < 4; a++) {
+                    const int c = jb + a;
+                    const int kd = c >= start && c < e ? spiv[c] : CTP_PIVKIND_ZERO;
+                    if (kd != CTP_PIVKIND_ZERO) {  // zero pivots have an all-zero L column
+                        const double yc = __shfl_sync(0xffffffffu, x[g], c & 31);
+                        // the (c + 1, c) slot of a 2x2 pivot holds D
+                        const int from = c + (kd == CTP_PIVKIND_2X2_FIRST ? 2 : 1);
+#pragma unroll
+                        for (int s = g; s < NG; s++)
+                            if (lane + 32 * s >= from) x[s] = fma(-yc, l[a][s], x[s]);
                     }
+#pragma unroll
+                    for (int s = g; s < NG; s++) l[a][s] = entry(c + 4, lane + 32 * s);
                 }
-                j += 1;  // zero pivots have an all-zero L column
             }
-            __syncwarp();  // the next pivot's y is written by another lane
         }
+    }
+    if (w < kPrepRows) {
+#pragma unroll
+        for (int s = 0; s < NG; s++) rows[w][lane + 32 * s] = x[s];
     }
     __syncthreads();
     // Z^T columns of these rows: thread (o, r) writes Zt[o * Kp + k0 + r]
@@ -710,7 +719,7 @@ cudaError_t launch_solve_tc(double *A, int64_t n, int p, int64_t lda, const int3
     const size_t smem = sizeof(double) * (size_t)p * (kRowsG + 1);
     cudaError_t err = smem_at_least((const void *)k_stc_gather, smem);
     if (err != cudaSuccess) return err;
-    k_stc_prep<<<Kp / kPrepRows, 32 * kPrepRows, 0, st>>>(A, p, lda, piv, Dinv, nelim, Zt, Kp, zoff, spieces);
+    k_stc_prep<<<Kp / kPrepRows, kPrepT, 0, st>>>(A, p, lda, piv, Dinv, nelim, Zt, Kp, zoff, spieces);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     k_stc_gather<<<(unsigned)((m + kRowsG - 1) / kRowsG), kRowsG * kWarpsG, smem, st>>>(
