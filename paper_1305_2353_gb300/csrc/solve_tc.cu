@@ -195,6 +195,43 @@ __global__ void __launch_bounds__(kPrepT)
     }
 }
 
+// The BF16 pieces of two neighbours.  v is held as two floats first, v = f + g to 2^-48,
+// so that only two conversions and a subtraction per value go through the FP64 pipe
+// (five with put_pieces); each piece rounds what the ones before it left, kept in f
+// and g exactly.  Values that a float does not hold normally take put_pieces.
+__device__ __forceinline__ bool float_pair(double v, float &f, float &g) {
+    f = (float)v;
+    const unsigned b = __float_as_uint(f), ex = (b >> 23) & 0xFFu;
+    if (ex - 64u > 126u) {  // below 2^-63, above 2^64, zero, Inf or NaN
+        g = 0.0f;
+        return v == 0.0;
+    }
+    const unsigned long long d = ((unsigned long long)(b >> 31) << 63) |
+                                 ((unsigned long long)(ex + 896u) << 52) | ((unsigned long long)(b & 0x7FFFFFu) << 29);
+    g = (float)(v - __longlong_as_double((long long)d));
+    return true;
+}
+__device__ __forceinline__ void put_pieces_pair(__nv_bfloat16 *dst, int64_t piece_off, int pieces, double v0,
+                                                double v1) {
+    float f0, g0, f1, g1;
+    const bool ok0 = float_pair(v0, f0, g0), ok1 = float_pair(v1, f1, g1);
+    if (!ok0 || !ok1) {
+        put_pieces(dst, piece_off, pieces, v0);
+        put_pieces(dst + 1, piece_off, pieces, v1);
+        return;
+    }
+    for (int pc = 0; pc < pieces; pc++) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(f0 + g0, f1 + g1);
+        *reinterpret_cast<__nv_bfloat162 *>(dst + pc * piece_off) = b;
+        // f - b is exact, and so is moving what it no longer needs of g into it
+        float r0 = f0 - __low2float(b), r1 = f1 - __high2float(b);
+        f0 = r0 + g0;
+        f1 = r1 + g1;
+        g0 -= f0 - r0;
+        g1 -= f1 - r1;
+    }
+}
+
 // Gather of x through perm; x_e to BF16 pieces, x_d back in place (FP64), and
 // the zero tails (K >= e) of the Form's operand pieces.
 __global__ void __launch_bounds__(kRowsG * kWarpsG)
@@ -211,21 +248,41 @@ __global__ void __launch_bounds__(kRowsG * kWarpsG)
     const int64_t row = row0 + lane;
     const bool valid = row < m;
     double *A21 = A + p;
-    for (int k = w; k < p; k += kWarpsG) {
-        const int c = perm[k];
-        xs[k * LDX + lane] = valid ? A21[(int64_t)c * lda + row] : 0.0;
+#pragma unroll 1
+    for (int k0 = w; k0 < p; k0 += 8 * kWarpsG) {  // eight columns' loads in flight per warp
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            const int k = k0 + q * kWarpsG;
+            v[q] = k < p && valid ? A21[(int64_t)perm[k] * lda + row] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+            if (k0 + q * kWarpsG < p) xs[(k0 + q * kWarpsG) * LDX + lane] = v[q];
     }
     __syncthreads();
-    // x_e pieces and the Form operands' zero tails: a warp writes one row at a time
+    // x_e pieces and the Form operands' zero tails: a warp writes one row at a time, two
+    // columns per lane (Kp and the pieces' offsets are even)
+    const __nv_bfloat162 z = __floats2bfloat162_rn(0.0f, 0.0f);
     for (int rr = w; rr < kRowsG; rr += kWarpsG) {
         const int64_t rw = row0 + rr;
         if (rw >= m) break;
-        for (int k = lane; k < Kp; k += 32) {
-            const double v = k < e ? xs[k * LDX + rr] : 0.0;
-            put_pieces(Xb + rw * Kp + k, xoff, xpieces, v);
-            if (k >= e && Lb != nullptr) {
-                put_pieces(Lb + rw * Kp + k, foff, fpieces, 0.0);
-                put_pieces(Wb + rw * Kp + k, foff, fpieces, 0.0);
+        for (int k = 2 * lane; k < Kp; k += 64) {
+            const int64_t at = rw * Kp + k;
+            if (k < e) {
+                put_pieces_pair(Xb + at, xoff, xpieces, xs[k * LDX + rr], k + 1 < e ? xs[(k + 1) * LDX + rr] : 0.0);
+            } else {
+                for (int pc = 0; pc < xpieces; pc++) *reinterpret_cast<__nv_bfloat162 *>(Xb + at + pc * xoff) = z;
+            }
+            if (k + 1 >= e && Lb != nullptr) {
+                for (int pc = 0; pc < fpieces; pc++) {
+                    if (k >= e) {
+                        *reinterpret_cast<__nv_bfloat162 *>(Lb + at + pc * foff) = z;
+                        *reinterpret_cast<__nv_bfloat162 *>(Wb + at + pc * foff) = z;
+                    } else {
+                        Lb[at + 1 + pc * foff] = Wb[at + 1 + pc * foff] = __float2bfloat16_rn(0.0f);
+                    }
+                }
             }
         }
     }
