@@ -130,6 +130,8 @@ __global__ void __launch_bounds__(kPrepT)
     k_stc_prep(const double *__restrict__ A, int p, int64_t lda, const int32_t *__restrict__ piv,
                const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p, __nv_bfloat16 *__restrict__ Zt,
                int Kp, int64_t zoff, int pieces) {
+    // the gather behind this kernel depends on nothing that it writes
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ double rows[kPrepRows][kMaxP];
     __shared__ int spiv[kMaxP];
     constexpr int NG = kMaxP / 32;
@@ -289,6 +291,8 @@ __global__ void __launch_bounds__(kRowsG * kWarpsG)
     // x_d at the delayed positions, in place (this tile's rows only)
     if (valid)
         for (int k = e + w; k < p; k += kWarpsG) A21[(int64_t)k * lda + row] = xs[k * LDX + lane];
+    // launched beside the preparation of Z^T: what follows needs both
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---- batched forms: x_e and Z^T of every front in 128 x 64 BF16 tiles (the
@@ -779,9 +783,20 @@ cudaError_t launch_solve_tc(double *A, int64_t n, int p, int64_t lda, const int3
     k_stc_prep<<<Kp / kPrepRows, kPrepT, 0, st>>>(A, p, lda, piv, Dinv, nelim, Zt, Kp, zoff, spieces);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    k_stc_gather<<<(unsigned)((m + kRowsG - 1) / kRowsG), kRowsG * kWarpsG, smem, st>>>(
-        A, n, p, lda, perm, nelim, Xb, xoff, spieces, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, foff, fpieces, Kp);
-    err = cudaGetLastError();
+    // beside the preparation (a chain of pivots that leaves most of the chip idle), by
+    // programmatic dependent launch: n = 40000, p = 256, both: 262 -> 238 us of Solve
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)((m + kRowsG - 1) / kRowsG));
+    cfg.blockDim = dim3(kRowsG * kWarpsG);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    err = cudaLaunchKernelEx(&cfg, k_stc_gather, A, n, p, lda, perm, nelim, Xb, xoff, spieces, (__nv_bfloat16 *)Wb,
+                             (__nv_bfloat16 *)Lb, foff, fpieces, Kp);
     if (err != cudaSuccess) return err;
     CUtensorMap mX[3], mZ[3];
     for (int pc = 0; pc < 3; pc++) {
