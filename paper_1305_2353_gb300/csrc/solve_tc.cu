@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(kPrepT)
         const int start = (k > 0 && spiv[k] == CTP_PIVKIND_2X2_SECOND) ? k - 1 : k;
         auto entry = [&](int c, int q) { return (c < e && q > c && q < p) ? __ldg(A + (int64_t)c * lda + q) : 0.0; };
         double l[4][NG];  // the columns of L11 of this and the next three pivots
+        double l0[NG], y0 = 0.0;  // the first column of the 2x2 pivot at hand and its y
 #pragma unroll
         for (int a = 0; a < 4; a++)
 #pragma unroll
@@ -161,11 +162,19 @@ __global__ void __launch_bounds__(kPrepT)
                     const int kd = c >= start && c < e ? spiv[c] : CTP_PIVKIND_ZERO;
                     if (kd != CTP_PIVKIND_ZERO) {  // zero pivots have an all-zero L column
                         const double yc = __shfl_sync(0xffffffffu, x[g], c & 31);
-                        // the (c + 1, c) slot of a 2x2 pivot holds D
-                        const int from = c + (kd == CTP_PIVKIND_2X2_FIRST ? 2 : 1);
+                        if (kd == CTP_PIVKIND_2X2_FIRST) {  // applied with its second column
+                            y0 = yc;
 #pragma unroll
-                        for (int s = g; s < NG; s++)
-                            if (lane + 32 * s >= from) x[s] = fma(-yc, l[a][s], x[s]);
+                            for (int s = g; s < NG; s++) l0[s] = l[a][s];
+                        } else if (kd == CTP_PIVKIND_2X2_SECOND) {
+#pragma unroll
+                            for (int s = g; s < NG; s++)
+                                if (lane + 32 * s > c) x[s] -= fma(y0, l0[s], yc * l[a][s]);
+                        } else {
+#pragma unroll
+                            for (int s = g; s < NG; s++)
+                                if (lane + 32 * s > c) x[s] = fma(-yc, l[a][s], x[s]);
+                        }
                     }
 #pragma unroll
                     for (int s = g; s < NG; s++) l[a][s] = entry(c + 4, lane + 32 * s);
@@ -197,40 +206,58 @@ __global__ void __launch_bounds__(kPrepT)
     }
 }
 
-// The BF16 pieces of two neighbours.  v is held as two floats first, v = f + g to 2^-48,
-// so that only two conversions and a subtraction per value go through the FP64 pipe
-// (five with put_pieces); each piece rounds what the ones before it left, kept in f
-// and g exactly.  Values that a float does not hold normally take put_pieces.
-__device__ __forceinline__ bool float_pair(double v, float &f, float &g) {
-    f = (float)v;
-    const unsigned b = __float_as_uint(f), ex = (b >> 23) & 0xFFu;
-    if (ex - 64u > 126u) {  // below 2^-63, above 2^64, zero, Inf or NaN
-        g = 0.0f;
-        return v == 0.0;
+// put_pieces of two neighbours, bit for bit, without the FP64 pipe: a value in the
+// middle of FP64's range is its 53-bit integer significand, kept normalized in 64
+// bits; a piece rounds it to 24 bits (to FP32) and those to 8, and what is
+// left is exact in 64-bit integers.  `at` is the exponent of the value's top bit.
+struct PieceInt {
+    unsigned long long n;  // top bit set, or 0
+    unsigned sign;         // in bit 15
+    int at;
+};
+__device__ __forceinline__ bool piece_int(double v, PieceInt &x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int ex = (int)((b >> 52) & 0x7FFu);
+    x.n = (b << 11) | (1ull << 63);
+    x.sign = (unsigned)(b >> 48) & 0x8000u;
+    x.at = ex - 1023;
+    if ((b << 1) == 0ull) {
+        x.n = 0ull;
+        return true;
     }
-    const unsigned long long d = ((unsigned long long)(b >> 31) << 63) |
-                                 ((unsigned long long)(ex + 896u) << 52) | ((unsigned long long)(b & 0x7FFFFFu) << 29);
-    g = (float)(v - __longlong_as_double((long long)d));
-    return true;
+    return (unsigned)(x.at + 63) <= 126u;  // the third piece is a normal BF16 too
+}
+__device__ __forceinline__ unsigned next_piece(PieceInt &x) {
+    if (x.n == 0ull) {
+        const unsigned z = x.sign;
+        x.sign = 0u;  // -0 leaves +0
+        return z;
+    }
+    const unsigned h = (unsigned)(x.n >> 32);
+    const unsigned q = (h >> 1) | (h & 1u) | ((unsigned)x.n != 0u ? 1u : 0u);  // sticky
+    const unsigned t24 = (q + 0x3Fu + ((q >> 7) & 1u)) >> 7;
+    const unsigned t8 = (t24 + 0x7FFFu + ((t24 >> 16) & 1u)) >> 16;  // 128 .. 256
+    const unsigned out = x.sign + (unsigned)((x.at + 127) << 7) + t8 - 128u;
+    const long long left = (long long)(x.n - ((unsigned long long)t8 << 56));  // modulo 2^64: also for 256
+    const unsigned long long a = left < 0 ? 0ull - (unsigned long long)left : (unsigned long long)left;
+    const int lz = __clzll((long long)a);
+    x.sign = a == 0ull ? 0u : (left < 0 ? x.sign ^ 0x8000u : x.sign);
+    x.n = a << (lz & 63);
+    x.at -= lz;
+    return out;
 }
 __device__ __forceinline__ void put_pieces_pair(__nv_bfloat16 *dst, int64_t piece_off, int pieces, double v0,
                                                 double v1) {
-    float f0, g0, f1, g1;
-    const bool ok0 = float_pair(v0, f0, g0), ok1 = float_pair(v1, f1, g1);
+    PieceInt x0, x1;
+    const bool ok0 = piece_int(v0, x0), ok1 = piece_int(v1, x1);
     if (!ok0 || !ok1) {
         put_pieces(dst, piece_off, pieces, v0);
         put_pieces(dst + 1, piece_off, pieces, v1);
         return;
     }
     for (int pc = 0; pc < pieces; pc++) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(f0 + g0, f1 + g1);
-        *reinterpret_cast<__nv_bfloat162 *>(dst + pc * piece_off) = b;
-        // f - b is exact, and so is moving what it no longer needs of g into it
-        float r0 = f0 - __low2float(b), r1 = f1 - __high2float(b);
-        f0 = r0 + g0;
-        f1 = r1 + g1;
-        g0 -= f0 - r0;
-        g1 -= f1 - r1;
+        const unsigned lo = next_piece(x0), hi = next_piece(x1);
+        *reinterpret_cast<uint32_t *>(dst + pc * piece_off) = lo | (hi << 16);
     }
 }
 
