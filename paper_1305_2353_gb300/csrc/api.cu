@@ -58,6 +58,10 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     off += align256(sizeof(int32_t) * (size_t)ms);
     L.el = off;
     off += align256(sizeof(int32_t) * (size_t)ms);
+    L.gw = off;
+    off += align256(slice_gw_bytes(ms, p));
+    L.gl = off;
+    off += align256(slice_gl_bytes(ms, p));
     // the blocked FP64 Solve
     const int blocks = opt->pivot != CTP_PIV_TPP && !solve_on_tc(opt) ? solve_blocks(m, p, opt->pivot) : 0;
     L.Yb = off;
@@ -68,6 +72,13 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     off += align256(sizeof(int32_t) * (size_t)(blocks > 0 ? m : 0));
     L.ex = off;
     off += align256(sizeof(int32_t) * (size_t)blocks * kMaxP);
+    L.gy = off;
+    off += align256(slice_gw_bytes(blocks > 0 ? m : 0, kSliceK));
+    L.gx = off;
+    off += align256(blocks * slice_gl_bytes(p, kSliceK));
+    L.marks = off;
+    const int64_t ut = blocks > 0 ? update_tiles(m, p) : 0, ft = form_fp64_slots(ms);
+    off += align256(sizeof(TileMarks) * (size_t)(ut > ft ? ut : ft));
     // BF16 operand copies (hi, and for the split form the lo parts after them)
     const size_t nb = tc ? 2 * (size_t)m * form_tc_kpad(p) * prec_pieces(opt->prec) : 0;
     L.Wb = off;
@@ -267,10 +278,10 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
     char *ws = (char *)workspace;
     int32_t *info = (int32_t *)(ws + L.info);
     double *Dinv = (double *)(ws + L.Dinv);
-    SliceBuf sb = {nullptr, nullptr, nullptr, nullptr, 0};
+    SliceBuf sb = {};
     if (opt->smode != CTP_S_NONE && !tc)
         sb = {(unsigned char *)(ws + L.Ws), (unsigned char *)(ws + L.Ls), (int32_t *)(ws + L.ew),
-              (int32_t *)(ws + L.el), slice_kb(p)};
+              (int32_t *)(ws + L.el), (uint16_t *)(ws + L.gw), (uint16_t *)(ws + L.gl), slice_kb(p)};
     void *Wb = tc ? (void *)(ws + L.Wb) : nullptr;
     void *Lbf = tc ? (void *)(ws + L.Lb) : nullptr;
     const int Kp = form_tc_kpad(p);
@@ -289,8 +300,8 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
                 return launch_slices_from_l(A, lda, p, m, piv, D, Dinv, nelim, sb, st);
             }));
             CTP_CUDA(timed(ctx, K_FORM, st, [&] {
-                return launch_form_fp64(sb, A + p, lda, piv, D, m, nelim, S, lds, opt->smode, info, ctx->num_sms,
-                                        st);
+                return launch_form_fp64(sb, A + p, lda, piv, D, m, nelim, S, lds, opt->smode, (TileMarks *)(ws + L.marks),
+                                        info, ctx->num_sms, st);
             }));
         }
         return CTP_OK;
@@ -353,9 +364,10 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
     else if (m > 0)
         CTP_CUDA(timed(ctx, K_SOLVE, st, [&] {
             const SliceBuf blk = {(unsigned char *)(ws + L.Yb), (unsigned char *)(ws + L.Lx),
-                                  (int32_t *)(ws + L.ey), (int32_t *)(ws + L.ex), 1};
+                                  (int32_t *)(ws + L.ey), (int32_t *)(ws + L.ex), (uint16_t *)(ws + L.gy),
+                                  (uint16_t *)(ws + L.gx), 1};
             return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, sb, blk, solve_blocks(m, p, opt->pivot), Wb,
-                                     Lbf, Kp, lo_off, pieces, info, ctx->num_sms, st);
+                                     Lbf, Kp, lo_off, pieces, (TileMarks *)(ws + L.marks), info, ctx->num_sms, st);
         }));
     if (opt->smode != CTP_S_NONE && m > 0) {
         if (tc)
@@ -367,8 +379,8 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
             }));
         else
             CTP_CUDA(timed(ctx, K_FORM, st, [&] {
-                return launch_form_fp64(sb, A + p, lda, piv, D, m, nelim, S, lds, opt->smode, info, ctx->num_sms,
-                                        st);
+                return launch_form_fp64(sb, A + p, lda, piv, D, m, nelim, S, lds, opt->smode, (TileMarks *)(ws + L.marks),
+                                        info, ctx->num_sms, st);
             }));
     }
     return CTP_OK;

@@ -223,7 +223,8 @@ struct ctp_plan {
     bool tc;
     // workspace layout
     size_t off_ginfo, off_tab, off_citem, off_sitem, off_fitem, off_lists, off_flags, off_sections, off_wb,
-        off_lb, off_qitem, off_ritem, off_xt, off_zt, off_csitem, off_cstile, off_cfitem, off_cftile, off_cuitem, off_cutile;
+        off_lb, off_qitem, off_ritem, off_xt, off_zt, off_csitem, off_cstile, off_cfitem, off_cftile, off_cuitem, off_cutile,
+        off_fmarks, off_umarks;
     size_t total;
     int64_t c_items, s_items, f_items, total_rows, q_items, r_items, nxt, nzt;
     int64_t cbucket[5] = {0, 0, 0, 0, 0};  // compression items of fronts with p <= 32, 64, 128, 256
@@ -548,6 +549,11 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     off += align256(stc ? 2 * 3 * (size_t)P->bo.xoff : 0);
     P->off_zt = off;
     off += align256(stc ? 2 * 3 * (size_t)P->bo.zoff : 0);
+    const bool slices = P->opt.smode != CTP_S_NONE && P->opt.prec == CTP_FP64;
+    P->off_fmarks = off;
+    off += align256(slices ? sizeof(TileMarks) * (size_t)P->f_items : 0);
+    P->off_umarks = off;
+    off += align256(sizeof(TileMarks) * cuitem.size());
     P->total = off;
     // section offsets are relative to the sections base: shift them to the workspace base
     for (int f = 0; f < nb; f++) tab[f].ws += (int64_t)P->off_sections;
@@ -659,7 +665,8 @@ cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, ch
             reinterpret_cast<const int *>(w + P->off_cuitem) + c.u_off,
             reinterpret_cast<const int *>(w + P->off_cutile) + c.u_off, c.u_count, P->bo,
             P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax,
-            reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
+            reinterpret_cast<TileMarks *>(w + P->off_umarks) + c.u_off, reinterpret_cast<int32_t *>(w + P->off_ginfo),
+            num_sms, st);
     return launch_solve_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
                               reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off, c.s_count, c.s_rows, P->bo,
                               P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax, st,
@@ -678,6 +685,7 @@ cudaError_t batch_form_class(const ctp_plan *P, int ci, const ctp_front *fr, cha
                                     P->bo.pieces, P->opt.smode == CTP_S_FP64_SUB ? 3 : 2,
                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st, ftile);
     return launch_form_fp64_batch(fr, tab, w, fitem, c.f_count, P->bo,
+                                  reinterpret_cast<TileMarks *>(w + P->off_fmarks) + c.f_off,
                                   reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st, ftile);
 }
 cudaError_t batch_form(const ctp_plan *P, const ctp_front *fr, char *w, int num_sms, cudaStream_t st) {
@@ -689,6 +697,7 @@ cudaError_t batch_form(const ctp_plan *P, const ctp_front *fr, char *w, int num_
                                     P->bo.pieces, P->opt.smode == CTP_S_FP64_SUB ? 3 : 2,
                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
     return launch_form_fp64_batch(fr, tab, w, fitem, P->f_items, P->bo,
+                                  reinterpret_cast<TileMarks *>(w + P->off_fmarks),
                                   reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
 }
 

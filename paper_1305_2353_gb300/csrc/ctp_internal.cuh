@@ -21,13 +21,17 @@ constexpr int kSliceK = 32;                       // pivots per K block
 constexpr int kWRows = 128, kLRows = 64;          // rows per block
 constexpr uint32_t kWSlice = kWRows * 64, kLSlice = kLRows * 64;  // bytes of one slice of one K block
 constexpr uint32_t kWBlock = kSlices * kWSlice, kLBlock = kSlices * kLSlice;
-constexpr int kExpZero = -100000, kExpNonfinite = 1 << 20, kExpWide = 1 << 24;
+constexpr int kExpZero = -100000, kExpNonfinite = 1 << 20;
+constexpr int kGroup = 4;  // rows that share a lower bound of their entries
+constexpr uint32_t kWGroup = kWRows / kGroup * kSliceK * 2, kLGroup = kLRows / kGroup * kSliceK * 2;  // a block's bytes
 
 // Where a supernode's slices live: blocks at (row block * kb + K block), the
-// rows' exponents E; kb = ceil(p / 32).
+// rows' exponents E, the groups' lower bounds (FP16) in blocks like the slices'; kb =
+// ceil(p / 32).
 struct SliceBuf {
     unsigned char *W, *L;
     int32_t *ew, *el;
+    uint16_t *gw, *gl;
     int kb;
 };
 __host__ __device__ inline int slice_kb(int p) { return (p + kSliceK - 1) / kSliceK; }
@@ -37,19 +41,34 @@ __host__ __device__ inline size_t slice_w_bytes(int64_t m, int p) {
 __host__ __device__ inline size_t slice_l_bytes(int64_t m, int p) {
     return (size_t)((m + kLRows - 1) / kLRows) * slice_kb(p) * kLBlock;
 }
+__host__ __device__ inline size_t slice_gw_bytes(int64_t m, int p) {
+    return (size_t)((m + kWRows - 1) / kWRows) * slice_kb(p) * kWGroup;
+}
+__host__ __device__ inline size_t slice_gl_bytes(int64_t m, int p) {
+    return (size_t)((m + kLRows - 1) / kLRows) * slice_kb(p) * kLGroup;
+}
+
+// Which entries of a tile of the FP64 Form (or of the Solve's update) digits do not serve,
+// for the kernel's own use: a bit per column for every row of a warp's block, and
+// the CTA's tile before it that has any.
+struct TileMarks {
+    uint16_t out[kWRows * kLRows / 512][32];
+    int64_t prev, pad;
+};
 
 // Workspace layout (all offsets 256-byte aligned):
 //   [0, 256)            info word + scratch counters
 //   C                   p*p doubles, row-major compressed matrix (strict: as uint64 keys)
 //   Dinv                2p doubles: inverse pivot blocks, same slots as D
-//   Ws, Ls, ew, el      digit slices of Y = L21 D11 and L21 and their row exponents
-//                       (slices.cuh) when the FP64 Form step runs
-//   Yb, Lx, ey, ex      digit slices of one block's y and of L11, and their row
-//                       exponents, for the blocked FP64 Solve
+//   Ws, Ls, ew, el,     digit slices of Y = L21 D11 and L21, their row exponents and
+//     gw, gl            lower bounds (slices.cuh) when the FP64 Form step runs
+//   Yb, Lx, ey, ex,     the same of one block's y and of L11 for the blocked FP64 Solve
+//     gy, gx
+//   marks               a TileMarks per tile of the FP64 Form and of the Solve's updates
 //   Wb, Lb              m*Kp BF16 copies of Y and L21 for the tensor-core Form
 //   aux                 method-specific scratch (relaxed candidate lists)
 struct WsLayout {
-    size_t info, C, Dinv, Ws, Ls, ew, el, Yb, Lx, ey, ex, Wb, Lb, aux, Xs, flags, total;
+    size_t info, C, Dinv, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, marks, Wb, Lb, aux, Xs, flags, total;
 };
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -126,7 +145,7 @@ struct BFront {
 // offsets inside a front's section: info word, compressed matrix (strict),
 // Dinv, and the digit slices of L21 D11 and L21 when an FP64 Form follows
 struct BSection {
-    size_t info, C, Dinv, Ws, Ls, ew, el, Yb, Lx, ey, ex, nz, total;
+    size_t info, C, Dinv, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, nz, total;
 };
 __host__ __device__ inline size_t align256hd(size_t x) { return (x + 255) & ~size_t(255); }
 __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options *opt) {
@@ -147,6 +166,10 @@ __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options
     off += align256hd(sizeof(int32_t) * (size_t)ms);
     s.el = off;
     off += align256hd(sizeof(int32_t) * (size_t)ms);
+    s.gw = off;
+    off += align256hd(slice_gw_bytes(ms, p));
+    s.gl = off;
+    off += align256hd(slice_gl_bytes(ms, p));
     // the blocked Solve's first block: slices of y and of L11's rows below it
     const int64_t mb = p > kSliceK ? n - p : 0;
     s.Yb = off;
@@ -157,6 +180,10 @@ __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options
     off += align256hd(sizeof(int32_t) * (size_t)mb);
     s.ex = off;
     off += align256hd(mb > 0 ? sizeof(int32_t) * (size_t)p : 0);
+    s.gy = off;
+    off += align256hd(slice_gw_bytes(mb, kSliceK));
+    s.gx = off;
+    off += align256hd(mb > 0 ? slice_gl_bytes(p, kSliceK) : 0);
     s.nz = off;  // strict: which rows of C receive an A21 row (one bit per row)
     off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
     s.total = off;
@@ -169,6 +196,8 @@ __host__ __device__ inline SliceBuf bsection_slices(char *base, const BSection &
     b.L = reinterpret_cast<unsigned char *>(base + s.Ls);
     b.ew = reinterpret_cast<int32_t *>(base + s.ew);
     b.el = reinterpret_cast<int32_t *>(base + s.el);
+    b.gw = reinterpret_cast<uint16_t *>(base + s.gw);
+    b.gl = reinterpret_cast<uint16_t *>(base + s.gl);
     b.kb = slice_kb(p);
     return b;
 }
@@ -179,6 +208,8 @@ __host__ __device__ inline SliceBuf bsection_block(char *base, const BSection &s
     b.L = reinterpret_cast<unsigned char *>(base + s.Lx);
     b.ew = reinterpret_cast<int32_t *>(base + s.ey);
     b.el = reinterpret_cast<int32_t *>(base + s.ex);
+    b.gw = reinterpret_cast<uint16_t *>(base + s.gy);
+    b.gl = reinterpret_cast<uint16_t *>(base + s.gx);
     b.kb = 1;
     return b;
 }
@@ -211,8 +242,8 @@ int solve_rows(int64_t tiles, bool blocked, int num_sms);
 // item_tile (optional, both batched Forms): each item's tile of its front;
 // without it the items of a front are consecutive, from tab[front].f0 on
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                                   const int *item_front, int64_t items, BatchOpts o, int32_t *info, int num_sms,
-                                   cudaStream_t st, const int *item_tile = nullptr);
+                                   const int *item_front, int64_t items, BatchOpts o, TileMarks *marks, int32_t *info,
+                                   int num_sms, cudaStream_t st, const int *item_tile = nullptr);
 cudaError_t launch_form_tc_batch(const ctp_front *fronts, const BFront *tab, const int *item_front,
                                  int64_t items, int64_t total_rows, const void *Wb, const void *Lb,
                                  int pieces, int layout /* 2 tiled, 3 subtract */, int32_t *info, int num_sms,
@@ -270,21 +301,22 @@ cudaError_t launch_solve_tc_batch(const ctp_front *fronts, const BFront *tab, ch
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
                               const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
-                              int64_t lo_off, int pieces, int32_t *info, int num_sms, cudaStream_t st);
+                              int64_t lo_off, int pieces, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st);
 int solve_blocks(int64_t m, int p, int pivot);  // 0: a whole pass
 // A21(:, 32 (blk+1)..p-1) -= y_blk L11(32 (blk+1).., block blk)^T from the slices (form.cu)
 cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int64_t m, int blk, const int32_t *piv,
-                          const int32_t *nelim, int32_t *info, int num_sms, cudaStream_t st);
+                          const int32_t *nelim, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st);
 // the same for block 0 of a batch's fronts, by (front, tile) items
 cudaError_t launch_update_batch(const ctp_front *fronts, const BFront *tab, char *ws, const int *item_front,
-                                const int *item_tile, int64_t items, BatchOpts o, int32_t *info, int num_sms,
-                                cudaStream_t st);
+                                const int *item_tile, int64_t items, BatchOpts o, TileMarks *marks, int32_t *info,
+                                int num_sms, cudaStream_t st);
 int64_t update_tiles(int64_t m, int p);  // of a front, for block 0
+int64_t form_fp64_slots(int64_t m);      // of a single supernode's Form
 // a batch class's Solve in one block of 32 columns, its update and the tail
 cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
                                        int count, const int *item_front, const int *item_tile, int64_t items,
                                        int rows, const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
-                                       void *Lb, int pmax, int32_t *info, int num_sms, cudaStream_t st);
+                                       void *Lb, int pmax, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st);
 
 // Threshold partial pivoting on all n rows (the comparator of the compressed path).
 size_t tpp_ws_bytes(int p);
@@ -305,7 +337,7 @@ cudaError_t launch_form_tc(const void *Wb, const void *Lb, int64_t piece_off, in
 // (L21, D and the pivot kinds serve the rows that the slices do not represent)
 cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda, const int32_t *piv,
                              const double *D, int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
-                             int32_t *info, int num_sms, cudaStream_t st);
+                             TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st);
 // the slices from a stored L21 and its D, D^-1 (full-column pivoting)
 cudaError_t launch_slices_from_l(const double *A, int64_t lda, int p, int64_t m, const int32_t *piv,
                                  const double *D, const double *Dinv, const int32_t *nelim, const SliceBuf &sb,

@@ -6,9 +6,9 @@
 // eight digit slices each (slices.cuh), the products d_s d_t' of slices with
 // g = s + t <= 7 are summed per g in FP32 without rounding, and the epilogue
 // adds the eight sums, which are integers, in 64-bit integer arithmetic and
-// rounds once to FP64.  slices.cuh says what this loses (less than the rounding
-// of FP64 multiply-adds) and which rows it is not good enough for: those are
-// marked, and the epilogue takes their entries by FP64 multiply-adds.
+// rounds once to FP64.  slices.cuh says what this loses: less than FP64
+// multiply-adds may, of every entry whose rows are large in common pivots.  The epilogue
+// makes sure of that for every entry and takes the others by FP64 multiply-adds.
 //
 // Kernel: persistent, one CTA per SM, tiles of 128 rows x 64 columns.
 //   warp 0      producer: bulk copies of K blocks of 32 pivots (W 64 KB, L 32 KB:
@@ -19,13 +19,21 @@
 //               its results land in the accumulators of g = s..7 (64 TMEM
 //               columns each, all 512 in use): twelve MMAs of N <= 256 per
 //               16 pivots for all 36 products.
+//   warp 18     scheduler: looks the tiles up (some 3000 clocks each: a walk over the
+//               triangle or a chain of a batch's descriptors) and hands them to the others
+//               through a ring of four.
+//   warp 19     checker: tells for every 4 x 4 block of a tile's entries whether digits
+//               serve it, from the groups' lower bounds (3 KB per K block): 512 sums of
+//               e products, four rows and columns of them per lane.  The epilogue finds
+//               a bit per block when the accumulators are full, and leaves entries of the
+//               others out; they are computed after the CTA's last tile.
 //   warps 2-17  epilogue: a thread holds 16 columns of one row of S as 64-bit
 //               integers; the accumulators are handed back as soon as they have
 //               been added up, and rounding and stores overlap the next tile.
 // The same kernel, kMode kUpdate, is the Solve's update of the later columns of A21
 // with a block of 32 columns: A21(:, c0 + j) -= y L11(c0 + j, block)^T, all rows
 // by all j, one K block.
-// Bound: tensor pipe for e from about 100 on (n = 20000, p = e = 256: 2.26 ms, 1.6
+// Bound: tensor pipe for e from about 100 on (n = 20000, p = e = 256: 2.31 ms, 1.6
 // PFLOP/s of executed products, against 80.6 ms for FP64 multiply-adds at 0.99 of
 // their pipe's rate); below, S traffic and the epilogue's instructions: the
 // update of 224 columns of 200000 rows took 446 us with 144 instructions per entry,
@@ -33,6 +41,8 @@
 // values brought to L2 ahead (HBM's share: 121 us).
 // Every mbarrier wait is bounded; on timeout the kernel records CTP_ETIMEOUT,
 // waits (bounded) for its copies in flight, frees its tensor memory and returns.
+#include <cuda_fp16.h>
+
 #include "slices.cuh"
 #include "tc_common.cuh"
 
@@ -43,16 +53,33 @@ using namespace tc;
 namespace {
 
 constexpr int kBM = kWRows, kBN = kLRows;
-constexpr int kEpiWarps = 16, kThreads = 32 * (2 + kEpiWarps);
+constexpr int kEpiWarps = 16, kThreads = 32 * (4 + kEpiWarps);
 constexpr int kCols = kBN / (kEpiWarps / 4);  // columns of S per epilogue thread
 constexpr int kStages = 2;
 constexpr uint32_t kStageBytes = kWBlock + kLBlock;
-constexpr size_t kSmem = kStages * (size_t)kStageBytes + 1024;
+constexpr size_t kSmem = kStages * (size_t)kStageBytes + kWGroup + kLGroup + 1024;
 constexpr int kPanel = 8;  // column blocks of a panel of the walk
 constexpr int kUpdate = 100;  // kMode of the Solve's update (the others are a ctp_smode)
 
+struct Tile {
+    int64_t t;             // item or slot
+    int ti, tj, e, m, nc;  // m, nc: rows, columns (a Form: nc = m); ti < 0: no tile
+    int c0;                // kUpdate: first column updated, 32 past the block's first
+    int64_t lds, ldl;
+    SliceBuf sb;
+    const double *L21, *D;
+    const int32_t *piv;
+    void *S;
+};
+
+constexpr int kRing = 4;
 struct Bars {
-    unsigned long long full[kStages], empty[kStages], acc_full, acc_empty;
+    unsigned long long full[kStages], empty[kStages], acc_full, acc_empty, grp_full, tile_full[kRing], tile_empty[kRing];
+    Tile tile[kRing];
+    int64_t marked;                 // the last tile of that list, -1: none
+    uint32_t unsure[2][kEpiWarps];  // by turns: blocks that digits may not serve,
+    int linked[2];                  // the tile is in the list of those with entries left out
+    int nmarks;
     uint32_t tmem_base;
     int abort;
 };
@@ -83,15 +110,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
     tmem_wait_ld();
 }
 
-struct Tile {
-    int ti, tj, e, m, nc;  // m, nc: rows, columns (a Form: nc = m)
-    int64_t lds, ldl;
-    SliceBuf sb;
-    const double *L21, *D;
-    const int32_t *piv;
-    void *S;
-};
-
 struct Work {
     // one supernode
     SliceBuf sb;
@@ -108,6 +126,7 @@ struct Work {
     const int *item_front, *item_tile;
     BatchOpts o;
     int64_t count;  // items, or slots of the walk
+    TileMarks *marks;  // one per item or slot
     int c0;         // kUpdate: first column updated, 32 past the block's first
     int64_t nc;     // kUpdate, one supernode: columns updated
 };
@@ -125,97 +144,104 @@ __host__ __device__ inline int64_t walk_slots(int64_t m) {
     return slots_before((nN + kPanel - 1) / kPanel, nM);
 }
 
-// The k-th tile of this CTA; false past the end.  ti < 0: a slot without a tile.
+// Looks this CTA's tiles up, one after another.
 template <bool kUpd>
-__device__ __forceinline__ bool tile_at(const Work &w, int64_t k, Tile &x) {
-    const int64_t t = blockIdx.x + k * (int64_t)gridDim.x;
-    if (t >= w.count) return false;
-    if (kUpd) {
-        // row block by row block, its column blocks one after another
-        int64_t q = t;
-        x.nc = (int)w.nc;
+struct Walk {
+    const Work &w;
+    int64_t t, panel = 0, before = 0, next;  // one supernode's Form: slots before this panel and the next
+    int e = 0;
+    __device__ __forceinline__ explicit Walk(const Work &w_) : w(w_), t(blockIdx.x) {
+        if (w.fronts == nullptr) e = *w.nelim;
+        next = slots_before(1, (w.m + kBM - 1) / kBM);
+    }
+    // the next tile; ti < 0 past the end
+    __device__ __forceinline__ void step(Tile &x) {
+        for (x.ti = -1; t < w.count && x.ti < 0; t += gridDim.x) look(x);
+    }
+    // tile `to` is looked up next (any)
+    __device__ __forceinline__ void seek(int64_t to) {
+        t = to;
+        panel = before = 0;
+        next = slots_before(1, (w.m + kBM - 1) / kBM);
+    }
+    __device__ __forceinline__ void look(Tile &x) {
+        int64_t q = x.t = t;
         x.sb = w.sb;
-        x.m = (int)w.m;
-        x.e = w.fronts != nullptr ? 0 : *w.nelim;
+        x.m = x.nc = (int)w.m;
+        x.e = e;
         x.L21 = w.L21;
         x.ldl = w.ldl;
+        x.D = w.D;
         x.piv = w.piv;
+        x.S = w.S;
+        x.lds = w.lds;
+        x.c0 = w.c0;
+        if (kUpd) x.nc = (int)w.nc;
         if (w.fronts != nullptr) {
             const int f = w.item_front[t];
             const BFront b = w.tab[f];
             const ctp_front &fr = w.fronts[f];
-            q = w.item_tile[t];
+            q = w.item_tile != nullptr ? (int64_t)w.item_tile[t] : t - b.f0;
             ctp_options oo;
             oo.pivot = w.o.pivot;
             oo.smode = w.o.smode;
             oo.prec = w.o.prec;
-            x.sb = bsection_block(w.ws + b.ws, bsection(b.n, b.p, &oo));
+            const BSection sec = bsection(b.n, b.p, &oo);
+            x.sb = kUpd ? bsection_block(w.ws + b.ws, sec) : bsection_slices(w.ws + b.ws, sec, b.p);
             x.m = (int)b.m;
-            x.nc = b.p - w.c0;
+            x.nc = kUpd ? b.p - w.c0 : x.m;
             x.e = *fr.nelim;
             x.L21 = fr.A + b.p;
             x.ldl = fr.lda;
+            x.D = fr.D;
             x.piv = fr.piv;
+            x.S = fr.S;
+            x.lds = fr.lds;
         }
-        x.e = min(x.e - (w.c0 - kSliceK), kSliceK);
-        x.S = const_cast<double *>(x.L21 + (int64_t)w.c0 * x.ldl);
-        x.lds = x.ldl;
-        const int nN = (x.nc + kBN - 1) / kBN;
-        x.ti = x.e > 0 ? (int)(q / nN) : -1;  // nothing eliminated in the block: nothing to do
-        x.tj = (int)(q % nN);
-        return true;
+        if (kUpd) {
+            // row block by row block, its column blocks one after another
+            x.e = min(x.e - (w.c0 - kSliceK), kSliceK);
+            x.S = const_cast<double *>(x.L21 + (int64_t)w.c0 * x.ldl);
+            x.lds = x.ldl;
+            const int nN = (x.nc + kBN - 1) / kBN;
+            x.ti = x.e > 0 ? (int)(q / nN) : -1;  // nothing eliminated in the block: nothing to do
+            x.tj = (int)(q % nN);
+        } else if (w.fronts != nullptr) {
+            // row block i has 2 (i + 1) tiles, i (i + 1) precede it
+            int64_t i = (int64_t)((sqrtf(4.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
+            while ((i + 1) * (i + 2) <= q) i++;
+            while (i * (i + 1) > q) i--;
+            x.ti = (int)i;
+            x.tj = (int)(q - i * (i + 1));
+        } else {
+            const int64_t nM = (w.m + kBM - 1) / kBM;
+            while (q >= next) {
+                panel++;
+                before = next;
+                next = slots_before(panel + 1, nM);
+            }
+            const int64_t r = q - before, ti = panel * (kPanel / 2) + r / kPanel, tj = panel * kPanel + r % kPanel;
+            x.tj = (int)tj;
+            x.ti = (tj * kBN < w.m && tj <= 2 * ti + 1) ? (int)ti : -1;
+        }
     }
-    if (w.fronts != nullptr) {
-        const int f = w.item_front[t];
-        const BFront b = w.tab[f];
-        const int64_t q = w.item_tile != nullptr ? (int64_t)w.item_tile[t] : t - b.f0;
-        // row block i has 2 (i + 1) tiles, i (i + 1) precede it
-        int64_t i = (int64_t)((sqrtf(4.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
-        while ((i + 1) * (i + 2) <= q) i++;
-        while (i * (i + 1) > q) i--;
-        x.ti = (int)i;
-        x.tj = (int)(q - i * (i + 1));
-        ctp_options oo;
-        oo.pivot = w.o.pivot;
-        oo.smode = w.o.smode;
-        oo.prec = w.o.prec;
-        const BSection sec = bsection(b.n, b.p, &oo);
-        x.sb = bsection_slices(w.ws + b.ws, sec, b.p);
-        const ctp_front &fr = w.fronts[f];
-        x.m = x.nc = (int)b.m;
-        x.e = *fr.nelim;
-        x.L21 = fr.A + b.p;
-        x.ldl = fr.lda;
-        x.D = fr.D;
-        x.piv = fr.piv;
-        x.S = fr.S;
-        x.lds = fr.lds;
-        return true;
+};
+
+// A role's way through the ring of tiles.
+struct Ring {
+    int slot = 0;
+    uint32_t phase = 0;
+    // the next tile is there; false on timeout
+    __device__ __forceinline__ bool wait(Bars &b) { return mbar_wait(&b.tile_full[slot], phase, &b.abort); }
+    // done with it (one lane of each role's warp)
+    __device__ __forceinline__ void release(Bars &b) { mbar_arrive(&b.tile_empty[slot]); }
+    __device__ __forceinline__ void step() {
+        if (++slot == kRing) {
+            slot = 0;
+            phase ^= 1u;
+        }
     }
-    x.sb = w.sb;
-    x.m = x.nc = (int)w.m;
-    x.e = *w.nelim;
-    x.L21 = w.L21;
-    x.ldl = w.ldl;
-    x.D = w.D;
-    x.piv = w.piv;
-    x.S = w.S;
-    x.lds = w.lds;
-    const int64_t nM = (w.m + kBM - 1) / kBM, nN = (w.m + kBN - 1) / kBN;
-    int64_t lo = 0, hi = (nN + kPanel - 1) / kPanel;
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (slots_before(mid, nM) <= t)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    const int64_t r = t - slots_before(lo, nM);
-    const int64_t ti = lo * (kPanel / 2) + r / kPanel, tj = lo * kPanel + r % kPanel;
-    x.tj = (int)tj;
-    x.ti = (tj < nN && tj <= 2 * ti + 1) ? (int)ti : -1;
-    return true;
-}
+};
 
 // V 2^ex rounded to nearest even in integer instructions, for results in the normal
 // range of FP64 (the FP64 pipe takes 17 cycles per warp instruction and SM)
@@ -234,35 +260,82 @@ __device__ __noinline__ double to_fp64_any(long long V, int ex) {
     return ex > -900 && ex < 900 ? to_fp64(V, ex) : (V == 0 ? 0.0 : scalbn((double)V, ex));
 }
 
-// Entries (i, j..j+7) of the k-th tile's result by FP64 multiply-adds (i < m; columns
-// past the result count as 0): the marked rows' path.  It looks its tile up again,
-// so that the epilogue keeps no registers for it.
-template <bool kUpd>
-__device__ __noinline__ void plain_entries(const Work &wk, int64_t kt, int64_t i, int64_t j, double (&acc)[8]) {
-    Tile x;
-    tile_at<kUpd>(wk, kt, x);
+// Which 4 x 4 blocks of a tile have pivots in which all their rows are large
+// (slices.cuh): the dot products of four groups of rows (4 (lane / 4)..) by four of
+// columns (4 (lane % 4)..) per lane, from the groups' bounds, a K block of them at a time
+// (`fetch(kb)` brings it to shared memory).  Bit 4 a + b: group a of the lane's rows by
+// group b of its columns has not, and neither are they without a pivot in common
+// (their results are then zero).  Rounded in FP16: a part in 2^11 per term of up to 128
+// per sum.  From the last pivot on, where growth puts the large entries, and no
+// further than needed: random data stop after the first block, which matters to the
+// traffic from L2 (all blocks: 3% at e = 256).
+constexpr float kSure = 0x1p-7f;
+template <typename F>
+__device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, F &&fetch) {
+    const int lane = threadIdx.x & 31;
+    const uint4 *pa = reinterpret_cast<const uint4 *>(grp) + 4 * (lane >> 2);
+    const uint4 *pb = reinterpret_cast<const uint4 *>(grp + kWGroup) + 4 * (lane & 3);
+    auto h2 = [](unsigned v) { return *reinterpret_cast<const __half2 *>(&v); };
+    __half2 s[16];
 #pragma unroll
-    for (int c = 0; c < 8; c++) acc[c] = 0.0;
-    const int first = kUpd ? wk.c0 - kSliceK : 0;
-    for (int k = first; k < first + x.e; k++) {
-        const int kd = x.piv[k];
-        if (kd == CTP_PIVKIND_ZERO) continue;
-        const double *col = x.L21 + (int64_t)k * x.ldl;
-        double w = col[i];  // kUpd: y itself, in the block's columns of A21
-        const double *l = col;
-        if (kUpd) {
-            l = col - (x.nc + wk.c0) + wk.c0;  // rows c0.. of L11's column
-        } else {
-            w *= x.D[2 * k];
-            if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(col[i + x.ldl], x.D[2 * k + 1], w);
-            if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(col[i - x.ldl], x.D[2 * k - 1], w);
+    for (int j = 0; j < 16; j++) s[j] = __floats2half2_rn(0.0f, 0.0f);
+    unsigned bad = 0xFFFFu;
+    const int KB = (e + kSliceK - 1) / kSliceK;
+#pragma unroll 1
+    for (int kb = KB - 1; kb >= 0 && __any_sync(0xffffffffu, bad); kb--) {
+        fetch(kb);
+        const int chunks = min(4, (e - kb * kSliceK + 7) / 8);
+#pragma unroll 1
+        for (int c = 0; c < chunks; c++) {
+            uint4 v[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) v[j] = pb[c * (kBN / kGroup) + j];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint4 u = pa[c * (kBM / kGroup) + i];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    __half2 &t = s[4 * i + j];
+                    t = __hfma2(h2(u.x), h2(v[j].x), t);
+                    t = __hfma2(h2(u.y), h2(v[j].y), t);
+                    t = __hfma2(h2(u.z), h2(v[j].z), t);
+                    t = __hfma2(h2(u.w), h2(v[j].w), t);
+                }
+            }
         }
+        bad = 0u;
 #pragma unroll
-        for (int c = 0; c < 8; c++) {
-            const bool d21 = kUpd && wk.c0 + j + c == k + 1 && kd == CTP_PIVKIND_2X2_FIRST;  // that slot holds D
-            if (j + c <= (kUpd ? x.nc - 1 : i) && !d21) acc[c] = fma(w, l[j + c], acc[c]);
+        for (int j = 0; j < 16; j++) {
+            const float2 t = __half22float2(s[j]);
+            if (!(t.x + t.y >= kSure)) bad |= 1u << j;
         }
     }
+    if (!__any_sync(0xffffffffu, bad)) return 0u;
+    unsigned none[16];  // signs: no pivot in common
+#pragma unroll
+    for (int j = 0; j < 16; j++) none[j] = 0x80008000u;
+#pragma unroll 1
+    for (int kb = 0; kb < KB; kb++) {
+        if (KB > 1) fetch(kb);
+        const int chunks = min(4, (e - kb * kSliceK + 7) / 8);
+#pragma unroll 1
+        for (int c = 0; c < chunks; c++) {
+            uint4 v[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) v[j] = pb[c * (kBN / kGroup) + j];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint4 u = pa[c * (kBM / kGroup) + i];
+#pragma unroll
+                for (int j = 0; j < 4; j++)
+                    none[4 * i + j] &= (u.x | v[j].x) & (u.y | v[j].y) & (u.z | v[j].z) & (u.w | v[j].w);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 16; j++)
+        if (none[j] == 0x80008000u) bad &= ~(1u << j);
+    return bad;
 }
 
 // The eight accumulators of 8 columns (group g at column g kBN) added up: V = sum_g
@@ -322,11 +395,117 @@ __device__ __forceinline__ void add_groups(uint32_t ta, int f, long long *V) {
 
 // kMode: ctp_smode of S, or kUpdate
 template <int kMode>
-__global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_t *__restrict__ info) {
-    using OutT = typename std::conditional<kMode == CTP_S_FP32 || kMode == CTP_S_FP32_PACKED, float, double>::type;
-    constexpr bool kPacked = kMode == CTP_S_FP64_PACKED || kMode == CTP_S_FP32_PACKED;
-    constexpr bool kUpd = kMode == kUpdate;
-    constexpr bool kSub = kMode == CTP_S_FP64_SUB || kUpd;
+struct FormOut {
+    using T = typename std::conditional<kMode == CTP_S_FP32 || kMode == CTP_S_FP32_PACKED, float, double>::type;
+    static constexpr bool kPacked = kMode == CTP_S_FP64_PACKED || kMode == CTP_S_FP32_PACKED;
+    static constexpr bool kSub = kMode == CTP_S_FP64_SUB || kMode == kUpdate;
+};
+// 2^(40 + weight) is the weight of g = 0: as large as the 64 bits allow for e pivots
+__device__ __forceinline__ int weight(int e) { return e <= 16 ? 6 : (e <= 32 ? 5 : (e <= 64 ? 4 : (e <= 128 ? 3 : 2))); }
+
+// The entries that digits do not serve, after the CTA's last tile: by FP64 multiply-adds,
+// tile by tile (all threads, four columns of a row each, or up to four times that
+// where a tile has many; 32 pivots of W21 and L21 at a time in shared memory).  Sparse
+// rows leave a few entries of a tile out; a tile with all of them left out takes what
+// FP64's pipe takes for it.
+constexpr int kFixW = kBM + 1, kFixL = kBN + 1;  // padded rows of the slabs
+template <int kMode>
+__device__ __noinline__ void fix_tiles(const Work &wk, Bars &bars, uint8_t *smem) {
+    typedef typename FormOut<kMode>::T OutT;
+    constexpr bool kPacked = FormOut<kMode>::kPacked, kUpd = kMode == kUpdate, kSub = FormOut<kMode>::kSub;
+    constexpr int kItems = (kBM * kBN / 4 + kThreads - 1) / kThreads;
+    double *ws = reinterpret_cast<double *>(smem), *ls = ws + kSliceK * kFixW;
+    uint16_t *ids = reinterpret_cast<uint16_t *>(ls + kSliceK * kFixL);
+    const Tile &x = bars.tile[0];
+    for (int64_t t = bars.marked; t >= 0; t = wk.marks[t].prev) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            Walk<kUpd> walk(wk);
+            Tile y;
+            walk.seek(t);
+            walk.look(y);
+            bars.tile[0] = y;
+            bars.nmarks = 0;
+        }
+        __syncthreads();
+        const int lane = threadIdx.x & 31;
+        if (threadIdx.x < kBM * kBN / kCols) {  // a row's sixteen columns: which fours have any
+            const unsigned mask = wk.marks[t].out[threadIdx.x >> 5][lane];
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const unsigned has = __ballot_sync(0xffffffffu, (mask >> (4 * c)) & 0xFu);
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&bars.nmarks, __popc(has));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(has & ((1u << lane) - 1u));
+                if ((has >> lane) & 1u) ids[at] = (uint16_t)(threadIdx.x * 4 + c);
+            }
+        }
+        __syncthreads();
+        const int n = bars.nmarks;
+        double acc[kItems][4] = {};
+        int row[kItems], col[kItems];
+#pragma unroll
+        for (int it = 0; it < kItems; it++) {
+            const int q = threadIdx.x + it * kThreads, id = q < n ? ids[q] : 0;  // warp's block, lane, four
+            row[it] = (id >> 9) * 32 + ((id >> 2) & 31);
+            col[it] = ((id >> 7) & 3) * kCols + (id & 3) * 4;
+        }
+        const int i0 = x.ti * kBM, j0 = x.tj * kBN, first = kUpd ? x.c0 - kSliceK : 0;
+        const double *rows = kUpd ? x.L21 - x.nc : x.L21;  // kUpd: rows c0.. of L11
+        for (int k0 = 0; k0 < x.e; k0 += kSliceK) {
+            const int cnt = min(kSliceK, x.e - k0);
+            for (int idx = threadIdx.x; idx < cnt * kBM; idx += kThreads) {
+                const int k = first + k0 + idx / kBM, r = idx % kBM, kd = x.piv[k];
+                double w = 0.0;
+                if (i0 + r < x.m && kd != CTP_PIVKIND_ZERO) {
+                    const double *c = x.L21 + (int64_t)k * x.ldl + i0 + r;
+                    w = *c;  // kUpd: y itself, in the block's columns of A21
+                    if (!kUpd) {
+                        w *= x.D[2 * k];
+                        if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(c[x.ldl], x.D[2 * k + 1], w);
+                        if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(c[-x.ldl], x.D[2 * k - 1], w);
+                    }
+                }
+                ws[idx / kBM * kFixW + r] = w;
+            }
+            for (int idx = threadIdx.x; idx < cnt * kBN; idx += kThreads) {
+                const int k = first + k0 + idx / kBN, c = idx % kBN, kd = x.piv[k];
+                const bool d21 = kUpd && x.c0 + j0 + c == k + 1 && kd == CTP_PIVKIND_2X2_FIRST;  // that slot holds D
+                ls[idx / kBN * kFixL + c] =
+                    kd != CTP_PIVKIND_ZERO && j0 + c < x.nc && !d21 ? rows[(int64_t)k * x.ldl + j0 + c] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int it = 0; it < kItems; it++) {
+                if (threadIdx.x + it * kThreads >= n) break;
+                for (int k = 0; k < cnt; k++) {
+                    const double w = ws[k * kFixW + row[it]];
+#pragma unroll
+                    for (int c = 0; c < 4; c++) acc[it][c] = fma(w, ls[k * kFixL + col[it] + c], acc[it][c]);
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int it = 0; it < kItems; it++) {
+            if (threadIdx.x + it * kThreads >= n) break;
+            const int i = i0 + row[it];
+            const unsigned mask = wk.marks[t].out[row[it] / 32 * 4 + col[it] / kCols][row[it] % 32] >> (col[it] % kCols);
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                const int64_t j = j0 + col[it] + c;
+                if (!((mask >> c) & 1u)) continue;
+                OutT *ptr = reinterpret_cast<OutT *>(x.S) + (kPacked ? j * x.m - j * (j + 1) / 2 : j * x.lds) + i;
+                *ptr = kSub ? (OutT)(*ptr - acc[it][c]) : (OutT)acc[it][c];
+            }
+        }
+    }
+}
+
+template <int kMode>
+__global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant__ Work wk, int32_t *__restrict__ info) {
+    typedef typename FormOut<kMode>::T OutT;
+    constexpr bool kPacked = FormOut<kMode>::kPacked, kUpd = kMode == kUpdate, kSub = FormOut<kMode>::kSub;
     extern __shared__ unsigned char smraw[];
     __shared__ Bars bars;
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
@@ -336,9 +515,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
             mbar_init(&bars.full[s], 1);
             mbar_init(&bars.empty[s], 1);
         }
-        mbar_init(&bars.acc_full, 1);
+        mbar_init(&bars.acc_full, 2);  // the MMAs and the checker
         mbar_init(&bars.acc_empty, kEpiWarps);
+        mbar_init(&bars.grp_full, 1);
+        for (int s = 0; s < kRing; s++) {
+            mbar_init(&bars.tile_full[s], 1);
+            mbar_init(&bars.tile_empty[s], 3 + kEpiWarps);
+        }
         bars.abort = 0;
+        bars.marked = -1;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(&bars.tmem_base, 512);
@@ -346,16 +531,110 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = bars.tmem_base;
+    uint8_t *grp = smem + kStages * (size_t)kStageBytes;
 
-    if (warp == 0) {
-        // ---------------- producer
+    Ring ring;
+    if (warp == 2 + kEpiWarps) {
+        // ---------------- scheduler
+        if (lane == 0) {
+            Walk<kUpd> walk(wk);
+            Tile x;
+            bool ok = true;
+            do {
+                walk.step(x);
+                ok = mbar_wait(&bars.tile_empty[ring.slot], ring.phase ^ 1u, &bars.abort);
+                if (!ok) break;
+                bars.tile[ring.slot] = x;
+                mbar_arrive(&bars.tile_full[ring.slot]);
+                ring.step();
+            } while (x.ti >= 0);
+            if (!ok) atomicExch(&bars.abort, 1);
+        }
+    } else if (warp == 3 + kEpiWarps) {
+        // ---------------- checker
+        uint32_t accphase = 0, grpphase = 0;
+        bool ok, first = true;
+        int64_t marked = -1;
+        while ((ok = ring.wait(bars))) {
+            const Tile &x = bars.tile[ring.slot];
+            if (x.ti < 0) break;
+            unsigned bits = 0u;
+            bool linked = false;
+            if (x.e > 0) {
+                // rows that hold an Inf or NaN
+                const int r0 = x.ti * kBM + 4 * lane, c0 = x.tj * kBN + 2 * lane;
+                int4 er = make_int4(0, 0, 0, 0);
+                int2 ec = make_int2(0, 0);
+                if (r0 < x.m) er = *reinterpret_cast<const int4 *>(x.sb.ew + r0);
+                if (c0 < x.nc) ec = *reinterpret_cast<const int2 *>(x.sb.el + c0);
+                auto fetch = [&](int kb) {
+                    __syncwarp();
+                    if (lane == 0) {
+                        const uint32_t chunks = min(4u, (uint32_t)(x.e - kb * kSliceK + 7) / 8);
+                        const uint32_t bw = chunks * (kWGroup / 4), bl = chunks * (kLGroup / 4);
+                        mbar_expect_tx(&bars.grp_full, bw + bl);
+                        bulk_load(grp, x.sb.gw + ((size_t)x.ti * x.sb.kb + kb) * (kWGroup / 2), bw, &bars.grp_full);
+                        bulk_load(grp + kWGroup, x.sb.gl + ((size_t)x.tj * x.sb.kb + kb) * (kLGroup / 2), bl,
+                                  &bars.grp_full);
+                    }
+                    int never = 0;  // no CTA leaves with copies in flight
+                    ok = mbar_wait(&bars.grp_full, grpphase, &never) && ok;
+                    grpphase ^= 1u;
+                };
+                bits = unsure_blocks(grp, x.e, fetch);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
+                const bool nonfinite =
+                    __any_sync(0xffffffffu, er.x >= kExpNonfinite || (r0 + 1 < x.m && er.y >= kExpNonfinite) ||
+                                                (r0 + 2 < x.m && er.z >= kExpNonfinite) ||
+                                                (r0 + 3 < x.m && er.w >= kExpNonfinite) || ec.x >= kExpNonfinite ||
+                                                (c0 + 1 < x.nc && ec.y >= kExpNonfinite));
+#pragma unroll
+                for (int j = 0; j < 4; j++) {  // rows and columns past the result
+                    if (x.ti * kBM + 16 * (lane >> 2) + 4 * j >= x.m) bits &= ~(0xFu << (4 * j));
+                    if (x.tj * kBN + 16 * (lane & 3) + 4 * j >= x.nc) bits &= ~(0x1111u << j);
+                }
+                // a warp of the epilogue: rows of two of these lanes, bit 4 (row group) + column group
+                bits <<= 16 * ((lane >> 2) & 1);
+                bits |= __shfl_xor_sync(0xffffffffu, bits, 4);
+                linked = __any_sync(0xffffffffu, bits) || nonfinite;
+                if (linked) {
+                    if (lane == 0) wk.marks[x.t].prev = marked;
+                    marked = x.t;
+                }
+            }
+            __syncwarp();
+            if (lane == 0) ring.release(bars);
+            ring.step();
+            // the bits of the tile before last have been read once the last one's accumulators are full
+            if (!first) {
+                ok = mbar_wait(&bars.acc_full, accphase, &bars.abort);
+                if (!ok) break;
+                accphase ^= 1u;
+            }
+            first = false;
+            if (!((lane >> 2) & 1)) bars.unsure[accphase][(lane >> 3) * 4 + (lane & 3)] = bits;
+            if (lane == 0) bars.linked[accphase] = linked;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.acc_full);
+        }
+        if (lane == 0) {
+            bars.marked = marked;
+            if (!ok) atomicExch(&bars.abort, 1);
+        }
+    } else if (warp == 0) {
+        // ---------------- producer of the slices
         if (lane == 0) {
             int stage = 0, issued = 0;
             uint32_t phase = 0;
-            Tile x;
             bool ok = true;
-            for (int64_t k = 0; ok && tile_at<kUpd>(wk, k, x); k++) {
-                if (x.ti < 0) continue;
+            while (ok && (ok = ring.wait(bars))) {
+                const Tile x = bars.tile[ring.slot];
+                ring.release(bars);
+                ring.step();
+                if (x.ti < 0) break;
                 // rows of the tile in use, in groups of 8
                 const uint32_t rw = (uint32_t)(min(kBM, x.m - x.ti * kBM) + 7) & ~7u;
                 const uint32_t rl = (uint32_t)(min(kBN, x.nc - x.tj * kBN) + 7) & ~7u;
@@ -403,10 +682,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0, accphase = 0;
-            Tile x;
             bool ok = true;
-            for (int64_t k = 0; ok && tile_at<kUpd>(wk, k, x); k++) {
-                if (x.ti < 0) continue;
+            while (ok && (ok = ring.wait(bars))) {
+                const Tile &slot = bars.tile[ring.slot];
+                const struct { int ti, e; } x = {slot.ti, slot.e};
+                ring.release(bars);
+                ring.step();
+                if (x.ti < 0) break;
                 if (!mbar_wait(&bars.acc_empty, accphase ^ 1u, &bars.abort)) {
                     ok = false;
                     break;
@@ -451,40 +733,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
         const int q = warp & 3;                        // TMEM lane quarter this warp may access
         const int cg = (warp - 2) >> 2;                // its 16 columns of the tile
         uint32_t accphase = 0;
-        Tile x;
-        for (int64_t k = 0; tile_at<kUpd>(wk, k, x); k++) {
-            if (x.ti < 0) continue;
-            const int i = x.ti * kBM + q * 32 + lane, j0 = x.tj * kBN + cg * kCols, m = x.m;
+        for (;; ring.step()) {
+            if (!ring.wait(bars)) {
+                if (lane == 0) atomicExch(&bars.abort, 1);
+                break;
+            }
+            const Tile &x = bars.tile[ring.slot];
+            if (x.ti < 0) break;
+            const int i = x.ti * kBM + q * 32 + lane, j0 = x.tj * kBN + cg * kCols, m = x.m, e = x.e;
+            const int64_t lds = x.lds;
             // entries (i, j) with i < m and j <= jmax belong to the result
             const int jmax = kUpd ? x.nc - 1 : i;
             const bool any = j0 <= (kUpd ? jmax : i - lane + 31) && j0 < x.nc && i - lane < m;  // warp-uniform
             const bool interior = j0 + kCols - 1 <= (kUpd ? jmax : i - lane) && i - lane + 31 < m;
             OutT *ptr = reinterpret_cast<OutT *>(x.S) +
-                        (kPacked ? (int64_t)j0 * m - (int64_t)j0 * (j0 + 1) / 2 : j0 * x.lds) + i;
+                        (kPacked ? (int64_t)j0 * m - (int64_t)j0 * (j0 + 1) / 2 : j0 * lds) + i;
             int ei = kExpZero, ej = kExpZero;
-            if (x.e > 0 && i < m) ei = x.sb.ew[i];
-            if (x.e > 0 && lane < kCols && j0 + lane < x.nc) ej = x.sb.el[j0 + lane];
+            if (e > 0 && i < m) ei = x.sb.ew[i];
+            if (e > 0 && lane < kCols && j0 + lane < x.nc) ej = x.sb.el[j0 + lane];
             // subtracting: the old values come to L2 while the products are computed
             if (kSub && any && i < m) {
 #pragma unroll
                 for (int c = 0; c < kCols; c++)
                     if (interior || j0 + c <= jmax)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr + (int64_t)c * x.lds));
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr + (int64_t)c * lds));
             }
             if (!mbar_wait(&bars.acc_full, accphase, &bars.abort)) {
                 if (lane == 0) atomicExch(&bars.abort, 1);
                 break;
             }
+            const unsigned unsure = *(volatile uint32_t *)&bars.unsure[accphase][q * 4 + cg];
+            const bool linked = *(volatile int *)&bars.linked[accphase] != 0;
             accphase ^= 1u;
             tc_fence_after();
-            // 2^(40 + f) is the weight of g = 0: as large as the 64 bits allow for e pivots
-            const int f = x.e <= 16 ? 6 : (x.e <= 32 ? 5 : (x.e <= 64 ? 4 : (x.e <= 128 ? 3 : 2)));
+            const int f = weight(e);
             long long V[kCols];
-            if (any && x.e > 0) {
+            if (any && e > 0) {
                 const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * kCols);
 #pragma unroll
                 for (int h = 0; h < kCols; h += 8)
-                    if (kUpd || x.e <= 32)
+                    if (kUpd || e <= 32)
                         add_groups<true>(ta + h, f, V + h);
                     else
                         add_groups<false>(ta + h, f, V + h);
@@ -492,15 +780,25 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.acc_empty);
-            if (!any) continue;
-            // marked rows and columns of this warp's block
-            const bool wide_i = ei >= kExpWide / 2, wide_j = ej >= kExpWide / 2;
-            const unsigned wides = __ballot_sync(0xffffffffu, wide_j);
-            const bool any_wide = wides != 0u || __any_sync(0xffffffffu, wide_i);
-            // the plain case -- every entry of the warp's block belongs to the result, no
-            // row is marked, exponents are moderate -- has no test in its loop
-            const bool mild = abs(ei) < 400 && (lane >= kCols || abs(ej) < 400);
-            if (interior && !any_wide && __all_sync(0xffffffffu, mild)) {
+            // this row's entries left out: of a block that digits may not serve, they do serve
+            // those of which they make 2^-7 of the scales (a lower bound of P)
+            unsigned weak = 0u;
+            const bool nonfinite = ei >= kExpNonfinite || ej >= kExpNonfinite;
+            if (linked && any && (unsure || __any_sync(0xffffffffu, nonfinite))) {
+#pragma unroll
+                for (int c = 0; c < kCols; c++) {
+                    const int ejc = __shfl_sync(0xffffffffu, ej, c);
+                    const unsigned long long a = V[c] < 0 ? 0ull - (unsigned long long)V[c] : (unsigned long long)V[c];
+                    const bool low = ((unsure >> ((lane & ~3) | (c >> 2))) & 1u) && a >> (45 + f) == 0ull &&
+                                     ei != kExpZero && ejc != kExpZero;
+                    if (i < m && j0 + c <= jmax && (low || ei >= kExpNonfinite || ejc >= kExpNonfinite)) weak |= 1u << c;
+                }
+            }
+            // the plain case -- every entry of the warp's block belongs to the result, its
+            // digits serve all of them, exponents are moderate -- has no test in its loop
+            const bool mild = weak == 0u && abs(ei) < 400 && (lane >= kCols || abs(ej) < 400);
+            if (!any) {
+            } else if (interior && __all_sync(0xffffffffu, mild)) {
 #pragma unroll
                 for (int h = 0; h < kCols; h += 8) {
                     double old[8];  // eight old values loaded before any is stored
@@ -509,7 +807,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
 #pragma unroll
                         for (int c = 0; c < 8; c++) {
                             old[c] = *pl;
-                            pl += x.lds;
+                            pl += lds;
                         }
                     }
 #pragma unroll
@@ -519,37 +817,40 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const Work wk, int32_
                             *ptr = (OutT)(old[c] - v);
                         else
                             __stcs(ptr, (OutT)v);
-                        ptr += kPacked ? m - 1 - (j0 + h + c) : x.lds;
+                        ptr += kPacked ? m - 1 - (j0 + h + c) : lds;
                     }
                 }
-                continue;
-            }
+            } else {
 #pragma unroll
-            for (int h = 0; h < kCols; h += 8) {
-                double pl[8], old[8];
-                if (any_wide && i < m) plain_entries<kUpd>(wk, k, i, j0 + h, pl);
-                if (kSub) {
+                for (int h = 0; h < kCols; h += 8) {
+                    double old[8];
+                    if (kSub) {
 #pragma unroll
-                    for (int c = 0; c < 8; c++) old[c] = i < m && j0 + h + c <= jmax ? ptr[(int64_t)c * x.lds] : 0.0;
-                }
-#pragma unroll
-                for (int c = 0; c < 8; c++) {
-                    const int ex = ei + __shfl_sync(0xffffffffu, ej, h + c) - 52 - f;
-                    if (i < m && j0 + h + c <= jmax) {
-                        double v = x.e > 0 ? to_fp64_any(V[h + c], ex) : 0.0;
-                        if (any_wide && (wide_i || ((wides >> (h + c)) & 1u))) v = pl[c];
-                        if (kSub)
-                            *ptr = (OutT)(old[c] - v);
-                        else
-                            __stcs(ptr, (OutT)v);
+                        for (int c = 0; c < 8; c++) old[c] = i < m && j0 + h + c <= jmax ? ptr[(int64_t)c * lds] : 0.0;
                     }
-                    ptr += kPacked ? m - 1 - (j0 + h + c) : x.lds;
+#pragma unroll
+                    for (int c = 0; c < 8; c++) {
+                        const int ex = ei + __shfl_sync(0xffffffffu, ej, h + c) - 52 - f;
+                        if (i < m && j0 + h + c <= jmax && !((weak >> (h + c)) & 1u)) {
+                            const double v = e > 0 ? to_fp64_any(V[h + c], ex) : 0.0;
+                            if (kSub)
+                                *ptr = (OutT)(old[c] - v);
+                            else
+                                __stcs(ptr, (OutT)v);
+                        }
+                        ptr += kPacked ? m - 1 - (j0 + h + c) : lds;
+                    }
                 }
             }
+            if (linked) wk.marks[x.t].out[q * 4 + cg][lane] = (uint16_t)weak;
+            __syncwarp();
+            if (lane == 0) ring.release(bars);
         }
     }
     __syncthreads();
     if (threadIdx.x == 0 && bars.abort) atomicCAS(info, kInfoOk, (int32_t)CTP_ETIMEOUT);
+    if (bars.marked >= 0 && !bars.abort) fix_tiles<kMode>(wk, bars, smem);
+    __syncwarp();
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
@@ -565,14 +866,14 @@ __global__ void __launch_bounds__(32 * kSW)
                     SliceBuf sb) {
     extern __shared__ __align__(16) double xs[];  // [p][33]
     __shared__ short cexp[kMaxP];
-    __shared__ int red[2 * kSW * 32], rexp[32];
+    __shared__ int red[kSW * 32], rexp[32];
     const int e = *nelim, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = (int64_t)blockIdx.x * 32;
     const int nrows = (int)min((int64_t)32, m - row0);
     for (int k = threadIdx.x; k < e; k += 32 * kSW) cexp[k] = (short)slice_col_exp(piv, Dinv, k);
     for (int k = w; k < e; k += kSW) xs[k * 33 + lane] = lane < nrows ? A[(int64_t)k * lda + p + row0 + lane] : 0.0;
     __syncthreads();
-    write_slices<kLRows, kSW>(xs, e, row0, nrows, cexp, 1, sb.L, sb.el, sb.kb, red, rexp);
+    write_slices<kLRows, kSW>(xs, e, row0, nrows, cexp, 1, sb.L, sb.el, sb.gl, sb.kb, red, rexp);
     __syncthreads();
     for (int k = w; k < e; k += kSW) {
         const int kd = piv[k];
@@ -585,7 +886,7 @@ __global__ void __launch_bounds__(32 * kSW)
         }
     }
     __syncthreads();
-    write_slices<kWRows, kSW>(xs, e, row0, nrows, cexp, -1, sb.W, sb.ew, sb.kb, red, rexp);
+    write_slices<kWRows, kSW>(xs, e, row0, nrows, cexp, -1, sb.W, sb.ew, sb.gw, sb.kb, red, rexp);
 }
 
 template <int kMode>
@@ -612,7 +913,7 @@ cudaError_t launch_any(const Work &wk, int smode, int32_t *info, int num_sms, cu
 
 cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda, const int32_t *piv,
                              const double *D, int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
-                             int32_t *info, int num_sms, cudaStream_t st) {
+                             TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
     Work wk = {};
     wk.sb = sb;
@@ -625,12 +926,13 @@ cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda,
     wk.nelim = nelim;
     wk.S = S;
     wk.count = walk_slots(m);
+    wk.marks = marks;
     return launch_any(wk, smode, info, num_sms, st);
 }
 
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                                   const int *item_front, int64_t items, BatchOpts o, int32_t *info, int num_sms,
-                                   cudaStream_t st, const int *item_tile) {
+                                   const int *item_front, int64_t items, BatchOpts o, TileMarks *marks, int32_t *info,
+                                   int num_sms, cudaStream_t st, const int *item_tile) {
     if (items == 0) return cudaSuccess;
     Work wk = {};
     wk.fronts = fronts;
@@ -640,13 +942,15 @@ cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, c
     wk.item_tile = item_tile;
     wk.o = o;
     wk.count = items;
+    wk.marks = marks;
     return launch_any(wk, o.smode, info, num_sms, st);
 }
 
 cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int64_t m, int blk, const int32_t *piv,
-                          const int32_t *nelim, int32_t *info, int num_sms, cudaStream_t st) {
+                          const int32_t *nelim, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st) {
     Work wk = {};
     wk.sb = u;
+    wk.marks = marks;
     wk.L21 = A + p;
     wk.ldl = lda;
     wk.piv = piv;
@@ -659,13 +963,15 @@ cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int6
     return launch_any(wk, kUpdate, info, num_sms, st);
 }
 
+int64_t form_fp64_slots(int64_t m) { return m > 0 ? walk_slots(m) : 0; }
+
 int64_t update_tiles(int64_t m, int p) {
     return p > kSliceK ? (m + kBM - 1) / kBM * ((p - kSliceK + kBN - 1) / kBN) : 0;
 }
 
 cudaError_t launch_update_batch(const ctp_front *fronts, const BFront *tab, char *ws, const int *item_front,
-                                const int *item_tile, int64_t items, BatchOpts o, int32_t *info, int num_sms,
-                                cudaStream_t st) {
+                                const int *item_tile, int64_t items, BatchOpts o, TileMarks *marks, int32_t *info,
+                                int num_sms, cudaStream_t st) {
     if (items == 0) return cudaSuccess;
     Work wk = {};
     wk.fronts = fronts;
@@ -676,6 +982,7 @@ cudaError_t launch_update_batch(const ctp_front *fronts, const BFront *tab, char
     wk.o = o;
     wk.c0 = kSliceK;
     wk.count = items;
+    wk.marks = marks;
     return launch_any(wk, kUpdate, info, num_sms, st);
 }
 

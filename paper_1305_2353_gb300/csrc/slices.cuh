@@ -17,17 +17,26 @@
 // 2^c_k about |d_k|^(1/2) (their products are unchanged): both operands then
 // look like L |D|^(1/2), whose rows do not mix the scales of the pivots.
 //
-// Accuracy: a digit product with s + t > 7 is dropped and X is cut at 2^-62, in
-// all about 2^-62 e^(1/2) of the two rows' scales 2^(E_i + E_j): less than the
-// rounding of e FP64 multiply-adds wherever the large entries of one row meet
-// entries of the other that are not much below its own largest, as they do in
-// random data and under the growth of the pivots' columns, which all rows share.
-// A row is marked, by kExpWide added to its exponent, when none of its entries
-// does -- in no column is its entry, relative to its scale, times the typical
-// entry (the geometric mean of the nonzero ones of the tile's 32 rows, relative
-// to theirs) above 2^-kWideBits -- or when it holds an Inf or NaN, and the Form
-// takes its entries of S by FP64 multiply-adds.  (Entries scattered over 2^40
-// lost up to 8 bits without the mark.)
+// Accuracy: cutting X and dropping the digit products with s + t > 7 costs an
+// entry of S at most e 2^-59, and rounding the two lowest sums to whole units 2^-(53+f)
+// with f = 6, 5, 4, 3, 2 for e <= 16, 32, 64, 128, 256, both times the two rows' scales
+// 2^(E_i + E_j): together less than 1.1 e 2^-59 2^(E_i + E_j).  (Past 128 pivots
+// the sums of g = 5 are exact only below 2^24; their digits would have to lie within
+// a tenth of their extremes in nearly all pivots to pass it.)  FP64
+// multiply-adds may lose e 2^-53 (|W21||L21|^T)_ij.  So digits serve an entry as well when
+//     P_ij = sum_k |w_ik| |l_jk| / 2^(E_i + E_j) >= 2^-7
+// (then they lose less than (2 e + 8) 2^-53 (|W21||L21|^T)_ij at the very most, and
+// in the mean what FP64 multiply-adds lose), that is unless the two rows are
+// large in different pivots.  The Form makes sure of that before it uses them, for 4 x 4
+// entries at a time, from a lower bound of P_ij: the sum over the least entries of
+// four rows each (the groups' bounds, written here).  Where that falls short
+// although the rows have pivots in common, the entry's own result may still bound P_ij
+// from below; where that falls short too, or a row holds an Inf or NaN, the entry is
+// taken by FP64 multiply-adds.  (Two blocks of rows, each large in columns where the
+// other is 2^-40 of its scale, lost 26 bits between them while rows were
+// compared within their tile only.)  Random rows pass the first test from about 8 pivots
+// on; of the entries of 36^3 multifrontal fronts one in 40 does not, and one in 1300
+// passes neither.
 //
 // Layout (what a bulk copy puts into shared memory as the MMA reads it): W in
 // blocks of 128 rows, L in blocks of 64; per row block and block of 32 pivots
@@ -46,7 +55,6 @@ __device__ __forceinline__ int biased_exp(double x) { return (int)((hi_word(x) >
 // the largest entry of D^-1 in the pivot's row.  A zero pivot has no part in S
 // (its column of L21 is zero): kSliceSkip, its entries count as zero.
 constexpr short kSliceSkip = 32767;
-constexpr int kWideBits = 5;
 __device__ __forceinline__ int slice_col_exp(const int32_t *__restrict__ piv, const double *__restrict__ Dinv, int k) {
     const int kd = piv[k];
     if (kd == CTP_PIVKIND_ZERO) return kSliceSkip;
@@ -94,15 +102,23 @@ __device__ __forceinline__ uint32_t slice_pair(unsigned long long y0, unsigned l
     return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
 }
 
+// A lower bound of |x| 2^(sh - E) < 1 as FP16 bits, 0 below 2^-14.
+__device__ __forceinline__ unsigned slice_low(double x, int sh, int E) {
+    const int h = slice_exp(x, sh) - E + 14;  // its exponent field (subnormal x: far below)
+    return h >= 1 ? (unsigned)(h << 10) | ((hi_word(x) >> 10) & 0x3FFu) : 0u;
+}
+
 // The slices of a tile of 32 rows, by a CTA of kWarps warps: columns k < e of the
 // tile in xs ([k][33], rows row0 .. row0 + nrows of the operand), column k times
 // 2^(sgn * cexp[k]); kBlk rows per block of the image.  Zeros from e to the
-// next multiple of 16 (the MMA reads no further).  red: 2 * kWarps * 32 ints,
-// rexp: 32 ints of shared memory.  Three CTA barriers; xs is only read.
+// next multiple of 16 (the MMA reads no further).  grp: per block of rows and chunk of 8
+// columns the groups' FP16 lower bounds of their rows' entries, 16 bytes each; -0
+// where all four rows hold zeros.  red: kWarps * 32 ints, rexp: 32 ints of
+// shared memory.  Two CTA barriers; xs is only read.
 template <int kBlk, int kWarps>
 __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t row0, int nrows, const short *cexp,
                                              int sgn, unsigned char *__restrict__ img, int32_t *__restrict__ rowexp,
-                                             int kb, int *red, int *rexp) {
+                                             uint16_t *__restrict__ grp, int kb, int *red, int *rexp) {
     constexpr int LDX = 33;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int E = kExpZero;
@@ -110,42 +126,54 @@ __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t ro
         if (cexp[k] != kSliceSkip) E = max(E, slice_exp(xs[k * LDX + lane], sgn * cexp[k]));
     red[w * 32 + lane] = E;
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kWarps; q++) E = max(E, red[q * 32 + lane]);
-    int best = kExpZero;  // the row's best column: log2 of its entry times the typical one
-    for (int k = w; k < e; k += kWarps) {
-        if (cexp[k] == kSliceSkip) continue;
-        const int x = slice_exp(xs[k * LDX + lane], sgn * cexp[k]);
-        const bool in = x > kExpZero && x < kExpNonfinite;
-        const int cnt = __popc(__ballot_sync(0xffffffffu, in));
-        const int sum = __reduce_add_sync(0xffffffffu, in ? E - x : 0);
-        if (in) best = max(best, x - E - sum / cnt);
-    }
-    red[(kWarps + w) * 32 + lane] = best;
-    __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int q = 1; q < kWarps; q++) best = max(best, red[(kWarps + q) * 32 + lane]);
+        for (int q = 1; q < kWarps; q++) E = max(E, red[q * 32 + lane]);
         rexp[lane] = E;
-        const bool wide = E >= kExpNonfinite || (E > kExpZero && best < -kWideBits);
-        if (lane < nrows) rowexp[row0 + lane] = wide ? E + kExpWide : E;
+        if (lane < nrows) rowexp[row0 + lane] = E;
     }
     __syncthreads();
     const int e16 = (e + 15) & ~15, nkb = (e + kSliceK - 1) / kSliceK;
     // an item: 8 rows by the four 16-byte chunks of a K block, a lane per (row, chunk)
     for (int it = w; it < 4 * nkb; it += kWarps) {
         const int kblk = it >> 2, r = (it & 3) * 8 + (lane >> 2), c = lane & 3, k0 = kblk * kSliceK + c * 8;
-        if (r >= nrows || k0 >= e16) continue;
+        if ((it & 3) * 8 >= nrows) continue;  // the whole warp
+        const bool on = r < nrows && k0 < e16;
         const int Er = rexp[r];
         unsigned long long y[8];
+        unsigned low[4], some = 0u;  // FP16 pairs; which columns hold an entry
 #pragma unroll
         for (int j = 0; j < 8; j++) {
-            const bool in = k0 + j < e && cexp[k0 + j] != kSliceSkip && Er < kExpNonfinite;
-            y[j] = in ? slice_digits(xs[(k0 + j) * LDX + r], sgn * cexp[k0 + j], Er) : 0x8080808080808080ull;
+            const bool in = k0 + j < e && cexp[k0 + j] != kSliceSkip;
+            unsigned h = 0u;
+            y[j] = 0x8080808080808080ull;
+            if (in && Er < kExpNonfinite) {
+                const double x = xs[(k0 + j) * LDX + r];
+                y[j] = slice_digits(x, sgn * cexp[k0 + j], Er);
+                h = Er > kExpZero ? slice_low(x, sgn * cexp[k0 + j], Er) : 0x3C00u;  // a zero row lowers nothing
+                some |= (x != 0.0 ? 1u : 0u) << j;
+            } else if (in) {
+                h = 0x3C00u;  // nor does one with an Inf or NaN, whose entries are known by its exponent
+            }
+            low[j >> 1] = (j & 1) ? low[j >> 1] | (h << 16) : h;
         }
-        const int64_t row = row0 + r;
+#pragma unroll
+        for (int o = 4; o <= 8; o <<= 1) {
+            some |= __shfl_xor_sync(0xffffffffu, some, o);
+#pragma unroll
+            for (int q = 0; q < 4; q++) low[q] = __vminu2(low[q], __shfl_xor_sync(0xffffffffu, low[q], o));
+        }
+        if (!on) continue;
+        const int64_t row = row0 + r, blk = row / kBlk * kb + kblk;
+        if (r % kGroup == 0) {
+#pragma unroll
+            for (int j = 0; j < 8; j++)
+                if (!((some >> j) & 1u)) low[j >> 1] = (j & 1) ? (low[j >> 1] & 0xFFFFu) | 0x80000000u : (low[j >> 1] & 0xFFFF0000u) | 0x8000u;
+            *reinterpret_cast<uint4 *>(grp + ((blk * 4 + c) * (kBlk / kGroup) + row % kBlk / kGroup) * 8) =
+                make_uint4(low[0], low[1], low[2], low[3]);
+        }
         const int rb = (int)(row % kBlk);
-        unsigned char *dst = img + ((size_t)(row / kBlk) * kb + kblk) * ((size_t)kSlices * kBlk * 64) + rb * 64 +
+        unsigned char *dst = img + (size_t)blk * ((size_t)kSlices * kBlk * 64) + rb * 64 +
                              ((c ^ ((rb >> 1) & 3)) << 4);
 #pragma unroll
         for (int s = 0; s < kSlices; s++) {

@@ -168,13 +168,13 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
 
     const int tile_rows = m - row0 < RT ? (int)(m - row0) : RT;
     __shared__ short cexp[kMaxP];
-    __shared__ int red[2 * kWarps * 32], rexp[32];
+    __shared__ int red[kWarps * 32], rexp[32];
     if (part) {
         if (c0 + kSliceK < p) {  // columns are left to update
             for (int k = c0 + threadIdx.x; k < j1; k += blockDim.x) cexp[k - c0] = (short)slice_col_exp(piv, Dinv, k);
             __syncthreads();
-            write_slices<kWRows, kWarps>(xs, j1 - c0, row0, tile_rows, cexp, -1, ps.yb.W, ps.yb.ew, ps.yb.kb, red,
-                                         rexp);
+            write_slices<kWRows, kWarps>(xs, j1 - c0, row0, tile_rows, cexp, -1, ps.yb.W, ps.yb.ew, ps.yb.gw,
+                                         ps.yb.kb, red, rexp);
         }
         if (valid)
             for (int k = c0 + w; k < c1; k += CW) A21[(int64_t)k * lda + row] = xs[(k - c0) * LDX + r];
@@ -188,7 +188,7 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     if (sb.W != nullptr) {
         for (int k = threadIdx.x; k < e; k += blockDim.x) cexp[k] = (short)slice_col_exp(piv, Dinv, k);
         __syncthreads();
-        write_slices<kWRows, kWarps>(xs, e, row0, tile_rows, cexp, -1, sb.W, sb.ew, sb.kb, red, rexp);
+        write_slices<kWRows, kWarps>(xs, e, row0, tile_rows, cexp, -1, sb.W, sb.ew, sb.gw, sb.kb, red, rexp);
     }
     if (Wb != nullptr) write_pieces(Wb, brow0 + row0, tile_rows, Kp, e, Kz, pieces, lo_off, xs);
     __syncthreads();
@@ -215,12 +215,13 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     if (Lb == nullptr && sb.L == nullptr) return;
     __syncthreads();
     // the Form's copies of L21
-    if (sb.L != nullptr) write_slices<kLRows, kWarps>(xs, e, row0, tile_rows, cexp, 1, sb.L, sb.el, sb.kb, red, rexp);
+    if (sb.L != nullptr)
+        write_slices<kLRows, kWarps>(xs, e, row0, tile_rows, cexp, 1, sb.L, sb.el, sb.gl, sb.kb, red, rexp);
     if (Lb != nullptr) write_pieces(Lb, brow0 + row0, tile_rows, Kp, e, Kz, pieces, lo_off, xs);
 }
 
 template <int RT>
-__global__ void __launch_bounds__(kRows * kWarps)
+__global__ void __launch_bounds__(kRows * kWarps, 6)
     k_solve_fp64(SolvePass ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                  const int32_t *__restrict__ perm, const int32_t *__restrict__ piv,
                  const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p,
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(kRows * kWarps)
 // Batched: CTA b takes work item b = (front, RT-row tile of its A21): the
 // front is item_front[b], the tile item_tile[b].
 template <int RT>
-__global__ void __launch_bounds__(kRows * kWarps)
+__global__ void __launch_bounds__(kRows * kWarps, 6)
     k_solve_batch(int mode, const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
                   const int *__restrict__ item_front, const int *__restrict__ item_tile, BatchOpts o,
                   __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb) {
@@ -247,9 +248,9 @@ __global__ void __launch_bounds__(kRows * kWarps)
     oo.prec = o.prec;
     const BSection sec = bsection(bt.n, bt.p, &oo);
     char *base = ws + bt.ws;
-    SliceBuf sb = {nullptr, nullptr, nullptr, nullptr, 0};
+    SliceBuf sb = {};
     if (o.smode != CTP_S_NONE && o.prec == CTP_FP64) sb = bsection_slices(base, sec, bt.p);
-    SolvePass ps = {mode, mode == kTail ? 1 : 0, {nullptr, nullptr, nullptr, nullptr, 0}};
+    SolvePass ps = {mode, mode == kTail ? 1 : 0, {}};
     if (mode == kFirst) ps.yb = bsection_block(base, sec);
     solve_tile<RT>(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
                *fr.nelim, sb, Wb, Lb, kBatchKp, bt.row0, o.lo_off, o.pieces,
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(kRows * kWarps)
 
 // The columns of A21 into pivot order, in place: a tile of 32 rows by all columns per
 // CTA; columns that stay are left alone.
-__global__ void __launch_bounds__(kRows * kWarps)
+__global__ void __launch_bounds__(kRows * kWarps, 6)
     k_move_columns(double *__restrict__ A21, int64_t m, int p, int64_t lda, const int32_t *__restrict__ perm) {
     extern __shared__ __align__(16) double xs[];  // [p][kRows]
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -322,7 +323,7 @@ __device__ __forceinline__ void l11_tile(const double *__restrict__ A, int64_t l
     constexpr int LDX = kRows + 1;
     __shared__ double xs[kSliceK * LDX];
     __shared__ short cexp[kSliceK];
-    __shared__ int red[2 * kWarps * 32], rexp[32];
+    __shared__ int red[kWarps * 32], rexp[32];
     const int c0 = blk * kSliceK, cnt = min(kSliceK, e - c0), first = c0 + kSliceK;
     if (cnt <= 0 || r0 < first || r0 >= p) return;  // the whole CTA
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r = r0 + lane;
@@ -333,16 +334,19 @@ __device__ __forceinline__ void l11_tile(const double *__restrict__ A, int64_t l
         xs[k * LDX + lane] = (r < p && !d21) ? A[(int64_t)c * lda + r] : 0.0;
     }
     __syncthreads();
-    write_slices<kLRows, kWarps>(xs, cnt, r0 - first, min(kRows, p - r0), cexp, 1, lb.L, lb.el, lb.kb, red, rexp);
+    write_slices<kLRows, kWarps>(xs, cnt, r0 - first, min(kRows, p - r0), cexp, 1, lb.L, lb.el, lb.gl, lb.kb, red,
+                                 rexp);
 }
-__global__ void __launch_bounds__(kRows * kWarps)
+__global__ void __launch_bounds__(kRows * kWarps, 6)
     k_l11_slices(const double *__restrict__ A, int64_t lda, int p, const int32_t *__restrict__ piv,
-                 const double *__restrict__ Dinv, const int32_t *__restrict__ nelim, SliceBuf lb, size_t blk_bytes) {
+                 const double *__restrict__ Dinv, const int32_t *__restrict__ nelim, SliceBuf lb, size_t blk_bytes,
+                 size_t grp_elems) {
     lb.L += blockIdx.y * blk_bytes;
     lb.el += blockIdx.y * kMaxP;
+    lb.gl += blockIdx.y * grp_elems;
     l11_tile(A, lda, p, blockIdx.y, blockIdx.x * kRows, piv, Dinv, *nelim, lb);
 }
-__global__ void __launch_bounds__(kRows * kWarps)
+__global__ void __launch_bounds__(kRows * kWarps, 6)
     k_l11_slices_batch(const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
                        const int *__restrict__ list, BatchOpts o) {
     const int f = list[blockIdx.x];
@@ -404,7 +408,7 @@ constexpr int64_t kApart = 6000000;
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
                               const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
-                              int64_t lo_off, int pieces, int32_t *info, int num_sms, cudaStream_t st) {
+                              int64_t lo_off, int pieces, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st) {
     const int64_t m = n - p;
     if (m <= 0) return cudaSuccess;
     const size_t smem_p = sizeof(double) * (size_t)p * (kRows + 1);
@@ -423,11 +427,11 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
         return cudaGetLastError();
     };
     if (blocks == 0) return pass(kWhole, 0, p);
-    const size_t lbytes = slice_l_bytes(p, kSliceK);
+    const size_t lbytes = slice_l_bytes(p, kSliceK), gelems = slice_gl_bytes(p, kSliceK) / sizeof(uint16_t);
     if (p > kSliceK) {
         const int nb = blocks < (p - 1) / kSliceK ? blocks : (p - 1) / kSliceK;  // the last block has nothing below
         k_l11_slices<<<dim3((unsigned)((p + kRows - 1) / kRows), (unsigned)nb), kRows * kWarps, 0, st>>>(
-            A, lda, p, piv, Dinv, nelim, blk, lbytes);
+            A, lda, p, piv, Dinv, nelim, blk, lbytes, gelems);
         err = cudaGetLastError();
         if (err != cudaSuccess) return err;
     }
@@ -445,7 +449,8 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
         SliceBuf u = blk;
         u.L += b * lbytes;
         u.el += b * kMaxP;
-        err = launch_update(u, A, lda, p, m, b, piv, nelim, info, num_sms, st);
+        u.gl += b * gelems;
+        err = launch_update(u, A, lda, p, m, b, piv, nelim, marks, info, num_sms, st);
         if (err != cudaSuccess) return err;
     }
     if (apart && blocks * kSliceK >= p && sb.W == nullptr && sb.L == nullptr && Wb == nullptr && Lb == nullptr) {
@@ -477,7 +482,8 @@ cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char 
 cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
                                        int count, const int *item_front, const int *item_tile, int64_t items,
                                        int rows, const int *uitem, const int *utile, int64_t uitems, BatchOpts o, void *Wb,
-                                       void *Lb, int pmax, int32_t *info, int num_sms, cudaStream_t st) {
+                                       void *Lb, int pmax, TileMarks *marks, int32_t *info, int num_sms,
+                                       cudaStream_t st) {
     if (items == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (size_t)pmax * (kRows + 1);
     auto *k = solve_batch_kernel(rows);
@@ -491,7 +497,7 @@ cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *ta
     k<<<(unsigned)items, kRows * kWarps, smem, st>>>(
         kFirst, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    err = launch_update_batch(fronts, tab, ws, uitem, utile, uitems, o, info, num_sms, st);
+    err = launch_update_batch(fronts, tab, ws, uitem, utile, uitems, o, marks, info, num_sms, st);
     if (err != cudaSuccess) return err;
     k<<<(unsigned)items, kRows * kWarps, smem, st>>>(
         kTail, fronts, tab, ws, item_front, item_tile, o, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb);
