@@ -49,33 +49,36 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     L.Dinv = off;
     off += align256(sizeof(double) * (2 * (size_t)p + 2));
     const bool tc = opt->prec != CTP_FP64 && opt->smode != CTP_S_NONE;
-    const int64_t ms = opt->smode != CTP_S_NONE && !tc ? m : 0;  // digit slices of the FP64 Form
+    const int64_t mf = opt->smode != CTP_S_NONE && !tc ? m : 0;
+    const int64_t ms = form_small(mf) ? 0 : mf;  // digit slices of the FP64 Form
+    L.W21 = off;
+    off += align256(opt->pivot != CTP_PIV_TPP ? sizeof(double) * (size_t)(mf - ms) * p : 0);
     L.Ws = off;
-    off += align256(slice_w_bytes(ms, p));
+    off += align256(slice_bytes(ms, p));
     L.Ls = off;
-    off += align256(slice_l_bytes(ms, p));
+    off += align256(slice_bytes(ms, p));
     L.ew = off;
     off += align256(sizeof(int32_t) * (size_t)ms);
     L.el = off;
     off += align256(sizeof(int32_t) * (size_t)ms);
     L.gw = off;
-    off += align256(slice_gw_bytes(ms, p));
+    off += align256(slice_g_bytes(ms, p));
     L.gl = off;
-    off += align256(slice_gl_bytes(ms, p));
+    off += align256(slice_g_bytes(ms, p));
     // the blocked FP64 Solve
     const int blocks = opt->pivot != CTP_PIV_TPP && !solve_on_tc(opt) ? solve_blocks(m, p, opt->pivot) : 0;
     L.Yb = off;
-    off += align256(slice_w_bytes(blocks > 0 ? m : 0, kSliceK));
+    off += align256(slice_bytes(blocks > 0 ? m : 0, kSliceK));
     L.Lx = off;
-    off += align256(blocks * slice_l_bytes(p, kSliceK));
+    off += align256(blocks * slice_bytes(p, kSliceK));
     L.ey = off;
     off += align256(sizeof(int32_t) * (size_t)(blocks > 0 ? m : 0));
     L.ex = off;
     off += align256(sizeof(int32_t) * (size_t)blocks * kMaxP);
     L.gy = off;
-    off += align256(slice_gw_bytes(blocks > 0 ? m : 0, kSliceK));
+    off += align256(slice_g_bytes(blocks > 0 ? m : 0, kSliceK));
     L.gx = off;
-    off += align256(blocks * slice_gl_bytes(p, kSliceK));
+    off += align256(blocks * slice_g_bytes(p, kSliceK));
     L.marks = off;
     const int64_t ut = blocks > 0 ? update_tiles(m, p) : 0, ft = form_fp64_slots(ms);
     off += align256(sizeof(TileMarks) * (size_t)(ut > ft ? ut : ft));
@@ -279,7 +282,9 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
     int32_t *info = (int32_t *)(ws + L.info);
     double *Dinv = (double *)(ws + L.Dinv);
     SliceBuf sb = {};
-    if (opt->smode != CTP_S_NONE && !tc)
+    const bool few = opt->smode != CTP_S_NONE && !tc && form_small(m);
+    double *W21 = few && opt->pivot != CTP_PIV_TPP ? (double *)(ws + L.W21) : nullptr;
+    if (opt->smode != CTP_S_NONE && !tc && !few)
         sb = {(unsigned char *)(ws + L.Ws), (unsigned char *)(ws + L.Ls), (int32_t *)(ws + L.ew),
               (int32_t *)(ws + L.el), (uint16_t *)(ws + L.gw), (uint16_t *)(ws + L.gl), slice_kb(p)};
     void *Wb = tc ? (void *)(ws + L.Wb) : nullptr;
@@ -295,7 +300,11 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
             return launch_tpp(A, n, p, lda, opt->u, opt->small, ws + L.aux, perm, piv, D, Dinv, nelim,
                               info, ctx->num_sms, ctx->tpp_spin, st);
         }));
-        if (opt->smode != CTP_S_NONE && m > 0) {
+        if (opt->smode != CTP_S_NONE && m > 0 && few) {
+            CTP_CUDA(timed(ctx, K_FORM, st, [&] {
+                return launch_form_small(A + p, lda, nullptr, piv, D, m, nelim, S, lds, opt->smode, st);
+            }));
+        } else if (opt->smode != CTP_S_NONE && m > 0) {
             CTP_CUDA(timed(ctx, K_W21, st, [&] {
                 return launch_slices_from_l(A, lda, p, m, piv, D, Dinv, nelim, sb, st);
             }));
@@ -366,7 +375,7 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
             const SliceBuf blk = {(unsigned char *)(ws + L.Yb), (unsigned char *)(ws + L.Lx),
                                   (int32_t *)(ws + L.ey), (int32_t *)(ws + L.ex), (uint16_t *)(ws + L.gy),
                                   (uint16_t *)(ws + L.gx), 1};
-            return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, sb, blk, solve_blocks(m, p, opt->pivot), Wb,
+            return launch_solve_fp64(A, n, p, lda, perm, piv, Dinv, nelim, W21, sb, blk, solve_blocks(m, p, opt->pivot), Wb,
                                      Lbf, Kp, lo_off, pieces, (TileMarks *)(ws + L.marks), info, ctx->num_sms, st);
         }));
     if (opt->smode != CTP_S_NONE && m > 0) {
@@ -376,6 +385,10 @@ ctp_status ctp_factor_supernode(ctp_ctx *ctx, int64_t n, int32_t p, double *A, i
                                       opt->smode == CTP_S_FP64_SUB ? 3
                                       : opt->smode == CTP_S_FP32_TILED ? 2 : (packed ? 1 : 0), info,
                                       ctx->num_sms, ctx->form_walk, st);
+            }));
+        else if (few)
+            CTP_CUDA(timed(ctx, K_FORM, st, [&] {
+                return launch_form_small(A + p, lda, W21, piv, D, m, nelim, S, lds, opt->smode, st);
             }));
         else
             CTP_CUDA(timed(ctx, K_FORM, st, [&] {

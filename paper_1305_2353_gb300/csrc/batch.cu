@@ -224,9 +224,9 @@ struct ctp_plan {
     // workspace layout
     size_t off_ginfo, off_tab, off_citem, off_sitem, off_fitem, off_lists, off_flags, off_sections, off_wb,
         off_lb, off_qitem, off_ritem, off_xt, off_zt, off_csitem, off_cstile, off_cfitem, off_cftile, off_cuitem, off_cutile,
-        off_fmarks, off_umarks;
+        off_fmarks, off_umarks, off_csmall;
     size_t total;
-    int64_t c_items, s_items, f_items, total_rows, q_items, r_items, nxt, nzt;
+    int64_t c_items, s_items, f_items, small, total_rows, q_items, r_items, nxt, nzt;
     int64_t cbucket[5] = {0, 0, 0, 0, 0};  // compression items of fronts with p <= 32, 64, 128, 256
     struct Class {
         int kind, G, count;  // kFactor*, cluster width
@@ -238,6 +238,7 @@ struct ctp_plan {
         int s_rows;              // rows per tile
         int64_t u_off, u_count;  // blocked Solve: the class's update items (none: a whole pass per tile)
         int64_t f_off, f_count;  // the class's Form items (front, tile) in the class Form lists
+        int64_t m_off, m_count;  // the class's fronts whose FP64 Form has few rows
     };
     std::vector<Class> classes;
     std::vector<unsigned char> blob;  // tables, in workspace order (up to off_sections)
@@ -443,7 +444,7 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
         };
         std::stable_sort(byKey[key].begin(), byKey[key].end(), [&](int x, int y) { return work(x) > work(y); });
     }
-    std::vector<int> lists, csitem, cstile, cfitem, cftile, cuitem, cutile;
+    std::vector<int> lists, csitem, cstile, cfitem, cftile, cuitem, cutile, csmall;
     for (int key = 0; key < kNumKeys; key++) {
         if (byKey[key].empty()) continue;
         ctp_plan::Class c;
@@ -480,6 +481,11 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
                 }
             }
         c.f_count = (int64_t)cfitem.size() - c.f_off;
+        c.m_off = (int64_t)csmall.size();
+        if (opt->smode != CTP_S_NONE && !tc)
+            for (int f : byKey[key])
+                if (tab[f].m > 0 && form_small(tab[f].m)) csmall.push_back(f);
+        c.m_count = (int64_t)csmall.size() - c.m_off;
         c.kind = key < 2 ? kFactorWarp : (key < 5 ? kFactorCta : kFactorCluster);
         c.G = key < 5 ? 1 : (2 << (key - 5));
         c.pcap = pmaxK[key];
@@ -528,6 +534,9 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     off += align256(sizeof(int) * cuitem.size());
     P->off_cutile = off;
     off += align256(sizeof(int) * cutile.size());
+    P->off_csmall = off;
+    off += align256(sizeof(int) * csmall.size());
+    P->small = (int64_t)csmall.size();
     P->off_flags = off;
     off += align256(sizeof(int32_t) * (size_t)nb);
     const size_t tables_end = off;
@@ -577,6 +586,7 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
         memcpy(P->blob.data() + P->off_cuitem, cuitem.data(), sizeof(int) * cuitem.size());
         memcpy(P->blob.data() + P->off_cutile, cutile.data(), sizeof(int) * cutile.size());
     }
+    if (!csmall.empty()) memcpy(P->blob.data() + P->off_csmall, csmall.data(), sizeof(int) * csmall.size());
     *plan = P;
     if (ws_bytes) *ws_bytes = P->total;
     return CTP_OK;
@@ -684,6 +694,9 @@ cudaError_t batch_form_class(const ctp_plan *P, int ci, const ctp_front *fr, cha
         return launch_form_tc_batch(fr, tab, fitem, c.f_count, P->total_rows, w + P->off_wb, w + P->off_lb,
                                     P->bo.pieces, P->opt.smode == CTP_S_FP64_SUB ? 3 : 2,
                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st, ftile);
+    const cudaError_t e = launch_form_small_batch(fr, tab, w, reinterpret_cast<const int *>(w + P->off_csmall) + c.m_off,
+                                                  c.m_count, P->bo, st);
+    if (e != cudaSuccess) return e;
     return launch_form_fp64_batch(fr, tab, w, fitem, c.f_count, P->bo,
                                   reinterpret_cast<TileMarks *>(w + P->off_fmarks) + c.f_off,
                                   reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st, ftile);
@@ -696,6 +709,9 @@ cudaError_t batch_form(const ctp_plan *P, const ctp_front *fr, char *w, int num_
         return launch_form_tc_batch(fr, tab, fitem, P->f_items, P->total_rows, w + P->off_wb, w + P->off_lb,
                                     P->bo.pieces, P->opt.smode == CTP_S_FP64_SUB ? 3 : 2,
                                     reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
+    const cudaError_t e = launch_form_small_batch(fr, tab, w, reinterpret_cast<const int *>(w + P->off_csmall), P->small,
+                                                  P->bo, st);
+    if (e != cudaSuccess) return e;
     return launch_form_fp64_batch(fr, tab, w, fitem, P->f_items, P->bo,
                                   reinterpret_cast<TileMarks *>(w + P->off_fmarks),
                                   reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);

@@ -25,6 +25,12 @@ constexpr int kExpZero = -100000, kExpNonfinite = 1 << 20;
 constexpr int kGroup = 4;  // rows that share a lower bound of their entries
 constexpr uint32_t kWGroup = kWRows / kGroup * kSliceK * 2, kLGroup = kLRows / kGroup * kSliceK * 2;  // a block's bytes
 
+// Fronts of at most this many rows below the pivots form S by FP64 multiply-adds from W21 itself
+// (form.cu): a tile of slices is 128 rows by 32 pivots, and they would take up to 40 times
+// the room of W21.
+constexpr int kFormSmall = 32;
+__host__ __device__ inline bool form_small(int64_t m) { return m <= kFormSmall; }
+
 // Where a supernode's slices live: blocks at (row block * kb + K block), the
 // rows' exponents E, the groups' lower bounds (FP16) in blocks like the slices'; kb =
 // ceil(p / 32).
@@ -35,17 +41,14 @@ struct SliceBuf {
     int kb;
 };
 __host__ __device__ inline int slice_kb(int p) { return (p + kSliceK - 1) / kSliceK; }
-__host__ __device__ inline size_t slice_w_bytes(int64_t m, int p) {
-    return (size_t)((m + kWRows - 1) / kWRows) * slice_kb(p) * kWBlock;
+// Rows are rounded up to 8 (what the MMA's layout and a bulk copy want), also in the last
+// block: a front with few rows takes room for those only.
+__host__ __device__ inline int64_t slice_rows(int64_t m) { return (m + 7) & ~int64_t(7); }
+__host__ __device__ inline size_t slice_bytes(int64_t m, int p) {
+    return (size_t)slice_rows(m) * slice_kb(p) * (kSlices * 64);
 }
-__host__ __device__ inline size_t slice_l_bytes(int64_t m, int p) {
-    return (size_t)((m + kLRows - 1) / kLRows) * slice_kb(p) * kLBlock;
-}
-__host__ __device__ inline size_t slice_gw_bytes(int64_t m, int p) {
-    return (size_t)((m + kWRows - 1) / kWRows) * slice_kb(p) * kWGroup;
-}
-__host__ __device__ inline size_t slice_gl_bytes(int64_t m, int p) {
-    return (size_t)((m + kLRows - 1) / kLRows) * slice_kb(p) * kLGroup;
+__host__ __device__ inline size_t slice_g_bytes(int64_t m, int p) {
+    return (size_t)(slice_rows(m) / kGroup) * slice_kb(p) * (kSliceK * 2);
 }
 
 // Which entries of a tile of the FP64 Form (or of the Solve's update) digits do not serve,
@@ -60,6 +63,7 @@ struct TileMarks {
 //   [0, 256)            info word + scratch counters
 //   C                   p*p doubles, row-major compressed matrix (strict: as uint64 keys)
 //   Dinv                2p doubles: inverse pivot blocks, same slots as D
+//   W21                 m*p doubles (Y = L21 D11) when the FP64 Form of few rows runs
 //   Ws, Ls, ew, el,     digit slices of Y = L21 D11 and L21, their row exponents and
 //     gw, gl            lower bounds (slices.cuh) when the FP64 Form step runs
 //   Yb, Lx, ey, ex,     the same of one block's y and of L11 for the blocked FP64 Solve
@@ -68,7 +72,7 @@ struct TileMarks {
 //   Wb, Lb              m*Kp BF16 copies of Y and L21 for the tensor-core Form
 //   aux                 method-specific scratch (relaxed candidate lists)
 struct WsLayout {
-    size_t info, C, Dinv, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, marks, Wb, Lb, aux, Xs, flags, total;
+    size_t info, C, Dinv, W21, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, marks, Wb, Lb, aux, Xs, flags, total;
 };
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -143,9 +147,10 @@ struct BFront {
     int32_t kbx, nwz;
 };
 // offsets inside a front's section: info word, compressed matrix (strict),
-// Dinv, and the digit slices of L21 D11 and L21 when an FP64 Form follows
+// Dinv, and when an FP64 Form follows W21 = L21 D11 (few rows) or the digit slices of
+// W21 and L21
 struct BSection {
-    size_t info, C, Dinv, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, nz, total;
+    size_t info, C, Dinv, W21, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, nz, total;
 };
 __host__ __device__ inline size_t align256hd(size_t x) { return (x + 255) & ~size_t(255); }
 __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options *opt) {
@@ -157,35 +162,38 @@ __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options
     off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(double) * (size_t)p * p : 0);
     s.Dinv = off;
     off += align256hd(sizeof(double) * (2 * (size_t)p + 2));
-    const int64_t ms = opt->smode != CTP_S_NONE && opt->prec == CTP_FP64 ? n - p : 0;
+    s.nz = off;  // strict: which rows of C receive an A21 row (one bit per row)
+    off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
+    const int64_t mf = opt->smode != CTP_S_NONE && opt->prec == CTP_FP64 ? n - p : 0;
+    const int64_t ms = form_small(mf) ? 0 : mf;
+    s.W21 = off;
+    off += align256hd(sizeof(double) * (size_t)(mf - ms) * p);
     s.Ws = off;
-    off += align256hd(slice_w_bytes(ms, p));
+    off += align256hd(slice_bytes(ms, p));
     s.Ls = off;
-    off += align256hd(slice_l_bytes(ms, p));
+    off += align256hd(slice_bytes(ms, p));
     s.ew = off;
     off += align256hd(sizeof(int32_t) * (size_t)ms);
     s.el = off;
     off += align256hd(sizeof(int32_t) * (size_t)ms);
     s.gw = off;
-    off += align256hd(slice_gw_bytes(ms, p));
+    off += align256hd(slice_g_bytes(ms, p));
     s.gl = off;
-    off += align256hd(slice_gl_bytes(ms, p));
+    off += align256hd(slice_g_bytes(ms, p));
     // the blocked Solve's first block: slices of y and of L11's rows below it
     const int64_t mb = p > kSliceK ? n - p : 0;
     s.Yb = off;
-    off += align256hd(slice_w_bytes(mb, kSliceK));
+    off += align256hd(slice_bytes(mb, kSliceK));
     s.Lx = off;
-    off += align256hd(mb > 0 ? slice_l_bytes(p, kSliceK) : 0);
+    off += align256hd(mb > 0 ? slice_bytes(p, kSliceK) : 0);
     s.ey = off;
     off += align256hd(sizeof(int32_t) * (size_t)mb);
     s.ex = off;
     off += align256hd(mb > 0 ? sizeof(int32_t) * (size_t)p : 0);
     s.gy = off;
-    off += align256hd(slice_gw_bytes(mb, kSliceK));
+    off += align256hd(slice_g_bytes(mb, kSliceK));
     s.gx = off;
-    off += align256hd(mb > 0 ? slice_gl_bytes(p, kSliceK) : 0);
-    s.nz = off;  // strict: which rows of C receive an A21 row (one bit per row)
-    off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
+    off += align256hd(mb > 0 ? slice_g_bytes(p, kSliceK) : 0);
     s.total = off;
     return s;
 }
@@ -244,6 +252,9 @@ int solve_rows(int64_t tiles, bool blocked, int num_sms);
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
                                    const int *item_front, int64_t items, BatchOpts o, TileMarks *marks, int32_t *info,
                                    int num_sms, cudaStream_t st, const int *item_tile = nullptr);
+// the fronts of few rows, by number (W21 from their sections)
+cudaError_t launch_form_small_batch(const ctp_front *fronts, const BFront *tab, char *ws, const int *list, int64_t count,
+                                    BatchOpts o, cudaStream_t st);
 cudaError_t launch_form_tc_batch(const ctp_front *fronts, const BFront *tab, const int *item_front,
                                  int64_t items, int64_t total_rows, const void *Wb, const void *Lb,
                                  int pieces, int layout /* 2 tiled, 3 subtract */, int32_t *info, int num_sms,
@@ -300,7 +311,7 @@ cudaError_t launch_solve_tc_batch(const ctp_front *fronts, const BFront *tab, ch
 
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
-                              const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
+                              double *W21, const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
                               int64_t lo_off, int pieces, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st);
 int solve_blocks(int64_t m, int p, int pivot);  // 0: a whole pass
 // A21(:, 32 (blk+1)..p-1) -= y_blk L11(32 (blk+1).., block blk)^T from the slices (form.cu)
@@ -338,6 +349,9 @@ cudaError_t launch_form_tc(const void *Wb, const void *Lb, int64_t piece_off, in
 cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda, const int32_t *piv,
                              const double *D, int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
                              TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st);
+// the same for few rows (W21 null: from L21 and D)
+cudaError_t launch_form_small(const double *L21, int64_t lda, const double *W21, const int32_t *piv, const double *D,
+                              int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode, cudaStream_t st);
 // the slices from a stored L21 and its D, D^-1 (full-column pivoting)
 cudaError_t launch_slices_from_l(const double *A, int64_t lda, int p, int64_t m, const int32_t *piv,
                                  const double *D, const double *Dinv, const int32_t *nelim, const SliceBuf &sb,

@@ -39,6 +39,7 @@
 // update of 224 columns of 200000 rows took 446 us with 144 instructions per entry,
 // 210 with the test-free path, the 32-bit sums of neighbouring groups and the old
 // values brought to L2 ahead (HBM's share: 121 us).
+// Fronts of few rows have a kernel of their own, k_form_small.
 // Every mbarrier wait is bounded; on timeout the kernel records CTP_ETIMEOUT,
 // waits (bounded) for its copies in flight, frees its tensor memory and returns.
 #include <cuda_fp16.h>
@@ -263,7 +264,7 @@ __device__ __noinline__ double to_fp64_any(long long V, int ex) {
 // Which 4 x 4 blocks of a tile have pivots in which all their rows are large
 // (slices.cuh): the dot products of four groups of rows (4 (lane / 4)..) by four of
 // columns (4 (lane % 4)..) per lane, from the groups' bounds, a K block of them at a time
-// (`fetch(kb)` brings it to shared memory).  Bit 4 a + b: group a of the lane's rows by
+// (`fetch(kb)` brings it to shared memory; gw and gl groups per chunk of 8 pivots).  Bit 4 a + b: group a of the lane's rows by
 // group b of its columns has not, and neither are they without a pivot in common
 // (their results are then zero).  Rounded in FP16: a part in 2^11 per term of up to 128
 // per sum.  From the last pivot on, where growth puts the large entries, and no
@@ -271,7 +272,7 @@ __device__ __noinline__ double to_fp64_any(long long V, int ex) {
 // traffic from L2 (all blocks: 3% at e = 256).
 constexpr float kSure = 0x1p-7f;
 template <typename F>
-__device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, F &&fetch) {
+__device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, int gw, int gl, F &&fetch) {
     const int lane = threadIdx.x & 31;
     const uint4 *pa = reinterpret_cast<const uint4 *>(grp) + 4 * (lane >> 2);
     const uint4 *pb = reinterpret_cast<const uint4 *>(grp + kWGroup) + 4 * (lane & 3);
@@ -289,10 +290,10 @@ __device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, F &
         for (int c = 0; c < chunks; c++) {
             uint4 v[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) v[j] = pb[c * (kBN / kGroup) + j];
+            for (int j = 0; j < 4; j++) v[j] = pb[c * gl + j];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
-                const uint4 u = pa[c * (kBM / kGroup) + i];
+                const uint4 u = pa[c * gw + i];
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     __half2 &t = s[4 * i + j];
@@ -322,10 +323,10 @@ __device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, F &
         for (int c = 0; c < chunks; c++) {
             uint4 v[4];
 #pragma unroll
-            for (int j = 0; j < 4; j++) v[j] = pb[c * (kBN / kGroup) + j];
+            for (int j = 0; j < 4; j++) v[j] = pb[c * gl + j];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
-                const uint4 u = pa[c * (kBM / kGroup) + i];
+                const uint4 u = pa[c * gw + i];
 #pragma unroll
                 for (int j = 0; j < 4; j++)
                     none[4 * i + j] &= (u.x | v[j].x) & (u.y | v[j].y) & (u.z | v[j].z) & (u.w | v[j].w);
@@ -561,6 +562,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
             unsigned bits = 0u;
             bool linked = false;
             if (x.e > 0) {
+                // groups of the tile's blocks of rows
+                const int gw = min(kBM, (int)slice_rows(x.m - x.ti * kBM)) / kGroup;
+                const int gl = min(kBN, (int)slice_rows(x.nc - x.tj * kBN)) / kGroup;
                 // rows that hold an Inf or NaN
                 const int r0 = x.ti * kBM + 4 * lane, c0 = x.tj * kBN + 2 * lane;
                 int4 er = make_int4(0, 0, 0, 0);
@@ -571,17 +575,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                     __syncwarp();
                     if (lane == 0) {
                         const uint32_t chunks = min(4u, (uint32_t)(x.e - kb * kSliceK + 7) / 8);
-                        const uint32_t bw = chunks * (kWGroup / 4), bl = chunks * (kLGroup / 4);
+                        const uint32_t bw = chunks * gw * 16, bl = chunks * gl * 16;
                         mbar_expect_tx(&bars.grp_full, bw + bl);
-                        bulk_load(grp, x.sb.gw + ((size_t)x.ti * x.sb.kb + kb) * (kWGroup / 2), bw, &bars.grp_full);
-                        bulk_load(grp + kWGroup, x.sb.gl + ((size_t)x.tj * x.sb.kb + kb) * (kLGroup / 2), bl,
+                        bulk_load(grp, x.sb.gw + (size_t)x.ti * x.sb.kb * (kWGroup / 2) + (size_t)kb * gw * 32, bw,
                                   &bars.grp_full);
+                        bulk_load(grp + kWGroup, x.sb.gl + (size_t)x.tj * x.sb.kb * (kLGroup / 2) + (size_t)kb * gl * 32,
+                                  bl, &bars.grp_full);
                     }
                     int never = 0;  // no CTA leaves with copies in flight
                     ok = mbar_wait(&bars.grp_full, grpphase, &never) && ok;
                     grpphase ^= 1u;
                 };
-                bits = unsure_blocks(grp, x.e, fetch);
+                bits = unsure_blocks(grp, x.e, gw, gl, fetch);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
                     break;
@@ -648,18 +653,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                     }
                     uint8_t *dW = smem + (size_t)stage * kStageBytes, *dL = dW + kWBlock;
                     mbar_expect_tx(&bars.full[stage], kSlices * 64 * (rw + rl));
+                    const unsigned char *kW = srcW + (size_t)kb * kSlices * 64 * rw, *kL = srcL + (size_t)kb * kSlices * 64 * rl;
                     if (rw == kBM)
-                        bulk_load(dW, srcW + (size_t)kb * kWBlock, kWBlock, &bars.full[stage]);
+                        bulk_load(dW, kW, kWBlock, &bars.full[stage]);
                     else
                         for (int s = 0; s < kSlices; s++)
-                            bulk_load(dW + s * kWSlice, srcW + (size_t)kb * kWBlock + s * kWSlice, rw * 64,
-                                      &bars.full[stage]);
+                            bulk_load(dW + s * kWSlice, kW + s * 64 * rw, rw * 64, &bars.full[stage]);
                     if (rl == kBN)
-                        bulk_load(dL, srcL + (size_t)kb * kLBlock, kLBlock, &bars.full[stage]);
+                        bulk_load(dL, kL, kLBlock, &bars.full[stage]);
                     else
                         for (int s = 0; s < kSlices; s++)
-                            bulk_load(dL + s * kLSlice, srcL + (size_t)kb * kLBlock + s * kLSlice, rl * 64,
-                                      &bars.full[stage]);
+                            bulk_load(dL + s * kLSlice, kL + s * 64 * rl, rl * 64, &bars.full[stage]);
                     issued++;
                     if (++stage == kStages) {
                         stage = 0;
@@ -857,6 +861,88 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
     }
 }
 
+// Few rows (kFormSmall at most): S by FP64 multiply-adds in the order of the pivots, a CTA
+// per front, 32 pivots of W21 and L21 at a time in shared memory, a thread an entry or
+// up to five.  A latency of a few microseconds per front, sixteen fronts per SM at a
+// time; a tile of slices takes 5 us of its SM whatever its rows.
+constexpr int kSmallT = 128, kSmallE = (kFormSmall * (kFormSmall + 1) / 2 + kSmallT - 1) / kSmallT;
+template <int kMode>
+__global__ void __launch_bounds__(kSmallT) k_form_small(const __grid_constant__ Work wk, const double *W21) {
+    typedef typename FormOut<kMode>::T OutT;
+    constexpr bool kPacked = FormOut<kMode>::kPacked, kSub = FormOut<kMode>::kSub;
+    __shared__ double ws[kSliceK][kFormSmall + 1], ls[kSliceK][kFormSmall + 1];
+    const double *L21 = wk.L21, *D = wk.D;
+    const int32_t *piv = wk.piv, *nelim = wk.nelim;
+    int64_t ldl = wk.ldl, lds = wk.lds;
+    int m = (int)wk.m;
+    OutT *S = reinterpret_cast<OutT *>(wk.S);
+    if (wk.fronts != nullptr) {
+        const int f = wk.item_front[blockIdx.x];
+        const BFront b = wk.tab[f];
+        const ctp_front fr = wk.fronts[f];
+        m = (int)b.m;
+        L21 = fr.A + b.p;
+        ldl = fr.lda;
+        lds = fr.lds;
+        S = reinterpret_cast<OutT *>(fr.S);
+        nelim = fr.nelim;
+        ctp_options oo;
+        oo.pivot = wk.o.pivot;
+        oo.smode = wk.o.smode;
+        oo.prec = wk.o.prec;
+        W21 = reinterpret_cast<const double *>(wk.ws + b.ws + bsection(b.n, b.p, &oo).W21);
+    }
+    const int e = *nelim, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // entries of the lower triangle, column by column
+    const int total = m * (m + 1) / 2;
+    int row[kSmallE], col[kSmallE];
+    double acc[kSmallE] = {};
+#pragma unroll
+    for (int q = 0; q < kSmallE; q++) {
+        const int t = min((int)threadIdx.x + q * kSmallT, total - 1);
+        int j = (int)((2 * m + 1 - sqrtf((float)((2 * m + 1) * (2 * m + 1) - 8 * t))) * 0.5f);
+        while (j > 0 && j * m - j * (j - 1) / 2 > t) j--;
+        while ((j + 1) * m - (j + 1) * j / 2 <= t) j++;
+        col[q] = j;
+        row[q] = t - (j * m - j * (j - 1) / 2) + j;
+    }
+    for (int k0 = 0; k0 < e; k0 += kSliceK) {
+        const int cnt = min(kSliceK, e - k0);
+        for (int k = warp; k < cnt; k += kSmallT / 32) {
+            if (lane >= m) continue;
+            const int kk = k0 + k;
+            const double *c = L21 + (int64_t)kk * ldl + lane;
+            const double l = *c;
+            double w;
+            if (W21 != nullptr) {
+                w = W21[(int64_t)kk * m + lane];
+            } else {  // W21 = L21 D11
+                const int kd = piv[kk];
+                w = kd == CTP_PIVKIND_ZERO ? 0.0 : l * D[2 * kk];
+                if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(c[ldl], D[2 * kk + 1], w);
+                if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(c[-ldl], D[2 * kk - 1], w);
+            }
+            ws[k][lane] = w;
+            ls[k][lane] = l;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kSmallE; q++) {
+            if ((int)threadIdx.x + q * kSmallT >= total) break;
+#pragma unroll 4
+            for (int k = 0; k < cnt; k++) acc[q] = fma(ws[k][row[q]], ls[k][col[q]], acc[q]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < kSmallE; q++) {
+        const int t = threadIdx.x + q * kSmallT;
+        if (t >= total) break;
+        OutT *ptr = S + (kPacked ? (int64_t)t : (int64_t)col[q] * lds + row[q]);
+        *ptr = kSub ? (OutT)(*ptr - acc[q]) : (OutT)acc[q];
+    }
+}
+
 // Slices of W21 = L21 D11 and L21 from a stored L21 (full-column pivoting writes no
 // slices itself): a CTA per 32 rows.
 constexpr int kSW = 8;
@@ -873,7 +959,7 @@ __global__ void __launch_bounds__(32 * kSW)
     for (int k = threadIdx.x; k < e; k += 32 * kSW) cexp[k] = (short)slice_col_exp(piv, Dinv, k);
     for (int k = w; k < e; k += kSW) xs[k * 33 + lane] = lane < nrows ? A[(int64_t)k * lda + p + row0 + lane] : 0.0;
     __syncthreads();
-    write_slices<kLRows, kSW>(xs, e, row0, nrows, cexp, 1, sb.L, sb.el, sb.gl, sb.kb, red, rexp);
+    write_slices<kLRows, kSW>(xs, e, row0, nrows, cexp, 1, sb.L, sb.el, sb.gl, sb.kb, m, red, rexp);
     __syncthreads();
     for (int k = w; k < e; k += kSW) {
         const int kd = piv[k];
@@ -886,7 +972,7 @@ __global__ void __launch_bounds__(32 * kSW)
         }
     }
     __syncthreads();
-    write_slices<kWRows, kSW>(xs, e, row0, nrows, cexp, -1, sb.W, sb.ew, sb.gw, sb.kb, red, rexp);
+    write_slices<kWRows, kSW>(xs, e, row0, nrows, cexp, -1, sb.W, sb.ew, sb.gw, sb.kb, m, red, rexp);
 }
 
 template <int kMode>
@@ -896,6 +982,22 @@ cudaError_t launch_mode(const Work &wk, int32_t *info, int num_sms, cudaStream_t
     const unsigned grid = (unsigned)(wk.count < num_sms ? wk.count : num_sms);
     k_form_fp64<kMode><<<grid, kThreads, kSmem, st>>>(wk, info);
     return cudaGetLastError();
+}
+
+template <int kMode>
+cudaError_t launch_small_mode(const Work &wk, const double *W21, cudaStream_t st) {
+    k_form_small<kMode><<<(unsigned)wk.count, kSmallT, 0, st>>>(wk, W21);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_small(const Work &wk, const double *W21, int smode, cudaStream_t st) {
+    switch (smode) {
+    case CTP_S_FP64: return launch_small_mode<CTP_S_FP64>(wk, W21, st);
+    case CTP_S_FP32: return launch_small_mode<CTP_S_FP32>(wk, W21, st);
+    case CTP_S_FP64_SUB: return launch_small_mode<CTP_S_FP64_SUB>(wk, W21, st);
+    case CTP_S_FP64_PACKED: return launch_small_mode<CTP_S_FP64_PACKED>(wk, W21, st);
+    default: return launch_small_mode<CTP_S_FP32_PACKED>(wk, W21, st);
+    }
 }
 
 cudaError_t launch_any(const Work &wk, int smode, int32_t *info, int num_sms, cudaStream_t st) {
@@ -928,6 +1030,35 @@ cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda,
     wk.count = walk_slots(m);
     wk.marks = marks;
     return launch_any(wk, smode, info, num_sms, st);
+}
+
+cudaError_t launch_form_small(const double *L21, int64_t lda, const double *W21, const int32_t *piv, const double *D,
+                              int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode, cudaStream_t st) {
+    if (m <= 0) return cudaSuccess;
+    Work wk = {};
+    wk.L21 = L21;
+    wk.ldl = lda;
+    wk.piv = piv;
+    wk.D = D;
+    wk.m = m;
+    wk.lds = lds;
+    wk.nelim = nelim;
+    wk.S = S;
+    wk.count = 1;
+    return launch_small(wk, W21, smode, st);
+}
+
+cudaError_t launch_form_small_batch(const ctp_front *fronts, const BFront *tab, char *ws, const int *list, int64_t count,
+                                    BatchOpts o, cudaStream_t st) {
+    if (count == 0) return cudaSuccess;
+    Work wk = {};
+    wk.fronts = fronts;
+    wk.tab = tab;
+    wk.ws = ws;
+    wk.item_front = list;
+    wk.o = o;
+    wk.count = count;
+    return launch_small(wk, nullptr, o.smode, st);
 }
 
 cudaError_t launch_form_fp64_batch(const ctp_front *fronts, const BFront *tab, char *ws,
@@ -1000,6 +1131,7 @@ cudaError_t launch_slices_from_l(const double *A, int64_t lda, int p, int64_t m,
 // Tiles of a front's Form: row blocks of 128 by column blocks of 64 on or below the
 // diagonal (the last row block may lack its last column block)
 int64_t form_fp64_tiles(int64_t m) {
+    if (form_small(m)) return 0;  // not of slices
     const int64_t nM = (m + kBM - 1) / kBM, nN = (m + kBN - 1) / kBN;
     return nM * (nM + 1) - (2 * nM - nN);
 }

@@ -39,7 +39,8 @@
 // passes neither.
 //
 // Layout (what a bulk copy puts into shared memory as the MMA reads it): W in
-// blocks of 128 rows, L in blocks of 64; per row block and block of 32 pivots
+// blocks of 128 rows, L in blocks of 64, the last of either as long as its rows, rounded
+// up to 8; per row block and block of 32 pivots
 // the eight slices one after another, each rows x 64 bytes, K-major with the
 // 64-byte swizzle (16-byte chunk c of row r at c ^ ((r >> 1) & 3)).
 #pragma once
@@ -110,7 +111,7 @@ __device__ __forceinline__ unsigned slice_low(double x, int sh, int E) {
 
 // The slices of a tile of 32 rows, by a CTA of kWarps warps: columns k < e of the
 // tile in xs ([k][33], rows row0 .. row0 + nrows of the operand), column k times
-// 2^(sgn * cexp[k]); kBlk rows per block of the image.  Zeros from e to the
+// 2^(sgn * cexp[k]); the operand's `rows` in blocks of kBlk.  Zeros from e to the
 // next multiple of 16 (the MMA reads no further).  grp: per block of rows and chunk of 8
 // columns the groups' FP16 lower bounds of their rows' entries, 16 bytes each; -0
 // where all four rows hold zeros.  red: kWarps * 32 ints, rexp: 32 ints of
@@ -118,7 +119,7 @@ __device__ __forceinline__ unsigned slice_low(double x, int sh, int E) {
 template <int kBlk, int kWarps>
 __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t row0, int nrows, const short *cexp,
                                              int sgn, unsigned char *__restrict__ img, int32_t *__restrict__ rowexp,
-                                             uint16_t *__restrict__ grp, int kb, int *red, int *rexp) {
+                                             uint16_t *__restrict__ grp, int kb, int64_t rows, int *red, int *rexp) {
     constexpr int LDX = 33;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int E = kExpZero;
@@ -133,6 +134,11 @@ __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t ro
         if (lane < nrows) rowexp[row0 + lane] = E;
     }
     __syncthreads();
+    // the block of the tile's rows (a tile lies in one)
+    const int64_t blk0 = row0 / kBlk * kBlk;
+    const int len = (int)min((int64_t)kBlk, slice_rows(rows - blk0)), at = (int)(row0 - blk0);
+    img += (size_t)blk0 * kb * (kSlices * 64);
+    grp += blk0 / kGroup * kb * kSliceK;
     const int e16 = (e + 15) & ~15, nkb = (e + kSliceK - 1) / kSliceK;
     // an item: 8 rows by the four 16-byte chunks of a K block, a lane per (row, chunk)
     for (int it = w; it < 4 * nkb; it += kWarps) {
@@ -164,17 +170,15 @@ __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t ro
             for (int q = 0; q < 4; q++) low[q] = __vminu2(low[q], __shfl_xor_sync(0xffffffffu, low[q], o));
         }
         if (!on) continue;
-        const int64_t row = row0 + r, blk = row / kBlk * kb + kblk;
+        const int rb = at + r;
         if (r % kGroup == 0) {
 #pragma unroll
             for (int j = 0; j < 8; j++)
                 if (!((some >> j) & 1u)) low[j >> 1] = (j & 1) ? (low[j >> 1] & 0xFFFFu) | 0x80000000u : (low[j >> 1] & 0xFFFF0000u) | 0x8000u;
-            *reinterpret_cast<uint4 *>(grp + ((blk * 4 + c) * (kBlk / kGroup) + row % kBlk / kGroup) * 8) =
+            *reinterpret_cast<uint4 *>(grp + ((kblk * 4 + c) * (len / kGroup) + rb / kGroup) * 8) =
                 make_uint4(low[0], low[1], low[2], low[3]);
         }
-        const int rb = (int)(row % kBlk);
-        unsigned char *dst = img + (size_t)blk * ((size_t)kSlices * kBlk * 64) + rb * 64 +
-                             ((c ^ ((rb >> 1) & 3)) << 4);
+        unsigned char *dst = img + (kblk * kSlices * len + rb) * 64 + ((c ^ ((rb >> 1) & 3)) << 4);
 #pragma unroll
         for (int s = 0; s < kSlices; s++) {
             uint4 v;
@@ -182,7 +186,7 @@ __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t ro
             v.y = slice_pair(y[2], y[3], s);
             v.z = slice_pair(y[4], y[5], s);
             v.w = slice_pair(y[6], y[7], s);
-            *reinterpret_cast<uint4 *>(dst + (size_t)s * kBlk * 64) = v;
+            *reinterpret_cast<uint4 *>(dst + s * len * 64) = v;
         }
     }
 }

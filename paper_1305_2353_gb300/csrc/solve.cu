@@ -102,7 +102,8 @@ template <int RT>
 __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                                            const int32_t *__restrict__ perm,
                                            const int32_t *__restrict__ piv,
-                                           const double *__restrict__ Dinv, int e, const SliceBuf &sb,
+                                           const double *__restrict__ Dinv, int e, double *__restrict__ W21,
+                                           const SliceBuf &sb,
                                            __nv_bfloat16 *__restrict__ Wb,
                                            __nv_bfloat16 *__restrict__ Lb, int Kp, int64_t brow0,
                                            int64_t lo_off, int pieces, int64_t tile, double *xs) {
@@ -174,7 +175,7 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
             for (int k = c0 + threadIdx.x; k < j1; k += blockDim.x) cexp[k - c0] = (short)slice_col_exp(piv, Dinv, k);
             __syncthreads();
             write_slices<kWRows, kWarps>(xs, j1 - c0, row0, tile_rows, cexp, -1, ps.yb.W, ps.yb.ew, ps.yb.gw,
-                                         ps.yb.kb, red, rexp);
+                                         ps.yb.kb, m, red, rexp);
         }
         if (valid)
             for (int k = c0 + w; k < c1; k += CW) A21[(int64_t)k * lda + row] = xs[(k - c0) * LDX + r];
@@ -188,8 +189,10 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     if (sb.W != nullptr) {
         for (int k = threadIdx.x; k < e; k += blockDim.x) cexp[k] = (short)slice_col_exp(piv, Dinv, k);
         __syncthreads();
-        write_slices<kWRows, kWarps>(xs, e, row0, tile_rows, cexp, -1, sb.W, sb.ew, sb.gw, sb.kb, red, rexp);
+        write_slices<kWRows, kWarps>(xs, e, row0, tile_rows, cexp, -1, sb.W, sb.ew, sb.gw, sb.kb, m, red, rexp);
     }
+    if (W21 != nullptr && valid)
+        for (int k = w; k < e; k += CW) W21[(int64_t)k * m + row] = xs[k * LDX + r];
     if (Wb != nullptr) write_pieces(Wb, brow0 + row0, tile_rows, Kp, e, Kz, pieces, lo_off, xs);
     __syncthreads();
     // L21 = Y D11^{-1} in place (1x1 and 2x2 blocks; zero pivots give 0), written
@@ -216,7 +219,7 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     __syncthreads();
     // the Form's copies of L21
     if (sb.L != nullptr)
-        write_slices<kLRows, kWarps>(xs, e, row0, tile_rows, cexp, 1, sb.L, sb.el, sb.gl, sb.kb, red, rexp);
+        write_slices<kLRows, kWarps>(xs, e, row0, tile_rows, cexp, 1, sb.L, sb.el, sb.gl, sb.kb, m, red, rexp);
     if (Lb != nullptr) write_pieces(Lb, brow0 + row0, tile_rows, Kp, e, Kz, pieces, lo_off, xs);
 }
 
@@ -225,10 +228,10 @@ __global__ void __launch_bounds__(kRows * kWarps, 6)
     k_solve_fp64(SolvePass ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                  const int32_t *__restrict__ perm, const int32_t *__restrict__ piv,
                  const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p,
-                 SliceBuf sb, __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb, int Kp,
+                 double *W21, SliceBuf sb, __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb, int Kp,
                  int64_t lo_off, int pieces) {
     extern __shared__ __align__(16) double xs[];  // [columns][kRows+1]
-    solve_tile<RT>(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
+    solve_tile<RT>(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, W21, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
 }
 
 // Batched: CTA b takes work item b = (front, RT-row tile of its A21): the
@@ -249,11 +252,17 @@ __global__ void __launch_bounds__(kRows * kWarps, 6)
     const BSection sec = bsection(bt.n, bt.p, &oo);
     char *base = ws + bt.ws;
     SliceBuf sb = {};
-    if (o.smode != CTP_S_NONE && o.prec == CTP_FP64) sb = bsection_slices(base, sec, bt.p);
+    double *W21 = nullptr;
+    if (o.smode != CTP_S_NONE && o.prec == CTP_FP64) {
+        if (form_small(bt.m))
+            W21 = reinterpret_cast<double *>(base + sec.W21);
+        else
+            sb = bsection_slices(base, sec, bt.p);
+    }
     SolvePass ps = {mode, mode == kTail ? 1 : 0, {}};
     if (mode == kFirst) ps.yb = bsection_block(base, sec);
     solve_tile<RT>(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
-               *fr.nelim, sb, Wb, Lb, kBatchKp, bt.row0, o.lo_off, o.pieces,
+               *fr.nelim, W21, sb, Wb, Lb, kBatchKp, bt.row0, o.lo_off, o.pieces,
                item_tile[blockIdx.x], xs);
 }
 
@@ -334,8 +343,8 @@ __device__ __forceinline__ void l11_tile(const double *__restrict__ A, int64_t l
         xs[k * LDX + lane] = (r < p && !d21) ? A[(int64_t)c * lda + r] : 0.0;
     }
     __syncthreads();
-    write_slices<kLRows, kWarps>(xs, cnt, r0 - first, min(kRows, p - r0), cexp, 1, lb.L, lb.el, lb.gl, lb.kb, red,
-                                 rexp);
+    write_slices<kLRows, kWarps>(xs, cnt, r0 - first, min(kRows, p - r0), cexp, 1, lb.L, lb.el, lb.gl, lb.kb, p - first,
+                                 red, rexp);
 }
 __global__ void __launch_bounds__(kRows * kWarps, 6)
     k_l11_slices(const double *__restrict__ A, int64_t lda, int p, const int32_t *__restrict__ piv,
@@ -407,7 +416,7 @@ constexpr int64_t kApart = 6000000;
 
 cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const int32_t *perm,
                               const int32_t *piv, const double *Dinv, const int32_t *nelim,
-                              const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
+                              double *W21, const SliceBuf &sb, const SliceBuf &blk, int blocks, void *Wb, void *Lb, int Kp,
                               int64_t lo_off, int pieces, TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st) {
     const int64_t m = n - p;
     if (m <= 0) return cudaSuccess;
@@ -423,11 +432,11 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
         const SolvePass ps = {mode, b, blk};
         auto *k = rt == kRows ? k_solve_fp64<kRows> : rt == kRows / 2 ? k_solve_fp64<kRows / 2> : k_solve_fp64<kRows / 4>;
         k<<<grid, kRows * kWarps, sizeof(double) * (size_t)cols * (kRows + 1), st>>>(
-            ps, A, n, p, lda, perm, piv, Dinv, nelim, sb, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, Kp, lo_off, pieces);
+            ps, A, n, p, lda, perm, piv, Dinv, nelim, W21, sb, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, Kp, lo_off, pieces);
         return cudaGetLastError();
     };
     if (blocks == 0) return pass(kWhole, 0, p);
-    const size_t lbytes = slice_l_bytes(p, kSliceK), gelems = slice_gl_bytes(p, kSliceK) / sizeof(uint16_t);
+    const size_t lbytes = slice_bytes(p, kSliceK), gelems = slice_g_bytes(p, kSliceK) / sizeof(uint16_t);
     if (p > kSliceK) {
         const int nb = blocks < (p - 1) / kSliceK ? blocks : (p - 1) / kSliceK;  // the last block has nothing below
         k_l11_slices<<<dim3((unsigned)((p + kRows - 1) / kRows), (unsigned)nb), kRows * kWarps, 0, st>>>(
@@ -453,7 +462,7 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
         err = launch_update(u, A, lda, p, m, b, piv, nelim, marks, info, num_sms, st);
         if (err != cudaSuccess) return err;
     }
-    if (apart && blocks * kSliceK >= p && sb.W == nullptr && sb.L == nullptr && Wb == nullptr && Lb == nullptr) {
+    if (apart && blocks * kSliceK >= p && W21 == nullptr && sb.W == nullptr && sb.L == nullptr && Wb == nullptr && Lb == nullptr) {
         k_scale_columns<<<dim3((unsigned)((m + kScaleRows - 1) / kScaleRows),
                                (unsigned)((p + kScaleCols - 1) / kScaleCols)),
                           kScaleRows, 0, st>>>(A + p, m, lda, piv, Dinv, nelim);
