@@ -67,16 +67,18 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     off += align256(slice_g_bytes(ms, p));
     // the blocked FP64 Solve
     const int blocks = opt->pivot != CTP_PIV_TPP && !solve_on_tc(opt) ? solve_blocks(m, p, opt->pivot) : 0;
-    L.Yb = off;
-    off += align256(slice_bytes(blocks > 0 ? m : 0, kSliceK));
+    // (its y where the slices of W21 come later, if there are any)
+    const int64_t mb = blocks > 0 && ms == 0 ? m : 0;
+    L.Yb = ms > 0 ? L.Ws : off;
+    off += align256(slice_bytes(mb, kSliceK));
     L.Lx = off;
     off += align256(blocks * slice_bytes(p, kSliceK));
-    L.ey = off;
-    off += align256(sizeof(int32_t) * (size_t)(blocks > 0 ? m : 0));
+    L.ey = ms > 0 ? L.ew : off;
+    off += align256(sizeof(int32_t) * (size_t)mb);
     L.ex = off;
     off += align256(sizeof(int32_t) * (size_t)blocks * kMaxP);
-    L.gy = off;
-    off += align256(slice_g_bytes(blocks > 0 ? m : 0, kSliceK));
+    L.gy = ms > 0 ? L.gw : off;
+    off += align256(slice_g_bytes(mb, kSliceK));
     L.gx = off;
     off += align256(blocks * slice_g_bytes(p, kSliceK));
     L.marks = off;

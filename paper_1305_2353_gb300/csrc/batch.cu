@@ -27,10 +27,10 @@ namespace {
 
 constexpr int kTR = 32;     // rows per compression item
 constexpr int kThreads = 256;
-// A class's Solve is blocked (solve.cu) when its fronts hold this many entries of A21
-// right of their first 32 columns: the Solves of a mixed 64^3 multifrontal
-// factorization took 67.8 ms whole, 45.9 with the line at 1e6, 46.4 at 1e5, those
-// of a 36^3 one 9.5, 9.3 and 8.3 ms, those of 1024 uneven fronts 0.79, 0.64, 0.68 ms
+// The fronts of a class that may solve in blocks (front_blocked) do when they hold this many
+// entries of A21 right of their first 32 columns together; fewer finish sooner in one
+// pass, which is three launches shorter (64 uneven fronts, the class that finishes
+// last: 30 us / 63).
 constexpr double kBlockedEntries = 3e5;
 constexpr unsigned long long kAbsMask = 0x7FFFFFFFFFFFFFFFull;
 
@@ -44,11 +44,7 @@ __global__ void k_batch_prepare(const BFront *__restrict__ tab, char *ws, BatchO
     const int f = blockIdx.x;
     if (f == 0 && threadIdx.x == 0) *ginfo = 0;
     const BFront bt = tab[f];
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    const BSection sec = bsection(bt.n, bt.p, &oo);
+    const BSection sec = bsection(bt.n, bt.p, o);
     char *base = ws + bt.ws;
     if (threadIdx.x == 0) *reinterpret_cast<int32_t *>(base + sec.info) = 0;
     if (o.pivot == CTP_PIV_STRICT) {
@@ -90,11 +86,7 @@ __global__ void __launch_bounds__(kThreads, KPL <= 2 ? 6 : (KPL == 4 ? 4 : 3))
     const int f = item_front[item];
     const BFront bt = tab[f];
     const ctp_front fr = fronts[f];
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    const BSection sec = bsection(bt.n, bt.p, &oo);
+    const BSection sec = bsection(bt.n, bt.p, o);
     char *base = ws + bt.ws;
     unsigned long long *Ckeys = reinterpret_cast<unsigned long long *>(base + sec.C);
     const int p = bt.p;
@@ -175,11 +167,7 @@ __global__ void k_batch_flags(const BFront *__restrict__ tab, const char *ws, Ba
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= nb) return;
     const BFront bt = tab[f];
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    const BSection sec = bsection(bt.n, bt.p, &oo);
+    const BSection sec = bsection(bt.n, bt.p, o);
     const int32_t v = *reinterpret_cast<const int32_t *>(ws + bt.ws + sec.info);
     flags[f] = v != kInfoOk ? v : *ginfo;
 }
@@ -234,9 +222,12 @@ struct ctp_plan {
         int pcap, ldcap;     // warp kernel: largest p and p + R of the class
         size_t list_off;     // element offset in the class-list array
         int pmax;            // largest p of the class
-        int64_t s_off, s_count;  // the class's Solve items (front, tile) in the class Solve lists
-        int s_rows;              // rows per tile
-        int64_t u_off, u_count;  // blocked Solve: the class's update items (none: a whole pass per tile)
+        struct Items {
+            int64_t off, count;  // Solve items (front, tile) in the class Solve lists
+            int rows;            // rows per tile
+            bool plain;          // no slices are written
+        } whole, blocked;        // of the fronts that solve in one pass, and in blocks
+        int64_t u_off, u_count;  // blocked Solves: the class's update items
         int64_t f_off, f_count;  // the class's Form items (front, tile) in the class Form lists
         int64_t m_off, m_count;  // the class's fronts whose FP64 Form has few rows
     };
@@ -356,6 +347,7 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     P->bo.pivot = opt->pivot;
     P->bo.smode = opt->smode;
     P->bo.prec = opt->prec;
+    P->bo.stc = stc ? 1 : 0;
     P->tc = tc;
     P->pmax = 1;
     std::vector<BFront> tab(nb);
@@ -369,7 +361,7 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
         b.m = b.n - b.p;
         b.nM = (int)((b.m + 127) / 128);
         b.ws = (int64_t)sec_off;
-        sec_off += bsection(b.n, b.p, opt).total;
+        sec_off += bsection(b.n, b.p, P->bo).total;
         b.row0 = row0;
         if (tc) row0 += (b.m + 255) / 256 * 256;
         const int64_t nt = (b.m + kTR - 1) / kTR;
@@ -449,28 +441,43 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
         if (byKey[key].empty()) continue;
         ctp_plan::Class c;
         c.pmax = pmaxK[key];
-        // the class's Solve is blocked (three more launches, one more pass over its
-        // rows) when its fronts hold enough entries of A21 right of the first block
-        c.u_off = (int64_t)cuitem.size();
+        // the fronts that solve in blocks (three more launches for the class, one more pass over
+        // their rows)
         double right = 0.0;
-        for (int f : byKey[key]) right += tab[f].p > kSliceK ? (double)tab[f].m * (tab[f].p - kSliceK) : 0.0;
-        if (!stc && right >= kBlockedEntries)
-            for (int f : byKey[key])
+        for (int f : byKey[key])
+            if (!stc && front_blocked(tab[f].m, tab[f].p, P->bo)) right += (double)tab[f].m * (tab[f].p - kSliceK);
+        auto in_blocks = [&](int f) { return right >= kBlockedEntries && front_blocked(tab[f].m, tab[f].p, P->bo); };
+        c.u_off = (int64_t)cuitem.size();
+        for (int f : byKey[key])
+            if (in_blocks(f))
                 for (int64_t t = 0; t < update_tiles(tab[f].m, tab[f].p); t++) {
                     cuitem.push_back(f);
                     cutile.push_back((int)t);
                 }
         c.u_count = (int64_t)cuitem.size() - c.u_off;
-        int64_t tiles = 0;
-        for (int f : byKey[key]) tiles += (tab[f].m + 31) / 32;
-        c.s_rows = solve_rows(tiles, c.u_count > 0, ctx_num_sms(ctx));
-        c.s_off = (int64_t)csitem.size();
-        for (int f : byKey[key])
-            for (int64_t t = 0; t < (tab[f].m + c.s_rows - 1) / c.s_rows; t++) {
-                csitem.push_back(f);
-                cstile.push_back((int)t);
+        auto items = [&](bool blocked) {
+            ctp_plan::Class::Items it = {(int64_t)csitem.size(), 0, 0, !blocked};
+            int64_t tiles = 0;
+            for (int pass = 0; pass < 2; pass++) {
+                for (int f : byKey[key]) {
+                    if (in_blocks(f) != blocked) continue;
+                    if (pass == 0) {
+                        tiles += (tab[f].m + 31) / 32;
+                        if (opt->smode != CTP_S_NONE && !tc && !form_small(tab[f].m)) it.plain = false;
+                        continue;
+                    }
+                    for (int64_t t = 0; t < (tab[f].m + it.rows - 1) / it.rows; t++) {
+                        csitem.push_back(f);
+                        cstile.push_back((int)t);
+                    }
+                }
+                it.rows = solve_rows(tiles, blocked, ctx_num_sms(ctx));
             }
-        c.s_count = (int64_t)csitem.size() - c.s_off;
+            it.count = (int64_t)csitem.size() - it.off;
+            return it;
+        };
+        c.whole = items(false);
+        c.blocked = items(true);
         c.f_off = (int64_t)cfitem.size();
         if (opt->smode != CTP_S_NONE)
             for (int f : byKey[key]) {
@@ -551,7 +558,6 @@ ctp_status ctp_batch_plan_create(ctp_ctx *ctx, int32_t nb, const int64_t *n_host
     P->bo.lo_off = pieces > 1 ? row0 * kBatchKp : 0;
     P->bo.pieces = pieces;
     // tensor-core Solve: x_e and Z^T tiles, three pieces each
-    P->bo.stc = stc ? 1 : 0;
     P->bo.xoff = (int64_t)xt * (int64_t)solve_tc_tile_elems();
     P->bo.zoff = (int64_t)zt * (int64_t)solve_tc_tile_elems();
     P->off_xt = off;
@@ -666,21 +672,19 @@ bool batch_solve_per_class(const ctp_plan *P) { return !P->bo.stc; }
 cudaError_t batch_solve_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, int num_sms,
                               cudaStream_t st) {
     const ctp_plan::Class &c = P->classes[ci];
-    if (c.u_count > 0)
-        return launch_solve_batch_blocked(
-            fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
-            reinterpret_cast<const int *>(w + P->off_lists) + c.list_off, c.count,
-            reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off,
-            reinterpret_cast<const int *>(w + P->off_cstile) + c.s_off, c.s_count, c.s_rows,
-            reinterpret_cast<const int *>(w + P->off_cuitem) + c.u_off,
-            reinterpret_cast<const int *>(w + P->off_cutile) + c.u_off, c.u_count, P->bo,
-            P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax,
-            reinterpret_cast<TileMarks *>(w + P->off_umarks) + c.u_off, reinterpret_cast<int32_t *>(w + P->off_ginfo),
-            num_sms, st);
-    return launch_solve_batch(fr, reinterpret_cast<const BFront *>(w + P->off_tab), w,
-                              reinterpret_cast<const int *>(w + P->off_csitem) + c.s_off, c.s_count, c.s_rows, P->bo,
-                              P->tc ? w + P->off_wb : nullptr, P->tc ? w + P->off_lb : nullptr, c.pmax, st,
-                              reinterpret_cast<const int *>(w + P->off_cstile) + c.s_off);
+    void *Wb = P->tc ? w + P->off_wb : nullptr, *Lb = P->tc ? w + P->off_lb : nullptr;
+    const BFront *tab = reinterpret_cast<const BFront *>(w + P->off_tab);
+    const int *item = reinterpret_cast<const int *>(w + P->off_csitem);
+    const int *tile = reinterpret_cast<const int *>(w + P->off_cstile);
+    cudaError_t e = launch_solve_batch(fr, tab, w, item + c.whole.off, c.whole.count, c.whole.rows, c.whole.plain, P->bo,
+                                       Wb, Lb, c.pmax, st, tile + c.whole.off);
+    if (e != cudaSuccess || c.blocked.count == 0) return e;
+    return launch_solve_batch_blocked(fr, tab, w, reinterpret_cast<const int *>(w + P->off_lists) + c.list_off, c.count,
+                                      item + c.blocked.off, tile + c.blocked.off, c.blocked.count, c.blocked.rows,
+                                      reinterpret_cast<const int *>(w + P->off_cuitem) + c.u_off,
+                                      reinterpret_cast<const int *>(w + P->off_cutile) + c.u_off, c.u_count, P->bo, Wb, Lb,
+                                      c.pmax, reinterpret_cast<TileMarks *>(w + P->off_umarks) + c.u_off,
+                                      reinterpret_cast<int32_t *>(w + P->off_ginfo), num_sms, st);
 }
 // The Form of one pivot-search class's fronts (after that class's Solve)
 cudaError_t batch_form_class(const ctp_plan *P, int ci, const ctp_front *fr, char *w, int num_sms,

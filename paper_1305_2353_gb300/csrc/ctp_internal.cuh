@@ -146,6 +146,28 @@ struct BFront {
     int64_t xt0, zt0, q0, r0;  // r0: first prep item (8 identity rows each)
     int32_t kbx, nwz;
 };
+struct BatchOpts {
+    double u, small;
+    int pivot;  // ctp_pivot
+    int smode, prec;
+    int64_t lo_off;  // elements between the BF16 pieces of the operand copies
+    int pieces;      // BF16 pieces per operand (1: plain; 2, 3: split)
+    int stc;         // the Solve runs on the tensor cores
+    int64_t xoff, zoff;  // elements between the pieces of the x_e / Z^T tile arrays
+};
+
+// Whether a front of a batch may solve for its rows in blocks (solve.cu): one block of 32
+// columns, the tensor cores' update of the others and the rest.  Measured, all Solves of
+// batches of equal fronts, one pass / in blocks, m x p.  Strict pivoting, a dozen
+// accepted: 60 x 96 430 / 518 us, 200 x 96 504 / 424, 60 x 128 512 / 618, 200 x 128 589 / 439,
+// 60 x 200 553 / 635, 60 x 256 612 / 600, 800 x 256 565 / 324; 200 x 64 475 / 563, 800 x 64
+// 485 / 440, 2400 x 64 385 / 393.  All accepted: 60 x 64 1396 / 1316, 60 x 96 1989 / 1612,
+// 800 x 200 3767 / 3187; 200 x 48 1143 / 1230, 800 x 48 1020 / 983.
+__host__ __device__ inline bool front_blocked(int64_t m, int p, const BatchOpts &o) {
+    const int64_t right = m * (p - kSliceK);  // entries that the update touches
+    return o.pivot == CTP_PIV_STRICT ? p > 56 && right >= 12000 : p > 48 && right >= 1900;
+}
+
 // offsets inside a front's section: info word, compressed matrix (strict),
 // Dinv, and when an FP64 Form follows W21 = L21 D11 (few rows) or the digit slices of
 // W21 and L21
@@ -153,18 +175,18 @@ struct BSection {
     size_t info, C, Dinv, W21, Ws, Ls, ew, el, gw, gl, Yb, Lx, ey, ex, gy, gx, nz, total;
 };
 __host__ __device__ inline size_t align256hd(size_t x) { return (x + 255) & ~size_t(255); }
-__host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options *opt) {
+__host__ __device__ inline BSection bsection(int64_t n, int p, const BatchOpts &o) {
     BSection s;
     size_t off = 0;
     s.info = off;
     off += 256;
     s.C = off;
-    off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(double) * (size_t)p * p : 0);
+    off += align256hd(o.pivot == CTP_PIV_STRICT ? sizeof(double) * (size_t)p * p : 0);
     s.Dinv = off;
     off += align256hd(sizeof(double) * (2 * (size_t)p + 2));
     s.nz = off;  // strict: which rows of C receive an A21 row (one bit per row)
-    off += align256hd(opt->pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
-    const int64_t mf = opt->smode != CTP_S_NONE && opt->prec == CTP_FP64 ? n - p : 0;
+    off += align256hd(o.pivot == CTP_PIV_STRICT ? sizeof(int32_t) * (size_t)p : 0);
+    const int64_t mf = o.smode != CTP_S_NONE && o.prec == CTP_FP64 ? n - p : 0;
     const int64_t ms = form_small(mf) ? 0 : mf;
     s.W21 = off;
     off += align256hd(sizeof(double) * (size_t)(mf - ms) * p);
@@ -180,20 +202,23 @@ __host__ __device__ inline BSection bsection(int64_t n, int p, const ctp_options
     off += align256hd(slice_g_bytes(ms, p));
     s.gl = off;
     off += align256hd(slice_g_bytes(ms, p));
-    // the blocked Solve's first block: slices of y and of L11's rows below it
-    const int64_t mb = p > kSliceK ? n - p : 0;
-    s.Yb = off;
+    // the blocked Solve's first block: slices of y (where those of W21 come later, if there
+    // are any) and of L11's rows below it
+    const bool blk = !o.stc && front_blocked(n - p, p, o);
+    const int64_t mb = blk && ms == 0 ? n - p : 0;
+    const int pb = blk ? p - kSliceK : 0;
+    s.Yb = blk && ms > 0 ? s.Ws : off;
     off += align256hd(slice_bytes(mb, kSliceK));
-    s.Lx = off;
-    off += align256hd(mb > 0 ? slice_bytes(p, kSliceK) : 0);
-    s.ey = off;
+    s.ey = blk && ms > 0 ? s.ew : off;
     off += align256hd(sizeof(int32_t) * (size_t)mb);
-    s.ex = off;
-    off += align256hd(mb > 0 ? sizeof(int32_t) * (size_t)p : 0);
-    s.gy = off;
+    s.gy = blk && ms > 0 ? s.gw : off;
     off += align256hd(slice_g_bytes(mb, kSliceK));
+    s.Lx = off;
+    off += align256hd(slice_bytes(pb, kSliceK));
+    s.ex = off;
+    off += align256hd(sizeof(int32_t) * (size_t)pb);
     s.gx = off;
-    off += align256hd(mb > 0 ? slice_g_bytes(p, kSliceK) : 0);
+    off += align256hd(slice_g_bytes(pb, kSliceK));
     s.total = off;
     return s;
 }
@@ -222,15 +247,6 @@ __host__ __device__ inline SliceBuf bsection_block(char *base, const BSection &s
     return b;
 }
 
-struct BatchOpts {
-    double u, small;
-    int pivot;  // ctp_pivot
-    int smode, prec;
-    int64_t lo_off;  // elements between the BF16 pieces of the operand copies
-    int pieces;      // BF16 pieces per operand (1: plain; 2, 3: split)
-    int stc;         // the Solve runs on the tensor cores
-    int64_t xoff, zoff;  // elements between the pieces of the x_e / Z^T tile arrays
-};
 // pivot search of the fronts list[0..count) of one class: kind (kFactor*), the
 // cluster width G, the dynamic shared memory per CTA, and for the warp kernel
 // the largest p and p + R of the class (its per-warp slice)
@@ -241,9 +257,9 @@ cudaError_t launch_factor_batch(const ctp_front *fronts, const BFront *tab, char
 cudaError_t launch_compress_strict_batch(const ctp_front *fronts, const BFront *tab, char *ws,
                                          const int *item_front, const int64_t (&bucket)[5], BatchOpts o,
                                          cudaStream_t st);
-// items: (front, 32-row tile) pairs
+// items: (front, tile) pairs; plain: no slices are written
 cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                               const int *item_front, int64_t items, int rows, BatchOpts o, void *Wb, void *Lb,
+                               const int *item_front, int64_t items, int rows, bool plain, BatchOpts o, void *Wb, void *Lb,
                                int pmax, cudaStream_t st, const int *item_tile);
 // rows per tile (32, 16 or 8) of a Solve with this many 32-row tiles
 int solve_rows(int64_t tiles, bool blocked, int num_sms);

@@ -736,11 +736,7 @@ __device__ __forceinline__ FactorArgs batch_args(const ctp_front *__restrict__ f
                                                  const BatchOpts &o) {
     const ctp_front fr = fronts[f];
     const BFront bt = tab[f];
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    const BSection sec = bsection(bt.n, bt.p, &oo);
+    const BSection sec = bsection(bt.n, bt.p, o);
     char *base = ws + bt.ws;
     FactorArgs a;
     a.A = fr.A;

@@ -73,13 +73,17 @@ struct Tile {
     void *S;
 };
 
-constexpr int kRing = 4;
+constexpr int kRing = 4, kList = 256, kKept = 16;
 struct Bars {
     unsigned long long full[kStages], empty[kStages], acc_full, acc_empty, grp_full, tile_full[kRing], tile_empty[kRing];
     Tile tile[kRing];
-    int64_t marked;                 // the last tile of that list, -1: none
+    int64_t list[kList];            // those tiles,
+    Tile kept[kKept];               // the first of them as they were looked up,
+    int64_t marked;                 // and the last that found no room there, -1: none
+    int nlist, next;
     uint32_t unsure[2][kEpiWarps];  // by turns: blocks that digits may not serve,
     int linked[2];                  // the tile is in the list of those with entries left out
+    int weak;                       // some entry was left out
     int nmarks;
     uint32_t tmem_base;
     int abort;
@@ -183,11 +187,7 @@ struct Walk {
             const BFront b = w.tab[f];
             const ctp_front &fr = w.fronts[f];
             q = w.item_tile != nullptr ? (int64_t)w.item_tile[t] : t - b.f0;
-            ctp_options oo;
-            oo.pivot = w.o.pivot;
-            oo.smode = w.o.smode;
-            oo.prec = w.o.prec;
-            const BSection sec = bsection(b.n, b.p, &oo);
+            const BSection sec = bsection(b.n, b.p, w.o);
             x.sb = kUpd ? bsection_block(w.ws + b.ws, sec) : bsection_slices(w.ws + b.ws, sec, b.p);
             x.m = (int)b.m;
             x.nc = kUpd ? b.p - w.c0 : x.m;
@@ -404,103 +404,191 @@ struct FormOut {
 // 2^(40 + weight) is the weight of g = 0: as large as the 64 bits allow for e pivots
 __device__ __forceinline__ int weight(int e) { return e <= 16 ? 6 : (e <= 32 ? 5 : (e <= 64 ? 4 : (e <= 128 ? 3 : 2))); }
 
-// The entries that digits do not serve, after the CTA's last tile: by FP64 multiply-adds,
-// tile by tile (all threads, four columns of a row each, or up to four times that
-// where a tile has many; 32 pivots of W21 and L21 at a time in shared memory).  Sparse
-// rows leave a few entries of a tile out; a tile with all of them left out takes what
-// FP64's pipe takes for it.
-constexpr int kFixW = kBM + 1, kFixL = kBN + 1;  // padded rows of the slabs
+// One pivot's entry of W21 (kUpd: of y) in row i, of kind kd, from L21 and D.
+template <bool kUpd>
+__device__ __forceinline__ double w21_entry(const Tile &x, int k, int kd, int i) {
+    if (kd == CTP_PIVKIND_ZERO) return 0.0;
+    const double *c = x.L21 + (int64_t)k * x.ldl + i;
+    double w = *c;  // kUpd: y itself, in the block's columns of A21
+    if (!kUpd) {
+        w *= x.D[2 * k];
+        if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(c[x.ldl], x.D[2 * k + 1], w);
+        if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(c[-x.ldl], x.D[2 * k - 1], w);
+    }
+    return w;
+}
+// The same of L21 in row j (kUpd: of the rows c0.. of L11).
+template <bool kUpd>
+__device__ __forceinline__ double l21_entry(const Tile &x, int k, int kd, int64_t j) {
+    const bool d21 = kUpd && x.c0 + j == k + 1 && kd == CTP_PIVKIND_2X2_FIRST;  // that slot holds D
+    if (kd == CTP_PIVKIND_ZERO || d21 || j >= x.nc) return 0.0;
+    return x.L21[(kUpd ? -(int64_t)x.nc : 0) + (int64_t)k * x.ldl + j];
+}
 template <int kMode>
-__device__ __noinline__ void fix_tiles(const Work &wk, Bars &bars, uint8_t *smem) {
+__device__ __forceinline__ void put_entry(const Tile &x, int i, int64_t j, double v) {
     typedef typename FormOut<kMode>::T OutT;
-    constexpr bool kPacked = FormOut<kMode>::kPacked, kUpd = kMode == kUpdate, kSub = FormOut<kMode>::kSub;
-    constexpr int kItems = (kBM * kBN / 4 + kThreads - 1) / kThreads;
-    double *ws = reinterpret_cast<double *>(smem), *ls = ws + kSliceK * kFixW;
-    uint16_t *ids = reinterpret_cast<uint16_t *>(ls + kSliceK * kFixL);
-    const Tile &x = bars.tile[0];
-    for (int64_t t = bars.marked; t >= 0; t = wk.marks[t].prev) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
+    OutT *ptr = reinterpret_cast<OutT *>(x.S) +
+                (FormOut<kMode>::kPacked ? j * x.m - j * (j + 1) / 2 : j * x.lds) + i;
+    *ptr = FormOut<kMode>::kSub ? (OutT)(*ptr - v) : (OutT)v;
+}
+
+// The entries that digits do not serve, after the CTA's last tile, by FP64 multiply-adds in
+// the order of the pivots.  Most tiles with any have a few (with two or three pivots
+// one entry in 10^4 of random rows is one, and a tile has 8192): a warp takes such a
+// tile, a lane an entry, and the CTA's warps hide each other's latency (4 us a tile).  A
+// tile with many is taken by all threads, four columns of a row each, or up to four
+// times that, 32 pivots of W21 and L21 at a time in shared memory; one with all of
+// them left out takes what FP64's pipe takes for it.
+constexpr int kFew = 32;  // entries of a tile that a warp takes
+template <int kMode>
+__device__ __forceinline__ void fix_few(const Work &wk, Bars &bars, uint8_t *smem) {
+    constexpr bool kUpd = kMode == kUpdate;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = bars.nlist;
+    uint16_t *ids = reinterpret_cast<uint16_t *>(smem) + warp * kFew;
+    Tile &x = reinterpret_cast<Tile *>(smem + kThreads / 32 * kFew * sizeof(uint16_t))[warp];
+    for (;;) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&bars.next, 1);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at >= n) break;
+        const int64_t t = bars.list[at];
+        unsigned mask[kEpiWarps];
+        int cnt = 0;
+#pragma unroll
+        for (int b = 0; b < kEpiWarps; b++) mask[b] = wk.marks[t].out[b][lane];
+#pragma unroll
+        for (int b = 0; b < kEpiWarps; b++) cnt += __popc(mask[b]);
+        int pos = cnt;  // inclusive prefix sum
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, pos, 31);
+        if (total > kFew) continue;  // left in the list
+        if (lane == 0) bars.list[at] = -1;
+        if (total == 0) continue;
+        pos -= cnt;
+#pragma unroll
+        for (int b = 0; b < kEpiWarps; b++)
+            for (unsigned w = mask[b]; w; w &= w - 1)
+                ids[pos++] = (uint16_t)(((b >> 2) * 32 + lane) * kBN + (b & 3) * kCols + __ffs(w) - 1);
+        if (lane == 0 && at < kKept) x = bars.kept[at];
+        if (lane == 0 && at >= kKept) {
             Walk<kUpd> walk(wk);
             Tile y;
             walk.seek(t);
             walk.look(y);
-            bars.tile[0] = y;
-            bars.nmarks = 0;
+            x = y;
+        }
+        __syncwarp();
+        const int first = kUpd ? x.c0 - kSliceK : 0, e = x.e;
+        for (int q0 = lane; q0 < total; q0 += 32) {
+            const int i = x.ti * kBM + ids[q0] / kBN;
+            const int64_t j = x.tj * kBN + ids[q0] % kBN;
+            double acc = 0.0;
+            for (int k0 = 0; k0 < e; k0 += 8) {
+                double w[8], l[8];
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const int kd = k0 + q < e ? x.piv[first + k0 + q] : CTP_PIVKIND_ZERO;
+                    w[q] = w21_entry<kUpd>(x, first + k0 + q, kd, i);
+                    l[q] = l21_entry<kUpd>(x, first + k0 + q, kd, j);
+                }
+#pragma unroll
+                for (int q = 0; q < 8; q++) acc = fma(w[q], l[q], acc);
+            }
+            put_entry<kMode>(x, i, j, acc);
+        }
+        __syncwarp();
+    }
+}
+
+constexpr int kFixW = kBM + 1, kFixL = kBN + 1;  // padded rows of the slabs
+template <int kMode>
+__device__ __forceinline__ void fix_tile(const Work &wk, Bars &bars, uint8_t *smem, int64_t t) {
+    constexpr bool kUpd = kMode == kUpdate;
+    constexpr int kItems = (kBM * kBN / 4 + kThreads - 1) / kThreads;
+    double *ws = reinterpret_cast<double *>(smem), *ls = ws + kSliceK * kFixW;
+    uint16_t *ids = reinterpret_cast<uint16_t *>(ls + kSliceK * kFixL);
+    const Tile &x = bars.tile[0];
+    const int lane = threadIdx.x & 31;
+    // a thread holds a row's sixteen columns
+    const unsigned mask = threadIdx.x < kBM * kBN / kCols ? wk.marks[t].out[threadIdx.x >> 5][lane] : 0u;
+    if (!__syncthreads_or(mask != 0u)) return;  // its own results served after all
+    if (threadIdx.x == 0) {
+        Walk<kUpd> walk(wk);
+        Tile y;
+        walk.seek(t);
+        walk.look(y);
+        bars.tile[0] = y;
+        bars.nmarks = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x < kBM * kBN / kCols) {  // which fours of columns have any
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const unsigned has = __ballot_sync(0xffffffffu, (mask >> (4 * c)) & 0xFu);
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&bars.nmarks, __popc(has));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(has & ((1u << lane) - 1u));
+            if ((has >> lane) & 1u) ids[at] = (uint16_t)(threadIdx.x * 4 + c);
+        }
+    }
+    __syncthreads();
+    const int n = bars.nmarks;
+    double acc[kItems][4] = {};
+    int row[kItems], col[kItems];
+#pragma unroll
+    for (int it = 0; it < kItems; it++) {
+        const int q = threadIdx.x + it * kThreads, id = q < n ? ids[q] : 0;  // warp's block, lane, four
+        row[it] = (id >> 9) * 32 + ((id >> 2) & 31);
+        col[it] = ((id >> 7) & 3) * kCols + (id & 3) * 4;
+    }
+    const int i0 = x.ti * kBM, j0 = x.tj * kBN, first = kUpd ? x.c0 - kSliceK : 0;
+    for (int k0 = 0; k0 < x.e; k0 += kSliceK) {
+        const int cnt = min(kSliceK, x.e - k0);
+        for (int idx = threadIdx.x; idx < cnt * kBM; idx += kThreads) {
+            const int k = first + k0 + idx / kBM, r = idx % kBM, kd = x.piv[k];
+            ws[idx / kBM * kFixW + r] = i0 + r < x.m ? w21_entry<kUpd>(x, k, kd, i0 + r) : 0.0;
+        }
+        for (int idx = threadIdx.x; idx < cnt * kBN; idx += kThreads) {
+            const int k = first + k0 + idx / kBN, c = idx % kBN, kd = x.piv[k];
+            ls[idx / kBN * kFixL + c] = l21_entry<kUpd>(x, k, kd, j0 + c);
         }
         __syncthreads();
-        const int lane = threadIdx.x & 31;
-        if (threadIdx.x < kBM * kBN / kCols) {  // a row's sixteen columns: which fours have any
-            const unsigned mask = wk.marks[t].out[threadIdx.x >> 5][lane];
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const unsigned has = __ballot_sync(0xffffffffu, (mask >> (4 * c)) & 0xFu);
-                int at = 0;
-                if (lane == 0) at = atomicAdd(&bars.nmarks, __popc(has));
-                at = __shfl_sync(0xffffffffu, at, 0) + __popc(has & ((1u << lane) - 1u));
-                if ((has >> lane) & 1u) ids[at] = (uint16_t)(threadIdx.x * 4 + c);
-            }
-        }
-        __syncthreads();
-        const int n = bars.nmarks;
-        double acc[kItems][4] = {};
-        int row[kItems], col[kItems];
-#pragma unroll
-        for (int it = 0; it < kItems; it++) {
-            const int q = threadIdx.x + it * kThreads, id = q < n ? ids[q] : 0;  // warp's block, lane, four
-            row[it] = (id >> 9) * 32 + ((id >> 2) & 31);
-            col[it] = ((id >> 7) & 3) * kCols + (id & 3) * 4;
-        }
-        const int i0 = x.ti * kBM, j0 = x.tj * kBN, first = kUpd ? x.c0 - kSliceK : 0;
-        const double *rows = kUpd ? x.L21 - x.nc : x.L21;  // kUpd: rows c0.. of L11
-        for (int k0 = 0; k0 < x.e; k0 += kSliceK) {
-            const int cnt = min(kSliceK, x.e - k0);
-            for (int idx = threadIdx.x; idx < cnt * kBM; idx += kThreads) {
-                const int k = first + k0 + idx / kBM, r = idx % kBM, kd = x.piv[k];
-                double w = 0.0;
-                if (i0 + r < x.m && kd != CTP_PIVKIND_ZERO) {
-                    const double *c = x.L21 + (int64_t)k * x.ldl + i0 + r;
-                    w = *c;  // kUpd: y itself, in the block's columns of A21
-                    if (!kUpd) {
-                        w *= x.D[2 * k];
-                        if (kd == CTP_PIVKIND_2X2_FIRST) w = fma(c[x.ldl], x.D[2 * k + 1], w);
-                        if (kd == CTP_PIVKIND_2X2_SECOND) w = fma(c[-x.ldl], x.D[2 * k - 1], w);
-                    }
-                }
-                ws[idx / kBM * kFixW + r] = w;
-            }
-            for (int idx = threadIdx.x; idx < cnt * kBN; idx += kThreads) {
-                const int k = first + k0 + idx / kBN, c = idx % kBN, kd = x.piv[k];
-                const bool d21 = kUpd && x.c0 + j0 + c == k + 1 && kd == CTP_PIVKIND_2X2_FIRST;  // that slot holds D
-                ls[idx / kBN * kFixL + c] =
-                    kd != CTP_PIVKIND_ZERO && j0 + c < x.nc && !d21 ? rows[(int64_t)k * x.ldl + j0 + c] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int it = 0; it < kItems; it++) {
-                if (threadIdx.x + it * kThreads >= n) break;
-                for (int k = 0; k < cnt; k++) {
-                    const double w = ws[k * kFixW + row[it]];
-#pragma unroll
-                    for (int c = 0; c < 4; c++) acc[it][c] = fma(w, ls[k * kFixL + col[it] + c], acc[it][c]);
-                }
-            }
-            __syncthreads();
-        }
 #pragma unroll
         for (int it = 0; it < kItems; it++) {
             if (threadIdx.x + it * kThreads >= n) break;
-            const int i = i0 + row[it];
-            const unsigned mask = wk.marks[t].out[row[it] / 32 * 4 + col[it] / kCols][row[it] % 32] >> (col[it] % kCols);
+            for (int k = 0; k < cnt; k++) {
+                const double w = ws[k * kFixW + row[it]];
 #pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const int64_t j = j0 + col[it] + c;
-                if (!((mask >> c) & 1u)) continue;
-                OutT *ptr = reinterpret_cast<OutT *>(x.S) + (kPacked ? j * x.m - j * (j + 1) / 2 : j * x.lds) + i;
-                *ptr = kSub ? (OutT)(*ptr - acc[it][c]) : (OutT)acc[it][c];
+                for (int c = 0; c < 4; c++) acc[it][c] = fma(w, ls[k * kFixL + col[it] + c], acc[it][c]);
             }
         }
+        __syncthreads();
     }
+#pragma unroll
+    for (int it = 0; it < kItems; it++) {
+        if (threadIdx.x + it * kThreads >= n) break;
+        const int i = i0 + row[it];
+        const unsigned mask = wk.marks[t].out[row[it] / 32 * 4 + col[it] / kCols][row[it] % 32] >> (col[it] % kCols);
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int64_t j = j0 + col[it] + c;
+            if (!((mask >> c) & 1u)) continue;
+            put_entry<kMode>(x, i, j, acc[it][c]);
+        }
+    }
+}
+
+template <int kMode>
+__device__ __noinline__ void fix_tiles(const Work &wk, Bars &bars, uint8_t *smem) {
+    fix_few<kMode>(wk, bars, smem);
+    __syncthreads();
+    for (int q = 0; q < bars.nlist; q++)
+        if (bars.list[q] >= 0) fix_tile<kMode>(wk, bars, smem, bars.list[q]);
+    for (int64_t t = bars.marked; t >= 0; t = wk.marks[t].prev) fix_tile<kMode>(wk, bars, smem, t);
 }
 
 template <int kMode>
@@ -524,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
             mbar_init(&bars.tile_empty[s], 3 + kEpiWarps);
         }
         bars.abort = 0;
-        bars.marked = -1;
+        bars.weak = bars.next = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(&bars.tmem_base, 512);
@@ -556,6 +644,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
         uint32_t accphase = 0, grpphase = 0;
         bool ok, first = true;
         int64_t marked = -1;
+        int nlist = 0;
         while ((ok = ring.wait(bars))) {
             const Tile &x = bars.tile[ring.slot];
             if (x.ti < 0) break;
@@ -605,7 +694,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                 bits <<= 16 * ((lane >> 2) & 1);
                 bits |= __shfl_xor_sync(0xffffffffu, bits, 4);
                 linked = __any_sync(0xffffffffu, bits) || nonfinite;
-                if (linked) {
+                if (linked && nlist < kList) {
+                    if (lane == 0) bars.list[nlist] = x.t;
+                    if (lane == 0 && nlist < kKept) bars.kept[nlist] = x;
+                    nlist++;
+                } else if (linked) {
                     if (lane == 0) wk.marks[x.t].prev = marked;
                     marked = x.t;
                 }
@@ -627,6 +720,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
         }
         if (lane == 0) {
             bars.marked = marked;
+            bars.nlist = nlist;
             if (!ok) atomicExch(&bars.abort, 1);
         }
     } else if (warp == 0) {
@@ -846,14 +940,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                     }
                 }
             }
-            if (linked) wk.marks[x.t].out[q * 4 + cg][lane] = (uint16_t)weak;
+            if (linked) {
+                wk.marks[x.t].out[q * 4 + cg][lane] = (uint16_t)weak;
+                if (weak) bars.weak = 1;
+            }
             __syncwarp();
             if (lane == 0) ring.release(bars);
         }
     }
     __syncthreads();
     if (threadIdx.x == 0 && bars.abort) atomicCAS(info, kInfoOk, (int32_t)CTP_ETIMEOUT);
-    if (bars.marked >= 0 && !bars.abort) fix_tiles<kMode>(wk, bars, smem);
+    if (bars.weak && !bars.abort) fix_tiles<kMode>(wk, bars, smem);
     __syncwarp();
     if (warp == 0) {
         tc_fence_after();
@@ -886,11 +983,7 @@ __global__ void __launch_bounds__(kSmallT) k_form_small(const __grid_constant__ 
         lds = fr.lds;
         S = reinterpret_cast<OutT *>(fr.S);
         nelim = fr.nelim;
-        ctp_options oo;
-        oo.pivot = wk.o.pivot;
-        oo.smode = wk.o.smode;
-        oo.prec = wk.o.prec;
-        W21 = reinterpret_cast<const double *>(wk.ws + b.ws + bsection(b.n, b.p, &oo).W21);
+        W21 = reinterpret_cast<const double *>(wk.ws + b.ws + bsection(b.n, b.p, wk.o).W21);
     }
     const int e = *nelim, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // entries of the lower triangle, column by column

@@ -92,22 +92,25 @@ struct SolvePass {
 // memory without a register copy, so that a CTA needs few
 // registers and as many CTAs fit on an SM as its shared memory allows (three at
 // p = 256, more for narrower fronts): enough warps for all four FP64 pipes.
-// One tile of RT rows: 32, a lane per row, or fewer, with the lanes of a warp on several
+// kPlain: a whole pass that writes no slices, in 40 registers without a spill (20000 fronts
+// of 24 x 8: 145 -> 125 us).  One tile of RT rows: 32, a lane per row, or fewer, with the lanes of a warp on several
 // columns (small supernodes, so that more SMs have a tile).  brow0: row of this front's first A21 row in the BF16
 // operand copies (0 for a single supernode; the stacked offset in a batch).
 // pieces > 1: also write the further BF16 pieces of the split operands (piece
 // k rounds what pieces 0..k-1 left), lo_off elements apart.  sb: the slices of
 // the FP64 Form (sb.W null: none).
-template <int RT>
-__device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
+template <int RT, bool kPlain>
+__device__ __forceinline__ void solve_tile(const SolvePass &ps_, double *__restrict__ A, int64_t n, int p, int64_t lda,
                                            const int32_t *__restrict__ perm,
                                            const int32_t *__restrict__ piv,
                                            const double *__restrict__ Dinv, int e, double *__restrict__ W21,
-                                           const SliceBuf &sb,
+                                           const SliceBuf &sb_,
                                            __nv_bfloat16 *__restrict__ Wb,
                                            __nv_bfloat16 *__restrict__ Lb, int Kp, int64_t brow0,
                                            int64_t lo_off, int pieces, int64_t tile, double *xs) {
     constexpr int LDX = kRows + 1, SUB = kRows / RT, CW = kWarps * SUB;
+    const SolvePass ps = kPlain ? SolvePass{kWhole, 0, {}} : ps_;
+    const SliceBuf sb = kPlain ? SliceBuf{} : sb_;
     const int64_t m = n - p;
     const int64_t row0 = tile * RT;
     const int r = (threadIdx.x & 31) % RT, w = (threadIdx.x >> 5) * SUB + (threadIdx.x & 31) / RT;
@@ -223,7 +226,7 @@ __device__ __forceinline__ void solve_tile(const SolvePass &ps, double *__restri
     if (Lb != nullptr) write_pieces(Lb, brow0 + row0, tile_rows, Kp, e, Kz, pieces, lo_off, xs);
 }
 
-template <int RT>
+template <int RT, bool kPlain>
 __global__ void __launch_bounds__(kRows * kWarps, 6)
     k_solve_fp64(SolvePass ps, double *__restrict__ A, int64_t n, int p, int64_t lda,
                  const int32_t *__restrict__ perm, const int32_t *__restrict__ piv,
@@ -231,13 +234,13 @@ __global__ void __launch_bounds__(kRows * kWarps, 6)
                  double *W21, SliceBuf sb, __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb, int Kp,
                  int64_t lo_off, int pieces) {
     extern __shared__ __align__(16) double xs[];  // [columns][kRows+1]
-    solve_tile<RT>(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, W21, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
+    solve_tile<RT, kPlain>(ps, A, n, p, lda, perm, piv, Dinv, *nelim_p, W21, sb, Wb, Lb, Kp, 0, lo_off, pieces, blockIdx.x, xs);
 }
 
 // Batched: CTA b takes work item b = (front, RT-row tile of its A21): the
 // front is item_front[b], the tile item_tile[b].
-template <int RT>
-__global__ void __launch_bounds__(kRows * kWarps, 6)
+template <int RT, bool kPlain>
+__global__ void __launch_bounds__(kRows * kWarps, kPlain ? 6 : 5)
     k_solve_batch(int mode, const ctp_front *__restrict__ fronts, const BFront *__restrict__ tab, char *ws,
                   const int *__restrict__ item_front, const int *__restrict__ item_tile, BatchOpts o,
                   __nv_bfloat16 *__restrict__ Wb, __nv_bfloat16 *__restrict__ Lb) {
@@ -245,23 +248,19 @@ __global__ void __launch_bounds__(kRows * kWarps, 6)
     const int f = item_front[blockIdx.x];
     const ctp_front fr = fronts[f];
     const BFront bt = tab[f];
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    const BSection sec = bsection(bt.n, bt.p, &oo);
+    const BSection sec = bsection(bt.n, bt.p, o);
     char *base = ws + bt.ws;
     SliceBuf sb = {};
     double *W21 = nullptr;
     if (o.smode != CTP_S_NONE && o.prec == CTP_FP64) {
-        if (form_small(bt.m))
+        if (kPlain || form_small(bt.m))
             W21 = reinterpret_cast<double *>(base + sec.W21);
         else
             sb = bsection_slices(base, sec, bt.p);
     }
     SolvePass ps = {mode, mode == kTail ? 1 : 0, {}};
     if (mode == kFirst) ps.yb = bsection_block(base, sec);
-    solve_tile<RT>(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
+    solve_tile<RT, kPlain>(ps, fr.A, bt.n, bt.p, fr.lda, fr.perm, fr.piv, reinterpret_cast<const double *>(base + sec.Dinv),
                *fr.nelim, W21, sb, Wb, Lb, kBatchKp, bt.row0, o.lo_off, o.pieces,
                item_tile[blockIdx.x], xs);
 }
@@ -361,12 +360,8 @@ __global__ void __launch_bounds__(kRows * kWarps, 6)
     const int f = list[blockIdx.x];
     const ctp_front fr = fronts[f];
     const BFront bt = tab[f];
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    if (bt.m == 0) return;  // no rows to solve for, and no room for slices in its section
-    const BSection sec = bsection(bt.n, bt.p, &oo);
+    if (!front_blocked(bt.m, bt.p, o)) return;  // no room for slices in its section
+    const BSection sec = bsection(bt.n, bt.p, o);
     char *base = ws + bt.ws;
     l11_tile(fr.A, fr.lda, bt.p, 0, (blockIdx.y + 1) * kRows, fr.piv,
              reinterpret_cast<const double *>(base + sec.Dinv), *fr.nelim, bsection_block(base, sec));
@@ -422,15 +417,18 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
     if (m <= 0) return cudaSuccess;
     const size_t smem_p = sizeof(double) * (size_t)p * (kRows + 1);
     const int rt = solve_rows((m + kRows - 1) / kRows, blocks > 0, num_sms);
-    const void *fn = rt == kRows       ? (const void *)k_solve_fp64<kRows>
-                     : rt == kRows / 2 ? (const void *)k_solve_fp64<kRows / 2>
-                                       : (const void *)k_solve_fp64<kRows / 4>;
-    cudaError_t err = smem_at_least(fn, smem_p);
+    const bool plain = blocks == 0 && sb.W == nullptr;
+    auto *k = plain ? (rt == kRows       ? k_solve_fp64<kRows, true>
+                       : rt == kRows / 2 ? k_solve_fp64<kRows / 2, true>
+                                         : k_solve_fp64<kRows / 4, true>)
+                    : (rt == kRows       ? k_solve_fp64<kRows, false>
+                       : rt == kRows / 2 ? k_solve_fp64<kRows / 2, false>
+                                         : k_solve_fp64<kRows / 4, false>);
+    cudaError_t err = smem_at_least((const void *)k, smem_p);
     if (err != cudaSuccess) return err;
     const unsigned grid = (unsigned)((m + rt - 1) / rt);
     auto pass = [&](int mode, int b, int cols) {
         const SolvePass ps = {mode, b, blk};
-        auto *k = rt == kRows ? k_solve_fp64<kRows> : rt == kRows / 2 ? k_solve_fp64<kRows / 2> : k_solve_fp64<kRows / 4>;
         k<<<grid, kRows * kWarps, sizeof(double) * (size_t)cols * (kRows + 1), st>>>(
             ps, A, n, p, lda, perm, piv, Dinv, nelim, W21, sb, (__nv_bfloat16 *)Wb, (__nv_bfloat16 *)Lb, Kp, lo_off, pieces);
         return cudaGetLastError();
@@ -471,16 +469,22 @@ cudaError_t launch_solve_fp64(double *A, int64_t n, int p, int64_t lda, const in
     return pass(kTail, blocks, p);
 }
 
-static decltype(&k_solve_batch<kRows>) solve_batch_kernel(int rows) {
-    return rows == kRows ? k_solve_batch<kRows> : rows == kRows / 2 ? k_solve_batch<kRows / 2> : k_solve_batch<kRows / 4>;
+static decltype(&k_solve_batch<kRows, false>) solve_batch_kernel(int rows, bool plain) {
+    if (plain)
+        return rows == kRows       ? k_solve_batch<kRows, true>
+               : rows == kRows / 2 ? k_solve_batch<kRows / 2, true>
+                                   : k_solve_batch<kRows / 4, true>;
+    return rows == kRows       ? k_solve_batch<kRows, false>
+           : rows == kRows / 2 ? k_solve_batch<kRows / 2, false>
+                               : k_solve_batch<kRows / 4, false>;
 }
 
 cudaError_t launch_solve_batch(const ctp_front *fronts, const BFront *tab, char *ws,
-                               const int *item_front, int64_t items, int rows, BatchOpts o, void *Wb, void *Lb,
+                               const int *item_front, int64_t items, int rows, bool plain, BatchOpts o, void *Wb, void *Lb,
                                int pmax, cudaStream_t st, const int *item_tile) {
     if (items == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (size_t)pmax * (kRows + 1);
-    auto *k = solve_batch_kernel(rows);
+    auto *k = solve_batch_kernel(rows, plain);
     cudaError_t err = smem_at_least((const void *)k, smem);
     if (err != cudaSuccess) return err;
     k<<<(unsigned)items, kRows * kWarps, smem, st>>>(
@@ -495,7 +499,7 @@ cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *ta
                                        cudaStream_t st) {
     if (items == 0) return cudaSuccess;
     const size_t smem = sizeof(double) * (size_t)pmax * (kRows + 1);
-    auto *k = solve_batch_kernel(rows);
+    auto *k = solve_batch_kernel(rows, false);
     cudaError_t err = smem_at_least((const void *)k, smem);
     if (err != cudaSuccess) return err;
     if (pmax > kSliceK) {

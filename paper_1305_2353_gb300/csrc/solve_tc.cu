@@ -339,11 +339,7 @@ __global__ void __launch_bounds__(256)
     const BFront b = tab[f];
     const ctp_front fr = fronts[f];
     if (b.m <= 0) return;
-    ctp_options oo;
-    oo.pivot = o.pivot;
-    oo.smode = o.smode;
-    oo.prec = o.prec;
-    const double *Dinv = reinterpret_cast<const double *>(ws + b.ws + bsection(b.n, b.p, &oo).Dinv);
+    const double *Dinv = reinterpret_cast<const double *>(ws + b.ws + bsection(b.n, b.p, o).Dinv);
     const int p = b.p, e = *fr.nelim;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int d = p - e, E = (e + 31) & ~31;
