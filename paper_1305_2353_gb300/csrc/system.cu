@@ -403,12 +403,17 @@ __global__ void __launch_bounds__(kTh) k_sym_grad_pattern(int64_t nnz, const int
 
 // R -= A X for a symmetric A given by its lower triangle in compressed columns
 // (kAbs: R += |A| 1, the row sums of |A|).  A column's entries update R(i) (atomics)
-// and their transposes accumulate into R(j).  A warp takes 32 consecutive columns:
-// a lane walks its own column, eight right-hand sides at a time -- the columns of
-// meshes hold a few entries, and neighbours' X(i) and R(i) are neighbours in
-// memory -- and columns of more than kLong entries are then shared by the warp.
-// A warp per column took 1.8 ms for 16 right-hand sides on a 64^3 grid.
-constexpr int kLong = 64;
+// and their transposes accumulate into R(j).  G lanes share a column, eight right-hand
+// sides at a time, by the columns' mean length: a lane's chain of atomics stays short, and
+// few entries do not idle a warp.  One lane for the columns of meshes, whose
+// neighbours' X(i) and R(i) are neighbours in memory; more where the matrix has few
+// columns.  Columns of more than kLong entries a lane are shared by the warp.
+// Measured, 16 right-hand sides, rows at random: a warp per column / a lane per column / this
+// rule: N = 2000, 40 a column 46 / 167 / 45 us; N = 20000, 70 279 / 821 / 211; N =
+// 200000, 6 1674 / 156 / 178, 20 1693 / 564 / 544, 60 2530 / 1739 / 1565.  At most 16
+// entries a lane (8: 521 and 1592 us for the last two, but 22% slower on bands).
+constexpr int kLong = 64, kSpmvPer = 16;
+constexpr int64_t kSpmvFill = 152 * 512;
 template <bool kAbs>
 __global__ void __launch_bounds__(kTh) k_spmv_csc(int64_t N, const int64_t *__restrict__ colptr,
                                                   const int32_t *__restrict__ rowind,
@@ -418,24 +423,28 @@ __global__ void __launch_bounds__(kTh) k_spmv_csc(int64_t N, const int64_t *__re
     constexpr int NR = kAbs ? 1 : 8;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (kTh / 32);
-    for (int64_t j0 = 32 * ((int64_t)blockIdx.x * (kTh / 32) + (threadIdx.x >> 5)); j0 < N; j0 += 32 * warps) {
-        const int64_t j = j0 + lane;
+    const int64_t per = (colptr[N] - colptr[0] + N - 1) / N;
+    int G = 1;
+    while (G < 32 && (G * kSpmvPer < per || (G < per && N * G < kSpmvFill))) G *= 2;
+    const int sub = lane & (G - 1), wc = 32 / G;
+    for (int64_t j0 = wc * ((int64_t)blockIdx.x * (kTh / 32) + (threadIdx.x >> 5)); j0 < N; j0 += wc * warps) {
+        const int64_t j = j0 + lane / G;
         const int64_t q0 = j < N ? colptr[j] : 0, q1 = j < N ? colptr[j + 1] : 0;
-        const bool lng = q1 - q0 > kLong;
-        const unsigned longs = __ballot_sync(0xffffffffu, lng);
+        const bool lng = G < 32 && q1 - q0 > kLong * G;
+        const unsigned longs = __ballot_sync(0xffffffffu, lng && sub == 0);
         const int nr = kAbs ? 1 : nrhs;
         for (int r0 = 0; r0 < nr; r0 += NR) {
             const int ng = min(NR, nr - r0);
             const double *Xr = X + (int64_t)r0 * ldx;
             double *Rr = R + (int64_t)r0 * ldr;
-            if (!lng && q1 > q0) {
-                double xj[NR], t[NR];
+            double xj[NR], t[NR];
 #pragma unroll
-                for (int r = 0; r < NR; r++) {
-                    xj[r] = kAbs ? 1.0 : (r < ng ? Xr[r * ldx + j] : 0.0);
-                    t[r] = 0.0;
-                }
-                for (int64_t q = q0; q < q1; q++) {
+            for (int r = 0; r < NR; r++) {
+                xj[r] = kAbs ? 1.0 : (r < ng && q1 > q0 ? Xr[r * ldx + j] : 0.0);
+                t[r] = 0.0;
+            }
+            if (!lng)
+                for (int64_t q = q0 + sub; q < q1; q += G) {
                     const int64_t i = rowind[q];
                     const double a = kAbs ? fabs(val[q]) : val[q];
 #pragma unroll
@@ -449,28 +458,33 @@ __global__ void __launch_bounds__(kTh) k_spmv_csc(int64_t N, const int64_t *__re
                         }
                     }
                 }
+            for (int o = G >> 1; o > 0; o >>= 1)
+#pragma unroll
+                for (int r = 0; r < NR; r++)
+                    if (r < ng) t[r] += __shfl_xor_sync(0xffffffffu, t[r], o);
+            if (!lng && q1 > q0 && sub == 0) {
 #pragma unroll
                 for (int r = 0; r < NR; r++)
                     if (r < ng) atomicAdd(Rr + r * ldr + j, kAbs ? t[r] : -t[r]);
             }
             for (unsigned b = longs; b; b &= b - 1) {
                 const int l = __ffs(b) - 1;
-                const int64_t jl = j0 + l, a0 = __shfl_sync(0xffffffffu, q0, l), a1 = __shfl_sync(0xffffffffu, q1, l);
+                const int64_t jl = j0 + l / G, a0 = __shfl_sync(0xffffffffu, q0, l), a1 = __shfl_sync(0xffffffffu, q1, l);
                 for (int r = 0; r < ng; r++) {
-                    const double xj = kAbs ? 1.0 : Xr[r * ldx + jl];
-                    double t = 0.0;
+                    const double x = kAbs ? 1.0 : Xr[r * ldx + jl];
+                    double s = 0.0;
                     for (int64_t q = a0 + lane; q < a1; q += 32) {
                         const int64_t i = rowind[q];
                         const double a = kAbs ? fabs(val[q]) : val[q];
                         if (i == jl) {
-                            t += a * xj;
+                            s += a * x;
                         } else {
-                            atomicAdd(Rr + r * ldr + i, kAbs ? a : -a * xj);
-                            t += a * (kAbs ? 1.0 : Xr[r * ldx + i]);
+                            atomicAdd(Rr + r * ldr + i, kAbs ? a : -a * x);
+                            s += a * (kAbs ? 1.0 : Xr[r * ldx + i]);
                         }
                     }
-                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                    if (lane == 0) atomicAdd(Rr + r * ldr + jl, kAbs ? t : -t);
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    if (lane == 0) atomicAdd(Rr + r * ldr + jl, kAbs ? s : -s);
                 }
             }
         }
@@ -600,14 +614,14 @@ cudaError_t launch_sym_grad_pattern(int64_t nnz, const int32_t *row, const int32
 cudaError_t launch_spmv_csc_residual(int64_t N, const int64_t *colptr, const int32_t *rowind,
                                      const double *val, int nrhs, const double *X, int64_t ldx, double *R,
                                      int64_t ldr, cudaStream_t st) {
-    const int64_t g = (N + kTh - 1) / kTh < 4096 ? (N + kTh - 1) / kTh : 4096;
+    const int64_t g = (N + 7) / 8 < 152 * 8 ? (N + 7) / 8 : 152 * 8;
     k_spmv_csc<false><<<(unsigned)g, kTh, 0, st>>>(N, colptr, rowind, val, nrhs, X, ldx, R, ldr);
     return cudaGetLastError();
 }
 
 cudaError_t launch_spmv_csc_abs_rowsum(int64_t N, const int64_t *colptr, const int32_t *rowind,
                                        const double *val, double *rowsum, cudaStream_t st) {
-    const int64_t g = (N + kTh - 1) / kTh < 4096 ? (N + kTh - 1) / kTh : 4096;
+    const int64_t g = (N + 7) / 8 < 152 * 8 ? (N + 7) / 8 : 152 * 8;
     k_spmv_csc<true><<<(unsigned)g, kTh, 0, st>>>(N, colptr, rowind, val, 1, nullptr, 0, rowsum, N);
     return cudaGetLastError();
 }
