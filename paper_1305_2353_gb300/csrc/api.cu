@@ -4,6 +4,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "chain.cuh"
@@ -119,7 +120,7 @@ ctp_status ctp_create(ctp_ctx **ctx, int32_t device) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return CTP_ECUDA;
-    ctp_ctx *c = (ctp_ctx *)malloc(sizeof(ctp_ctx));
+    ctp_ctx *c = new (std::nothrow) ctp_ctx();
     if (c == nullptr) return CTP_ENOMEM;
     c->device = device;
     c->num_sms = sms;
@@ -148,7 +149,7 @@ ctp_status ctp_destroy(ctp_ctx *ctx) {
         cudaStreamDestroy(s.main);
         cudaEventDestroy(s.fork_ev);
     }
-    free(ctx);
+    delete ctx;
     return CTP_OK;
 }
 
@@ -453,10 +454,6 @@ ctp_status ctp_profile_end(ctp_ctx *ctx, int32_t max_kernels, char *names, doubl
     return CTP_OK;
 }
 
-// Held while work is enqueued through a context's side streams: their events are
-// recorded and waited for in pairs, which calls from several threads must not mix.
-static std::mutex side_mutex;
-
 // The context's side streams, made on first use outside a stream capture
 // (false: run on st alone).  They belong to the context's device: when another
 // device is current the batch does not fork (the caller's stream is on the
@@ -496,7 +493,7 @@ static bool side_streams(ctp_ctx *ctx, cudaStream_t st, int set) {
 namespace ctp {
 
 bool second_stream(ctp_ctx *ctx, cudaStream_t st, cudaStream_t *out) {
-    std::lock_guard<std::mutex> lock(side_mutex);
+    std::lock_guard<std::mutex> lock(ctx->side_mutex);
     if (ctx->profiling || !side_streams(ctx, st, 1)) return false;
     ctp_ctx::SideSet &s = ctx->sides[1];
     if (cudaEventRecord(s.fork_ev, st) != cudaSuccess || cudaStreamWaitEvent(s.main, s.fork_ev, 0) != cudaSuccess) {
@@ -514,7 +511,7 @@ ctp_status factor_batch_on(ctp_ctx *ctx, const ctp_plan *plan, const ctp_front *
     CTP_CUDA(timed(ctx, K_B_PREPARE, st, [&] { return batch_prepare(plan, w, st); }));
     CTP_CUDA(timed(ctx, K_B_COMPRESS, st, [&] { return batch_compress(plan, fronts, w, ctx->num_sms, st); }));
     const int ncls = batch_num_classes(plan);
-    std::unique_lock<std::mutex> lock(side_mutex, std::defer_lock);
+    std::unique_lock<std::mutex> lock(ctx->side_mutex, std::defer_lock);
     if (!ctx->profiling && ncls > 1) lock.lock();
     if (!ctx->profiling && ncls > 1 && side_streams(ctx, st, set)) {
         ctp_ctx::SideSet &sd = ctx->sides[set];

@@ -2,6 +2,8 @@
 // the translation units that implement the C ABI.
 #pragma once
 
+#include <mutex>
+
 #include "ctp_internal.cuh"
 
 namespace ctp {
@@ -37,6 +39,9 @@ struct ctp_ctx {
         cudaEvent_t fork_ev, join_ev[ctp::kSideStreams];
         bool made;
     } sides[2];
+    // Held while work is enqueued through them: their events are recorded and waited for in
+    // pairs, which calls from several threads on one context must not mix.
+    std::mutex side_mutex;
 };
 
 namespace ctp {
