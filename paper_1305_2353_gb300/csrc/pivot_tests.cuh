@@ -5,6 +5,7 @@
 #pragma once
 
 #include "ctp_internal.cuh"
+#include "division.cuh"
 
 namespace ctp {
 
@@ -119,23 +120,6 @@ __device__ __forceinline__ int test_1x1_f32(unsigned long long kmm, unsigned lon
 // smallest binade; the rare others take the FP64 product.
 __device__ __forceinline__ unsigned long long half_key(unsigned long long k) {
     return (k >> 52) > 1 ? k - (1ull << 52) : akey(0.5 * key_val(k));
-}
-
-// x / d correctly rounded, given y = RN(1/d): two steps of Markstein's division
-// ("Computation of elementary functions on the IBM RISC System/6000 processor",
-// IBM J. Res. Dev. 34, 1990: with y the correctly rounded reciprocal, q within
-// one unit of x/d and the residual r = x - q d exact, RN(q + r y) is x/d
-// correctly rounded); the first step brings q within a unit.  Five FP64-pipe
-// instructions against the division's eight, where exponents leave room;
-// elsewhere the division.
-__device__ __forceinline__ double div_by(double x, double d, double y) {
-    const unsigned ex = (unsigned)(akey(x) >> 52), ed = (unsigned)(akey(d) >> 52);
-    const bool zero = !nonzero_bits(x);
-    if ((ex - 400u > 1246u && !zero) || ed - 723u > 600u) return __ddiv_rn(x, d);
-    const double q0 = __dmul_rn(x, y);
-    const double q1 = __fma_rn(__fma_rn(-q0, d, x), y, q0);
-    const double q2 = __fma_rn(__fma_rn(-q1, d, x), y, q1);
-    return zero ? q0 : q2;
 }
 
 // Listing 1's test_2x2 with the nonsingularity/cancellation guard and the growth
