@@ -467,7 +467,7 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             for (int i = tid; i < p; i += kT) {
                 const int np = sh.lpos[i] - (cstar < i ? 1 : 0);
                 sh.lpos[i] = (unsigned short)np;
-                if (sh.live[i] && i != cstar) sh.lrow[np] = (unsigned short)i;
+                if (i != cstar && sh.live[i]) sh.lrow[np] = (unsigned short)i;
             }
             if (tid == 0) {
                 sh.nlive--;
@@ -501,7 +501,8 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
         {
             // copies of the pivot column(s), every row's multipliers, and the
             // bookkeeping of the pivot, in one phase (the pivot columns are not
-            // written in this round; live[] is read nowhere in this phase)
+            // written in this round; live[q0] and live[q1], cleared in this phase, are
+            // not read in it)
             // multipliers are stored with the sign of their term (-l on normal
             // rows, +l on abs rows) and the A11 pivot entries also as |.|, so
             // that the update loop needs no FP64 sign or abs operation
@@ -509,14 +510,14 @@ __device__ __forceinline__ void factor_body(const FactorArgs &a, int G) {
             const double *s1 = q1 >= 0 ? colptr(q1) : s0;
             const double ad0 = abs_bits(dv.d0), ai0 = abs_bits(dv.i0), ai1 = abs_bits(dv.i1), ai2 = abs_bits(dv.i2);
             for (int i = tid; i < LD; i += kT) {
-                if (i < p && !sh.live[i]) continue;  // rows of earlier pivots take no part any more
+                if (i < p && i != q0 && i != q1 && !sh.live[i]) continue;  // rows of earlier pivots take no part any more
                 if (i < p) {
                     // the live-row list without the pivot rows: the rank of a
                     // row drops by the pivots above it (the pivots' own flags
                     // are cleared in this phase, so they are named explicitly)
                     const int np = sh.lpos[i] - (q0 < i ? 1 : 0) - (q1 >= 0 && q1 < i ? 1 : 0);
                     sh.lpos[i] = (unsigned short)np;
-                    if (sh.live[i] && i != q0 && i != q1) sh.lrow[np] = (unsigned short)i;
+                    if (i != q0 && i != q1) sh.lrow[np] = (unsigned short)i;
                 }
                 const double x = s0[i];
                 pc0[i] = x;
