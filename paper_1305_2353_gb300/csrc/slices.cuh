@@ -78,12 +78,14 @@ __device__ __forceinline__ int slice_exp(double x, int sh) {
 }
 
 // The 62-bit integer nearest x 2^sh 2^(62-E), plus 0x80 in every byte: byte s
-// (from the top) minus 128 is then the balanced digit d_s.
-__device__ __forceinline__ unsigned long long slice_digits(double x, int sh, int E) {
+// (from the top) minus 128 is then the balanced digit d_s.  low: a lower bound of
+// |x| 2^(sh - E) < 1 as FP16 bits, 0 below 2^-14.
+__device__ __forceinline__ unsigned long long slice_digits(double x, int sh, int E, unsigned &low) {
     const int e = biased_exp(x);
     const unsigned long long f = (unsigned long long)__double_as_longlong(x) & 0xFFFFFFFFFFFFFull;
     const unsigned long long t = (e ? (f | 0x10000000000000ull) : f) << 9;  // 62 bits, value t 2^(max(e,1)-1084)
     const int q = E - ((e ? e : 1) - 1022 + sh);                            // >= 0 but for subnormals
+    low = e && q <= 13 ? (unsigned)(14 - q) << 10 | ((hi_word(x) >> 10) & 0x3FFu) : 0u;
     unsigned long long X;
     if (q <= 0)
         X = t << (-q & 63);
@@ -101,12 +103,6 @@ __device__ __forceinline__ uint32_t slice_pair(unsigned long long y0, unsigned l
     const float f0 = __uint_as_float(__byte_perm(w0, 0x4B000000u, sel)) - 8388736.0f;
     const float f1 = __uint_as_float(__byte_perm(w1, 0x4B000000u, sel)) - 8388736.0f;
     return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-}
-
-// A lower bound of |x| 2^(sh - E) < 1 as FP16 bits, 0 below 2^-14.
-__device__ __forceinline__ unsigned slice_low(double x, int sh, int E) {
-    const int h = slice_exp(x, sh) - E + 14;  // its exponent field (subnormal x: far below)
-    return h >= 1 ? (unsigned)(h << 10) | ((hi_word(x) >> 10) & 0x3FFu) : 0u;
 }
 
 // The slices of a tile of 32 rows, by a CTA of kWarps warps: columns k < e of the
@@ -155,9 +151,9 @@ __device__ __forceinline__ void write_slices(const double *xs, int e, int64_t ro
             y[j] = 0x8080808080808080ull;
             if (in && Er < kExpNonfinite) {
                 const double x = xs[(k0 + j) * LDX + r];
-                y[j] = slice_digits(x, sgn * cexp[k0 + j], Er);
-                h = Er > kExpZero ? slice_low(x, sgn * cexp[k0 + j], Er) : 0x3C00u;  // a zero row lowers nothing
-                some |= (x != 0.0 ? 1u : 0u) << j;
+                y[j] = slice_digits(x, sgn * cexp[k0 + j], Er, h);
+                if (Er == kExpZero) h = 0x3C00u;  // a zero row lowers nothing
+                some |= (((unsigned long long)__double_as_longlong(x) << 1) != 0ull ? 1u : 0u) << j;
             } else if (in) {
                 h = 0x3C00u;  // nor does one with an Inf or NaN, whose entries are known by its exponent
             }
