@@ -205,8 +205,9 @@ struct Walk {
             x.S = const_cast<double *>(x.L21 + (int64_t)w.c0 * x.ldl);
             x.lds = x.ldl;
             const int nN = (x.nc + kBN - 1) / kBN;
-            x.ti = x.e > 0 ? (int)(q / nN) : -1;  // nothing eliminated in the block: nothing to do
-            x.tj = (int)(q % nN);
+            const unsigned r = (unsigned)q / (unsigned)nN;  // (fewer than 2^31 tiles)
+            x.ti = x.e > 0 ? (int)r : -1;  // nothing eliminated in the block: nothing to do
+            x.tj = (int)((unsigned)q - r * (unsigned)nN);
         } else if (w.fronts != nullptr) {
             // row block i has 2 (i + 1) tiles, i (i + 1) precede it
             int64_t i = (int64_t)((sqrtf(4.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
@@ -269,10 +270,12 @@ __device__ __noinline__ double to_fp64_any(long long V, int ex) {
 // (their results are then zero).  Rounded in FP16: a part in 2^11 per term of up to 128
 // per sum.  From the last pivot on, where growth puts the large entries, and no
 // further than needed: random data stop after the first block, which matters to the
-// traffic from L2 (all blocks: 3% at e = 256).
+// traffic from L2 (all blocks: 3% at e = 256).  From 24 pivots on, eight rows at a time are
+// tried first, a quarter of the products: the checker shares its issue slots with a
+// quarter of the epilogue.
 constexpr float kSure = 0x1p-7f;
 template <typename F>
-__device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, int gw, int gl, F &&fetch) {
+__device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, int gw, int gl, bool in, F &&fetch) {
     const int lane = threadIdx.x & 31;
     const uint4 *pa = reinterpret_cast<const uint4 *>(grp) + 4 * (lane >> 2);
     const uint4 *pb = reinterpret_cast<const uint4 *>(grp + kWGroup) + 4 * (lane & 3);
@@ -282,9 +285,49 @@ __device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, int
     for (int j = 0; j < 16; j++) s[j] = __floats2half2_rn(0.0f, 0.0f);
     unsigned bad = 0xFFFFu;
     const int KB = (e + kSliceK - 1) / kSliceK;
+    bool here = false;  // the last K block is in shared memory
+    if (e >= 24) {
+        const int kb = KB - 1, chunks = min(4, (e - kb * kSliceK + 7) / 8);
+        fetch(kb);
+        here = true;
+        __half2 c[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) c[j] = __floats2half2_rn(0.0f, 0.0f);
+#pragma unroll 1
+        for (int k = 0; k < chunks; k++) {
+            uint4 u[2], v[2];
+            auto least = [](const uint4 &x, const uint4 &y) {  // FP16 pairs of magnitudes, -0 below them
+                return make_uint4(__vminu2(x.x & 0x7FFF7FFFu, y.x & 0x7FFF7FFFu), __vminu2(x.y & 0x7FFF7FFFu, y.y & 0x7FFF7FFFu),
+                                  __vminu2(x.z & 0x7FFF7FFFu, y.z & 0x7FFF7FFFu), __vminu2(x.w & 0x7FFF7FFFu, y.w & 0x7FFF7FFFu));
+            };
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                u[i] = least(pa[k * gw + 2 * i], pa[k * gw + 2 * i + 1]);
+                v[i] = least(pb[k * gl + 2 * i], pb[k * gl + 2 * i + 1]);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int j = 0; j < 2; j++) {
+                    __half2 &t = c[2 * i + j];
+                    t = __hfma2(h2(u[i].x), h2(v[j].x), t);
+                    t = __hfma2(h2(u[i].y), h2(v[j].y), t);
+                    t = __hfma2(h2(u[i].z), h2(v[j].z), t);
+                    t = __hfma2(h2(u[i].w), h2(v[j].w), t);
+                }
+        }
+        // (rows and columns past the result hold anything: their lanes decide nothing)
+        bool all = true;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const float2 t = __half22float2(c[j]);
+            all = all && t.x + t.y >= kSure;
+        }
+        if (__all_sync(0xffffffffu, all || !in)) return 0u;
+    }
 #pragma unroll 1
     for (int kb = KB - 1; kb >= 0 && __any_sync(0xffffffffu, bad); kb--) {
-        fetch(kb);
+        if (!here || kb < KB - 1) fetch(kb);
         const int chunks = min(4, (e - kb * kSliceK + 7) / 8);
 #pragma unroll 1
         for (int c = 0; c < chunks; c++) {
@@ -304,12 +347,13 @@ __device__ __forceinline__ unsigned unsure_blocks(const uint8_t *grp, int e, int
                 }
             }
         }
-        bad = 0u;
+        bad = 0u;  // (two sums at a time; a NaN compares as false)
+        const __half2 sure = __float2half2_rn(kSure);
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-            const float2 t = __half22float2(s[j]);
-            if (!(t.x + t.y >= kSure)) bad |= 1u << j;
-        }
+        for (int j = 0; j < 16; j += 2)
+            bad |= ~__hge2_mask(__hadd2(__lows2half2(s[j], s[j + 1]), __highs2half2(s[j], s[j + 1])), sure) &
+                   (1u << j | 1u << (j + 1 + 15));
+        bad = (bad & 0xFFFFu) | bad >> 15;
     }
     if (!__any_sync(0xffffffffu, bad)) return 0u;
     unsigned none[16];  // signs: no pivot in common
@@ -675,7 +719,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                     ok = mbar_wait(&bars.grp_full, grpphase, &never) && ok;
                     grpphase ^= 1u;
                 };
-                bits = unsure_blocks(grp, x.e, gw, gl, fetch);
+                // (a lane whose 16 rows or columns are not all there takes no part in the first test)
+                const bool in = x.ti * kBM + 16 * (lane >> 2) < x.m && x.tj * kBN + 16 * (lane & 3) < x.nc;
+                bits = unsure_blocks(grp, x.e, gw, gl, in, fetch);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
                     break;
@@ -685,14 +731,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                                                 (r0 + 2 < x.m && er.z >= kExpNonfinite) ||
                                                 (r0 + 3 < x.m && er.w >= kExpNonfinite) || ec.x >= kExpNonfinite ||
                                                 (c0 + 1 < x.nc && ec.y >= kExpNonfinite));
+                if (__any_sync(0xffffffffu, bits)) {
 #pragma unroll
-                for (int j = 0; j < 4; j++) {  // rows and columns past the result
-                    if (x.ti * kBM + 16 * (lane >> 2) + 4 * j >= x.m) bits &= ~(0xFu << (4 * j));
-                    if (x.tj * kBN + 16 * (lane & 3) + 4 * j >= x.nc) bits &= ~(0x1111u << j);
+                    for (int j = 0; j < 4; j++) {  // rows and columns past the result
+                        if (x.ti * kBM + 16 * (lane >> 2) + 4 * j >= x.m) bits &= ~(0xFu << (4 * j));
+                        if (x.tj * kBN + 16 * (lane & 3) + 4 * j >= x.nc) bits &= ~(0x1111u << j);
+                    }
+                    // a warp of the epilogue: rows of two of these lanes, bit 4 (row group) + column group
+                    bits <<= 16 * ((lane >> 2) & 1);
+                    bits |= __shfl_xor_sync(0xffffffffu, bits, 4);
                 }
-                // a warp of the epilogue: rows of two of these lanes, bit 4 (row group) + column group
-                bits <<= 16 * ((lane >> 2) & 1);
-                bits |= __shfl_xor_sync(0xffffffffu, bits, 4);
                 linked = __any_sync(0xffffffffu, bits) || nonfinite;
                 if (linked && nlist < kList) {
                     if (lane == 0) bars.list[nlist] = x.t;
