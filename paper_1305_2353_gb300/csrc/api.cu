@@ -83,7 +83,7 @@ WsLayout ws_layout(int64_t n, int p, const ctp_options *opt, int num_sms) {
     L.gx = off;
     off += align256(blocks * slice_g_bytes(p, kSliceK));
     L.marks = off;
-    const int64_t ut = blocks > 0 ? update_tiles(m, p) : 0, ft = form_fp64_slots(ms);
+    const int64_t ut = blocks > 0 ? update_tiles(m, p) : 0, ft = form_fp64_marks(ms);
     off += align256(sizeof(TileMarks) * (size_t)(ut > ft ? ut : ft));
     // BF16 operand copies (hi, and for the split form the lo parts after them)
     const size_t nb = tc ? 2 * (size_t)m * form_tc_kpad(p) * prec_pieces(opt->prec) : 0;

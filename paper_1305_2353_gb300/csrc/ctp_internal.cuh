@@ -68,7 +68,7 @@ struct TileMarks {
 //     gw, gl            lower bounds (slices.cuh) when the FP64 Form step runs
 //   Yb, Lx, ey, ex,     the same of one block's y and of L11 for the blocked FP64 Solve
 //     gy, gx
-//   marks               a TileMarks per tile of the FP64 Form and of the Solve's updates
+//   marks               a TileMarks per tile of a launch of the FP64 Form or of the Solve's updates
 //   Wb, Lb              m*Kp BF16 copies of Y and L21 for the tensor-core Form
 //   aux                 method-specific scratch (relaxed candidate lists)
 struct WsLayout {
@@ -338,7 +338,7 @@ cudaError_t launch_update_batch(const ctp_front *fronts, const BFront *tab, char
                                 const int *item_tile, int64_t items, BatchOpts o, TileMarks *marks, int32_t *info,
                                 int num_sms, cudaStream_t st);
 int64_t update_tiles(int64_t m, int p);  // of a front, for block 0
-int64_t form_fp64_slots(int64_t m);      // of a single supernode's Form
+int64_t form_fp64_marks(int64_t m);      // TileMarks that a single supernode's Form needs
 // a batch class's Solve in one block of 32 columns, its update and the tail
 cudaError_t launch_solve_batch_blocked(const ctp_front *fronts, const BFront *tab, char *ws, const int *list,
                                        int count, const int *item_front, const int *item_tile, int64_t items,

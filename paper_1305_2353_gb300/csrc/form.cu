@@ -130,8 +130,8 @@ struct Work {
     char *ws;
     const int *item_front, *item_tile;
     BatchOpts o;
-    int64_t count;  // items, or slots of the walk
-    TileMarks *marks;  // one per item or slot
+    int64_t first, count;  // the launch's items, or slots of the walk: first .. count - 1
+    TileMarks *marks;      // one for each of them
     int c0;         // kUpdate: first column updated, 32 past the block's first
     int64_t nc;     // kUpdate, one supernode: columns updated
 };
@@ -155,7 +155,7 @@ struct Walk {
     const Work &w;
     int64_t t, panel = 0, before = 0, next;  // one supernode's Form: slots before this panel and the next
     int e = 0;
-    __device__ __forceinline__ explicit Walk(const Work &w_) : w(w_), t(blockIdx.x) {
+    __device__ __forceinline__ explicit Walk(const Work &w_) : w(w_), t(w_.first + blockIdx.x) {
         if (w.fronts == nullptr) e = *w.nelim;
         next = slots_before(1, (w.m + kBM - 1) / kBM);
     }
@@ -499,7 +499,7 @@ __device__ __forceinline__ void fix_few(const Work &wk, Bars &bars, uint8_t *sme
         unsigned mask[kEpiWarps];
         int cnt = 0;
 #pragma unroll
-        for (int b = 0; b < kEpiWarps; b++) mask[b] = wk.marks[t].out[b][lane];
+        for (int b = 0; b < kEpiWarps; b++) mask[b] = wk.marks[t - wk.first].out[b][lane];
 #pragma unroll
         for (int b = 0; b < kEpiWarps; b++) cnt += __popc(mask[b]);
         int pos = cnt;  // inclusive prefix sum
@@ -558,7 +558,7 @@ __device__ __forceinline__ void fix_tile(const Work &wk, Bars &bars, uint8_t *sm
     const Tile &x = bars.tile[0];
     const int lane = threadIdx.x & 31;
     // a thread holds a row's sixteen columns
-    const unsigned mask = threadIdx.x < kBM * kBN / kCols ? wk.marks[t].out[threadIdx.x >> 5][lane] : 0u;
+    const unsigned mask = threadIdx.x < kBM * kBN / kCols ? wk.marks[t - wk.first].out[threadIdx.x >> 5][lane] : 0u;
     if (!__syncthreads_or(mask != 0u)) return;  // its own results served after all
     if (threadIdx.x == 0) {
         Walk<kUpd> walk(wk);
@@ -616,7 +616,8 @@ __device__ __forceinline__ void fix_tile(const Work &wk, Bars &bars, uint8_t *sm
     for (int it = 0; it < kItems; it++) {
         if (threadIdx.x + it * kThreads >= n) break;
         const int i = i0 + row[it];
-        const unsigned mask = wk.marks[t].out[row[it] / 32 * 4 + col[it] / kCols][row[it] % 32] >> (col[it] % kCols);
+        const unsigned mask =
+            wk.marks[t - wk.first].out[row[it] / 32 * 4 + col[it] / kCols][row[it] % 32] >> (col[it] % kCols);
 #pragma unroll
         for (int c = 0; c < 4; c++) {
             const int64_t j = j0 + col[it] + c;
@@ -632,7 +633,7 @@ __device__ __noinline__ void fix_tiles(const Work &wk, Bars &bars, uint8_t *smem
     __syncthreads();
     for (int q = 0; q < bars.nlist; q++)
         if (bars.list[q] >= 0) fix_tile<kMode>(wk, bars, smem, bars.list[q]);
-    for (int64_t t = bars.marked; t >= 0; t = wk.marks[t].prev) fix_tile<kMode>(wk, bars, smem, t);
+    for (int64_t t = bars.marked; t >= 0; t = wk.marks[t - wk.first].prev) fix_tile<kMode>(wk, bars, smem, t);
 }
 
 template <int kMode>
@@ -747,7 +748,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                     if (lane == 0 && nlist < kKept) bars.kept[nlist] = x;
                     nlist++;
                 } else if (linked) {
-                    if (lane == 0) wk.marks[x.t].prev = marked;
+                    if (lane == 0) wk.marks[x.t - wk.first].prev = marked;
                     marked = x.t;
                 }
             }
@@ -989,7 +990,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_form_fp64(const __grid_constant
                 }
             }
             if (linked) {
-                wk.marks[x.t].out[q * 4 + cg][lane] = (uint16_t)weak;
+                wk.marks[x.t - wk.first].out[q * 4 + cg][lane] = (uint16_t)weak;
                 if (weak) bars.weak = 1;
             }
             __syncwarp();
@@ -1120,7 +1121,8 @@ template <int kMode>
 cudaError_t launch_mode(const Work &wk, int32_t *info, int num_sms, cudaStream_t st) {
     cudaError_t err = smem_at_least((const void *)k_form_fp64<kMode>, kSmem);
     if (err != cudaSuccess) return err;
-    const unsigned grid = (unsigned)(wk.count < num_sms ? wk.count : num_sms);
+    const int64_t items = wk.count - wk.first;
+    const unsigned grid = (unsigned)(items < num_sms ? items : num_sms);
     k_form_fp64<kMode><<<grid, kThreads, kSmem, st>>>(wk, info);
     return cudaGetLastError();
 }
@@ -1154,6 +1156,11 @@ cudaError_t launch_any(const Work &wk, int smode, int32_t *info, int num_sms, cu
 
 }  // namespace
 
+// Slots of the walk that one launch takes.  Their marks are 1/64 of S (2.5 GB at n =
+// 200000, p = 256), so larger Forms go in several launches that use the same ones, 273 MB
+// at most (there: ten launches, 233.5 ms; all tiles in one 233.7).
+constexpr int64_t kRoundSlots = 262144;
+
 cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda, const int32_t *piv,
                              const double *D, int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
                              TileMarks *marks, int32_t *info, int num_sms, cudaStream_t st) {
@@ -1168,9 +1175,15 @@ cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda,
     wk.lds = lds;
     wk.nelim = nelim;
     wk.S = S;
-    wk.count = walk_slots(m);
     wk.marks = marks;
-    return launch_any(wk, smode, info, num_sms, st);
+    const int64_t slots = walk_slots(m), rounds = (slots + kRoundSlots - 1) / kRoundSlots;
+    cudaError_t err = cudaSuccess;
+    for (int64_t r = 0; r < rounds && err == cudaSuccess; r++) {
+        wk.first = slots * r / rounds;
+        wk.count = slots * (r + 1) / rounds;
+        err = launch_any(wk, smode, info, num_sms, st);
+    }
+    return err;
 }
 
 cudaError_t launch_form_small(const double *L21, int64_t lda, const double *W21, const int32_t *piv, const double *D,
@@ -1235,7 +1248,10 @@ cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int6
     return launch_any(wk, kUpdate, info, num_sms, st);
 }
 
-int64_t form_fp64_slots(int64_t m) { return m > 0 ? walk_slots(m) : 0; }
+int64_t form_fp64_marks(int64_t m) {
+    const int64_t slots = m > 0 ? walk_slots(m) : 0;
+    return slots < kRoundSlots ? slots : kRoundSlots;
+}
 
 int64_t update_tiles(int64_t m, int p) {
     return p > kSliceK ? (m + kBM - 1) / kBM * ((p - kSliceK + kBN - 1) / kBN) : 0;
