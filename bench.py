@@ -58,9 +58,9 @@ NCU_TRAFFIC = {
     "form_tc_bf16x3": {"file": "form_tc.cu", "sha1": "488eb8cb39a135fe2b96ff90b589d43a008cdf37",
                        "unit": "tiled_entry", "bytes_per_unit": (89.629184e6 + 3118.794e6) / (48516 * 16384)},
     # ncu --set full, n=40000 p=256 relaxed, tensor-core Solve before a split-BF16
-    # Form (prep + gather + GEMM): 145.21 MB read + 122.34 MB written for 39,744 rows
-    "solve_tc": {"file": "solve_tc.cu", "sha1": "e210f4414d4a3177580a3d09e17f9d41b70d04d8", "prec": "bf16x3",
-                 "unit": "row", "bytes_per_unit": (145.21472e6 + 122.337e6) / 39744},
+    # Form (prep + gather + GEMM): 145.23 MB read + 122.33 MB written for 39,744 rows
+    "solve_tc": {"file": "solve_tc.cu", "sha1": "ccb2ef343ae6bb8f30406838d4af597437b6472f", "prec": "bf16x3",
+                 "unit": "row", "bytes_per_unit": (145.233e6 + 122.330e6) / 39744},
     # ncu --set full, n=200000 p=256 strict: 409.64 MB read + 3.59 MB written for
     # 199,744 A21 rows
     "compress_strict": {"file": "compress.cu", "sha1": "64d01d59c6c3d5f92ce7b20d803e44db5ce0659b",

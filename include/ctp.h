@@ -66,7 +66,10 @@ typedef enum {
  * inversions and D11 are always FP64; the Solve is FP64 unless the options ask
  * for the tensor-core Solve (ctp_solve_kind below). */
 typedef enum {
-    CTP_FP64 = 0,  /* FP64 throughout */
+    CTP_FP64 = 0,  /* FP64 throughout.  The Form, and the updates of a large Solve, run as
+                      exact digit slices on the tensor cores where these lose no more than
+                      FP64 multiply-adds may, and as FP64 multiply-adds elsewhere: an entry
+                      of S is off by less than (2 e + 8) 2^-53 (|W21| |L21|^T) */
     CTP_BF16 = 1,  /* Form on the tensor cores: BF16 operands, FP32 accumulation and
                       FP32 S (requires smode CTP_S_FP32, CTP_S_FP32_PACKED,
                       CTP_S_FP32_TILED or CTP_S_FP64_SUB); products carry the
@@ -273,7 +276,11 @@ ctp_status ctp_read_info(ctp_ctx *ctx, const void *workspace, int32_t *info_host
 
 /* ------------------------------------------------------------------------ */
 /* Batched factorization of many independent supernodes (the fronts of an
- * assembly tree), each exactly as ctp_factor_supernode would factor it.
+ * assembly tree), each as ctp_factor_supernode would factor it: the same
+ * compression, pivots and D.  L21, the delayed columns and S may be rounded differently:
+ * whether a front's Solve runs in blocks is decided from its size and from the size of
+ * the other fronts that it is launched with, and the two Solves, equally
+ * accurate, differ in their last bits.  The same plan gives the same bits again.
  *
  * Device-visible descriptor of one front (an array of them lives in device
  * memory); all pointers are device pointers with the meaning they have in
@@ -460,7 +467,9 @@ ctp_status ctp_refine_csc(ctp_ctx *ctx, int32_t nf, const ctp_sfront *fronts, in
  *   on a stream of the context's, ordered behind `stream` and finished when the
  *   call goes on to the next level.
  *   Device memory for the fronts is allocated by the call and held by *mf, as is
- *   pinned host memory for the passes' tables.
+ *   pinned host memory for the passes' tables.  The factors are held a second time, packed
+ *   for ctp_mf_solve in the order in which it reads them (after a tensor-core Form a third
+ *   time, in FP32, for the solves inside the refinement).
  *   The host waits for every pass.
  * ctp_mf_fronts: the factored panels, in elimination order, as fronts for
  *   ctp_solve / ctp_refine_csc (host array valid until the next factor or

@@ -33,12 +33,15 @@
 // The same kernel, kMode kUpdate, is the Solve's update of the later columns of A21
 // with a block of 32 columns: A21(:, c0 + j) -= y L11(c0 + j, block)^T, all rows
 // by all j, one K block.
-// Bound: tensor pipe for e from about 100 on (n = 20000, p = e = 256: 2.31 ms, 1.6
+// Bound: tensor pipe for e from about 100 on (n = 20000, p = e = 256: 2.33 ms, 1.55
 // PFLOP/s of executed products, against 80.6 ms for FP64 multiply-adds at 0.99 of
 // their pipe's rate); below, S traffic and the epilogue's instructions: the
 // update of 224 columns of 200000 rows took 446 us with 144 instructions per entry,
-// 210 with the test-free path, the 32-bit sums of neighbouring groups and the old
-// values brought to L2 ahead (HBM's share: 121 us).
+// 236 with the test-free path, the 32-bit sums of neighbouring groups and the old
+// values brought to L2 ahead (HBM's share: 121 us).  The checker shares its issue slots with
+// a quarter of the epilogue: without it the two take 2.26 ms and 196 us.  Where no two rows are
+// large in a common pivot, nearly all entries go to FP64 multiply-adds (n = 20000, p = 256:
+// 91 ms; 16 with 1% of such rows).
 // Fronts of few rows have a kernel of their own, k_form_small.
 // Every mbarrier wait is bounded; on timeout the kernel records CTP_ETIMEOUT,
 // waits (bounded) for its copies in flight, frees its tensor memory and returns.

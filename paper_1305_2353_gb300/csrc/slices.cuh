@@ -35,8 +35,8 @@
 // taken by FP64 multiply-adds.  (Two blocks of rows, each large in columns where the
 // other is 2^-40 of its scale, lost 26 bits between them while rows were
 // compared within their tile only.)  Random rows pass the first test from about 8 pivots
-// on; of the entries of 36^3 multifrontal fronts one in 40 does not, and one in 1300
-// passes neither.
+// on; of the 4 x 4 blocks of 36^3 multifrontal fronts one in 80 does not, and of their
+// entries one in 1400 passes neither.
 //
 // Layout (what a bulk copy puts into shared memory as the MMA reads it): W in
 // blocks of 128 rows, L in blocks of 64, the last of either as long as its rows, rounded

@@ -68,7 +68,7 @@ __device__ __forceinline__ void write_pieces(__nv_bfloat16 *__restrict__ B, int6
 // What a pass over a tile does.  A whole Solve in one pass updates every later
 // column with every y_j in FP64: p^2/2 multiply-adds per row on a pipe of 2 per
 // clock and SM (n = 200000, p = e = 256: 12.9 ms, 0.8 of that pipe).  The blocked
-// Solve (3.06 ms: 2.0 ms in the diagonal blocks, 0.84 in the updates, the rest moving
+// Solve (3.10 ms: 1.9 ms in the diagonal blocks, 0.95 in the updates, the rest moving
 // and scaling columns) keeps only the 32-column diagonal blocks of
 // that and leaves the rest -- columns times y's block by block -- to the
 // tensor cores, as products of exact digit slices (k_update in form.cu):

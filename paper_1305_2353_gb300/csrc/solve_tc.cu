@@ -125,7 +125,8 @@ constexpr int kPrepT = 128;   // threads: the others help to write the outputs
 // positions behind it per pivot, the columns of L11 loaded four pivots ahead (row k is
 // zero before position k, so its pivots start at k's block).  The CTA then writes the
 // Z^T column of its row.  p = 256: 140 -> 97 us (the row in shared memory, an L2 round
-// trip and all positions' instructions per pivot before).
+// trip and all positions' instructions per pivot before), 108 with the two columns of a 2x2
+// pivot applied as one sum.
 __global__ void __launch_bounds__(kPrepT)
     k_stc_prep(const double *__restrict__ A, int p, int64_t lda, const int32_t *__restrict__ piv,
                const double *__restrict__ Dinv, const int32_t *__restrict__ nelim_p, __nv_bfloat16 *__restrict__ Zt,
@@ -807,7 +808,8 @@ cudaError_t launch_solve_tc(double *A, int64_t n, int p, int64_t lda, const int3
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     // beside the preparation (a chain of pivots that leaves most of the chip idle), by
-    // programmatic dependent launch: n = 40000, p = 256, both: 262 -> 238 us of Solve
+    // programmatic dependent launch: n = 40000, p = 256, both: 262 -> 238 us of Solve,
+    // with pieces from two floats (254 with the integer pieces)
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
