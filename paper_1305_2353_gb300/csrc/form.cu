@@ -1162,7 +1162,7 @@ cudaError_t launch_any(const Work &wk, int smode, int32_t *info, int num_sms, cu
 // Slots of the walk that one launch takes.  Their marks are 1/64 of S (2.5 GB at n =
 // 200000, p = 256), so larger Forms go in several launches that use the same ones, 273 MB
 // at most (there: ten launches, 233.5 ms; all tiles in one 233.7).
-constexpr int64_t kRoundSlots = 262144;
+constexpr int64_t kLaunchSlots = 262144;
 
 cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda, const int32_t *piv,
                              const double *D, int64_t m, const int32_t *nelim, void *S, int64_t lds, int smode,
@@ -1179,11 +1179,11 @@ cudaError_t launch_form_fp64(const SliceBuf &sb, const double *L21, int64_t lda,
     wk.nelim = nelim;
     wk.S = S;
     wk.marks = marks;
-    const int64_t slots = walk_slots(m), rounds = (slots + kRoundSlots - 1) / kRoundSlots;
+    const int64_t slots = walk_slots(m), launches = (slots + kLaunchSlots - 1) / kLaunchSlots;
     cudaError_t err = cudaSuccess;
-    for (int64_t r = 0; r < rounds && err == cudaSuccess; r++) {
-        wk.first = slots * r / rounds;
-        wk.count = slots * (r + 1) / rounds;
+    for (int64_t r = 0; r < launches && err == cudaSuccess; r++) {
+        wk.first = slots * r / launches;
+        wk.count = slots * (r + 1) / launches;
         err = launch_any(wk, smode, info, num_sms, st);
     }
     return err;
@@ -1253,7 +1253,7 @@ cudaError_t launch_update(const SliceBuf &u, double *A, int64_t lda, int p, int6
 
 int64_t form_fp64_marks(int64_t m) {
     const int64_t slots = m > 0 ? walk_slots(m) : 0;
-    return slots < kRoundSlots ? slots : kRoundSlots;
+    return slots < kLaunchSlots ? slots : kLaunchSlots;
 }
 
 int64_t update_tiles(int64_t m, int p) {
